@@ -500,17 +500,20 @@ sadmm_status sadmm_project_groups_noalloc(const sadmm_conv_desc* d, const void* 
                                           int* filt_idx, int* col_idx, double* keys_out,
                                           void* stream);
 
-/* Device bytes of scratch for sadmm_conv_bwd to take the layer's output
- * pixels in chunks of at most 32768 (sized so a chunk's gathered bf16
- * operands and fp32 products stay in L2): the default.  0 on a bad plan. */
+/* Device bytes of scratch for sadmm_conv_bwd's default path.  A stride-1 layer
+ * whose pads are below its kernel extents runs whole on a zero-padded pixel grid
+ * (copies of x and dZ, a partial dW per pixel range); any other layer takes its
+ * output pixels in chunks of at most 32768 (sized so a chunk's gathered bf16
+ * operands and fp32 products stay in L2).  0 on a bad plan. */
 size_t sadmm_conv_bwd_workspace_size(const sadmm_plan* plan);
 
 /* Device bytes of scratch for chunks of `chunk_pixels` output pixels (rounded
  * up to a multiple of 256, at least 256, at most 32768).  sadmm_conv_bwd
- * accepts any workspace at least the size for 256 pixels and takes the pixels
- * in the largest chunks (up to 32768) the workspace holds: a smaller workspace
- * costs more launches and partial-sum passes, not results (the dW and db
- * reductions keep a fixed order for a given chunk size). */
+ * accepts any workspace at least the size for 256 pixels: a workspace that holds
+ * the default path's runs it, a smaller one takes the pixels in the largest
+ * chunks (up to 32768) it holds.  That costs more launches and partial-sum
+ * passes, not results (the dW and db reductions keep a fixed order for a given
+ * workspace size). */
 size_t sadmm_conv_bwd_workspace_size_chunk(const sadmm_plan* plan, long long chunk_pixels);
 
 /*
@@ -522,9 +525,11 @@ size_t sadmm_conv_bwd_workspace_size_chunk(const sadmm_plan* plan, long long chu
  *   db[f]      = sum of dZ over images and pixels for kept f; 0 for pruned f;
  *   dx         = the input gradient through the kept weights only.
  * The contractions run on the tensor cores (bf16 operands, fp32 accumulation);
- * dW and db are summed in a fixed order (deterministic); dx is summed with
- * fp32 atomics (its last bits depend on timing).  For an input-slab plan
- * (plan->xs_mode) with at most 128 kept filters, dW is contracted on the
+ * dW and db are summed in a fixed order (deterministic), and so is dx on the
+ * pixel grid, where a sum spans every kept filter and tap and a pruned entry's
+ * product with an infinity or NaN is left out as everywhere else; the chunked
+ * path sums dx with fp32 atomics (its last bits depend on timing).  There, for
+ * an input-slab plan (plan->xs_mode) with at most 128 kept filters, dW is contracted on the
  * plan's space-to-depth copy of x (rewritten by this call) instead of an
  * im2col copy; its workspace then also holds dZ in the output's block-pixel
  * grid and one fp32 partial dW per CTA.

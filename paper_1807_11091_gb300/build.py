@@ -28,7 +28,7 @@ LIB = os.path.join(BUILD, "libsadmm.so")
 DEBUG_LIB = os.path.join(BUILD, "debug", "libsadmm.so")
 
 SOURCES = ["abi.cu", "project.cu", "pack.cu", "conv_fwd.cu", "conv_slab.cu", "admm.cu", "elements.cu", "gemm.cu",
-           "bwd.cu", "bwd_slab.cu", "sparse.cu"]
+           "bwd.cu", "bwd_slab.cu", "bwd_grid.cu", "conv_grid.cu", "sparse.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -8,7 +8,9 @@
 //   dWp[i][j] = sum_m dZ[m][f_i] * A[m][j]          (weight gradient, kept only)
 //   dA[m][j]  = sum_i dZ[m][f_i] * Wp[i][j]         (then col2im into dx)
 //   db[f_i]   = sum_m dZ[m][f_i]
-// Per conv group and per chunk of output pixels the two contractions run on
+// Stride-1 layers run on the padded pixel grid (bwd_grid.cu) when the workspace
+// holds it.  For the others, and in smaller workspaces, the contractions run per
+// conv group and per chunk of output pixels on
 // the tensor cores (gemm.cu) over bf16 operands gathered here; the weight
 // gradient's few output tiles split each chunk's pixels over many CTAs that
 // add into dWp with fp32 atomics, and dx receives the col2im sums with fp32
@@ -16,6 +18,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "grid.cuh"
 #include "internal.h"
 
 namespace sadmm {
@@ -378,6 +381,10 @@ int pick_bn(long long n)
 
 size_t bwd_workspace_bytes(const sadmm_plan* plan, const Geometry& g, long long chunk)
 {
+    if (chunk <= 0) {
+        const size_t grid = grid_bwd_bytes(plan, g);
+        if (grid > 0) return std::max(grid, layout(geometry(plan, g, 256)).total);
+    }
     return layout(geometry(plan, g, chunk > 0 ? chunk : kBwdMaxChunk)).total;
 }
 
@@ -393,11 +400,17 @@ long long bwd_chunk_for(const sadmm_plan* plan, const Geometry& g, size_t ws_byt
     return 0;
 }
 
+// The grid path wherever the layer has a grid and the workspace holds it: over
+// 20 drawn stride-1 layers (1x1 to 5x5, 3-D, batch 1 to 128, densities 0.1 to 1)
+// it took 0.26 to 0.84 of the gathered path's time, AlexNet conv2 at batch 128
+// 841 -> 196 us, conv3 164 -> 64 us, and none took longer.
 sadmm_status launch_conv_bwd(const sadmm_plan* plan, const Geometry& g, const void* x, const void* dy, const void* y,
                              int ydt, int relu, float* dW, float* db, float* dx, void* ws, size_t ws_bytes,
                              cudaStream_t s)
 {
     if (g.m >= (1ll << 31)) return SADMM_EUNSUPPORTED;  // pixel indices decode in 32 bits
+    const size_t grid = grid_bwd_bytes(plan, g);
+    if (grid > 0 && grid <= ws_bytes) return launch_grid_bwd(plan, g, x, dy, y, ydt, relu, dW, db, dx, ws, s);
     const long long chunk = bwd_chunk_for(plan, g, ws_bytes);
     if (chunk <= 0) return SADMM_EINVAL;
     BwdGeo b = geometry(plan, g, chunk);

@@ -1,0 +1,869 @@
+// bwd_grid.cu -- backward of a packed pruned stride-1 CONV layer for masked
+// retraining (Sec. 4) on the padded pixel grid of grid.cuh: no im2col, no
+// col2im, no atomics.
+//
+//   k_grid_prep    the input gradient's weights (taps flipped, kept filters as
+//                  channels), its output map, dW zeroed
+//   k_grid_dz      dZ = dY * [y > 0] of the kept filters as a grid copy (each
+//                  element read once for dW, dx and db) and db's partial sums
+//   k_grid_x       x as a grid copy (conv_grid.cu)
+//   k_grid_wgrad   dW: for a tap of shift s, dW[f][c] = sum over grid pixels q
+//                  of x[c][q + s] * dZ[f][D0 + q].  Channels are the MMA's M
+//                  side, filters its N side, pixels its K side: both operands
+//                  are the copies themselves, read MN-major (core matrices of 8
+//                  channels x 8 pixels); dZ is zero off the output, so the
+//                  padded pixels add nothing.
+//   k_grid_wreduce the slices of the pixel ranges, in order, into dW's kept
+//                  entries
+//   k_grid_conv    dx: the slab GEMM over dZ (conv_grid.cu), every element
+//                  written once
+//
+// A layer of at most 64 channels fills half of the M side or less: its slab is
+// then staged up to 16 / chunks times, each copy a pixel further on, and one
+// MMA covers that many kernel columns.
+// The tensor core truncates as it accumulates (about 1e-8 of the result per
+// step of 16 pixels), so a slice takes at most kGwMaxTiles tiles of 128.
+//
+// AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5;
+// one cold launch each, against the six im2col / GEMM / col2im chunks before,
+// 841 us in all): dZ 28 us (99 MB moved), x copy 9, weight gradient 72 (57
+// cycles per 128 x 64 x 16 MMA: bound by the operands' shared-memory reads, 96
+// of the 128 rows in use), its reduction 14, input gradient 59 (57 cycles per
+// 128 x 48 x 16).  conv3: 8.5 / 7 / 18 / 10 / 19 us.
+#include <string.h>
+
+#include <algorithm>
+
+#include "grid.cuh"
+
+namespace sadmm {
+namespace {
+
+constexpr int kGwThreads = 10 * 32;
+constexpr int kGwMaxStages = 4;
+constexpr int kGwMaxTiles = 12;      // 128-pixel tiles summed in TMEM: 96 MMA steps
+constexpr long long kGwCtas = 152;   // work items come in multiples of about this many (fixed: it sizes the workspace)
+constexpr int kGwSmemLimit = 232448;
+constexpr int kGwCols = 512;         // accumulator columns
+
+struct WgradShape {
+    int nch;          // 8-channel chunks of x per conv group
+    int blk, mblks;   // chunks per M block, blocks
+    int rep, kwg;     // kernel columns per MMA, groups of them per kernel row
+    int rows;         // M rows in use: rep * blk * 8
+    int nst, nft;     // filters per N tile, tiles
+    int tpg, tgs;     // macro taps per item, items per kernel frame
+    int types;        // items per pixel range
+    int tiles, tps, Z;  // 128-pixel tiles, tiles per range, ranges
+    int spa;          // slots of a staged chunk
+    int stages, a_bytes, stage_stride;
+    size_t smem;
+    long long slice;  // floats of a pixel range's slice
+};
+
+bool wgrad_shape(const Grid& gr, int nck, int n_pad, int groups, WgradShape* out)
+{
+    WgradShape w;
+    if (nck < 1) return false;
+    w.nch = (nck + 7) / 8;
+    w.rep = 1;
+    if (w.nch <= 8) {
+        w.rep = std::min(16 / w.nch, gr.KW);
+        w.mblks = 1;
+    } else {
+        w.mblks = (w.nch + 15) / 16;
+    }
+    w.blk = (w.nch + w.mblks - 1) / w.mblks;
+    w.kwg = (gr.KW + w.rep - 1) / w.rep;
+    w.rows = w.rep * w.blk * 8;
+    w.nft = (n_pad + 255) / 256;
+    w.nst = (int)round_up((n_pad + w.nft - 1) / w.nft, 16);
+    const int macro = gr.KH * w.kwg;
+    w.tpg = std::min(std::min(kGwCols / w.nst, macro), 32);
+    for (;; --w.tpg) {  // fewer taps per item until two stages of their slab fit
+        if (w.tpg < 1) return false;
+        w.tgs = (macro + w.tpg - 1) / w.tpg;
+        int span = 0;
+        for (int t0 = 0; t0 < macro; t0 += w.tpg) {
+            int lo = 1 << 30, hi = 0;
+            for (int t = t0; t < std::min(macro, t0 + w.tpg); ++t) {
+                const int s = (t / w.kwg) * gr.Wb + (t % w.kwg) * w.rep;
+                lo = std::min(lo, s);
+                hi = std::max(hi, s);
+            }
+            span = std::max(span, hi - lo);
+        }
+        w.spa = 128 + span;
+        w.a_bytes = (int)round_up((long long)w.rep * w.blk * w.spa * 16, 128);
+        w.stage_stride = w.a_bytes + w.nst / 8 * 2048;
+        // the MMA reads 16 chunks whatever the rows in use: room past the last stage
+        const long long fixed = 1024 + 512 + (long long)(16 - w.rep * w.blk) * w.spa * 16;
+        w.stages = (int)std::min<long long>(kGwMaxStages, (kGwSmemLimit - fixed) / w.stage_stride);
+        w.smem = (size_t)(fixed + (long long)w.stages * w.stage_stride);
+        if (w.spa < (1 << 14) && w.stages >= 2 && (w.stages >= 3 || w.tpg == 1)) break;
+    }
+    const long long types = (long long)groups * w.nft * w.mblks * gr.KT * w.tgs;
+    w.tiles = (gr.L + 127) / 128;
+    const long long work = types * w.tiles;
+    const long long waves = std::max<long long>(1, (work + kGwCtas * kGwMaxTiles - 1) / (kGwCtas * kGwMaxTiles));
+    w.tps = (int)std::max<long long>(1, std::min<long long>(kGwMaxTiles, (work + kGwCtas * waves - 1) / (kGwCtas * waves)));
+    w.Z = (w.tiles + w.tps - 1) / w.tps;
+    if (types * w.Z >= (1ll << 30)) return false;
+    w.types = (int)types;
+    w.slice = types * w.rows * w.tpg * w.nst;
+    *out = w;
+    return true;
+}
+
+struct GwArgs {
+    Grid gr;
+    WgradShape w;
+    const __nv_bfloat16* xs;
+    const __nv_bfloat16* dz;
+    long long xs_gstride, dz_gstride;
+    const int* counts;
+    const int* colidx;  // kept columns, ascending (NULL: every column of the kept channels)
+    int nck, n_cols, taps;
+    float* slices;
+    int groups, units;
+    FastDiv types_div;
+    int* status;
+};
+
+// One work item: pixel range z and (group, filter tile, channel block, kernel
+// frame, tap group).
+struct GwItem {
+    int z, type, g, ft, mb, kt, t0, nt, nr, base, span;
+};
+SADMM_DEV GwItem gw_item(const GwArgs& a, int u)
+{
+    GwItem it;
+    it.z = (int)fdiv((uint32_t)u, a.types_div);
+    it.type = u - it.z * a.w.types;
+    int r = it.type;
+    const int tg = r % a.w.tgs;
+    r /= a.w.tgs;
+    it.kt = r % a.gr.KT;
+    r /= a.gr.KT;
+    it.mb = r % a.w.mblks;
+    r /= a.w.mblks;
+    it.ft = r % a.w.nft;
+    it.g = r / a.w.nft;
+    it.t0 = tg * a.w.tpg;
+    it.nt = min(a.w.tpg, a.gr.KH * a.w.kwg - it.t0);
+    const int cnt = min(a.w.nst, __ldg(a.counts + 2 * it.g) - it.ft * a.w.nst);
+    it.nr = cnt > 0 ? (cnt + 15) & ~15 : 0;
+    int lo = 1 << 30, hi = 0;
+    for (int t = it.t0; t < it.t0 + it.nt; ++t) {
+        const int s = (t / a.w.kwg) * a.gr.Wb + (t % a.w.kwg) * a.w.rep;
+        lo = min(lo, s);
+        hi = max(hi, s);
+    }
+    it.base = lo;
+    it.span = hi - lo;
+    return it;
+}
+
+// Bit j: the item's macro tap j holds a kept GEMM column of accumulator row `row`.
+SADMM_DEV uint32_t gw_keep(const GwArgs& a, const GwItem& it, int row)
+{
+    const int per = a.w.blk * 8;
+    const int rp = row / per, c = it.mb * per + row - rp * per;
+    if (row >= a.w.rows || c >= a.nck) return 0;
+    uint32_t keep = 0;
+    for (int j = 0; j < it.nt; ++j) {
+        const int t = it.t0 + j, kh = t / a.w.kwg, kw = (t - kh * a.w.kwg) * a.w.rep + rp;
+        if (kw >= a.gr.KW) continue;
+        bool ok = true;
+        if (a.colidx) {
+            const int want = c * a.taps + (it.kt * a.gr.KH + kh) * a.gr.KW + kw;
+            int lo = 0, hi = a.n_cols;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (__ldg(a.colidx + mid) < want) lo = mid + 1;
+                else hi = mid;
+            }
+            ok = lo < a.n_cols && __ldg(a.colidx + lo) == want;
+        }
+        if (ok) keep |= 1u << j;
+    }
+    return keep;
+}
+
+__global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_constant__ GwArgs a)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem);  // the first 512 bytes
+    uint8_t* stage0 = smem + 512;
+    uint64_t* full = bars;
+    uint64_t* empty = bars + kGwMaxStages;
+    uint64_t* acc_full = bars + 2 * kGwMaxStages;
+    uint64_t* acc_empty = acc_full + 2;
+    uint64_t* drain = acc_empty + 2;
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kGwMaxStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 8); }
+        mbar_init(drain, 1);
+        *abort_flag = 0;
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(tmem_holder, (uint32_t)kGwCols);
+        tmem_relinquish();
+    }
+    pdl_wait();
+    pdl_trigger();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_holder;
+    // two accumulator sets when every item's columns fit half of TMEM
+    int most = 0;
+    for (int g = 0; g < a.groups; ++g) most = max(most, __ldg(a.counts + 2 * g));
+    const int nbuf = uniform(a.w.tpg * min(a.w.nst, (most + 15) & ~15) <= kGwCols / 2) ? 2 : 1;
+
+    if (warp == 0) {
+        int s = 0;
+        uint32_t ph = 0, last = 0, issued = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x) {
+            const GwItem it = gw_item(a, u);
+            if (it.nr == 0) continue;
+            const int nb = min(a.w.blk, a.w.nch - it.mb * a.w.blk);  // chunks of this block
+            const int na = nb * a.w.rep, nd = it.nr / 8;
+            const uint32_t abytes = (uint32_t)(128 + it.span) * 16u;
+            const __nv_bfloat16* xg = a.xs + (size_t)it.g * a.xs_gstride;
+            const __nv_bfloat16* dg = a.dz + (size_t)it.g * a.dz_gstride;
+            const int e = min(a.w.tiles, (it.z + 1) * a.w.tps);
+            for (int t = it.z * a.w.tps; t < e; ++t) {
+                if (!mbar_wait_warp(&empty[s], ph ^ 1u, abort_flag, a.status)) { ok = false; break; }
+                if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)na * abytes + (uint32_t)nd * 2048u);
+                __syncwarp();
+                const uint32_t sa = smem_u32(stage0 + (size_t)s * a.w.stage_stride);
+                for (int i = lane; i < na + nd; i += 32) {
+                    if (i < na) {
+                        const int rp = i / nb, c = i - rp * nb;
+                        bulk_load(sa + (uint32_t)((rp * a.w.blk + c) * a.w.spa * 16),
+                                  xg + ((size_t)(it.mb * a.w.blk + c) * a.gr.slots +
+                                        (size_t)(t * 128 + it.kt * a.gr.HWb + it.base + rp)) * 8,
+                                  abytes, &full[s]);
+                    } else {
+                        const int c = i - na;
+                        bulk_load(sa + (uint32_t)(a.w.a_bytes + c * 2048),
+                                  dg + ((size_t)(it.ft * (a.w.nst / 8) + c) * a.gr.slots +
+                                        (size_t)(a.gr.D0 + t * 128)) * 8,
+                                  2048u, &full[s]);
+                    }
+                }
+                last = (last & ~(1u << s)) | (ph << s);
+                issued |= 1u << s;
+                if (++s == a.w.stages) { s = 0; ph ^= 1u; }
+            }
+        }
+        for (int q = 0; q < a.w.stages; ++q) {
+            if (!(issued & (1u << q))) continue;
+            const unsigned long long t0 = globaltimer();
+            while (!mbar_try_wait(&full[q], (last >> q) & 1u) && globaltimer() - t0 < kWaitLimitNs) {}
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // The whole warp runs the loop; one elected lane issues.
+        int s = 0, ab = 0;
+        uint32_t ph = 0, acc_ph = 0;
+        bool ok = true;
+        const uint64_t ad0 = sdesc_kmajor_none(smem_u32(stage0), 128u, (uint32_t)a.w.spa * 16u);
+        const uint64_t bd0 = sdesc_kmajor_none(smem_u32(stage0) + (uint32_t)a.w.a_bytes, 128u, 2048u);
+        const uint64_t ahi = ad0 & 0xffffffff00000000ull, bhi = bd0 & 0xffffffff00000000ull;
+        for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x) {
+            const GwItem it = gw_item(a, u);
+            if (uniform(it.nr == 0)) continue;
+            const uint32_t idesc = idesc_bf16_f32(128, it.nr) | (1u << 15) | (1u << 16);  // A and B MN-major
+            if (!mbar_wait_warp(&acc_empty[ab], acc_ph ^ 1u, abort_flag, a.status)) break;
+            const uint32_t d0 = tmem_base + (uint32_t)(ab * (kGwCols / 2));
+            const int b = it.z * a.w.tps, e = min(a.w.tiles, b + a.w.tps);
+            for (int t = b; t < e; ++t) {
+                if (!mbar_wait_warp(&full[s], ph, abort_flag, a.status)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t so = (uint32_t)(s * a.w.stage_stride) >> 4;
+                const uint32_t blo = (uint32_t)bd0 + so;
+                for (int j = 0; j < it.nt; ++j) {
+                    const int tap = it.t0 + j;
+                    const uint32_t alo = (uint32_t)ad0 + so +
+                                         (uint32_t)((tap / a.w.kwg) * a.gr.Wb + (tap % a.w.kwg) * a.w.rep - it.base);
+                    const uint32_t d = d0 + (uint32_t)(j * it.nr);
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk)  // 16 grid pixels each
+                        mma_bf16_ss_elect(d, ahi | (alo + kk * 16u), bhi | (blo + kk * 16u), idesc,
+                                          (t > b || kk > 0) ? 1u : 0u);
+                }
+                mma_commit_elect(&empty[s]);
+                if (++s == a.w.stages) { s = 0; ph ^= 1u; }
+            }
+            if (!ok) break;
+            mma_commit_elect(&acc_full[ab]);
+            if (++ab == nbuf) { ab = 0; acc_ph ^= 1u; }
+        }
+        mma_commit_elect(drain);
+        if (lane == 0) {
+            const unsigned long long t0 = globaltimer();
+            while (!mbar_try_wait(drain, 0) && globaltimer() - t0 < kWaitLimitNs) {}
+        }
+        __syncwarp();
+    } else {
+        // epilogue: the item's accumulator into its slice, lane = channel row
+        const int q4 = warp & 3, h = (warp - 2) >> 2;
+        const int row = q4 * 32 + lane;
+        int ab = 0;
+        uint32_t acc_ph = 0;
+        for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+            const GwItem it = gw_item(a, u);
+            if (it.nr == 0) continue;
+            // the item's taps whose column of this lane's channel is kept: only
+            // those are written (found while the MMAs run)
+            const uint32_t keep = gw_keep(a, it, row);
+            if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[ab], acc_ph, abort_flag, a.status))) break;
+            tc_fence_after();
+            const uint32_t taddr = tmem_base + (uint32_t)(ab * (kGwCols / 2)) + ((uint32_t)(q4 * 32) << 16);
+            float* dst = a.slices + (size_t)it.z * a.w.slice +
+                         ((size_t)it.type * a.w.rows + row) * (size_t)(a.w.tpg * a.w.nst);
+            const int per = it.nr / kEpiCols, n = it.nt * per;
+            if (q4 * 32 < a.w.rows) {
+                for (int k = h; k < n; k += 2) {
+                    uint32_t r[kEpiCols];
+                    tmem_ld_32x32b_x16(taddr + (uint32_t)(k * kEpiCols), r);
+                    tmem_ld_wait();
+                    const int j = k / per;
+                    if ((keep >> j) & 1u) {
+                        float4* d4 = reinterpret_cast<float4*>(dst + j * a.w.nst + (k - j * per) * kEpiCols);
+#pragma unroll
+                        for (int e = 0; e < kEpiCols / 4; ++e)
+                            d4[e] = make_float4(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]),
+                                                __uint_as_float(r[4 * e + 2]), __uint_as_float(r[4 * e + 3]));
+                    }
+                    __syncwarp();
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_empty[ab]);
+            if (++ab == nbuf) { ab = 0; acc_ph ^= 1u; }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, (uint32_t)kGwCols);
+    }
+}
+
+// The weight gradient of one kept entry over the layer's output pixels alone:
+// what its grid sum is, unless a padded pixel's zero met an infinity or a NaN.
+__device__ __noinline__ float wgrad_exact(const __nv_bfloat16* xc, const __nv_bfloat16* dc, int shift, int D0, int N, int P,
+                                          int HWb, int Wb, int OT, int OH, int OW)
+{
+    float acc = 0.0f;
+    for (int n = 0; n < N; ++n)
+        for (int t = 0; t < OT; ++t)
+            for (int h = 0; h < OH; ++h)
+                for (int w = 0; w < OW; ++w) {
+                    const size_t q = (size_t)n * P + (size_t)t * HWb + h * Wb + w;
+                    acc += __bfloat162float(dc[(q + D0) * 8]) * __bfloat162float(xc[(q + shift) * 8]);
+                }
+    return acc;
+}
+
+struct WrArgs {
+    Grid gr;
+    WgradShape w;
+    const float* slices;
+    const int* rowmap;
+    const int* colidx;
+    const int* counts;
+    const __nv_bfloat16* xs;
+    const __nv_bfloat16* dz;
+    long long xs_gstride, dz_gstride;
+    float* dW;
+    int n_pad, n_cols, taps, chan_kind;
+    long long K;
+};
+
+// dW[f_i][col_j] = sum over the pixel ranges of their slices: eight threads per
+// entry take every eighth range, then their sums are added in order
+// (deterministic).  Block (bx, by, g): packed columns bx*kWrCols .., packed rows
+// by*32 .. +31; the slices are read along the filters.
+constexpr int kWrCols = 4;
+
+__global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a)
+{
+    pdl_wait();  // after the kernel before it in the stream
+    __shared__ float s_v[8][kWrCols][32];
+    const int g = blockIdx.z, cnt = __ldg(a.counts + 2 * g);
+    const int i0 = blockIdx.y * 32, j0 = blockIdx.x * kWrCols;
+    if (i0 >= cnt) return;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int i = i0 + tx;
+    const int ft = i / a.w.nst;
+    const float* src[kWrCols];
+    int shift[kWrCols], chan[kWrCols];
+    float v[kWrCols];
+#pragma unroll
+    for (int e = 0; e < kWrCols; ++e) {
+        const int j = j0 + e;
+        const int col = j < a.n_cols ? __ldg(a.colidx + j) : -1;
+        v[e] = 0.0f;
+        src[e] = nullptr;
+        if (col < 0 || i >= cnt) continue;
+        const int c = a.chan_kind ? j / a.taps : col / a.taps, tap = col % a.taps;
+        const int kw = tap % a.gr.KW, kh = (tap / a.gr.KW) % a.gr.KH, kt = tap / (a.gr.KW * a.gr.KH);
+        const int mb = (c >> 3) / a.w.blk, mt = kh * a.w.kwg + kw / a.w.rep;
+        const int m = (((kw % a.w.rep) * a.w.blk + ((c >> 3) - mb * a.w.blk)) << 3) + (c & 7);
+        const int type = (((g * a.w.nft + ft) * a.w.mblks + mb) * a.gr.KT + kt) * a.w.tgs + mt / a.w.tpg;
+        chan[e] = c;
+        shift[e] = kt * a.gr.HWb + kh * a.gr.Wb + kw;
+        src[e] = a.slices + ((size_t)type * a.w.rows + m) * (size_t)(a.w.tpg * a.w.nst) + (mt % a.w.tpg) * a.w.nst +
+                 (i - ft * a.w.nst);
+    }
+#pragma unroll 4
+    for (int z = ty; z < a.w.Z; z += 8)
+#pragma unroll
+        for (int e = 0; e < kWrCols; ++e)
+            if (src[e]) v[e] += __ldcs(src[e] + (size_t)z * a.w.slice);
+#pragma unroll
+    for (int e = 0; e < kWrCols; ++e) s_v[ty][e][tx] = v[e];
+    __syncthreads();
+    if (ty >= kWrCols || i >= cnt) return;
+    float acc = 0.0f;
+    for (int z = 0; z < 8; ++z) acc += s_v[z][ty][tx];
+#pragma unroll
+    for (int e = 0; e < kWrCols; ++e) {
+        if (e != ty || !src[e]) continue;
+        if (acc != acc)
+            acc = wgrad_exact(a.xs + (size_t)g * a.xs_gstride + (size_t)(chan[e] >> 3) * a.gr.slots * 8 + (chan[e] & 7),
+                              a.dz + (size_t)g * a.dz_gstride + (size_t)(i >> 3) * a.gr.slots * 8 + (i & 7), shift[e],
+                              a.gr.D0, a.gr.N, a.gr.P, a.gr.HWb, a.gr.Wb, a.gr.OT, a.gr.OH, a.gr.OW);
+        const int f = __ldg(a.rowmap + g * a.n_pad + i);
+        if (f >= 0) a.dW[(long long)f * a.K + __ldg(a.colidx + j0 + e)] = acc;
+    }
+}
+
+struct DzArgs {
+    Grid gr;
+    const __nv_bfloat16* dy;
+    const void* y;
+    const int* rowmap;
+    const int* counts;
+    int n_pad, F, plane, chunks, cb;
+    __nv_bfloat16* dz;  // NULL: the bias gradient alone
+    float* part;        // [groups*n_pad][gridDim.x], or NULL
+};
+
+// Grid copy of dZ and the bias gradient's partial sums.  Block (bx, by): slots
+// bx*kDzSlots .. of chunk by % chunks (8 kept filters) of conv group by / chunks.
+constexpr int kDzSlots = 512;
+
+// One pixel's dZ of a chunk's filters (nf of them, 8 when FULL): every load
+// first, then the products, the running bias sums and the packed octet.
+template <bool RELU, typename Y, bool FULL>
+SADMM_DEV void dz_octet(const unsigned short* dp, const Y* yp, const int (&off)[8], int nf, float (&sum)[8], uint32_t (&o)[4])
+{
+    uint32_t dyv[8];
+    Y yv[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        dyv[e] = (FULL || e < nf) ? (uint32_t)__ldg(dp + off[e]) : 0u;
+        if (RELU) yv[e] = (FULL || e < nf) ? __ldg(yp + off[e]) : Y(0);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        float v = __uint_as_float(dyv[e] << 16);
+        if (RELU) {
+            const float yf = sizeof(Y) == 2 ? __uint_as_float((uint32_t)yv[e] << 16) : (float)yv[e];
+            v *= yf > 0.0f ? 1.0f : 0.0f;
+        }
+        sum[e] += v;
+        // v is a bf16 value (or a NaN, whose upper half is one)
+        const uint32_t u = __float_as_uint(v);
+        o[e >> 1] = (e & 1) ? __byte_perm(o[e >> 1], u, 0x7610) : u >> 16;
+    }
+}
+
+template <bool RELU, typename Y>
+__global__ void __launch_bounds__(256) k_grid_dz(const DzArgs a)
+{
+    pdl_wait();  // after the kernel before it in the stream
+    __shared__ int s_off[8];
+    __shared__ float s_part[8][8];
+    const int g = blockIdx.y / a.chunks, ck = blockIdx.y - g * a.chunks;
+    const int cnt = __ldg(a.counts + 2 * g);
+    if (ck * 8 >= (cnt + a.cb - 1) / a.cb * a.cb && ck * 8 >= cnt + 15) return;  // past every reader's last filter
+    const int nf = min(8, cnt - ck * 8);  // kept filters of this chunk (they come first)
+    if (threadIdx.x < 8 && (int)threadIdx.x < nf)
+        s_off[threadIdx.x] = __ldg(a.rowmap + g * a.n_pad + ck * 8 + threadIdx.x) * a.plane;
+    __syncthreads();
+    int off[8];
+    float sum[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        off[e] = e < nf ? s_off[e] : 0;
+        sum[e] = 0.0f;
+    }
+#pragma unroll 1
+    for (int k = 0; k < kDzSlots / 256; ++k) {
+        const int s = blockIdx.x * kDzSlots + k * 256 + threadIdx.x;
+        if (s >= a.gr.slots) break;
+        int n = 0, t = 0, h = 0, w = 0;
+        const int q = s - a.gr.D0;
+        if (q >= 0) grid_decode(a.gr, q, n, t, h, w);
+        uint32_t o[4] = {0u, 0u, 0u, 0u};
+        if (q >= 0 && n < a.gr.N && t < a.gr.OT && h < a.gr.OH && w < a.gr.OW) {
+            // every load first (32-bit offsets from the image's pixel), then the products
+            const long long base = (long long)n * a.F * a.plane + (t * a.gr.OH + h) * a.gr.OW + w;
+            const unsigned short* dp = reinterpret_cast<const unsigned short*>(a.dy) + base;
+            const Y* yp = static_cast<const Y*>(a.y) + base;
+            if (nf == 8) dz_octet<RELU, Y, true>(dp, yp, off, 8, sum, o);
+            else dz_octet<RELU, Y, false>(dp, yp, off, nf, sum, o);
+        }
+        if (a.dz)
+            reinterpret_cast<uint4*>(a.dz)[((size_t)g * a.chunks + ck) * a.gr.slots + s] =
+                make_uint4(o[0], o[1], o[2], o[3]);
+    }
+    if (!a.part) return;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        for (int o = 16; o > 0; o >>= 1) sum[e] += __shfl_down_sync(0xffffffffu, sum[e], o);
+        if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5][e] = sum[e];
+    }
+    __syncthreads();
+    const int i = ck * 8 + threadIdx.x;
+    if (threadIdx.x < 8 && i < a.n_pad) {
+        float r = 0.0f;
+        for (int w = 0; w < 8; ++w) r += s_part[w][threadIdx.x];
+        a.part[(size_t)(g * a.n_pad + i) * gridDim.x + blockIdx.x] = r;
+    }
+}
+
+// db: a warp per packed row adds its partial sums (fixed order); zeros for the
+// pruned filters.
+__global__ void __launch_bounds__(256) k_grid_db(const float* part, int nparts, const int* rowmap, const int* zeromap,
+                                                 const int* counts, int groups, int n_pad, int Fg, float* db)
+{
+    pdl_wait();  // after the kernel before it in the stream
+    const int lane = threadIdx.x & 31;
+    const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (r < groups * n_pad) {
+        const int f = __ldg(rowmap + r);
+        if (f >= 0) {
+            float s = 0.0f;
+            for (int k = lane; k < nparts; k += 32) s += __ldg(part + (size_t)r * nparts + k);
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+            if (lane == 0) db[f] = s;
+        }
+    }
+    for (int z = blockIdx.x * 256 + threadIdx.x; z < groups * Fg; z += gridDim.x * 256) {
+        const int g = z / Fg;
+        if (z - g * Fg < __ldg(counts + 2 * g + 1)) db[__ldg(zeromap + z)] = 0.0f;
+    }
+}
+
+struct PrepArgs {
+    const __nv_bfloat16* wp;
+    const int* colidx;
+    const int* counts;
+    int n_pad, k_pad, n_cols, taps, Cg, groups, nck, chan_kind;
+    int rows, ncpad, bn, cb, ksteps;  // rows 0: no input gradient
+    __nv_bfloat16* wd;
+    int* colmap;
+    int* zmap;
+    int* counts2;
+    float* zero;  // dW (or NULL)
+    long long zero_n;
+};
+
+// Blocks below `rows`: one output column (input channel) of the input
+// gradient's weights each, a quarter of its K columns per blockIdx.y; the
+// others zero dW.
+__global__ void __launch_bounds__(128) k_grid_prep(const PrepArgs a)
+{
+    pdl_wait();  // after the kernel before it in the stream
+    __shared__ int s_j[256];  // flipped tap -> packed column (-1: pruned)
+    if ((int)blockIdx.x >= a.rows) {
+        const long long nb = (long long)(gridDim.x - a.rows) * gridDim.y * 128;
+        for (long long i = ((long long)(blockIdx.x - a.rows) * gridDim.y + blockIdx.y) * 128 + threadIdx.x; i < a.zero_n; i += nb) a.zero[i] = 0.0f;
+        return;
+    }
+    const int g = blockIdx.x / a.ncpad, jc = blockIdx.x - g * a.ncpad;
+    const int cnt = __ldg(a.counts + 2 * g);
+    int c = jc < a.nck ? jc : -1;
+    if (c >= 0 && a.chan_kind) {
+        const int col = __ldg(a.colidx + jc * a.taps);
+        c = col >= 0 ? col / a.taps : -1;
+    }
+    if (threadIdx.x == 0 && blockIdx.y == 0) a.colmap[blockIdx.x] = c >= 0 ? g * a.Cg + c : -1;
+    for (int t = threadIdx.x; t < a.taps; t += 128) {
+        int j = -1;
+        if (c >= 0) {
+            const int want = c * a.taps + t;
+            int lo = 0, hi = a.n_cols;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (__ldg(a.colidx + mid) < want) lo = mid + 1;
+                else hi = mid;
+            }
+            if (lo < a.n_cols && __ldg(a.colidx + lo) == want) j = lo;
+        }
+        s_j[a.taps - 1 - t] = j;
+    }
+    __syncthreads();
+    // [step][K half][bn][8] of this column's tile: a thread fills the 8 filters
+    // of one half of a step
+    const int nt = jc / a.bn, h8 = a.cb / 8;
+    uint4* wd = reinterpret_cast<uint4*>(a.wd) + ((size_t)(blockIdx.x / a.bn) * a.ksteps * 2) * a.bn + (jc - nt * a.bn);
+    const unsigned short* wp = reinterpret_cast<const unsigned short*>(a.wp) + (size_t)g * a.n_pad * a.k_pad;
+    const int kuse = min(a.ksteps, (cnt + a.cb - 1) / a.cb * a.taps * (a.cb / 16)) * 2;  // what an item may load
+    for (int k = blockIdx.y * 128 + threadIdx.x; k < kuse; k += gridDim.y * 128) {
+        int t = k / h8;
+        const int c8 = k - t * h8;
+        const int blk = t / a.taps;
+        t -= blk * a.taps;  // kt * KH*KW + tap
+        const int i = blk * a.cb + c8 * 8, j = s_j[t];
+        uint32_t v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            v[e] = 0;
+            if (i + e < cnt) {
+                v[e] = j >= 0 ? __ldg(wp + (size_t)(i + e) * a.k_pad + j) : 0x8000u;
+                if (j >= 0 && v[e] == 0x8000u) v[e] = 0;
+            }
+        }
+        wd[(size_t)k * a.bn] = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+    }
+    if (jc == 0 && blockIdx.y == 0) {
+        // the group's output columns and the pruned channels' planes
+        const bool none = a.chan_kind && (a.n_cols == 0 || __ldg(a.colidx) < 0);
+        const int ncols = none ? 0 : a.nck;
+        if (threadIdx.x == 0) {
+            a.counts2[2 * g] = ncols;
+            a.counts2[2 * g + 1] = a.Cg - ncols;
+        }
+        if (a.chan_kind)
+            for (int ch = threadIdx.x; ch < a.Cg; ch += 128) {
+                int lo = 0, hi = ncols;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (__ldg(a.colidx + mid * a.taps) / a.taps < ch) lo = mid + 1;
+                    else hi = mid;
+                }
+                if (!(lo < ncols && __ldg(a.colidx + lo * a.taps) / a.taps == ch)) a.zmap[g * a.Cg + ch - lo] = g * a.Cg + ch;
+            }
+    }
+}
+
+struct GridBwd {
+    Grid gr;
+    GridConvShape cs;
+    WgradShape ws;
+    int nck;      // channels of x per group that hold a kept column
+    int dchunks;  // 8-filter chunks of dZ per group
+    int nparts;   // blocks of k_grid_dz along the slots
+    size_t off_xs, off_dz, off_wd, off_maps, off_slices, off_part, total;
+};
+
+bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, GridBwd* out)
+{
+    GridBwd b;
+    if (plan->n_cols < 1 || plan->n_filt < 1 || g.taps > 256) return false;
+    if (!grid_of(g, &b.gr)) return false;
+    b.nck = plan->colkind == SADMM_COL_CHANNEL ? plan->n_colgroups : (int)g.cg;
+    if (!grid_conv_shape(b.gr, plan->n_pad, b.nck, (int)g.groups, (int)kGwCtas, &b.cs)) return false;
+    if (!wgrad_shape(b.gr, b.nck, plan->n_pad, (int)g.groups, &b.ws)) return false;
+    b.dchunks = std::max(b.cs.k16 * 2, b.ws.nft * b.ws.nst / 8);
+    b.nparts = (b.gr.slots + kDzSlots - 1) / kDzSlots;
+    if (g.groups * b.dchunks > 65535 || g.groups * ((b.ws.nch + 1) / 2) > 65535) return false;
+    size_t off = 0;
+    auto take = [&off](long long bytes) {
+        const size_t at = off;
+        off += (size_t)round_up(bytes, 1024);
+        return at;
+    };
+    b.off_xs = take(g.groups * b.ws.nch * (long long)b.gr.slots * 16);
+    b.off_dz = take(g.groups * b.dchunks * (long long)b.gr.slots * 16);
+    b.off_wd = take(g.groups * b.cs.npad * (long long)b.cs.ksteps * 32);
+    b.off_maps = take((g.groups * b.cs.npad + g.c + 2 * g.groups) * 4);
+    b.off_slices = take(b.ws.Z * b.ws.slice * 4);
+    b.off_part = take(g.groups * plan->n_pad * (long long)b.nparts * 4);
+    b.total = off;
+    *out = b;
+    return true;
+}
+
+}  // namespace
+
+size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g)
+{
+    GridBwd b;
+    return grid_bwd_shape(plan, g, &b) ? b.total : 0;
+}
+
+sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const void* x, const void* dy, const void* y,
+                             int ydt, int relu, float* dW, float* db, float* dx, void* ws, cudaStream_t s)
+{
+    GridBwd b;
+    if (!grid_bwd_shape(plan, g, &b)) return SADMM_EINVAL;
+    const char* base = static_cast<const char*>(plan->dev);
+    char* w = static_cast<char*>(ws);
+    const int* rowmap = reinterpret_cast<const int*>(base + plan->off_rowmap);
+    const int* zeromap = reinterpret_cast<const int*>(base + plan->off_zeromap);
+    const int* counts = reinterpret_cast<const int*>(base + plan->off_counts);
+    const int* colidx = reinterpret_cast<const int*>(base + plan->off_colidx);
+    __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(w + b.off_xs);
+    __nv_bfloat16* dz = reinterpret_cast<__nv_bfloat16*>(w + b.off_dz);
+    __nv_bfloat16* wd = reinterpret_cast<__nv_bfloat16*>(w + b.off_wd);
+    int* colmap = reinterpret_cast<int*>(w + b.off_maps);
+    int* zmap = colmap + g.groups * b.cs.npad;
+    int* counts2 = zmap + g.c;
+    float* slices = reinterpret_cast<float*>(w + b.off_slices);
+    float* part = reinterpret_cast<float*>(w + b.off_part);
+    const int chan_kind = plan->colkind == SADMM_COL_CHANNEL ? 1 : 0;
+    const int* chans = chan_kind ? colidx : nullptr;
+    const long long xs_g = (long long)b.ws.nch * b.gr.slots * 8, dz_g = (long long)b.dchunks * b.gr.slots * 8;
+
+    if (dW || dx) {
+        PrepArgs p;
+        memset(&p, 0, sizeof(p));
+        p.wp = reinterpret_cast<const __nv_bfloat16*>(base + plan->off_wp);
+        p.colidx = colidx;
+        p.counts = counts;
+        p.n_pad = plan->n_pad;
+        p.k_pad = plan->k_pad;
+        p.n_cols = plan->n_cols;
+        p.taps = (int)g.taps;
+        p.Cg = (int)g.cg;
+        p.groups = (int)g.groups;
+        p.nck = b.nck;
+        p.chan_kind = chan_kind;
+        p.ncpad = b.cs.npad;
+        p.rows = dx ? (int)g.groups * b.cs.npad : 0;
+        p.bn = b.cs.bn;
+        p.cb = b.cs.cb;
+        p.ksteps = b.cs.ksteps;
+        p.wd = wd;
+        p.colmap = colmap;
+        p.zmap = zmap;
+        p.counts2 = counts2;
+        p.zero = dW;
+        p.zero_n = dW ? g.f * g.k : 0;
+        const long long nz = dW ? std::min<long long>(256, (p.zero_n + 2047) / 2048) : 0;
+        if (launch_pdl(k_grid_prep, dim3((unsigned)(p.rows + nz), 4), dim3(128), 0, s, p) != cudaSuccess) return SADMM_ECUDA;
+    }
+    DzArgs d;
+    memset(&d, 0, sizeof(d));
+    d.gr = b.gr;
+    d.dy = static_cast<const __nv_bfloat16*>(dy);
+    d.y = y;
+    d.rowmap = rowmap;
+    d.counts = counts;
+    d.n_pad = plan->n_pad;
+    d.F = (int)g.f;
+    d.plane = (int)g.plane;
+    d.chunks = b.dchunks;
+    d.cb = b.cs.cb;
+    d.dz = (dW || dx) ? dz : nullptr;
+    d.part = db ? part : nullptr;
+    const dim3 dgrid((unsigned)b.nparts, (unsigned)(g.groups * b.dchunks));
+    const cudaError_t de =
+        !relu ? launch_pdl(k_grid_dz<false, float>, dgrid, dim3(256), 0, s, d)
+              : (ydt == SADMM_BF16 ? launch_pdl(k_grid_dz<true, unsigned short>, dgrid, dim3(256), 0, s, d)
+                                   : launch_pdl(k_grid_dz<true, float>, dgrid, dim3(256), 0, s, d));
+    if (de != cudaSuccess) return SADMM_ECUDA;
+    if (db &&
+        launch_pdl(k_grid_db, dim3((unsigned)((g.groups * plan->n_pad + 7) / 8)), dim3(256), 0, s,
+                   static_cast<const float*>(part), b.nparts, rowmap, zeromap, counts, (int)g.groups, plan->n_pad,
+                   (int)g.fg, db) != cudaSuccess)
+        return SADMM_ECUDA;
+    if (dW) {
+        const sadmm_status st = launch_grid_x(b.gr, g, x, chans, b.nck, b.ws.nch, xs, s);
+        if (st != SADMM_OK) return st;
+        GwArgs a;
+        memset(&a, 0, sizeof(a));
+        a.gr = b.gr;
+        a.w = b.ws;
+        a.xs = xs;
+        a.dz = dz;
+        a.xs_gstride = xs_g;
+        a.dz_gstride = dz_g;
+        a.counts = counts;
+        a.colidx = plan->colkind == SADMM_COL_SHAPE ? colidx : nullptr;
+        a.nck = b.nck;
+        a.n_cols = plan->n_cols;
+        a.taps = (int)g.taps;
+        a.slices = slices;
+        a.groups = (int)g.groups;
+        a.units = b.ws.types * b.ws.Z;
+        a.types_div = make_fastdiv((uint32_t)b.ws.types);
+        a.status = device_status_ptr();
+        static int configured_dev = -1;
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (configured_dev != dev) {
+            if (cudaFuncSetAttribute(k_grid_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kGwSmemLimit) != cudaSuccess)
+                return SADMM_ECUDA;
+            configured_dev = dev;
+        }
+        const int grid = std::min(a.units, device_sm_count());
+        if (launch_pdl(k_grid_wgrad, dim3((unsigned)grid), dim3(kGwThreads), b.ws.smem, s, a) != cudaSuccess)
+            return SADMM_ECUDA;
+        WrArgs r;
+        memset(&r, 0, sizeof(r));
+        r.gr = b.gr;
+        r.w = b.ws;
+        r.slices = slices;
+        r.rowmap = rowmap;
+        r.colidx = colidx;
+        r.counts = counts;
+        r.xs = xs;
+        r.dz = dz;
+        r.xs_gstride = xs_g;
+        r.dz_gstride = dz_g;
+        r.dW = dW;
+        r.n_pad = plan->n_pad;
+        r.n_cols = plan->n_cols;
+        r.taps = (int)g.taps;
+        r.chan_kind = chan_kind;
+        r.K = g.k;
+        if (launch_pdl(k_grid_wreduce,
+                       dim3((unsigned)((plan->n_cols + kWrCols - 1) / kWrCols), (unsigned)((plan->n_pad + 31) / 32),
+                            (unsigned)g.groups),
+                       dim3(256), 0, s, r) != cudaSuccess)
+            return SADMM_ECUDA;
+    }
+    if (dx) {
+        GridConvCall c;
+        memset(&c, 0, sizeof(c));
+        c.src = dz;
+        c.chunks = b.dchunks;
+        c.wd = wd;
+        c.out = dx;
+        c.colmap = colmap;
+        c.zmap = zmap;
+        c.zstride = (int)g.cg;
+        c.counts = counts2;
+        c.kcounts = counts;
+        c.groups = (int)g.groups;
+        c.planes = (int)g.c;
+        c.VT = (int)g.t;
+        c.VH = (int)g.h;
+        c.VW = (int)g.w;
+        c.out_total = g.n * g.c * g.t * g.h * g.w;
+        const sadmm_status st = launch_grid_conv(b.gr, b.cs, c, s);
+        if (st != SADMM_OK) return st;
+    }
+    return cudaGetLastError() == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
+}
+
+}  // namespace sadmm

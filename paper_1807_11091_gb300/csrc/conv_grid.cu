@@ -1,0 +1,682 @@
+// conv_grid.cu -- stride-1 convolution as a slab GEMM on the tensor cores: the
+// input gradient of a pruned layer (its forward with the taps flipped, over the
+// kept filters; Sec. 4, masked retraining).
+//
+// GEMM row i of tile t is grid pixel 128t + i of the padded line (grid.cuh);
+// every tap of a block of CB channels is the same shared-memory slab of
+// 128*MT + maxshift slots, shifted: a K-major no-swizzle operand whose start
+// moves by 16 bytes a slot.  So x is read about once per tile instead of once
+// per tap, no element is gathered by a thread, and no thread touches the A
+// operand: bulk copies bring the slabs, TMA the weights, one warp issues.
+// Pruned columns cost tensor time (their weights are zero) but no traffic: at
+// a quarter of the columns the 128 x 96 x 16 MMA of four times the steps is
+// still shorter than gathering the kept ones 2 bytes at a time.
+//
+//   warp 0       slabs: CB/8 bulk copies per stage
+//   warp 1       TMEM allocator, MMA issuer
+//   warp 2       weights: resident, or a ring of a few MMA steps per slot
+//   warps 3-10   epilogue: every `sps` stages (at most about 54 MMA steps) the
+//                accumulator is read from TMEM and added to fp32 registers
+//                (the tensor core truncates when it accumulates, about 1e-8 of
+//                the result per step; short chains keep that below 5e-7), the
+//                other TMEM buffer meanwhile taking the next stages; after the
+//                last, bias, ReLU and coalesced stores (lane = pixel).
+// A 0 * inf of a pruned weight would put a NaN where the kept sum has none:
+// pruned entries are stored as -0.0 and an output that comes out NaN is summed
+// again over the kept entries alone (grid_exact).
+#include <string.h>
+
+#include <algorithm>
+
+#include "grid.cuh"
+
+namespace sadmm {
+
+namespace {
+
+constexpr int kGcWarps = 11;
+constexpr int kGcThreads = kGcWarps * 32;
+constexpr int kGcEpiWarps = 8;
+constexpr int kGcMaxA = 4, kGcMaxB = 8;
+constexpr int kGcSegSteps = 54;    // MMA steps accumulated in TMEM before the fp32 registers take over
+constexpr int kGcTables = 2 * 256 * 4;
+constexpr int kGcZcap = 1024;
+constexpr int kGcBars = 512;
+constexpr int kGcSmemLimit = 232448;
+
+struct GcArgs {
+    Grid gr;
+    const __nv_bfloat16* src;
+    const __nv_bfloat16* wd;
+    void* out;
+    const float* bias;
+    const int* colmap;
+    const int* zmap;
+    const int* counts;
+    const int* kcounts;
+    int* status;
+    long long out_total;
+    long long gstride;  // source elements per group
+    int zstride, groups, planes, plane, VT, VH, VW, VHW;
+    int units, mtiles, ntiles;
+    FastDiv mt_div, nt_div;
+    int bn, ksteps;
+    int cb, ncb, spt;   // channels per block, blocks (static), MMA steps per stage
+    int h16, rsteps;    // 16-channel steps per tap, MMA steps per kernel row (a slot of the weight ring)
+    int sp;             // slots of a slab
+    int sps;            // stages per accumulation segment
+    int cap_b, stages_a, a_bytes, a_stride;
+    int tmem_stride, tmem_cols;
+    int relu;
+};
+
+// The sum of one output (column `col` of the tile whose weights wd are, grid
+// pixel q) over the kept K columns only, as the gathered path forms it (pruned
+// entries are -0.0).
+__device__ __noinline__ float grid_exact(const __nv_bfloat16* wd, int bn, int col, const __nv_bfloat16* src, int q,
+                                         int kch, int cb, int KT, int KH, int KW, int HWb, int Wb, int slots)
+{
+    const unsigned short* w = reinterpret_cast<const unsigned short*>(wd) + col * 8;
+    float acc = 0.0f;
+    for (int c0 = 0; c0 < kch; c0 += cb)
+        for (int kt = 0; kt < KT; ++kt)
+            for (int kh = 0; kh < KH; ++kh)
+                for (int kw = 0; kw < KW; ++kw)
+                    for (int c8 = c0; c8 < c0 + cb; c8 += 8, w += bn * 8)
+                        for (int e = 0; e < 8; ++e) {
+                            const unsigned short b = __ldg(w + e);
+                            if (b == 0x8000u || c8 + e >= kch) continue;
+                            const size_t slot = (size_t)(c8 >> 3) * slots + (q + kt * HWb + kh * Wb + kw);
+                            acc += __uint_as_float((uint32_t)b << 16) * __bfloat162float(src[slot * 8 + e]);
+                        }
+    return acc;
+}
+
+// Channel blocks a group's items contract over.
+SADMM_DEV int gc_blocks(const GcArgs& a, int g)
+{
+    return a.kcounts ? min(a.ncb, (__ldg(a.kcounts + 2 * g) + a.cb - 1) / a.cb) : a.ncb;
+}
+
+// Work item u: pixel tile (fastest), column tile, group.
+SADMM_DEV void gc_unit(const GcArgs& a, int u, int& g, int& nt, int& mt)
+{
+    const int t = (int)fdiv((uint32_t)u, a.mt_div);
+    mt = u - t * a.mtiles;
+    g = (int)fdiv((uint32_t)t, a.nt_div);
+    nt = t - g * a.ntiles;
+}
+
+// The barriers and operand bases of a CTA, for its issuing warp.
+struct GcPipe {
+    uint64_t *full_a, *empty_a, *full_b, *empty_b, *acc_full, *acc_empty, *b_full, *b_empty;
+    volatile int* abort_flag;
+    uint32_t sA, sB, tmem_base;
+    int stages_b;
+};
+
+// The issuing warp's run over its work items.  The whole warp runs the loop,
+// every branch on a parameter or a vote, and one elected lane issues.  KW taps
+// of H steps of 16 channels make a kernel row, unrolled: an MMA then issues in
+// the 48 cycles that a 128 x 64 x 16 takes (71 with the offsets read from a
+// table in the parameters, 103 with the row chosen by a switch inside the loop,
+// 120 and more with bounds the compiler cannot prove uniform).  KW = 0: any
+// other row, one MMA at a time.
+template <int KW, int H, int MT>
+SADMM_DEV void gc_issue(const GcArgs& a, const GcPipe& p, const bool resident)
+{
+    int s = 0, sb = 0, ab = 0;
+    uint32_t ph = 0, phb = 0, acc_ph = 0, bf_ph = 0;
+    int cur = -1;
+    bool ok = true;
+    const uint64_t ad0 = sdesc_kmajor_none(p.sA, (uint32_t)a.sp * 16u, 128u);
+    const uint64_t bd0 = sdesc_kmajor_none(p.sB, (uint32_t)a.bn * 16u, 128u);
+    const uint64_t ahi = ad0 & 0xffffffff00000000ull, bhi = bd0 & 0xffffffff00000000ull;
+    const uint32_t alo0 = (uint32_t)ad0, blo0 = (uint32_t)bd0;
+    const uint32_t bs16 = (uint32_t)a.bn * 2u;   // one step of the weights, in 16-byte units
+    const uint32_t half = 2u * (uint32_t)a.sp;   // 16 channels of a slab
+    for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x) {
+        int g, nt, mt;
+        gc_unit(a, u, g, nt, mt);
+        const int cnt = min(a.bn, __ldg(a.counts + 2 * g) - nt * a.bn);
+        const int nst = gc_blocks(a, g) * a.gr.KT;
+        if (uniform(cnt <= 0 || nst == 0)) continue;
+        const uint32_t idesc = idesc_bf16_f32(128, (cnt + 15) & ~15);
+        if (resident && g != cur) {
+            if (cur >= 0) mma_commit_elect(p.b_empty);  // the old weights are free once these MMAs finish
+            if (!mbar_wait_warp(p.b_full, bf_ph, p.abort_flag, a.status)) break;
+            bf_ph ^= 1u;
+            cur = g;
+        }
+        uint32_t d = 0, blo = blo0;
+        int in_seg = 0;
+        for (int st = 0; st < a.ncb * a.gr.KT; ++st) {
+            if (uniform(st >= nst)) break;
+            if (in_seg == 0) {
+                if (!mbar_wait_warp(&p.acc_empty[ab], acc_ph ^ 1u, p.abort_flag, a.status)) { ok = false; break; }
+                d = p.tmem_base + (uint32_t)(ab * MT * a.tmem_stride);
+            }
+            if (!mbar_wait_warp(&p.full_a[s], ph, p.abort_flag, a.status)) { ok = false; break; }
+            tc_fence_after();
+            uint32_t ar = alo0 + ((uint32_t)(s * a.a_stride) >> 4);
+            for (int kh = 0; kh < a.gr.KH; ++kh) {
+                if (!resident) {
+                    if (!mbar_wait_warp(&p.full_b[sb], phb, p.abort_flag, a.status)) { ok = false; break; }
+                    tc_fence_after();
+                    blo = blo0 + (uint32_t)(sb * a.rsteps) * bs16;
+                }
+                const uint32_t acc = (in_seg > 0 || kh > 0) ? 1u : 0u;
+                if (KW > 0) {
+#pragma unroll
+                    for (int kw = 0; kw < KW; ++kw)
+#pragma unroll
+                        for (int j = 0; j < H; ++j) {
+                            const uint32_t al = ar + kw + j * half, bl = blo + (kw * H + j) * bs16;
+                            const uint32_t ac = (kw || j) ? 1u : acc;
+                            mma_bf16_ss_elect(d, ahi | al, bhi | bl, idesc, ac);
+                            if (MT == 2) mma_bf16_ss_elect(d + (uint32_t)a.tmem_stride, ahi | (al + 128u), bhi | bl, idesc, ac);
+                        }
+                } else {
+                    for (int i = 0; i < a.rsteps; ++i) {
+                        const int kw = i / a.h16;
+                        const uint32_t al = ar + kw + (i - kw * a.h16) * half, bl = blo + i * bs16;
+                        const uint32_t ac = i > 0 ? 1u : acc;
+                        mma_bf16_ss_elect(d, ahi | al, bhi | bl, idesc, ac);
+                        if (MT == 2) mma_bf16_ss_elect(d + (uint32_t)a.tmem_stride, ahi | (al + 128u), bhi | bl, idesc, ac);
+                    }
+                }
+                ar += (uint32_t)a.gr.Wb;
+                blo += (uint32_t)a.rsteps * bs16;
+                if (!resident) {
+                    mma_commit_elect(&p.empty_b[sb]);
+                    if (++sb == p.stages_b) { sb = 0; phb ^= 1u; }
+                }
+            }
+            if (!ok) break;
+            mma_commit_elect(&p.empty_a[s]);
+            if (++s == a.stages_a) { s = 0; ph ^= 1u; }
+            if (++in_seg == a.sps || uniform(st + 1 == nst)) {
+                mma_commit_elect(&p.acc_full[ab]);
+                if (++ab == 2) { ab = 0; acc_ph ^= 1u; }
+                in_seg = 0;
+            }
+        }
+    }
+}
+
+template <bool OUT_BF16, int MT>
+__global__ void __launch_bounds__(kGcThreads, 1)
+    k_grid_conv(const __grid_constant__ GcArgs a)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const uint32_t bstep = (uint32_t)a.bn * 32u;  // one step of the weights
+    uint8_t* sB = smem;
+    uint8_t* sA = sB + (size_t)a.cap_b * bstep;
+    int* t_off = reinterpret_cast<int*>(sA + (size_t)a.stages_a * a.a_stride);
+    float* t_bias = reinterpret_cast<float*>(t_off + 256);
+    int* z_off = reinterpret_cast<int*>(t_bias + 256);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(z_off + kGcZcap);
+    uint64_t* full_a = bars;
+    uint64_t* empty_a = full_a + kGcMaxA;
+    uint64_t* full_b = empty_a + kGcMaxA;
+    uint64_t* empty_b = full_b + kGcMaxB;
+    uint64_t* acc_full = empty_b + kGcMaxB;
+    uint64_t* acc_empty = acc_full + 2;
+    uint64_t* b_full = acc_empty + 2;
+    uint64_t* b_empty = b_full + 1;
+    uint64_t* drain = b_empty + 1;
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kGcMaxA; ++s) { mbar_init(&full_a[s], 1); mbar_init(&empty_a[s], 1); }
+        for (int s = 0; s < kGcMaxB; ++s) { mbar_init(&full_b[s], 1); mbar_init(&empty_b[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], kGcEpiWarps); }
+        mbar_init(b_full, 1);
+        mbar_init(b_empty, 1);
+        mbar_init(drain, 1);
+        *abort_flag = 0;
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(tmem_holder, (uint32_t)a.tmem_cols);
+        tmem_relinquish();
+    }
+    // Nothing above reads global memory: it overlaps the previous kernel's tail.
+    pdl_wait();
+    pdl_trigger();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_holder;
+    // The weights of a group stay in shared memory when there is one column
+    // tile and every group's (as many steps as its channels need) fit.
+    int most = 0;
+    for (int g = 0; g < a.groups; ++g) most = max(most, gc_blocks(a, g) * a.gr.KT * a.spt);
+    const bool resident = a.ntiles == 1 && uniform(most <= a.cap_b);
+    const int stages_b = min(a.cap_b / a.rsteps, kGcMaxB);
+
+    if (warp == 0) {
+        // --------------------------------------------------- slab producer
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        uint32_t last = 0, issued = 0;  // bit s: parity of the last copy into stage s; whether there was one
+        for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x) {
+            int g, nt, mt;
+            gc_unit(a, u, g, nt, mt);
+            if (__ldg(a.counts + 2 * g) <= nt * a.bn) continue;
+            const int nblk = gc_blocks(a, g);
+            const __nv_bfloat16* src = a.src + (size_t)g * a.gstride + (size_t)mt * (MT * 128) * 8;
+            for (int c = 0; ok && c < nblk; ++c) {
+                for (int kt = 0; kt < a.gr.KT; ++kt) {
+                    if (!mbar_wait_warp(&empty_a[s], ph ^ 1u, abort_flag, a.status)) { ok = false; break; }
+                    if (lane == 0) mbar_arrive_expect_tx(&full_a[s], (uint32_t)a.a_bytes);
+                    __syncwarp();
+                    if (lane < a.cb / 8)
+                        bulk_load(smem_u32(sA + (size_t)s * a.a_stride) + (uint32_t)(lane * a.sp * 16),
+                                  src + ((size_t)(c * (a.cb / 8) + lane) * a.gr.slots + (size_t)kt * a.gr.HWb) * 8,
+                                  (uint32_t)a.sp * 16u, &full_a[s]);
+                    last = (last & ~(1u << s)) | (ph << s);
+                    issued |= 1u << s;
+                    if (++s == a.stages_a) { s = 0; ph ^= 1u; }
+                }
+            }
+        }
+        // every copy issued has landed before the CTA retires
+        for (int q = 0; q < a.stages_a; ++q) {
+            if (!(issued & (1u << q))) continue;
+            const unsigned long long t0 = globaltimer();
+            while (!mbar_try_wait(&full_a[q], (last >> q) & 1u) && globaltimer() - t0 < kWaitLimitNs) {}
+        }
+        __syncwarp();
+    } else if (warp == 2) {
+        // ------------------------------------------------- weight producer
+        if (lane == 0 && resident) {
+            int cur = -1, loads = 0;
+            uint32_t e_ph = 0;
+            for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+                int g, nt, mt;
+                gc_unit(a, u, g, nt, mt);
+                const int nst = gc_blocks(a, g) * a.gr.KT;
+                if (__ldg(a.counts + 2 * g) <= 0 || nst == 0 || g == cur) continue;
+                if (loads > 0) {
+                    if (!mbar_wait(b_empty, e_ph, abort_flag, a.status)) break;
+                    e_ph ^= 1u;
+                }
+                const uint32_t sbytes = bstep * (uint32_t)a.spt;
+                mbar_arrive_expect_tx(b_full, sbytes * (uint32_t)nst);
+                const char* w = reinterpret_cast<const char*>(a.wd) + (size_t)g * a.ksteps * bstep;
+                for (int i = 0; i < nst; ++i)
+                    bulk_load(smem_u32(sB) + (uint32_t)i * sbytes, w + (size_t)i * sbytes, sbytes, b_full);
+                cur = g;
+                ++loads;
+            }
+            if (loads > 0) {
+                const unsigned long long t0 = globaltimer();
+                while (!mbar_try_wait(b_full, (uint32_t)((loads - 1) & 1)) && globaltimer() - t0 < kWaitLimitNs) {}
+            }
+        } else if (lane == 0) {
+            int s = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            uint32_t last = 0, issued = 0;
+            const uint32_t sbytes = bstep * (uint32_t)a.rsteps;
+            for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x) {
+                int g, nt, mt;
+                gc_unit(a, u, g, nt, mt);
+                if (__ldg(a.counts + 2 * g) <= nt * a.bn) continue;
+                const int nb = gc_blocks(a, g) * a.gr.KT * a.gr.KH;
+                const char* w = reinterpret_cast<const char*>(a.wd) + (size_t)(g * a.ntiles + nt) * a.ksteps * bstep;
+                for (int i = 0; i < nb; ++i) {
+                    if (!mbar_wait(&empty_b[s], ph ^ 1u, abort_flag, a.status)) { ok = false; break; }
+                    mbar_arrive_expect_tx(&full_b[s], sbytes);
+                    bulk_load(smem_u32(sB) + (uint32_t)s * sbytes, w + (size_t)i * sbytes, sbytes, &full_b[s]);
+                    last = (last & ~(1u << s)) | (ph << s);
+                    issued |= 1u << s;
+                    if (++s == stages_b) { s = 0; ph ^= 1u; }
+                }
+            }
+            for (int q = 0; q < stages_b; ++q) {
+                if (!(issued & (1u << q))) continue;
+                const unsigned long long t0 = globaltimer();
+                while (!mbar_try_wait(&full_b[q], (last >> q) & 1u) && globaltimer() - t0 < kWaitLimitNs) {}
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ------------------------------------------------------- MMA issuer
+        const GcPipe p{full_a, empty_a, full_b, empty_b, acc_full, acc_empty, b_full, b_empty, abort_flag,
+                       smem_u32(sA), smem_u32(sB), tmem_base, stages_b};
+        const int row = a.gr.KW * 8 + a.h16;
+        // (resident or streamed weights: two loops each, so that the choice is not in them)
+#define SADMM_ROW(KW, H)                                       \
+    if (row == KW * 8 + H) {                                   \
+        if (resident) gc_issue<KW, H, MT>(a, p, true);         \
+        else gc_issue<KW, H, MT>(a, p, false);                 \
+    } else
+        SADMM_ROW(1, 1) SADMM_ROW(1, 2) SADMM_ROW(1, 3) SADMM_ROW(1, 4)
+        SADMM_ROW(3, 1) SADMM_ROW(3, 2) SADMM_ROW(3, 3) SADMM_ROW(3, 4)
+        SADMM_ROW(5, 1) SADMM_ROW(5, 2)
+        if (resident) gc_issue<0, 0, MT>(a, p, true);
+        else gc_issue<0, 0, MT>(a, p, false);
+#undef SADMM_ROW
+        // Every MMA issued has completed before TMEM is freed.
+        mma_commit_elect(drain);
+        if (lane == 0) {
+            const unsigned long long t0 = globaltimer();
+            while (!mbar_try_wait(drain, 0) && globaltimer() - t0 < kWaitLimitNs) {}
+        }
+        __syncwarp();
+    } else {
+        // --------------------------------------------------------- epilogue
+        // Two warps per TMEM lane quadrant: with one pixel tile they take its
+        // 16-column chunks in turn, with two a tile each.
+        const int q4 = warp & 3;
+        const int h = (warp - 3) >> 2;
+        const int et = threadIdx.x - 3 * 32;
+        int ab = 0, key = -1;
+        uint32_t acc_ph = 0;
+        bool alive = true;
+        for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+            int g, nt, mt;
+            gc_unit(a, u, g, nt, mt);
+            const int cnt = min(a.bn, __ldg(a.counts + 2 * g) - nt * a.bn);
+            const int zc = nt == 0 ? __ldg(a.counts + 2 * g + 1) : 0;
+            if (g * a.ntiles + nt != key) {
+                key = g * a.ntiles + nt;
+                asm volatile("bar.sync 1, %0;" ::"n"(kGcEpiWarps * 32) : "memory");  // the old tables are read
+                for (int i = et; i < cnt; i += kGcEpiWarps * 32) {
+                    const int p = __ldg(a.colmap + (g * a.ntiles + nt) * a.bn + i);
+                    t_off[i] = p >= 0 ? p * a.plane : 0;
+                    t_bias[i] = (p >= 0 && a.bias) ? __ldg(a.bias + p) : 0.0f;
+                }
+                for (int z = et; z < min(zc, kGcZcap); z += kGcEpiWarps * 32)
+                    z_off[z] = __ldg(a.zmap + g * a.zstride + z) * a.plane;
+                asm volatile("bar.sync 1, %0;" ::"n"(kGcEpiWarps * 32) : "memory");
+            }
+            const int q = mt * (MT * 128) + (MT == 2 ? h * 128 : 0) + q4 * 32 + lane;
+            int n, t, hh, w;
+            grid_decode(a.gr, q, n, t, hh, w);
+            const bool valid = q < a.gr.L && t < a.VT && hh < a.VH && w < a.VW;
+            const long long pix =
+                valid ? (long long)n * a.planes * a.plane + (long long)t * a.VHW + (long long)hh * a.VW + w : 0;
+            float* yf = reinterpret_cast<float*>(a.out) + pix;
+            __nv_bfloat16* yh = reinterpret_cast<__nv_bfloat16*>(a.out) + pix;
+            const YCheck yc{pix, a.out_total, a.status};
+            // zero planes, while the item's MMAs run
+            if (alive && valid) {
+                for (int z = MT == 2 ? 0 : h; z < zc; z += MT == 2 ? 1 : 2) {
+                    const long long off = z < kGcZcap ? z_off[z] : (long long)__ldg(a.zmap + g * a.zstride + z) * a.plane;
+                    if (!y_ok(yc, off)) continue;
+                    if (OUT_BF16)
+                        yh[off] = __float2bfloat16_rn(0.0f);
+                    else
+                        __stcs(yf + off, 0.0f);
+                }
+            }
+            if (cnt <= 0) continue;
+            const int nch = (cnt + kEpiCols - 1) / kEpiCols;
+            const int nst = gc_blocks(a, g) * a.gr.KT;
+            float v[8][kEpiCols];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+#pragma unroll
+                for (int j = 0; j < kEpiCols; ++j) v[k][j] = 0.0f;
+            for (int st = 0; alive && st < nst; st += a.sps) {
+                // warp-uniform outcome: the TMEM loads below are .sync.aligned
+                if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[ab], acc_ph, abort_flag, a.status))) {
+                    alive = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t taddr = tmem_base + (uint32_t)((ab * MT + (MT == 2 ? h : 0)) * a.tmem_stride) +
+                                       ((uint32_t)(q4 * 32) << 16);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int c = MT == 2 ? k : 2 * k + h;
+                    if (c < nch) {
+                        uint32_t r[kEpiCols];
+                        tmem_ld_32x32b_x16(taddr + (uint32_t)(c * kEpiCols), r);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int j = 0; j < kEpiCols; ++j) v[k][j] += __uint_as_float(r[j]);
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acc_empty[ab]);
+                if (++ab == 2) { ab = 0; acc_ph ^= 1u; }
+            }
+            uint32_t nan = 0;  // chunks with a NaN
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int c = MT == 2 ? k : 2 * k + h;
+                if (alive && valid && c < nch) {
+                    bool bad = false;
+#pragma unroll
+                    for (int j = 0; j < kEpiCols; ++j) bad |= v[k][j] != v[k][j];
+                    if (bad) nan |= 1u << k;
+                    store_cols<OUT_BF16>(v[k], c * kEpiCols, cnt, t_off, t_bias, a.relu, yf, yh, yc);
+                }
+            }
+            if (nan) {
+                const int kch = a.kcounts ? __ldg(a.kcounts + 2 * g) : a.ncb * a.cb;
+                for (int i = 0; i < nch * kEpiCols; ++i) {
+                    const int c = i / kEpiCols;
+                    if (i >= cnt || (MT == 1 && (c & 1) != h) || !((nan >> (MT == 2 ? c : c >> 1)) & 1u)) continue;
+                    float e = grid_exact(a.wd + (size_t)(g * a.ntiles + nt) * a.ksteps * a.bn * 16, a.bn, i,
+                                         a.src + (size_t)g * a.gstride, q, kch, a.cb, a.gr.KT, a.gr.KH, a.gr.KW, a.gr.HWb,
+                                         a.gr.Wb, a.gr.slots) + t_bias[i];
+                    if (a.relu) e = fmaxf(e, 0.0f);
+                    if (!y_ok(yc, t_off[i])) continue;
+                    if (OUT_BF16)
+                        yh[t_off[i]] = __float2bfloat16_rn(e);
+                    else
+                        yf[t_off[i]] = e;
+                }
+            }
+            __syncwarp();
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, (uint32_t)a.tmem_cols);
+    }
+}
+
+// Grid copy of x.  Thread t of block (bx, by): slot 256*bx + t, two chunks of
+// conv group by / pairs (16 loads in flight, each coalesced along the row).
+__global__ void __launch_bounds__(256) k_grid_x(const __nv_bfloat16* __restrict__ x, const int* __restrict__ colidx,
+                                                const Grid gr, int C, int Cg, int nck, int chunks, int taps,
+                                                long long x_total, int* status, __nv_bfloat16* __restrict__ xs)
+{
+    __shared__ int s_off[16];  // channel plane offset (-1: zero)
+    pdl_wait();  // after the kernel before it in the stream
+    const int pairs = (chunks + 1) / 2;
+    const int g = blockIdx.y / pairs, c0 = (blockIdx.y - g * pairs) * 2;
+    const int thw = gr.T * gr.H * gr.W;
+    if (threadIdx.x < 16) {
+        const int ci = c0 * 8 + threadIdx.x;
+        int ch = ci < nck ? ci : -1;
+        if (ch >= 0 && colidx) {
+            const int col = __ldg(colidx + ci * taps);
+            ch = col >= 0 ? col / taps : -1;
+        }
+        s_off[threadIdx.x] = ch >= 0 ? (g * Cg + ch) * thw : -1;
+    }
+    __syncthreads();
+    const int s = blockIdx.x * 256 + threadIdx.x;
+    if (s >= gr.slots) return;
+    int n, t, h, w;
+    grid_decode(gr, s, n, t, h, w);
+    const bool valid = n < gr.N && t >= gr.pt && h >= gr.ph && w >= gr.pw;
+    const long long base = (long long)n * C * thw + (long long)(t - gr.pt) * (gr.H * gr.W) +
+                           (long long)(h - gr.ph) * gr.W + (w - gr.pw);
+    const unsigned short* xi = reinterpret_cast<const unsigned short*>(x);
+    uint32_t v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const int off = s_off[e];
+        v[e] = (valid && off >= 0 && dbg_in(base + off, x_total, status)) ? (uint32_t)__ldg(xi + base + off) : 0u;
+    }
+    uint4* dst = reinterpret_cast<uint4*>(xs) + ((size_t)g * chunks + c0) * gr.slots + s;
+    dst[0] = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+    if (c0 + 1 < chunks)
+        dst[gr.slots] =
+            make_uint4(v[8] | (v[9] << 16), v[10] | (v[11] << 16), v[12] | (v[13] << 16), v[14] | (v[15] << 16));
+}
+
+template <bool OUT_BF16, int MT>
+cudaError_t launch_gc(const GcArgs& a, int grid, size_t smem, cudaStream_t s)
+{
+    auto kern = k_grid_conv<OUT_BF16, MT>;
+    static int configured_dev = -1;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (configured_dev != dev) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGcSmemLimit);
+        if (e != cudaSuccess) return e;
+        configured_dev = dev;
+    }
+    return launch_pdl(kern, dim3((unsigned)grid), dim3(kGcThreads), smem, s, a);
+}
+
+}  // namespace
+
+bool grid_conv_shape(const Grid& gr, int chans, int cols, int groups, int sms, GridConvShape* out)
+{
+    if (chans < 1 || cols < 1) return false;
+    GridConvShape r;
+    const int taps = gr.KH * gr.KW;
+    r.k16 = (chans + 15) / 16;
+    const long long ksteps = (long long)r.k16 * gr.KT * taps;
+    if (ksteps > (1 << 16)) return false;
+    r.ksteps = (int)ksteps;
+    const long long fixed = 1024 + kGcTables + kGcZcap * 4 + kGcBars;
+    const int n16 = (int)round_up(cols, 16);
+    if ((long long)(256 + (gr.KH - 1) * gr.Wb + gr.KW) >= (1 << 14)) return false;  // operand stride field
+    // The tiling of least estimated time: rounds of items over the SMs, each
+    // item the longest of its MMAs (M = 128: the operands' shared-memory reads,
+    // 32 + N/4 cycles, or N/2 at the tensor rate; about 400 more for a stage's
+    // waits and commits), its stores (25 cycles per column and tile: 512 bytes
+    // at 20 a cycle) and its streamed weights (32 bytes per step and column at
+    // about 40 a cycle).  A block is as many 16s of channels as divide them and
+    // keep a stage to one accumulation segment.
+    long long best = -1;
+    for (int mt = 1; mt <= 2; ++mt)
+        for (int m = 4; m >= 1; --m) {
+            if (r.k16 % m != 0 || (taps * m > kGcSegSteps && m > 1)) continue;
+            const int rsteps = gr.KW * m;
+            const long long stride =
+                round_up((long long)(mt * 128 + (gr.KH - 1) * gr.Wb + gr.KW - 1) * 16 * (m * 2), 128);
+            const int nt0 = (n16 + 256 / mt - 1) / (256 / mt);
+            for (int nt = nt0; nt <= nt0 + 3; ++nt) {
+                const int bn = (int)round_up((n16 + nt - 1) / nt, 16);
+                if (nt > nt0 && bn < 48) break;
+                // three slabs and three slots of weights, two of each where that is too much
+                long long room = kGcSmemLimit - fixed - 3 * stride;
+                if (room < std::min(ksteps, 3ll * rsteps) * bn * 32) room = kGcSmemLimit - fixed - 2 * stride;
+                if (room < std::min(ksteps, 2ll * rsteps) * bn * 32) continue;
+                const long long cap = std::min<long long>(room / (bn * 32), ksteps);
+                const bool res = nt == 1 && cap >= ksteps;
+                const long long units = (gr.L + mt * 128 - 1) / (mt * 128) * nt * groups;
+                const long long mma = ksteps * mt * std::max(32 + bn / 4, bn / 2) + r.k16 / m * gr.KT * 400;
+                const long long st = 25ll * mt * bn;
+                const long long item = std::max(std::max(mma, st), res ? 0 : ksteps * bn * 32 / 40);
+                const long long cost = (units + sms - 1) / sms * item + std::min(mma, st);
+                if (best < 0 || cost < best) {
+                    best = cost;
+                    r.mt = mt;
+                    r.cb = 16 * m;
+                    r.bn = bn;
+                    r.ntiles = nt;
+                    r.cap_b = (int)cap;
+                    const long long left = kGcSmemLimit - fixed - cap * bn * 32;
+                    r.stages_a = (int)std::min<long long>(kGcMaxA, left / stride);
+                    r.smem = (size_t)(fixed + cap * bn * 32 + r.stages_a * stride);
+                }
+            }
+        }
+    if (best < 0) return false;
+    r.npad = r.bn * r.ntiles;
+    *out = r;
+    return true;
+}
+
+sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const GridConvCall& c, cudaStream_t s)
+{
+    GcArgs a;
+    memset(&a, 0, sizeof(a));
+    a.gr = gr;
+    a.src = c.src;
+    a.wd = c.wd;
+    a.out = c.out;
+    a.bias = c.bias;
+    a.colmap = c.colmap;
+    a.zmap = c.zmap;
+    a.zstride = c.zstride;
+    a.counts = c.counts;
+    a.kcounts = c.kcounts;
+    a.status = device_status_ptr();
+    a.out_total = c.out_total;
+    a.gstride = (long long)c.chunks * gr.slots * 8;
+    a.groups = c.groups;
+    a.planes = c.planes;
+    a.VT = c.VT;
+    a.VH = c.VH;
+    a.VW = c.VW;
+    a.VHW = c.VH * c.VW;
+    a.plane = c.VT * c.VH * c.VW;
+    a.bn = sh.bn;
+    a.ksteps = sh.ksteps;
+    a.ntiles = sh.ntiles;
+    a.mtiles = (gr.L + sh.mt * 128 - 1) / (sh.mt * 128);
+    const long long units = (long long)a.mtiles * sh.ntiles * c.groups;
+    if (units >= (1ll << 31) - (1ll << 20)) return SADMM_EUNSUPPORTED;
+    a.units = (int)units;
+    a.mt_div = make_fastdiv((uint32_t)a.mtiles);
+    a.nt_div = make_fastdiv((uint32_t)a.ntiles);
+    a.cb = sh.cb;
+    a.ncb = sh.k16 * 16 / sh.cb;
+    a.sp = sh.mt * 128 + (gr.KH - 1) * gr.Wb + gr.KW - 1;
+    a.h16 = sh.cb / 16;
+    a.rsteps = gr.KW * a.h16;
+    a.spt = gr.KH * a.rsteps;
+    a.sps = std::max(1, kGcSegSteps / a.spt);
+    a.cap_b = sh.cap_b;
+    a.stages_a = sh.stages_a;
+    a.a_bytes = a.sp * 16 * (sh.cb / 8);
+    a.a_stride = (int)round_up(a.a_bytes, 128);
+    a.tmem_stride = (int)round_up(sh.bn, 32);
+    int cols = 32;
+    while (cols < 2 * sh.mt * a.tmem_stride) cols <<= 1;
+    a.tmem_cols = cols;
+    a.relu = c.relu ? 1 : 0;
+    long long grid = c.ctas > 0 ? c.ctas : device_sm_count();
+    if (grid > units) grid = units;
+    cudaError_t e;
+    if (sh.mt == 2)
+        e = c.out_bf16 ? launch_gc<true, 2>(a, (int)grid, sh.smem, s) : launch_gc<false, 2>(a, (int)grid, sh.smem, s);
+    else
+        e = c.out_bf16 ? launch_gc<true, 1>(a, (int)grid, sh.smem, s) : launch_gc<false, 1>(a, (int)grid, sh.smem, s);
+    return e == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
+}
+
+sadmm_status launch_grid_x(const Grid& gr, const Geometry& g, const void* x, const int* colidx, int nck, int chunks,
+                           __nv_bfloat16* xs, cudaStream_t s)
+{
+    const long long rows = g.groups * ((chunks + 1) / 2);
+    if (rows > 65535) return SADMM_EUNSUPPORTED;
+    const cudaError_t e =
+        launch_pdl(k_grid_x, dim3((unsigned)((gr.slots + 255) / 256), (unsigned)rows), dim3(256), 0, s,
+                   static_cast<const __nv_bfloat16*>(x), colidx, gr, (int)g.c, (int)g.cg, nck, chunks, (int)g.taps,
+                   g.n * g.c * g.t * g.h * g.w, device_status_ptr(), xs);
+    return e == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
+}
+
+}  // namespace sadmm

@@ -1,0 +1,140 @@
+// grid.cuh -- the zero-padded pixel grid shared by the stride-1 kernels that
+// read shifted slabs (conv_grid.cu, bwd_grid.cu).
+//
+// A stride-1 layer's input and output gradient are rewritten as channel-octet
+// copies src[group][chunk][slot][8 channels] (bf16).  Slots run over the whole
+// batch in one line: image n, frame t, row h, column w of the input sit at slot
+//   n*P + (t + pt)*HWb + (h + ph)*Wb + (w + pw),
+// Wb = W + pw, Hb = H + ph, Tb = T + pt, HWb = Hb*Wb, P = Tb*HWb.  Only the
+// leading zeros of each row, frame and image are stored: the trailing ones are
+// the next row's leading ones (pads are at most K - 1).  Output pixel
+// (n, ot, oh, ow) is grid pixel q = n*P + ot*HWb + oh*Wb + ow and its tap
+// (kt, kh, kw) reads slot q + kt*HWb + kh*Wb + kw, whatever the pixel: every
+// tap is one shift of the whole line.  The output gradient sits D0 slots later
+// (the flipped kernel's leading pad), so the same line serves the input
+// gradient (a conv with the flipped taps) and, read from slot D0 on, the
+// weight gradient.
+#pragma once
+
+#include "common.cuh"
+#include "conv_common.cuh"
+#include "internal.h"
+
+namespace sadmm {
+
+struct Grid {
+    int N, T, H, W, OT, OH, OW, KT, KH, KW, pt, ph, pw;
+    int Wb, HWb, P;
+    int L;         // grid pixels N*P
+    int slots;     // slots of a chunk, every one written: L to 256, the largest shift and 16 more, to 8
+    int D0;        // slot of output pixel 0 in the output gradient's copy
+    int maxshift;  // the last tap's shift
+    FastDiv p_div, hw_div, w_div;
+};
+
+// The grid of a layer; false when it has none (a stride above 1, or a pad of K or more).
+inline bool grid_of(const Geometry& g, Grid* out)
+{
+    if (g.st != 1 || g.sh != 1 || g.sw != 1 || g.pt >= g.kt || g.ph >= g.kh || g.pw >= g.kw) return false;
+    const long long wb = g.w + g.pw, hb = g.h + g.ph, tb = g.t + g.pt;
+    const long long p = wb * hb * tb, L = g.n * p;
+    const long long ms = (g.kt - 1) * hb * wb + (g.kh - 1) * wb + g.kw - 1;
+    const long long slots = round_up(round_up(L, 256) + ms + 16, 8);
+    if (slots >= (1ll << 30)) return false;
+    Grid r;
+    r.N = (int)g.n; r.T = (int)g.t; r.H = (int)g.h; r.W = (int)g.w;
+    r.OT = (int)g.ot; r.OH = (int)g.oh; r.OW = (int)g.ow;
+    r.KT = (int)g.kt; r.KH = (int)g.kh; r.KW = (int)g.kw;
+    r.pt = (int)g.pt; r.ph = (int)g.ph; r.pw = (int)g.pw;
+    r.Wb = (int)wb;
+    r.HWb = (int)(hb * wb);
+    r.P = (int)p;
+    r.L = (int)L;
+    r.slots = (int)slots;
+    r.maxshift = (int)ms;
+    r.D0 = (int)((g.kt - 1 - g.pt) * hb * wb + (g.kh - 1 - g.ph) * wb + (g.kw - 1 - g.pw));
+    r.p_div = make_fastdiv((uint32_t)p);
+    r.hw_div = make_fastdiv((uint32_t)(hb * wb));
+    r.w_div = make_fastdiv((uint32_t)wb);
+    *out = r;
+    return true;
+}
+
+// ---- slab GEMM over a grid copy (conv_grid.cu) ----
+// out[plane(col)][pixel] = bias + sum over the K columns of Wd[col][k] * src:
+// K column k = ((cb*KT + kt)*KH*KW + kh*KW + kw)*CB + ci reads channel
+// cb*CB + ci at shift kt*HWb + kh*Wb + kw.  Wd lies as the MMA reads it, a step
+// of 16 K columns at a time: [group][column tile][step][K half][bn][8].
+struct GridConvShape {
+    int cb;      // channels per block (multiple of 16)
+    int k16;     // 16-channel groups of the source (padded channels / 16)
+    int ksteps;  // MMA steps of 16 K columns
+    int mt;      // 128-pixel tiles per work item (1 or 2)
+    int bn, ntiles, npad;  // output columns per tile, tiles, and bn*ntiles
+    int cap_b;     // steps of weights shared memory holds: all of an item's stay there, or a ring streams
+    int stages_a;
+    size_t smem;
+};
+// The tiling for `chans` source channels and `cols` output columns per group
+// over `groups` groups; false when it does not fit.
+bool grid_conv_shape(const Grid& gr, int chans, int cols, int groups, int sms, GridConvShape* out);
+
+struct GridConvCall {
+    const __nv_bfloat16* src;  // [groups][chunks][slots][8]
+    int chunks;                // chunks per group (k16 * 2)
+    const __nv_bfloat16* wd;   // [groups][ntiles][ksteps][2][bn][8], -0.0 at pruned entries
+    void* out;
+    int out_bf16;
+    const float* bias;     // per plane, or NULL
+    int relu;
+    const int* colmap;     // [groups][npad] column -> plane of an image (-1: none)
+    const int* zmap;       // [groups][zstride] planes written as zeros
+    int zstride;
+    const int* counts;     // [groups][2] columns, zero planes
+    const int* kcounts;    // channels per group at [2*g] (NULL: all)
+    int groups, planes;    // planes per image of the output
+    int VT, VH, VW;        // its extents
+    long long out_total;
+    int ctas;
+};
+sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const GridConvCall& c, cudaStream_t s);
+
+// x (bf16 NCTHW) -> grid copy of `nck` channels per group (kept channels
+// colidx[ci*taps]/taps when colidx != NULL, else 0..nck-1), `chunks` chunks.
+sadmm_status launch_grid_x(const Grid& gr, const Geometry& g, const void* x, const int* colidx, int nck, int chunks,
+                           __nv_bfloat16* xs, cudaStream_t s);
+
+// ---- grid backward (bwd_grid.cu) ----
+size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g);  // 0: the layer takes the gathered backward
+sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const void* x, const void* dy, const void* y,
+                             int ydt, int relu, float* dW, float* db, float* dx, void* ws, cudaStream_t s);
+
+// ------------------------------------------------------------- device side --
+
+// Bulk copy of `bytes` (a multiple of 16) from 16-byte aligned global memory
+// into shared memory, completion as transaction bytes on `bar`.
+SADMM_DEV void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+
+// A condition every lane of the converged warp agrees on, as a vote: control
+// flow the compiler cannot prove warp-uniform keeps the issuing warp's
+// descriptors out of the uniform registers, and an MMA then takes about 140
+// cycles to issue instead of 50.
+SADMM_DEV bool uniform(bool c) { return __all_sync(0xffffffffu, c); }
+
+// Grid pixel q -> image and coordinates.
+SADMM_DEV void grid_decode(const Grid& gr, int q, int& n, int& t, int& h, int& w)
+{
+    n = (int)fdiv((uint32_t)q, gr.p_div);
+    int r = q - n * gr.P;
+    t = (int)fdiv((uint32_t)r, gr.hw_div);
+    r -= t * gr.HWb;
+    h = (int)fdiv((uint32_t)r, gr.w_div);
+    w = r - h * gr.Wb;
+}
+
+}  // namespace sadmm
