@@ -212,7 +212,7 @@ class LayerRun:
         cols_all = self.colkind != wl.COL_NONE and self.k_cols == G
         self.launches = (1 + (0 if rows_all else 1)
                          + (2 if self.colkind != wl.COL_NONE and not cols_all else 0) + 2
-                         + (2 if self.plan.splits > 1 or self.plan.xs_mode else 1))
+                         + (2 if self.plan.splits > 1 or self.plan.xs_mode or self.plan.gx_mode else 1))
 
     def flops(self):
         s = self.s

@@ -123,6 +123,18 @@ typedef struct {
     uint64_t tmap[16];    /* 128-byte TMA tensor map of the packed matrix       */
     uint64_t tmap_ws[16]; /* TMA map of the slab-ordered weights (xs_mode)      */
     uint64_t tmap_xs[16]; /* TMA map of the space-to-depth input (xs_mode)      */
+    /* Pixel-grid forward (gx_mode = 1, see sadmm_plan_init): its tiling and
+     * the regions of the device buffer it adds. */
+    int gx_mode;
+    int gx_cb;          /* channels per block of the contraction                */
+    int gx_mt;          /* 128-pixel tiles per work item                        */
+    int gx_bn, gx_ntiles; /* filters per tile, tiles per conv group             */
+    int gx_stages;      /* slabs in shared memory                               */
+    int gx_cap;         /* bytes of weights in shared memory                    */
+    int gx_smem;        /* shared memory of the kernel                          */
+    size_t off_gx;      /* grid copy of x [groups][chunk][slot][8] bf16         */
+    size_t off_gw;      /* weights [groups][tile][step][2][rows][8] bf16        */
+    size_t off_gcol;    /* K column -> GEMM column (-1 pruned, -2 none) int32   */
 } sadmm_plan;
 
 /* ------------------------------------------------------------------------ */
@@ -365,6 +377,18 @@ sadmm_status sadmm_sparse_conv_fwd(const sadmm_conv_desc* d, const void* plan, c
  * slab GEMM has xs_r * xs_q * xs_cs columns (the taps and channels past the
  * kernel or the kept channels hold zero weights): the same sums as the
  * gathered path, in another order.  No K' split or stream-K in this path.
+ */
+/*
+ * Pixel-grid path (plan->gx_mode = 1): a stride-1 layer whose pads are below
+ * its kernel extents and whose output tiles fill the device, where the rule in
+ * conv_grid.cu estimates it to be the faster.  The forward rewrites the kept
+ * channels of x as a channel-octet copy on one zero-padded line of pixels in the
+ * plan's buffer, on which every tap is a shift, and contracts shifted slabs of
+ * it on the tensor cores with the kept filters' weights of every tap, zero at
+ * the pruned columns.  A product of a pruned column never reaches the output,
+ * infinities and NaN included: the sums are the gathered path's, in another
+ * order.  The plan still holds the gathered packing (the chunked backward and
+ * larger strides use it).  Both passes belong to SADMM_FWD_REST.
  */
 sadmm_status sadmm_plan_init(sadmm_plan* plan, const sadmm_conv_desc* d,
                              int n_filt, int colkind, int n_colgroups);

@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "grid.cuh"
 #include "internal.h"
 
 namespace sadmm {
@@ -475,6 +476,15 @@ sadmm_status sadmm_plan_init_ctas(sadmm_plan* plan, const sadmm_conv_desc* d, in
                     p.off_sk = take((size_t)bytes);
                 }
             }
+        }
+    }
+    if (!p.xs_mode) {
+        size_t gx, gw, gcol;
+        if (grid_fwd_plan(g, &p, &gx, &gw, &gcol)) {
+            p.gx_mode = 1;
+            p.off_gx = take(gx);
+            p.off_gw = take(gw);
+            p.off_gcol = take(gcol);
         }
     }
     p.dev_bytes = off;

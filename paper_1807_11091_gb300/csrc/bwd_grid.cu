@@ -680,7 +680,7 @@ bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, GridBwd* out)
     if (plan->n_cols < 1 || plan->n_filt < 1 || g.taps > 256) return false;
     if (!grid_of(g, &b.gr)) return false;
     b.nck = plan->colkind == SADMM_COL_CHANNEL ? plan->n_colgroups : (int)g.cg;
-    if (!grid_conv_shape(b.gr, plan->n_pad, b.nck, (int)g.groups, (int)kGwCtas, &b.cs)) return false;
+    if (!grid_conv_shape(b.gr, plan->n_pad, b.nck, b.nck, (int)g.groups, (int)kGwCtas, &b.cs)) return false;
     if (!wgrad_shape(b.gr, b.nck, plan->n_pad, (int)g.groups, &b.ws)) return false;
     b.dchunks = std::max(b.cs.k16 * 2, b.ws.nft * b.ws.nst / 8);
     b.nparts = (b.gr.slots + kDzSlots - 1) / kDzSlots;
@@ -850,6 +850,7 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         c.wd = wd;
         c.out = dx;
         c.colmap = colmap;
+        c.cstride = b.cs.npad;
         c.zmap = zmap;
         c.zstride = (int)g.cg;
         c.counts = counts2;

@@ -30,6 +30,7 @@
 
 #include "common.cuh"
 #include "conv_common.cuh"
+#include "grid.cuh"
 #include "internal.h"
 
 namespace sadmm {
@@ -897,7 +898,8 @@ sadmm_status launch_conv_fwd(const sadmm_plan* plan, const Geometry& g, const vo
                              int relu, void* y, int ydt, int phase, cudaStream_t s)
 {
     if (plan->xs_mode) return launch_conv_slab(plan, g, x, bias, relu, y, ydt, phase, s);
-    if (phase == SADMM_FWD_INPUT) return SADMM_OK;  // the gathered path reads x in its own kernel
+    if (phase == SADMM_FWD_INPUT) return SADMM_OK;  // the other paths read x in the rest
+    if (plan->gx_mode) return launch_grid_fwd(plan, g, x, bias, relu, y, ydt, s);
     if (g.groups > kMaxGroups) return SADMM_EUNSUPPORTED;
     const char* base = static_cast<const char*>(plan->dev);
     ConvArgs a;

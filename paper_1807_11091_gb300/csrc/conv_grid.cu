@@ -1,6 +1,6 @@
 // conv_grid.cu -- stride-1 convolution as a slab GEMM on the tensor cores: the
-// input gradient of a pruned layer (its forward with the taps flipped, over the
-// kept filters; Sec. 4, masked retraining).
+// forward of a pruned layer (Sec. 3) and its input gradient (the forward with
+// the taps flipped, over the kept filters; Sec. 4, masked retraining).
 //
 // GEMM row i of tile t is grid pixel 128t + i of the padded line (grid.cuh);
 // every tap of a block of CB channels is the same shared-memory slab of
@@ -66,6 +66,7 @@ struct GcArgs {
     int sp;             // slots of a slab
     int sps;            // stages per accumulation segment
     int cap_b, stages_a, a_bytes, a_stride;
+    int cstride;
     int tmem_stride, tmem_cols;
     int relu;
 };
@@ -107,12 +108,26 @@ SADMM_DEV void gc_unit(const GcArgs& a, int u, int& g, int& nt, int& mt)
     nt = t - g * a.ntiles;
 }
 
+template <bool OUT_BF16>
+SADMM_DEV void zero_at(float* yf, __nv_bfloat16* yh, const YCheck& yc, int off)
+{
+    if (!y_ok(yc, off)) return;
+    if (OUT_BF16)
+        yh[off] = __float2bfloat16_rn(0.0f);
+    else
+        __stcs(yf + off, 0.0f);
+}
+
+// Where an item's weights come from: shared memory for the whole group, a ring
+// slot per stage, or one per kernel row where two stages of them do not fit.
+enum { kResident, kStageSlots, kRowSlots };
+
 // The barriers and operand bases of a CTA, for its issuing warp.
 struct GcPipe {
     uint64_t *full_a, *empty_a, *full_b, *empty_b, *acc_full, *acc_empty, *b_full, *b_empty;
     volatile int* abort_flag;
     uint32_t sA, sB, tmem_base;
-    int stages_b;
+    int stages_b, bnr;
 };
 
 // The issuing warp's run over its work items.  The whole warp runs the loop,
@@ -123,17 +138,18 @@ struct GcPipe {
 // 120 and more with bounds the compiler cannot prove uniform).  KW = 0: any
 // other row, one MMA at a time.
 template <int KW, int H, int MT>
-SADMM_DEV void gc_issue(const GcArgs& a, const GcPipe& p, const bool resident)
+SADMM_DEV void gc_issue(const GcArgs& a, const GcPipe& p, const int mode)
 {
+    const bool resident = mode == kResident;
     int s = 0, sb = 0, ab = 0;
     uint32_t ph = 0, phb = 0, acc_ph = 0, bf_ph = 0;
     int cur = -1;
     bool ok = true;
     const uint64_t ad0 = sdesc_kmajor_none(p.sA, (uint32_t)a.sp * 16u, 128u);
-    const uint64_t bd0 = sdesc_kmajor_none(p.sB, (uint32_t)a.bn * 16u, 128u);
+    const uint64_t bd0 = sdesc_kmajor_none(p.sB, (uint32_t)p.bnr * 16u, 128u);
     const uint64_t ahi = ad0 & 0xffffffff00000000ull, bhi = bd0 & 0xffffffff00000000ull;
     const uint32_t alo0 = (uint32_t)ad0, blo0 = (uint32_t)bd0;
-    const uint32_t bs16 = (uint32_t)a.bn * 2u;   // one step of the weights, in 16-byte units
+    const uint32_t bs16 = (uint32_t)p.bnr * 2u;   // one step of the weights, in 16-byte units
     const uint32_t half = 2u * (uint32_t)a.sp;   // 16 channels of a slab
     for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x) {
         int g, nt, mt;
@@ -160,10 +176,10 @@ SADMM_DEV void gc_issue(const GcArgs& a, const GcPipe& p, const bool resident)
             tc_fence_after();
             uint32_t ar = alo0 + ((uint32_t)(s * a.a_stride) >> 4);
             for (int kh = 0; kh < a.gr.KH; ++kh) {
-                if (!resident) {
+                if (mode == kRowSlots || (mode == kStageSlots && kh == 0)) {
                     if (!mbar_wait_warp(&p.full_b[sb], phb, p.abort_flag, a.status)) { ok = false; break; }
                     tc_fence_after();
-                    blo = blo0 + (uint32_t)(sb * a.rsteps) * bs16;
+                    blo = blo0 + (uint32_t)(sb * (mode == kRowSlots ? a.rsteps : a.spt)) * bs16;
                 }
                 const uint32_t acc = (in_seg > 0 || kh > 0) ? 1u : 0u;
                 if (KW > 0) {
@@ -187,12 +203,16 @@ SADMM_DEV void gc_issue(const GcArgs& a, const GcPipe& p, const bool resident)
                 }
                 ar += (uint32_t)a.gr.Wb;
                 blo += (uint32_t)a.rsteps * bs16;
-                if (!resident) {
+                if (mode == kRowSlots) {
                     mma_commit_elect(&p.empty_b[sb]);
                     if (++sb == p.stages_b) { sb = 0; phb ^= 1u; }
                 }
             }
             if (!ok) break;
+            if (mode == kStageSlots) {
+                mma_commit_elect(&p.empty_b[sb]);
+                if (++sb == p.stages_b) { sb = 0; phb ^= 1u; }
+            }
             mma_commit_elect(&p.empty_a[s]);
             if (++s == a.stages_a) { s = 0; ph ^= 1u; }
             if (++in_seg == a.sps || uniform(st + 1 == nst)) {
@@ -210,9 +230,8 @@ __global__ void __launch_bounds__(kGcThreads, 1)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const uint32_t bstep = (uint32_t)a.bn * 32u;  // one step of the weights
     uint8_t* sB = smem;
-    uint8_t* sA = sB + (size_t)a.cap_b * bstep;
+    uint8_t* sA = sB + a.cap_b;
     int* t_off = reinterpret_cast<int*>(sA + (size_t)a.stages_a * a.a_stride);
     float* t_bias = reinterpret_cast<float*>(t_off + 256);
     int* z_off = reinterpret_cast<int*>(t_bias + 256);
@@ -253,10 +272,15 @@ __global__ void __launch_bounds__(kGcThreads, 1)
     const uint32_t tmem_base = *tmem_holder;
     // The weights of a group stay in shared memory when there is one column
     // tile and every group's (as many steps as its channels need) fit.
+    const int bnr = grid_rows(a.counts, a.groups, a.ntiles, a.bn);
+    const uint32_t bstep = (uint32_t)bnr * 32u;               // one step of the weights
+    const size_t btile = (size_t)a.ksteps * a.bn * 32;        // room of a tile's weights
     int most = 0;
     for (int g = 0; g < a.groups; ++g) most = max(most, gc_blocks(a, g) * a.gr.KT * a.spt);
-    const bool resident = a.ntiles == 1 && uniform(most <= a.cap_b);
-    const int stages_b = min(a.cap_b / a.rsteps, kGcMaxB);
+    const bool resident = a.ntiles == 1 && uniform(most * (int)bstep <= a.cap_b);
+    const bool stage_slots = uniform(2 * a.spt * (int)bstep <= a.cap_b);
+    const int slot = stage_slots ? a.spt : a.rsteps;  // MMA steps of a ring slot
+    const int stages_b = min(a.cap_b / (int)(bstep * slot), kGcMaxB);
 
     if (warp == 0) {
         // --------------------------------------------------- slab producer
@@ -308,7 +332,7 @@ __global__ void __launch_bounds__(kGcThreads, 1)
                 }
                 const uint32_t sbytes = bstep * (uint32_t)a.spt;
                 mbar_arrive_expect_tx(b_full, sbytes * (uint32_t)nst);
-                const char* w = reinterpret_cast<const char*>(a.wd) + (size_t)g * a.ksteps * bstep;
+                const char* w = reinterpret_cast<const char*>(a.wd) + (size_t)g * btile;
                 for (int i = 0; i < nst; ++i)
                     bulk_load(smem_u32(sB) + (uint32_t)i * sbytes, w + (size_t)i * sbytes, sbytes, b_full);
                 cur = g;
@@ -323,17 +347,17 @@ __global__ void __launch_bounds__(kGcThreads, 1)
             uint32_t ph = 0;
             bool ok = true;
             uint32_t last = 0, issued = 0;
-            const uint32_t sbytes = bstep * (uint32_t)a.rsteps;
+            const uint32_t rbytes = bstep * (uint32_t)slot;
             for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x) {
                 int g, nt, mt;
                 gc_unit(a, u, g, nt, mt);
                 if (__ldg(a.counts + 2 * g) <= nt * a.bn) continue;
-                const int nb = gc_blocks(a, g) * a.gr.KT * a.gr.KH;
-                const char* w = reinterpret_cast<const char*>(a.wd) + (size_t)(g * a.ntiles + nt) * a.ksteps * bstep;
+                const int nb = gc_blocks(a, g) * a.gr.KT * (stage_slots ? 1 : a.gr.KH);
+                const char* w = reinterpret_cast<const char*>(a.wd) + (size_t)(g * a.ntiles + nt) * btile;
                 for (int i = 0; i < nb; ++i) {
                     if (!mbar_wait(&empty_b[s], ph ^ 1u, abort_flag, a.status)) { ok = false; break; }
-                    mbar_arrive_expect_tx(&full_b[s], sbytes);
-                    bulk_load(smem_u32(sB) + (uint32_t)s * sbytes, w + (size_t)i * sbytes, sbytes, &full_b[s]);
+                    mbar_arrive_expect_tx(&full_b[s], rbytes);
+                    bulk_load(smem_u32(sB) + (uint32_t)s * rbytes, w + (size_t)i * rbytes, rbytes, &full_b[s]);
                     last = (last & ~(1u << s)) | (ph << s);
                     issued |= 1u << s;
                     if (++s == stages_b) { s = 0; ph ^= 1u; }
@@ -349,20 +373,21 @@ __global__ void __launch_bounds__(kGcThreads, 1)
     } else if (warp == 1) {
         // ------------------------------------------------------- MMA issuer
         const GcPipe p{full_a, empty_a, full_b, empty_b, acc_full, acc_empty, b_full, b_empty, abort_flag,
-                       smem_u32(sA), smem_u32(sB), tmem_base, stages_b};
+                       smem_u32(sA), smem_u32(sB), tmem_base, stages_b, bnr};
         const int row = a.gr.KW * 8 + a.h16;
-        // (resident or streamed weights: two loops each, so that the choice is not in them)
-#define SADMM_ROW(KW, H)                                       \
-    if (row == KW * 8 + H) {                                   \
-        if (resident) gc_issue<KW, H, MT>(a, p, true);         \
-        else gc_issue<KW, H, MT>(a, p, false);                 \
-    } else
+        const int mode = resident ? kResident : stage_slots ? kStageSlots : kRowSlots;
+        // (a loop for each, so that the choice is not in them)
+#define SADMM_ISSUE(KW, H)                                                 \
+    if (mode == kResident) gc_issue<KW, H, MT>(a, p, kResident);           \
+    else if (mode == kStageSlots) gc_issue<KW, H, MT>(a, p, kStageSlots);  \
+    else gc_issue<KW, H, MT>(a, p, kRowSlots);
+#define SADMM_ROW(KW, H) if (row == KW * 8 + H) { SADMM_ISSUE(KW, H) } else
         SADMM_ROW(1, 1) SADMM_ROW(1, 2) SADMM_ROW(1, 3) SADMM_ROW(1, 4)
         SADMM_ROW(3, 1) SADMM_ROW(3, 2) SADMM_ROW(3, 3) SADMM_ROW(3, 4)
         SADMM_ROW(5, 1) SADMM_ROW(5, 2)
-        if (resident) gc_issue<0, 0, MT>(a, p, true);
-        else gc_issue<0, 0, MT>(a, p, false);
+        { SADMM_ISSUE(0, 0) }
 #undef SADMM_ROW
+#undef SADMM_ISSUE
         // Every MMA issued has completed before TMEM is freed.
         mma_commit_elect(drain);
         if (lane == 0) {
@@ -389,7 +414,7 @@ __global__ void __launch_bounds__(kGcThreads, 1)
                 key = g * a.ntiles + nt;
                 asm volatile("bar.sync 1, %0;" ::"n"(kGcEpiWarps * 32) : "memory");  // the old tables are read
                 for (int i = et; i < cnt; i += kGcEpiWarps * 32) {
-                    const int p = __ldg(a.colmap + (g * a.ntiles + nt) * a.bn + i);
+                    const int p = __ldg(a.colmap + g * a.cstride + nt * a.bn + i);
                     t_off[i] = p >= 0 ? p * a.plane : 0;
                     t_bias[i] = (p >= 0 && a.bias) ? __ldg(a.bias + p) : 0.0f;
                 }
@@ -406,16 +431,22 @@ __global__ void __launch_bounds__(kGcThreads, 1)
             float* yf = reinterpret_cast<float*>(a.out) + pix;
             __nv_bfloat16* yh = reinterpret_cast<__nv_bfloat16*>(a.out) + pix;
             const YCheck yc{pix, a.out_total, a.status};
-            // zero planes, while the item's MMAs run
+            // zero planes, while the item's MMAs run: 16 at a time, the table read
+            // four offsets to a load
             if (alive && valid) {
-                for (int z = MT == 2 ? 0 : h; z < zc; z += MT == 2 ? 1 : 2) {
-                    const long long off = z < kGcZcap ? z_off[z] : (long long)__ldg(a.zmap + g * a.zstride + z) * a.plane;
-                    if (!y_ok(yc, off)) continue;
-                    if (OUT_BF16)
-                        yh[off] = __float2bfloat16_rn(0.0f);
-                    else
-                        __stcs(yf + off, 0.0f);
+                const int zt = min(zc, kGcZcap) & ~15;
+                for (int z = MT == 2 ? 0 : 16 * h; z < zt; z += MT == 2 ? 16 : 32) {
+#pragma unroll
+                    for (int j = 0; j < 16; j += 4) {
+                        const int4 o = *reinterpret_cast<const int4*>(z_off + z + j);
+                        zero_at<OUT_BF16>(yf, yh, yc, o.x);
+                        zero_at<OUT_BF16>(yf, yh, yc, o.y);
+                        zero_at<OUT_BF16>(yf, yh, yc, o.z);
+                        zero_at<OUT_BF16>(yf, yh, yc, o.w);
+                    }
                 }
+                for (int z = zt + (MT == 2 ? 0 : h); z < zc; z += MT == 2 ? 1 : 2)
+                    zero_at<OUT_BF16>(yf, yh, yc, z < kGcZcap ? z_off[z] : __ldg(a.zmap + g * a.zstride + z) * a.plane);
             }
             if (cnt <= 0) continue;
             const int nch = (cnt + kEpiCols - 1) / kEpiCols;
@@ -467,7 +498,7 @@ __global__ void __launch_bounds__(kGcThreads, 1)
                 for (int i = 0; i < nch * kEpiCols; ++i) {
                     const int c = i / kEpiCols;
                     if (i >= cnt || (MT == 1 && (c & 1) != h) || !((nan >> (MT == 2 ? c : c >> 1)) & 1u)) continue;
-                    float e = grid_exact(a.wd + (size_t)(g * a.ntiles + nt) * a.ksteps * a.bn * 16, a.bn, i,
+                    float e = grid_exact(a.wd + (size_t)(g * a.ntiles + nt) * btile / 2, bnr, i,
                                          a.src + (size_t)g * a.gstride, q, kch, a.cb, a.gr.KT, a.gr.KH, a.gr.KW, a.gr.HWb,
                                          a.gr.Wb, a.gr.slots) + t_bias[i];
                     if (a.relu) e = fmaxf(e, 0.0f);
@@ -548,7 +579,7 @@ cudaError_t launch_gc(const GcArgs& a, int grid, size_t smem, cudaStream_t s)
 
 }  // namespace
 
-bool grid_conv_shape(const Grid& gr, int chans, int cols, int groups, int sms, GridConvShape* out)
+bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups, int sms, GridConvShape* out)
 {
     if (chans < 1 || cols < 1) return false;
     GridConvShape r;
@@ -560,49 +591,53 @@ bool grid_conv_shape(const Grid& gr, int chans, int cols, int groups, int sms, G
     const long long fixed = 1024 + kGcTables + kGcZcap * 4 + kGcBars;
     const int n16 = (int)round_up(cols, 16);
     if ((long long)(256 + (gr.KH - 1) * gr.Wb + gr.KW) >= (1 << 14)) return false;  // operand stride field
+    const long long span = (gr.KH - 1) * gr.Wb + gr.KW - 1;
+    // A block: as many 16s of channels as divide them, keep a stage to one
+    // accumulation segment and its slab to 24 KB.
+    int m = 4;
+    while (m > 1 && (r.k16 % m != 0 || taps * m > kGcSegSteps || (128 + span) * 32 * m > 24576)) --m;
+    r.cb = 16 * m;
+    const int rsteps = gr.KW * m;
     // The tiling of least estimated time: rounds of items over the SMs, each
     // item the longest of its MMAs (M = 128: the operands' shared-memory reads,
-    // 32 + N/4 cycles, or N/2 at the tensor rate; about 400 more for a stage's
-    // waits and commits), its stores (25 cycles per column and tile: 512 bytes
-    // at 20 a cycle) and its streamed weights (32 bytes per step and column at
-    // about 40 a cycle).  A block is as many 16s of channels as divide them and
-    // keep a stage to one accumulation segment.
+    // 32 + N/4 cycles, or N/2 at the tensor rate, and 9 more as issued; about
+    // 400 a stage for its waits and commits), its stores (25 cycles per column
+    // and tile: 512 bytes at 20 a cycle) and its streamed weights (32 bytes per
+    // step and column at about 40 a cycle).
     long long best = -1;
-    for (int mt = 1; mt <= 2; ++mt)
-        for (int m = 4; m >= 1; --m) {
-            if (r.k16 % m != 0 || (taps * m > kGcSegSteps && m > 1)) continue;
-            const int rsteps = gr.KW * m;
-            const long long stride =
-                round_up((long long)(mt * 128 + (gr.KH - 1) * gr.Wb + gr.KW - 1) * 16 * (m * 2), 128);
-            const int nt0 = (n16 + 256 / mt - 1) / (256 / mt);
-            for (int nt = nt0; nt <= nt0 + 3; ++nt) {
-                const int bn = (int)round_up((n16 + nt - 1) / nt, 16);
-                if (nt > nt0 && bn < 48) break;
-                // three slabs and three slots of weights, two of each where that is too much
-                long long room = kGcSmemLimit - fixed - 3 * stride;
-                if (room < std::min(ksteps, 3ll * rsteps) * bn * 32) room = kGcSmemLimit - fixed - 2 * stride;
-                if (room < std::min(ksteps, 2ll * rsteps) * bn * 32) continue;
-                const long long cap = std::min<long long>(room / (bn * 32), ksteps);
-                const bool res = nt == 1 && cap >= ksteps;
-                const long long units = (gr.L + mt * 128 - 1) / (mt * 128) * nt * groups;
-                const long long mma = ksteps * mt * std::max(32 + bn / 4, bn / 2) + r.k16 / m * gr.KT * 400;
-                const long long st = 25ll * mt * bn;
-                const long long item = std::max(std::max(mma, st), res ? 0 : ksteps * bn * 32 / 40);
-                const long long cost = (units + sms - 1) / sms * item + std::min(mma, st);
-                if (best < 0 || cost < best) {
-                    best = cost;
-                    r.mt = mt;
-                    r.cb = 16 * m;
-                    r.bn = bn;
-                    r.ntiles = nt;
-                    r.cap_b = (int)cap;
-                    const long long left = kGcSmemLimit - fixed - cap * bn * 32;
-                    r.stages_a = (int)std::min<long long>(kGcMaxA, left / stride);
-                    r.smem = (size_t)(fixed + cap * bn * 32 + r.stages_a * stride);
-                }
+    for (int mt = 1; mt <= 2; ++mt) {
+        const long long stride = round_up((mt * 128 + span) * 16 * (m * 2), 128);
+        const int nt0 = (n16 + 256 / mt - 1) / (256 / mt);
+        for (int nt = nt0; nt <= nt0 + 3; ++nt) {
+            const int bn = (int)round_up((n16 + nt - 1) / nt, 16);
+            if (nt > nt0 && bn < 48) break;
+            // three slabs and three slots of weights, two of each where that is too much
+            long long room = kGcSmemLimit - fixed - 3 * stride;
+            if (room < std::min(ksteps, 3ll * rsteps) * bn * 32) room = kGcSmemLimit - fixed - 2 * stride;
+            if (room < std::min(ksteps, 2ll * rsteps) * bn * 32) continue;
+            const long long cap = std::min(room / 128 * 128, ksteps * bn * 32);
+            const int lb = nt == 1 ? std::min(bn, (int)round_up(likely, 16)) : bn;  // rows a tile is likely to have
+            const bool res = nt == 1 && cap >= ksteps * lb * 32;
+            const long long units = (gr.L + mt * 128 - 1) / (mt * 128) * nt * groups;
+            const long long mma = ksteps * mt * (std::max(32 + lb / 4, lb / 2) + 9) + r.k16 / m * gr.KT * 400;
+            const long long st = 25ll * mt * lb;
+            // (an item's stores overlap the next one's MMAs about by half)
+            const long long item = std::max(std::max(mma, st) + std::min(mma, st) / 2, res ? 0 : ksteps * lb * 32 / 40);
+            const long long cost = (units + sms - 1) / sms * item + std::min(mma, st) / 2;
+            if (best < 0 || cost < best) {
+                best = cost;
+                r.mt = mt;
+                r.bn = bn;
+                r.ntiles = nt;
+                r.cap_b = (int)cap;
+                const long long left = kGcSmemLimit - fixed - cap;
+                r.stages_a = (int)std::min<long long>(kGcMaxA, left / stride);
+                r.smem = (size_t)(fixed + cap + r.stages_a * stride);
             }
         }
+    }
     if (best < 0) return false;
+    r.cycles = best;
     r.npad = r.bn * r.ntiles;
     *out = r;
     return true;
@@ -618,6 +653,7 @@ sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const Gri
     a.out = c.out;
     a.bias = c.bias;
     a.colmap = c.colmap;
+    a.cstride = c.cstride;
     a.zmap = c.zmap;
     a.zstride = c.zstride;
     a.counts = c.counts;
@@ -677,6 +713,119 @@ sadmm_status launch_grid_x(const Grid& gr, const Geometry& g, const void* x, con
                    static_cast<const __nv_bfloat16*>(x), colidx, gr, (int)g.c, (int)g.cg, nck, chunks, (int)g.taps,
                    g.n * g.c * g.t * g.h * g.w, device_status_ptr(), xs);
     return e == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
+}
+
+// The rule for the forward compares estimated times on a whole GB300, whatever
+// the plan's cap: of 80 layers measured both ways (AlexNet conv2-5, ResNet-50,
+// C3D and sweep layers, 1x1 to 5x5, densities 0.05 to 1, batch 8 to 128; each
+// graph-replayed) it takes the slower one by more than 5 % on two, by at most
+// 20 %.  Dense-in-taps work pays where the gathered kernel's rate is the gather's
+// (up to 128 filters a group) or columns are mostly kept: AlexNet conv2 at half
+// density 77 -> 50 us, all columns of conv3 63 -> 37, 64-channel 5x5 51 -> 23;
+// conv3 at a quarter stays gathered (22 against 29 us), the 512-filter layer at
+// half too (125 against 185).
+constexpr long long kRuleSms = 152;
+
+// Channels of x per conv group that hold a kept column.
+static int fwd_channels(const sadmm_plan* plan, const Geometry& g)
+{
+    return plan->colkind == SADMM_COL_CHANNEL ? plan->n_colgroups : (int)g.cg;
+}
+
+int grid_fwd_ksteps(const sadmm_plan* plan, const Geometry& g)
+{
+    return (fwd_channels(plan, g) + 15) / 16 * (int)g.taps;
+}
+
+bool grid_fwd_plan(const Geometry& g, sadmm_plan* plan, size_t* gx, size_t* gw, size_t* gcol)
+{
+    Grid gr;
+    GridConvShape sh;
+    if (plan->n_cols < 1 || plan->n_filt < 1 || plan->splits > 1 || g.groups > 64 || !grid_of(g, &gr)) return false;
+    if (g.taps == 1) return false;  // one tap reads contiguous rows: no slab to share
+    const long long units = (g.m + 127) / 128 * g.groups * ((plan->n_tiles + 1) / 2);
+    if (units < kRuleSms) return false;
+    const int nck = fwd_channels(plan, g);
+    const int per = (int)((plan->n_filt + g.groups - 1) / g.groups);
+    if (!grid_conv_shape(gr, nck, plan->n_pad, per, (int)g.groups, plan->ctas, &sh)) return false;
+    const int chunks = sh.k16 * 2;
+    if (g.groups * sh.k16 > 65535) return false;
+    plan->gx_cb = sh.cb;
+    plan->gx_mt = sh.mt;
+    plan->gx_bn = sh.bn;
+    plan->gx_ntiles = sh.ntiles;
+    plan->gx_stages = sh.stages_a;
+    plan->gx_cap = sh.cap_b;
+    plan->gx_smem = (int)sh.smem;
+    // The estimates, in ns.  Grid: launches and drain, the copy at 4 TB/s of x
+    // read and written, the slab GEMM's cycles at 1.95 GHz, and y at 60 TB/s
+    // for what its stores add.  Gathered: start-up, the busiest CTA's 64-column
+    // stages (the gather's rate up to 128 filters, the MMAs' above), and the
+    // stores, which overlap less when one accumulator set fills TMEM.
+    GridConvShape rule;
+    if (!grid_conv_shape(gr, nck, plan->n_pad, per, (int)g.groups, kRuleSms, &rule)) return false;
+    const long long xb = 2 * g.n * g.groups * (long long)nck * g.t * g.h * g.w + 2 * g.groups * 16ll * sh.k16 * gr.L;
+    const long long yb = 4 * g.m * g.f;
+    const long long grid_ns = 8000 + xb / 4000 + rule.cycles * 100 / 195 + yb / 60000;
+    const long long nks = plan->k_pad / 64, rows = (long long)std::min(plan->n_tiles, 2) * plan->bn;
+    const long long whole = (units + kRuleSms - 1) / kRuleSms * nks, even = (units * nks + kRuleSms - 1) / kRuleSms;
+    const bool sk = 2 * std::min(plan->n_tiles, 2) * round_up(plan->bn, 32) <= 512 && plan->k_pad >= 4ll * plan->bn &&
+                    even >= nks && (whole - even) * 8 >= whole;
+    const long long stages = sk ? even : whole;
+    const long long gather_ns = 7000 + stages * (rows <= 128 ? 680 : rows <= 256 ? 800 : 950) +
+                                yb / (plan->n_tiles > 1 ? 20000 : 40000);
+    if (grid_ns * 100 > gather_ns * 95) return false;
+    *gx = (size_t)(g.groups * chunks * (long long)gr.slots * 16);
+    *gw = (size_t)(g.groups * sh.npad * (long long)sh.ksteps * 32);
+    *gcol = (size_t)sh.ksteps * 16 * 4;
+    return true;
+}
+
+sadmm_status launch_grid_fwd(const sadmm_plan* plan, const Geometry& g, const void* x, const float* bias, int relu,
+                             void* y, int ydt, cudaStream_t s)
+{
+    Grid gr;
+    if (!grid_of(g, &gr)) return SADMM_EINVAL;
+    const int nck = fwd_channels(plan, g);
+    GridConvShape sh;
+    memset(&sh, 0, sizeof(sh));
+    sh.cb = plan->gx_cb;
+    sh.k16 = (nck + 15) / 16;
+    sh.ksteps = grid_fwd_ksteps(plan, g);
+    sh.mt = plan->gx_mt;
+    sh.bn = plan->gx_bn;
+    sh.ntiles = plan->gx_ntiles;
+    sh.npad = sh.bn * sh.ntiles;
+    sh.cap_b = plan->gx_cap;
+    sh.stages_a = plan->gx_stages;
+    sh.smem = (size_t)plan->gx_smem;
+    const char* base = static_cast<const char*>(plan->dev);
+    __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(const_cast<char*>(base) + plan->off_gx);
+    const int* colidx = reinterpret_cast<const int*>(base + plan->off_colidx);
+    sadmm_status st = launch_grid_x(gr, g, x, plan->colkind == SADMM_COL_CHANNEL ? colidx : nullptr, nck, sh.k16 * 2, xs, s);
+    if (st != SADMM_OK) return st;
+    GridConvCall c;
+    memset(&c, 0, sizeof(c));
+    c.src = xs;
+    c.chunks = sh.k16 * 2;
+    c.wd = reinterpret_cast<const __nv_bfloat16*>(base + plan->off_gw);
+    c.out = y;
+    c.out_bf16 = ydt == SADMM_BF16;
+    c.bias = bias;
+    c.relu = relu;
+    c.colmap = reinterpret_cast<const int*>(base + plan->off_rowmap);
+    c.cstride = plan->n_pad;
+    c.zmap = reinterpret_cast<const int*>(base + plan->off_zeromap);
+    c.zstride = (int)g.fg;
+    c.counts = reinterpret_cast<const int*>(base + plan->off_counts);
+    c.groups = (int)g.groups;
+    c.planes = (int)g.f;
+    c.VT = (int)g.ot;
+    c.VH = (int)g.oh;
+    c.VW = (int)g.ow;
+    c.out_total = g.n * g.f * g.plane;
+    c.ctas = plan->ctas;
+    return launch_grid_conv(gr, sh, c, s);
 }
 
 }  // namespace sadmm

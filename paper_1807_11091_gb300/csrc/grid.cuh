@@ -64,30 +64,45 @@ inline bool grid_of(const Geometry& g, Grid* out)
 // out[plane(col)][pixel] = bias + sum over the K columns of Wd[col][k] * src:
 // K column k = ((cb*KT + kt)*KH*KW + kh*KW + kw)*CB + ci reads channel
 // cb*CB + ci at shift kt*HWb + kh*Wb + kw.  Wd lies as the MMA reads it, a step
-// of 16 K columns at a time: [group][column tile][step][K half][bn][8].
+// of 16 K columns at a time: [group][column tile][step][K half][row][8].
 struct GridConvShape {
     int cb;      // channels per block (multiple of 16)
     int k16;     // 16-channel groups of the source (padded channels / 16)
     int ksteps;  // MMA steps of 16 K columns
     int mt;      // 128-pixel tiles per work item (1 or 2)
     int bn, ntiles, npad;  // output columns per tile, tiles, and bn*ntiles
-    int cap_b;     // steps of weights shared memory holds: all of an item's stay there, or a ring streams
+    int cap_b;     // bytes of weights shared memory holds: all of an item's stay there, or a ring streams
     int stages_a;
     size_t smem;
+    long long cycles;  // its estimated time
 };
-// The tiling for `chans` source channels and `cols` output columns per group
-// over `groups` groups; false when it does not fit.
-bool grid_conv_shape(const Grid& gr, int chans, int cols, int groups, int sms, GridConvShape* out);
+// The tiling for `chans` source channels and at most `cols`, likely `likely`,
+// output columns per group over `groups` groups; false when it does not fit.
+// The blocks of channels (the order of the sums) follow the layer alone, not its
+// batch or the device.
+bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups, int sms, GridConvShape* out);
+
+// Rows of a column tile in the weights' layout: the most columns any group has,
+// to 16, when there is one tile (the groups' counts are known on the device
+// alone), else bn.
+SADMM_DEV int grid_rows(const int* counts, int groups, int ntiles, int bn)
+{
+    if (ntiles > 1) return bn;
+    int m = 16;
+    for (int g = 0; g < groups; ++g) m = max(m, (__ldg(counts + 2 * g) + 15) & ~15);
+    return min(m, bn);
+}
 
 struct GridConvCall {
     const __nv_bfloat16* src;  // [groups][chunks][slots][8]
     int chunks;                // chunks per group (k16 * 2)
-    const __nv_bfloat16* wd;   // [groups][ntiles][ksteps][2][bn][8], -0.0 at pruned entries
+    const __nv_bfloat16* wd;   // [groups][ntiles][ksteps][2][rows][8], rows = grid_rows() (a tile's room: bn); -0.0 at pruned entries
     void* out;
     int out_bf16;
     const float* bias;     // per plane, or NULL
     int relu;
-    const int* colmap;     // [groups][npad] column -> plane of an image (-1: none)
+    const int* colmap;     // [groups][cstride] column -> plane of an image (-1: none)
+    int cstride;
     const int* zmap;       // [groups][zstride] planes written as zeros
     int zstride;
     const int* counts;     // [groups][2] columns, zero planes
@@ -103,6 +118,14 @@ sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const Gri
 // colidx[ci*taps]/taps when colidx != NULL, else 0..nck-1), `chunks` chunks.
 sadmm_status launch_grid_x(const Grid& gr, const Geometry& g, const void* x, const int* colidx, int nck, int chunks,
                            __nv_bfloat16* xs, cudaStream_t s);
+
+// ---- grid forward (conv_grid.cu) ----
+// Whether the plan's forward takes the grid; its tiling then, and the bytes of
+// the regions it adds to the plan's buffer.
+bool grid_fwd_plan(const Geometry& g, sadmm_plan* plan, size_t* gx, size_t* gw, size_t* gcol);
+int grid_fwd_ksteps(const sadmm_plan* plan, const Geometry& g);
+sadmm_status launch_grid_fwd(const sadmm_plan* plan, const Geometry& g, const void* x, const float* bias, int relu,
+                             void* y, int ydt, cudaStream_t s);
 
 // ---- grid backward (bwd_grid.cu) ----
 size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g);  // 0: the layer takes the gathered backward

@@ -17,6 +17,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "grid.cuh"
 #include "internal.h"
 
 namespace sadmm {
@@ -42,6 +43,9 @@ struct PackArgs {
     int* scol;   // [xs_kpad] slab column -> GEMM column (-1: zero)
     int* chan;   // [xs_cs] kept input channels (-1 past them)
     int C, xs_cs, xs_kpad, xs_r, xs_q, sh, sw;
+    // pixel-grid plans (gcol != NULL): K column -> GEMM column
+    int* gcol;
+    int gx_k, gx_cb;    // K columns, channels per block
     int* skcnt;         // stream-K arrival counters, zeroed here
     int sk_n;
     int lists_in_smem;  // 1: the filter and column lists are staged in shared memory
@@ -63,6 +67,11 @@ struct WpLayer {
     __nv_bfloat16* wps;
     long long rows, first;
     int K, k_pad, kpad_s;
+    // pixel-grid plans: rows past rows + srows pack a row of wg each
+    const int* gcol;
+    const int* counts;
+    __nv_bfloat16* wg;
+    int srows, n_pad, groups, gx_bn, gx_ntiles, gx_ksteps;
 };
 
 template <int N>
@@ -139,6 +148,7 @@ SADMM_DEV void pack_meta(PackArgs a, int* status)
             for (int j = tid; j < a.xs_kpad; j += blockDim.x) a.scol[j] = -1;
             for (int ci = tid; ci < a.xs_cs; ci += blockDim.x) a.chan[ci] = -1;
         }
+        for (int k = tid; k < a.gx_k; k += blockDim.x) a.gcol[k] = -2;
         return;
     }
     // kept-filter range of each conv group in the ascending filter list
@@ -197,6 +207,23 @@ SADMM_DEV void pack_meta(PackArgs a, int* status)
         const int j0 = st * 64, j1 = min(j0 + 63, a.n_cols - 1);
         a.stage_chan[st] = (j1 < j0) ? make_int2(0, -1) : make_int2(a.colidx[j0] / a.taps, a.colidx[j1] / a.taps);
     }
+    // Grid column order: column k = ((blk*taps + tap)*gx_cb + ci) is channel
+    // blk*gx_cb + ci (a kept one, or any when columns are pruned shape-wise) at
+    // `tap`; -1 where that GEMM column is pruned, -2 past the channels.
+    for (int k = tid; k < a.gx_k; k += blockDim.x) {
+        const int t = k / a.gx_cb, blk = t / a.taps;
+        const int ci = blk * a.gx_cb + (k - t * a.gx_cb);
+        const int nck = a.colkind == SADMM_COL_CHANNEL ? a.n_colgroups : a.K / a.taps;
+        int col = -2;
+        if (ci < nck) {
+            col = (a.colkind == SADMM_COL_CHANNEL ? a.col_idx[ci] : ci) * a.taps + (t - blk * a.taps);
+            if (a.colkind == SADMM_COL_SHAPE) {
+                const int pos = lower_bound(a.col_idx, a.n_colgroups, col);
+                if (pos >= a.n_colgroups || a.col_idx[pos] != col) col = -1;
+            }
+        }
+        a.gcol[k] = col;
+    }
     if (a.scol) {
         // Slab column order of the input-slab path: column j is block tap
         // (r, q) = (j / cs / Q, j / cs % Q) and slab channel cc = j % cs =
@@ -239,9 +266,43 @@ SADMM_DEV float load_f32<float>(const float* p) { return *p; }
 
 // Row r of a layer: rows past `rows` pack the input-slab plan's weights, row
 // r - rows of conv group 0 through the slab column map scol, into wps [bn][kpad_s].
+// Row r (kept filter i of conv group g) of a pixel-grid plan's weights
+// [g][tile][step][K half][row][8]: a thread writes the 8 channels of one half of
+// a step, -0.0 at pruned columns (a kept weight that is -0.0 as +0.0: no product
+// or sum tells them apart).
+template <typename T>
+SADMM_DEV void pack_wg_row(const WpLayer& L, int r)
+{
+    const T* W = static_cast<const T*>(L.W);
+    const int npad = L.gx_bn * L.gx_ntiles;
+    const int g = r / npad, i = r - g * npad;
+    const int rows = grid_rows(L.counts, L.groups, L.gx_ntiles, L.gx_bn);
+    const int nt = i / L.gx_bn, il = i - nt * L.gx_bn;
+    if (il >= rows) return;
+    const int f = i < L.n_pad ? L.rowmap[g * L.n_pad + i] : -1;
+    uint4* dst = reinterpret_cast<uint4*>(L.wg) + (size_t)(g * L.gx_ntiles + nt) * L.gx_ksteps * 2 * L.gx_bn + il;
+    for (int k = threadIdx.x; k < L.gx_ksteps * 2; k += blockDim.x) {
+        uint32_t v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int col = __ldg(L.gcol + k * 8 + e);
+            v[e] = col == -1 ? 0x8000u : 0u;
+            if (f >= 0 && col >= 0) {
+                v[e] = __bfloat16_as_ushort(__float2bfloat16_rn(load_f32<T>(W + (long long)f * L.K + col)));
+                if (v[e] == 0x8000u) v[e] = 0u;
+            }
+        }
+        dst[(size_t)k * rows] = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+    }
+}
+
 template <typename T>
 SADMM_DEV void pack_wp_row(const WpLayer& L, long long r)
 {
+    if (r >= L.rows + L.srows) {
+        pack_wg_row<T>(L, (int)(r - L.rows - L.srows));
+        return;
+    }
     const T* W = static_cast<const T*>(L.W);
     const int* colidx = L.colidx;
     int k_pad = L.k_pad;
@@ -347,6 +408,11 @@ PackArgs pack_args(const sadmm_plan* plan, const Geometry& g, const int* filt_id
         a.sh = (int)g.sh;
         a.sw = (int)g.sw;
     }
+    if (plan->gx_mode) {
+        a.gcol = reinterpret_cast<int*>(base + plan->off_gcol);
+        a.gx_k = grid_fwd_ksteps(plan, g) * 16;
+        a.gx_cb = plan->gx_cb;
+    }
     if (plan->sk_len > 0) {
         a.skcnt = reinterpret_cast<int*>(base + plan->off_sk);
         a.sk_n = plan->sk_grid;
@@ -422,7 +488,18 @@ sadmm_status launch_batch(const PackJob* jobs, int n, int wdt, cudaStream_t s)
         L.kpad_s = plan->xs_kpad;
         L.wps = plan->xs_mode ? reinterpret_cast<__nv_bfloat16*>(base + plan->off_wps) : nullptr;
         L.first = blocks;
-        blocks += L.rows + (plan->xs_mode ? plan->bn : 0);
+        L.srows = plan->xs_mode ? plan->bn : 0;
+        if (plan->gx_mode) {
+            L.gcol = pb.L[i].gcol;
+            L.counts = pb.L[i].counts;
+            L.wg = reinterpret_cast<__nv_bfloat16*>(base + plan->off_gw);
+            L.n_pad = plan->n_pad;
+            L.groups = (int)g.groups;
+            L.gx_bn = plan->gx_bn;
+            L.gx_ntiles = plan->gx_ntiles;
+            L.gx_ksteps = pb.L[i].gx_k / 16;
+        }
+        blocks += L.rows + L.srows + (plan->gx_mode ? g.groups * (long long)plan->gx_bn * plan->gx_ntiles : 0);
     }
     wb.n = n;
     if (blocks >= (1ll << 31)) return SADMM_EUNSUPPORTED;

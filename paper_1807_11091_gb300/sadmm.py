@@ -96,6 +96,17 @@ class Plan(ctypes.Structure):
         ("tmap", ctypes.c_uint64 * 16),
         ("tmap_ws", ctypes.c_uint64 * 16),
         ("tmap_xs", ctypes.c_uint64 * 16),
+        ("gx_mode", ctypes.c_int),
+        ("gx_cb", ctypes.c_int),
+        ("gx_mt", ctypes.c_int),
+        ("gx_bn", ctypes.c_int),
+        ("gx_ntiles", ctypes.c_int),
+        ("gx_stages", ctypes.c_int),
+        ("gx_cap", ctypes.c_int),
+        ("gx_smem", ctypes.c_int),
+        ("off_gx", ctypes.c_size_t),
+        ("off_gw", ctypes.c_size_t),
+        ("off_gcol", ctypes.c_size_t),
     ]
 
 
