@@ -125,16 +125,32 @@ struct ConvArgs {
     int sk_cols;     // nacc * bn
 };
 
+// How the output tiles become work items; an instantiation of the kernel each, so
+// that the whole-tile loops carry no state of the others (a runtime split count
+// in their zero-plane loop alone cost the 1x1 layers 2 %: 41.5 us against 39.5 for
+// 64 channels to 256 at 56x56).  kStreamK keeps the runtime split count, always 1
+// there: without its branch the compiler's schedule is 1 % slower (48.9 against
+// 48.3 us on the 3-D layer).
+enum { kWhole, kStreamK, kSplit };
+
 // Work item w is split sp (stages ks0 .. ks1-1 of K') of unit w / splits; a
 // unit covers filter tiles p*nacc .. p*nacc+nacc-1 of conv group g for pixel
 // tile mt.  Groups are outermost, so a CTA (items w, w + grid, ...) stays in
 // one conv group for long runs and rarely reloads resident weights.
+// (kWhole: the unit itself, all stages.)
+template <int MODE>
 SADMM_DEV void decode_unit(const ConvArgs& a, int w, int& p, int& g, int& mt, int& sp, int& ks0, int& ks1)
 {
-    const uint32_t u = fdiv((uint32_t)w, a.split_div);
-    sp = w - (int)(u * a.split_div.d);
-    ks0 = sp * a.ksps;
-    ks1 = min(a.nks, ks0 + a.ksps);
+    uint32_t u = (uint32_t)w;
+    sp = 0;
+    ks0 = 0;
+    ks1 = a.nks;
+    if (MODE != kWhole) {
+        u = fdiv((uint32_t)w, a.split_div);
+        sp = w - (int)(u * a.split_div.d);
+        ks0 = sp * a.ksps;
+        ks1 = min(a.nks, ks0 + a.ksps);
+    }
     const uint32_t t = fdiv(u, a.upairs_div);
     p = (int)(u - t * a.upairs_div.d);
     const uint32_t gq = fdiv(t, a.mtiles_div);
@@ -154,11 +170,11 @@ struct Work {
     int phase;    // stream-K: 0 start piece next, 1 end piece next, 2 whole units
 };
 
-template <bool SK>
+template <int MODE>
 SADMM_DEV Work work_begin(const ConvArgs& a)
 {
     Work w;
-    if (SK) {
+    if (MODE == kStreamK) {
         const int s0 = blockIdx.x * a.sk_len;
         const int e0 = min(s0 + a.sk_len, a.units * a.nks);
         // sk_len >= nks: a run that starts inside a unit goes past that unit's end
@@ -175,10 +191,10 @@ SADMM_DEV Work work_begin(const ConvArgs& a)
 }
 
 // Next work item: its unit and stage range ks0 .. ks1-1; false at the end.
-template <bool SK>
+template <int MODE>
 SADMM_DEV bool work_next(const ConvArgs& a, Work& w, int& p, int& g, int& mt, int& sp, int& ks0, int& ks1)
 {
-    if (SK) {
+    if (MODE == kStreamK) {
         int b = 0, e = 0;
         while (w.phase < 2 && b == e) {
             const int s0 = blockIdx.x * a.sk_len;
@@ -196,13 +212,13 @@ SADMM_DEV bool work_next(const ConvArgs& a, Work& w, int& p, int& g, int& mt, in
             w.it = e;
         }
         const int u = (int)fdiv((uint32_t)b, a.nks_div);
-        decode_unit(a, u, p, g, mt, sp, ks0, ks1);  // one split: sp = 0
+        decode_unit<MODE>(a, u, p, g, mt, sp, ks0, ks1);  // one split: sp = 0
         ks0 = b - u * a.nks;
         ks1 = ks0 + (e - b);
         return true;
     }
     if (w.it >= w.end) return false;
-    decode_unit(a, w.it, p, g, mt, sp, ks0, ks1);
+    decode_unit<MODE>(a, w.it, p, g, mt, sp, ks0, ks1);
     w.it += gridDim.x;
     return true;
 }
@@ -251,9 +267,7 @@ SADMM_DEV uint32_t ldg_u16_if(const unsigned short* p, uint32_t bits, uint32_t n
     return v;
 }
 
-// SK: stream-K work items (a.sk_len > 0); a separate instantiation keeps the
-// whole-tile loops free of the extra state.
-template <bool OUT_BF16, bool SK>
+template <bool OUT_BF16, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
     k_conv_fwd(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ ConvArgs a)
 {
@@ -330,9 +344,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             long long cur = -1;
             uint32_t e_ph = 0;
             int loads = 0;
-            Work wk = work_begin<SK>(a);
+            Work wk = work_begin<MODE>(a);
             int p, g, sp, ks0, ks1, mt;
-            while (work_next<SK>(a, wk, p, g, mt, sp, ks0, ks1)) {
+            while (work_next<MODE>(a, wk, p, g, mt, sp, ks0, ks1)) {
                 if (s_counts[2 * g] <= p * a.bn) continue;
                 const long long key = (long long)g * a.upairs + p;
                 if (key == cur) continue;
@@ -358,9 +372,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t issued_parity[kMaxStages];
             uint32_t issued_mask = 0;
             bool ok = true;
-            Work wk = work_begin<SK>(a);
+            Work wk = work_begin<MODE>(a);
             int p, g, sp, ks0, ks1, mt;
-            while (ok && work_next<SK>(a, wk, p, g, mt, sp, ks0, ks1)) {
+            while (ok && work_next<MODE>(a, wk, p, g, mt, sp, ks0, ks1)) {
                 const int nt0 = p * a.nacc;
                 if (s_counts[2 * g] <= nt0 * a.bn) continue;
                 int nbox = 0;  // filter tiles of this unit with kept rows
@@ -400,9 +414,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             long long cur = -1;    // (group, filter tile) of the resident weights
             uint32_t bf_ph = 0;
             const uint32_t sB0 = smem_u32(sB);
-            Work wk = work_begin<SK>(a);
+            Work wk = work_begin<MODE>(a);
             int p, g, sp, ks0, ks1, mt;
-            while (ok && work_next<SK>(a, wk, p, g, mt, sp, ks0, ks1)) {
+            while (ok && work_next<MODE>(a, wk, p, g, mt, sp, ks0, ks1)) {
                 const int cnt = s_counts[2 * g] - p * a.nacc * a.bn;  // kept rows from the unit's first tile
                 if (cnt <= 0) continue;
                 if (a.b_res) {
@@ -483,9 +497,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         // After a failed wait (another role aborted) the warp keeps walking the
         // units, without TMEM or stores, so the named barrier stays balanced.
         bool alive = true;
-        Work wk = work_begin<SK>(a);
+        Work wk = work_begin<MODE>(a);
         int p, g, sp, ks0, ks1, mt;
-        while (work_next<SK>(a, wk, p, g, mt, sp, ks0, ks1)) {
+        while (work_next<MODE>(a, wk, p, g, mt, sp, ks0, ks1)) {
             const int nt0 = p * a.nacc;
             const int cnt = s_counts[2 * g] - nt0 * a.bn;  // kept rows from the unit's first tile
             const int zc = (p == 0) ? s_counts[2 * g + 1] : 0;  // pruned filters whose planes this unit zeroes
@@ -514,7 +528,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const float* u_bias = s_ebias + ub * kTabCap;
             // stream-K: a unit cut at the start of CTA b's run has piece 0 (its
             // first stages) in CTA b-1 and piece 1 in CTA b, and cut index b-1
-            const bool cut = SK && (ks0 > 0 || ks1 < a.nks);
+            const bool cut = MODE == kStreamK && (ks0 > 0 || ks1 < a.nks);
             const int piece = ks0 > 0 ? 1 : 0;
             const int cut_idx = (int)blockIdx.x - piece;
             const int m = mt * kBM + row;
@@ -525,7 +539,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             __nv_bfloat16* yh = reinterpret_cast<__nv_bfloat16*>(a.y) + (n_img * (long long)a.F * a.plane + pix);
             const YCheck yc{n_img * (long long)a.F * a.plane + pix, a.y_total, a.status};
             int chunks = 0;  // chunks of this unit so far (zero planes, then accumulator columns)
-            if (zc > 0 && alive && (a.splits > 1 || ks0 == 0)) {
+            if (zc > 0 && alive && (MODE == kSplit || (a.splits == 1 && ks0 == 0))) {
                 // Pruned filters of this conv group: their planes are zero.  They
                 // need no accumulator, so they go out while the unit's MMAs run;
                 // these chunks of 16 planes start the unit's chunk sequence
@@ -534,7 +548,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int* zmap = a.zeromap + (long long)g * a.Fg;
                 const int* u_zero = s_zoff + ub * a.zcap;
                 const int nzc = (zc + kEpiCols - 1) / kEpiCols;
-                for (int k = sp * kHalves + h; valid && k < nzc; k += a.splits * kHalves) {
+                for (int k = MODE == kSplit ? sp * kHalves + h : h; valid && k < nzc;
+                     k += MODE == kSplit ? a.splits * kHalves : kHalves) {
                     const int z0 = k * kEpiCols;
                     if (z0 + kEpiCols <= a.zcap && z0 + kEpiCols <= zc) {
 #pragma unroll
@@ -612,7 +627,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             for (int j = 0; j < kEpiCols; ++j)
                                 v[j] = __uint_as_float(r[j]) + __ldcg(other + col0 + (size_t)j * kBM);
                             if (valid) store_cols<OUT_BF16>(v, c0, nrows, t_off, t_bias, a.relu, yf, yh, yc);
-                        } else if (valid && a.splits > 1) {
+                        } else if (MODE != kWhole && valid && a.splits > 1) {
                             // split K': raw fp32 partial sums, [split][column][pixel]
                             float* pp = a.partial +
                                         ((size_t)sp * a.ncols_all + (size_t)g * a.n_pad + (size_t)(nt0 + ti) * a.bn + c0) *
@@ -689,9 +704,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t ph = 0;
         int turn = 0;  // running stage index modulo kGatherSets
         bool ok = true;
-        Work wk = work_begin<SK>(a);
+        Work wk = work_begin<MODE>(a);
         int p, g, sp, ks0, ks1, mt;
-        while (ok && work_next<SK>(a, wk, p, g, mt, sp, ks0, ks1)) {
+        while (ok && work_next<MODE>(a, wk, p, g, mt, sp, ks0, ks1)) {
             if (s_counts[2 * g] <= p * a.nacc * a.bn) continue;
             uint32_t M[kPixPerThread];
             const unsigned short* xb[kPixPerThread];
@@ -854,10 +869,10 @@ __global__ void __launch_bounds__(256) k_splitk_finalize(const ConvArgs a)
     }
 }
 
-template <bool OUT_BF16, bool SK>
+template <bool OUT_BF16, int MODE>
 cudaError_t launch(const CUtensorMap& map, const ConvArgs& a, int grid, size_t smem, cudaStream_t s)
 {
-    auto kern = k_conv_fwd<OUT_BF16, SK>;
+    auto kern = k_conv_fwd<OUT_BF16, MODE>;
     static int configured_dev = -1;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -880,7 +895,7 @@ cudaError_t launch(const CUtensorMap& map, const ConvArgs& a, int grid, size_t s
     cfg.numAttrs = 1;
     cudaError_t e = cudaLaunchKernelEx(&cfg, kern, map, a);
     if (e != cudaSuccess) return e;
-    if (a.splits > 1) {
+    if (MODE == kSplit) {
         cfg.gridDim = dim3((unsigned)(((long long)a.ncols_all * (a.m_pad / kBM) + 7) / 8));
         cfg.blockDim = dim3(256);
         cfg.dynamicSmemBytes = 0;
@@ -1035,12 +1050,13 @@ sadmm_status launch_conv_fwd(const sadmm_plan* plan, const Geometry& g, const vo
     CUtensorMap map;
     memcpy(&map, plan->tmap, sizeof(map));
     cudaError_t e;
+    const bool bf16 = ydt == SADMM_BF16;
     if (a.sk_len > 0)
-        e = (ydt == SADMM_BF16) ? launch<true, true>(map, a, (int)grid, smem, s)
-                                : launch<false, true>(map, a, (int)grid, smem, s);
+        e = bf16 ? launch<true, kStreamK>(map, a, (int)grid, smem, s) : launch<false, kStreamK>(map, a, (int)grid, smem, s);
+    else if (a.splits > 1)
+        e = bf16 ? launch<true, kSplit>(map, a, (int)grid, smem, s) : launch<false, kSplit>(map, a, (int)grid, smem, s);
     else
-        e = (ydt == SADMM_BF16) ? launch<true, false>(map, a, (int)grid, smem, s)
-                                : launch<false, false>(map, a, (int)grid, smem, s);
+        e = bf16 ? launch<true, kWhole>(map, a, (int)grid, smem, s) : launch<false, kWhole>(map, a, (int)grid, smem, s);
     return e == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
 }
 
