@@ -2,11 +2,11 @@
 // retraining (Sec. 4) on the padded pixel grid of grid.cuh: no im2col, no
 // col2im, no atomics.
 //
-//   k_grid_prep    the input gradient's weights (taps flipped, kept filters as
-//                  channels), its output map, dW zeroed
-//   k_grid_dz      dZ = dY * [y > 0] of the kept filters as a grid copy (each
-//                  element read once for dW, dx and db) and db's partial sums
-//   k_grid_x       x as a grid copy (conv_grid.cu)
+//   k_grid_front   in one launch: dZ = dY * [y > 0] of the kept filters as a grid
+//                  copy (each element read once for dW, dx and db) with db's
+//                  partial sums; x as a grid copy; the input gradient's weights
+//                  (taps flipped, kept filters as channels) and output map; dW
+//                  zeroed
 //   k_grid_wgrad   dW: for a tap of shift s, dW[f][c] = sum over grid pixels q
 //                  of x[c][q + s] * dZ[f][D0 + q].  Channels are the MMA's M
 //                  side, filters its N side, pixels its K side: both operands
@@ -14,7 +14,7 @@
 //                  channels x 8 pixels); dZ is zero off the output, so the
 //                  padded pixels add nothing.
 //   k_grid_wreduce the slices of the pixel ranges, in order, into dW's kept
-//                  entries
+//                  entries, and db's partial sums
 //   k_grid_conv    dx: the slab GEMM over dZ (conv_grid.cu), every element
 //                  written once
 //
@@ -378,6 +378,41 @@ __device__ __noinline__ float wgrad_exact(const __nv_bfloat16* xc, const __nv_bf
     return acc;
 }
 
+struct DbArgs {
+    const float* part;  // NULL: no bias gradient
+    const int* rowmap;
+    const int* zeromap;
+    const int* counts;
+    int nparts, groups, n_pad, Fg;
+    float* db;
+};
+
+// db, by blocks b, b + nb, ... of 256 threads: a warp per packed row adds its
+// partial sums (fixed order); zeros for the pruned filters.
+SADMM_DEV void db_blocks(const DbArgs& a, int b, int nb)
+{
+    const int lane = threadIdx.x & 31;
+    for (int r = b * 8 + (threadIdx.x >> 5); r < a.groups * a.n_pad; r += nb * 8) {
+        const int f = __ldg(a.rowmap + r);
+        if (f < 0) continue;
+        float s = 0.0f;
+        for (int k = lane; k < a.nparts; k += 32) s += __ldg(a.part + (size_t)r * a.nparts + k);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) a.db[f] = s;
+    }
+    for (int z = b * 256 + threadIdx.x; z < a.groups * a.Fg; z += nb * 256) {
+        const int g = z / a.Fg;
+        if (z - g * a.Fg < __ldg(a.counts + 2 * g + 1)) a.db[__ldg(a.zeromap + z)] = 0.0f;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_grid_db(const DbArgs a)
+{
+    pdl_wait();  // after the kernel before it in the stream
+    pdl_trigger();
+    db_blocks(a, blockIdx.x, gridDim.x);
+}
+
 struct WrArgs {
     Grid gr;
     WgradShape w;
@@ -399,10 +434,15 @@ struct WrArgs {
 // by*32 .. +31; the slices are read along the filters.
 constexpr int kWrCols = 4;
 
-__global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a)
+__global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbArgs d)
 {
     pdl_wait();  // after the kernel before it in the stream
+    pdl_trigger();
     __shared__ float s_v[8][kWrCols][32];
+    if ((int)blockIdx.z == d.groups) {  // the last layer of blocks: the bias gradient
+        db_blocks(d, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+        return;
+    }
     const int g = blockIdx.z, cnt = __ldg(a.counts + 2 * g);
     const int i0 = blockIdx.y * 32, j0 = blockIdx.x * kWrCols;
     if (i0 >= cnt) return;
@@ -460,10 +500,11 @@ struct DzArgs {
     const int* counts;
     int n_pad, F, plane, chunks, cb;
     __nv_bfloat16* dz;  // NULL: the bias gradient alone
-    float* part;        // [groups*n_pad][gridDim.x], or NULL
+    float* part;        // [groups*n_pad][bx], or NULL
+    int bx, by;         // blocks
 };
 
-// Grid copy of dZ and the bias gradient's partial sums.  Block (bx, by): slots
+// Grid copy of dZ and the bias gradient's partial sums.  Block (bx, by), 256 threads: slots
 // bx*kDzSlots .. of chunk by % chunks (8 kept filters) of conv group by / chunks.
 constexpr int kDzSlots = 512;
 
@@ -494,12 +535,9 @@ SADMM_DEV void dz_octet(const unsigned short* dp, const Y* yp, const int (&off)[
 }
 
 template <bool RELU, typename Y>
-__global__ void __launch_bounds__(256) k_grid_dz(const DzArgs a)
+SADMM_DEV void dz_block(const DzArgs& a, int bx, int by, int* s_off, float (*s_part)[8])
 {
-    pdl_wait();  // after the kernel before it in the stream
-    __shared__ int s_off[8];
-    __shared__ float s_part[8][8];
-    const int g = blockIdx.y / a.chunks, ck = blockIdx.y - g * a.chunks;
+    const int g = by / a.chunks, ck = by - g * a.chunks;
     const int cnt = __ldg(a.counts + 2 * g);
     if (ck * 8 >= (cnt + a.cb - 1) / a.cb * a.cb && ck * 8 >= cnt + 15) return;  // past every reader's last filter
     const int nf = min(8, cnt - ck * 8);  // kept filters of this chunk (they come first)
@@ -515,7 +553,7 @@ __global__ void __launch_bounds__(256) k_grid_dz(const DzArgs a)
     }
 #pragma unroll 1
     for (int k = 0; k < kDzSlots / 256; ++k) {
-        const int s = blockIdx.x * kDzSlots + k * 256 + threadIdx.x;
+        const int s = bx * kDzSlots + k * 256 + threadIdx.x;
         if (s >= a.gr.slots) break;
         int n = 0, t = 0, h = 0, w = 0;
         const int q = s - a.gr.D0;
@@ -544,30 +582,7 @@ __global__ void __launch_bounds__(256) k_grid_dz(const DzArgs a)
     if (threadIdx.x < 8 && i < a.n_pad) {
         float r = 0.0f;
         for (int w = 0; w < 8; ++w) r += s_part[w][threadIdx.x];
-        a.part[(size_t)(g * a.n_pad + i) * gridDim.x + blockIdx.x] = r;
-    }
-}
-
-// db: a warp per packed row adds its partial sums (fixed order); zeros for the
-// pruned filters.
-__global__ void __launch_bounds__(256) k_grid_db(const float* part, int nparts, const int* rowmap, const int* zeromap,
-                                                 const int* counts, int groups, int n_pad, int Fg, float* db)
-{
-    pdl_wait();  // after the kernel before it in the stream
-    const int lane = threadIdx.x & 31;
-    const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (r < groups * n_pad) {
-        const int f = __ldg(rowmap + r);
-        if (f >= 0) {
-            float s = 0.0f;
-            for (int k = lane; k < nparts; k += 32) s += __ldg(part + (size_t)r * nparts + k);
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-            if (lane == 0) db[f] = s;
-        }
-    }
-    for (int z = blockIdx.x * 256 + threadIdx.x; z < groups * Fg; z += gridDim.x * 256) {
-        const int g = z / Fg;
-        if (z - g * Fg < __ldg(counts + 2 * g + 1)) db[__ldg(zeromap + z)] = 0.0f;
+        a.part[(size_t)(g * a.n_pad + i) * a.bx + bx] = r;
     }
 }
 
@@ -583,29 +598,31 @@ struct PrepArgs {
     int* counts2;
     float* zero;  // dW (or NULL)
     long long zero_n;
+    int zblocks;  // blocks that zero it
 };
 
-// Blocks below `rows`: one output column (input channel) of the input
-// gradient's weights each, a quarter of its K columns per blockIdx.y; the
-// others zero dW.
-__global__ void __launch_bounds__(128) k_grid_prep(const PrepArgs a)
+// Block b of 256 threads, of rows*kPrepSplit + zblocks: below rows*kPrepSplit, a
+// share of the K columns of one output column (input channel) of the input
+// gradient's weights; the others zero dW.
+constexpr int kPrepSplit = 2;
+
+SADMM_DEV void prep_block(const PrepArgs& a, int b, int* s_j)
 {
-    pdl_wait();  // after the kernel before it in the stream
-    __shared__ int s_j[256];  // flipped tap -> packed column (-1: pruned)
-    if ((int)blockIdx.x >= a.rows) {
-        const long long nb = (long long)(gridDim.x - a.rows) * gridDim.y * 128;
-        for (long long i = ((long long)(blockIdx.x - a.rows) * gridDim.y + blockIdx.y) * 128 + threadIdx.x; i < a.zero_n; i += nb) a.zero[i] = 0.0f;
+    if (b >= a.rows * kPrepSplit) {
+        const long long nb = (long long)a.zblocks * 256;
+        for (long long i = (long long)(b - a.rows * kPrepSplit) * 256 + threadIdx.x; i < a.zero_n; i += nb) a.zero[i] = 0.0f;
         return;
     }
-    const int g = blockIdx.x / a.ncpad, jc = blockIdx.x - g * a.ncpad;
+    const int row = b / kPrepSplit, share = b - row * kPrepSplit;
+    const int g = row / a.ncpad, jc = row - g * a.ncpad;
     const int cnt = __ldg(a.counts + 2 * g);
     int c = jc < a.nck ? jc : -1;
     if (c >= 0 && a.chan_kind) {
         const int col = __ldg(a.colidx + jc * a.taps);
         c = col >= 0 ? col / a.taps : -1;
     }
-    if (threadIdx.x == 0 && blockIdx.y == 0) a.colmap[blockIdx.x] = c >= 0 ? g * a.Cg + c : -1;
-    for (int t = threadIdx.x; t < a.taps; t += 128) {
+    if (threadIdx.x == 0 && share == 0) a.colmap[row] = c >= 0 ? g * a.Cg + c : -1;
+    for (int t = threadIdx.x; t < a.taps; t += 256) {
         int j = -1;
         if (c >= 0) {
             const int want = c * a.taps + t;
@@ -623,10 +640,10 @@ __global__ void __launch_bounds__(128) k_grid_prep(const PrepArgs a)
     // [step][K half][bn][8] of this column's tile: a thread fills the 8 filters
     // of one half of a step
     const int nt = jc / a.bn, h8 = a.cb / 8;
-    uint4* wd = reinterpret_cast<uint4*>(a.wd) + ((size_t)(blockIdx.x / a.bn) * a.ksteps * 2) * a.bn + (jc - nt * a.bn);
+    uint4* wd = reinterpret_cast<uint4*>(a.wd) + ((size_t)(row / a.bn) * a.ksteps * 2) * a.bn + (jc - nt * a.bn);
     const unsigned short* wp = reinterpret_cast<const unsigned short*>(a.wp) + (size_t)g * a.n_pad * a.k_pad;
     const int kuse = min(a.ksteps, (cnt + a.cb - 1) / a.cb * a.taps * (a.cb / 16)) * 2;  // what an item may load
-    for (int k = blockIdx.y * 128 + threadIdx.x; k < kuse; k += gridDim.y * 128) {
+    for (int k = share * 256 + threadIdx.x; k < kuse; k += kPrepSplit * 256) {
         int t = k / h8;
         const int c8 = k - t * h8;
         const int blk = t / a.taps;
@@ -643,7 +660,7 @@ __global__ void __launch_bounds__(128) k_grid_prep(const PrepArgs a)
         }
         wd[(size_t)k * a.bn] = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
     }
-    if (jc == 0 && blockIdx.y == 0) {
+    if (jc == 0 && share == 0) {
         // the group's output columns and the pruned channels' planes
         const bool none = a.chan_kind && (a.n_cols == 0 || __ldg(a.colidx) < 0);
         const int ncols = none ? 0 : a.nck;
@@ -652,7 +669,7 @@ __global__ void __launch_bounds__(128) k_grid_prep(const PrepArgs a)
             a.counts2[2 * g + 1] = a.Cg - ncols;
         }
         if (a.chan_kind)
-            for (int ch = threadIdx.x; ch < a.Cg; ch += 128) {
+            for (int ch = threadIdx.x; ch < a.Cg; ch += 256) {
                 int lo = 0, hi = ncols;
                 while (lo < hi) {
                     const int mid = (lo + hi) >> 1;
@@ -662,6 +679,31 @@ __global__ void __launch_bounds__(128) k_grid_prep(const PrepArgs a)
                 if (!(lo < ncols && __ldg(a.colidx + lo * a.taps) / a.taps == ch)) a.zmap[g * a.Cg + ch - lo] = g * a.Cg + ch;
             }
     }
+}
+
+// The copies and the input gradient's weights in one launch: blocks of dZ, then
+// of x, then of the weights and dW's zeros.
+struct FrontArgs {
+    DzArgs dz;
+    GridX x;
+    PrepArgs prep;
+    int ndz, nx, np;  // blocks of each
+};
+
+template <bool RELU, typename Y>
+__global__ void __launch_bounds__(256) k_grid_front(const __grid_constant__ FrontArgs a)
+{
+    pdl_wait();  // after the kernel before it in the stream
+    pdl_trigger();
+    __shared__ int s_i[256];
+    __shared__ float s_part[8][8];
+    const int b = blockIdx.x;
+    if (b < a.ndz)
+        dz_block<RELU, Y>(a.dz, b % a.dz.bx, b / a.dz.bx, s_i, s_part);
+    else if (b < a.ndz + a.nx)
+        grid_x_block(a.x, (b - a.ndz) % a.x.bx, (b - a.ndz) / a.x.bx, s_i);
+    else
+        prep_block(a.prep, b - a.ndz - a.nx, s_i);
 }
 
 struct GridBwd {
@@ -684,7 +726,10 @@ bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, GridBwd* out)
     if (!wgrad_shape(b.gr, b.nck, plan->n_pad, (int)g.groups, &b.ws)) return false;
     b.dchunks = std::max(b.cs.k16 * 2, b.ws.nft * b.ws.nst / 8);
     b.nparts = (b.gr.slots + kDzSlots - 1) / kDzSlots;
-    if (g.groups * b.dchunks > 65535 || g.groups * ((b.ws.nch + 1) / 2) > 65535) return false;
+    if ((long long)b.nparts * g.groups * b.dchunks + (b.gr.slots / 256 + 1) * g.groups * ((b.ws.nch + 1) / 2) +
+            2 * g.groups * b.cs.npad + 256 >= (1ll << 31) ||
+        g.groups * ((b.ws.nch + 1) / 2) > 65535)
+        return false;
     size_t off = 0;
     auto take = [&off](long long bytes) {
         const size_t at = off;
@@ -733,9 +778,10 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
     const int* chans = chan_kind ? colidx : nullptr;
     const long long xs_g = (long long)b.ws.nch * b.gr.slots * 8, dz_g = (long long)b.dchunks * b.gr.slots * 8;
 
+    FrontArgs fa;
+    memset(&fa, 0, sizeof(fa));
     if (dW || dx) {
-        PrepArgs p;
-        memset(&p, 0, sizeof(p));
+        PrepArgs& p = fa.prep;
         p.wp = reinterpret_cast<const __nv_bfloat16*>(base + plan->off_wp);
         p.colidx = colidx;
         p.counts = counts;
@@ -758,11 +804,10 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         p.counts2 = counts2;
         p.zero = dW;
         p.zero_n = dW ? g.f * g.k : 0;
-        const long long nz = dW ? std::min<long long>(256, (p.zero_n + 2047) / 2048) : 0;
-        if (launch_pdl(k_grid_prep, dim3((unsigned)(p.rows + nz), 4), dim3(128), 0, s, p) != cudaSuccess) return SADMM_ECUDA;
+        p.zblocks = dW ? (int)std::min<long long>(256, (p.zero_n + 2047) / 2048) : 0;
+        fa.np = p.rows * kPrepSplit + p.zblocks;
     }
-    DzArgs d;
-    memset(&d, 0, sizeof(d));
+    DzArgs& d = fa.dz;
     d.gr = b.gr;
     d.dy = static_cast<const __nv_bfloat16*>(dy);
     d.y = y;
@@ -775,20 +820,34 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
     d.cb = b.cs.cb;
     d.dz = (dW || dx) ? dz : nullptr;
     d.part = db ? part : nullptr;
-    const dim3 dgrid((unsigned)b.nparts, (unsigned)(g.groups * b.dchunks));
-    const cudaError_t de =
-        !relu ? launch_pdl(k_grid_dz<false, float>, dgrid, dim3(256), 0, s, d)
-              : (ydt == SADMM_BF16 ? launch_pdl(k_grid_dz<true, unsigned short>, dgrid, dim3(256), 0, s, d)
-                                   : launch_pdl(k_grid_dz<true, float>, dgrid, dim3(256), 0, s, d));
-    if (de != cudaSuccess) return SADMM_ECUDA;
-    if (db &&
-        launch_pdl(k_grid_db, dim3((unsigned)((g.groups * plan->n_pad + 7) / 8)), dim3(256), 0, s,
-                   static_cast<const float*>(part), b.nparts, rowmap, zeromap, counts, (int)g.groups, plan->n_pad,
-                   (int)g.fg, db) != cudaSuccess)
+    d.bx = b.nparts;
+    d.by = (int)(g.groups * b.dchunks);
+    fa.ndz = d.bx * d.by;
+    if (dW) {
+        if (!grid_x_args(b.gr, g, x, chans, b.nck, b.ws.nch, xs, &fa.x)) return SADMM_EUNSUPPORTED;
+        fa.nx = fa.x.bx * fa.x.by;
+    }
+    const dim3 fgrid((unsigned)(fa.ndz + fa.nx + fa.np));
+    const cudaError_t fe =
+        !relu ? launch_pdl(k_grid_front<false, float>, fgrid, dim3(256), 0, s, fa)
+              : (ydt == SADMM_BF16 ? launch_pdl(k_grid_front<true, unsigned short>, fgrid, dim3(256), 0, s, fa)
+                                   : launch_pdl(k_grid_front<true, float>, fgrid, dim3(256), 0, s, fa));
+    if (fe != cudaSuccess) return SADMM_ECUDA;
+    DbArgs dd;
+    memset(&dd, 0, sizeof(dd));
+    dd.part = part;
+    dd.rowmap = rowmap;
+    dd.zeromap = zeromap;
+    dd.counts = counts;
+    dd.nparts = b.nparts;
+    dd.groups = (int)g.groups;
+    dd.n_pad = plan->n_pad;
+    dd.Fg = (int)g.fg;
+    dd.db = db;
+    if (db && !dW &&
+        launch_pdl(k_grid_db, dim3((unsigned)((g.groups * plan->n_pad + 7) / 8)), dim3(256), 0, s, dd) != cudaSuccess)
         return SADMM_ECUDA;
     if (dW) {
-        const sadmm_status st = launch_grid_x(b.gr, g, x, chans, b.nck, b.ws.nch, xs, s);
-        if (st != SADMM_OK) return st;
         GwArgs a;
         memset(&a, 0, sizeof(a));
         a.gr = b.gr;
@@ -838,8 +897,8 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         r.K = g.k;
         if (launch_pdl(k_grid_wreduce,
                        dim3((unsigned)((plan->n_cols + kWrCols - 1) / kWrCols), (unsigned)((plan->n_pad + 31) / 32),
-                            (unsigned)g.groups),
-                       dim3(256), 0, s, r) != cudaSuccess)
+                            (unsigned)g.groups + (db ? 1u : 0u)),
+                       dim3(256), 0, s, r, dd) != cudaSuccess)
             return SADMM_ECUDA;
     }
     if (dx) {

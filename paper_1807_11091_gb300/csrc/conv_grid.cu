@@ -520,46 +520,11 @@ __global__ void __launch_bounds__(kGcThreads, 1)
     }
 }
 
-// Grid copy of x.  Thread t of block (bx, by): slot 256*bx + t, two chunks of
-// conv group by / pairs (16 loads in flight, each coalesced along the row).
-__global__ void __launch_bounds__(256) k_grid_x(const __nv_bfloat16* __restrict__ x, const int* __restrict__ colidx,
-                                                const Grid gr, int C, int Cg, int nck, int chunks, int taps,
-                                                long long x_total, int* status, __nv_bfloat16* __restrict__ xs)
+__global__ void __launch_bounds__(256) k_grid_x(const GridX a)
 {
-    __shared__ int s_off[16];  // channel plane offset (-1: zero)
     pdl_wait();  // after the kernel before it in the stream
-    const int pairs = (chunks + 1) / 2;
-    const int g = blockIdx.y / pairs, c0 = (blockIdx.y - g * pairs) * 2;
-    const int thw = gr.T * gr.H * gr.W;
-    if (threadIdx.x < 16) {
-        const int ci = c0 * 8 + threadIdx.x;
-        int ch = ci < nck ? ci : -1;
-        if (ch >= 0 && colidx) {
-            const int col = __ldg(colidx + ci * taps);
-            ch = col >= 0 ? col / taps : -1;
-        }
-        s_off[threadIdx.x] = ch >= 0 ? (g * Cg + ch) * thw : -1;
-    }
-    __syncthreads();
-    const int s = blockIdx.x * 256 + threadIdx.x;
-    if (s >= gr.slots) return;
-    int n, t, h, w;
-    grid_decode(gr, s, n, t, h, w);
-    const bool valid = n < gr.N && t >= gr.pt && h >= gr.ph && w >= gr.pw;
-    const long long base = (long long)n * C * thw + (long long)(t - gr.pt) * (gr.H * gr.W) +
-                           (long long)(h - gr.ph) * gr.W + (w - gr.pw);
-    const unsigned short* xi = reinterpret_cast<const unsigned short*>(x);
-    uint32_t v[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        const int off = s_off[e];
-        v[e] = (valid && off >= 0 && dbg_in(base + off, x_total, status)) ? (uint32_t)__ldg(xi + base + off) : 0u;
-    }
-    uint4* dst = reinterpret_cast<uint4*>(xs) + ((size_t)g * chunks + c0) * gr.slots + s;
-    dst[0] = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
-    if (c0 + 1 < chunks)
-        dst[gr.slots] =
-            make_uint4(v[8] | (v[9] << 16), v[10] | (v[11] << 16), v[12] | (v[13] << 16), v[14] | (v[15] << 16));
+    __shared__ int s_off[16];
+    grid_x_block(a, blockIdx.x, blockIdx.y, s_off);
 }
 
 template <bool OUT_BF16, int MT>
@@ -703,16 +668,32 @@ sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const Gri
     return e == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
 }
 
-sadmm_status launch_grid_x(const Grid& gr, const Geometry& g, const void* x, const int* colidx, int nck, int chunks,
-                           __nv_bfloat16* xs, cudaStream_t s)
+bool grid_x_args(const Grid& gr, const Geometry& g, const void* x, const int* colidx, int nck, int chunks,
+                 __nv_bfloat16* xs, GridX* a)
 {
-    const long long rows = g.groups * ((chunks + 1) / 2);
-    if (rows > 65535) return SADMM_EUNSUPPORTED;
-    const cudaError_t e =
-        launch_pdl(k_grid_x, dim3((unsigned)((gr.slots + 255) / 256), (unsigned)rows), dim3(256), 0, s,
-                   static_cast<const __nv_bfloat16*>(x), colidx, gr, (int)g.c, (int)g.cg, nck, chunks, (int)g.taps,
-                   g.n * g.c * g.t * g.h * g.w, device_status_ptr(), xs);
-    return e == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
+    a->gr = gr;
+    a->x = static_cast<const __nv_bfloat16*>(x);
+    a->colidx = colidx;
+    a->xs = xs;
+    a->C = (int)g.c;
+    a->Cg = (int)g.cg;
+    a->nck = nck;
+    a->chunks = chunks;
+    a->taps = (int)g.taps;
+    a->x_total = g.n * g.c * g.t * g.h * g.w;
+    a->status = device_status_ptr();
+    a->bx = (gr.slots + 255) / 256;
+    a->by = (int)(g.groups * ((chunks + 1) / 2));
+    return a->by <= 65535;
+}
+
+static sadmm_status launch_grid_x(const Grid& gr, const Geometry& g, const void* x, const int* colidx, int nck, int chunks,
+                                  __nv_bfloat16* xs, cudaStream_t s)
+{
+    GridX a;
+    if (!grid_x_args(gr, g, x, colidx, nck, chunks, xs, &a)) return SADMM_EUNSUPPORTED;
+    return launch_pdl(k_grid_x, dim3((unsigned)a.bx, (unsigned)a.by), dim3(256), 0, s, a) == cudaSuccess ? SADMM_OK
+                                                                                                         : SADMM_ECUDA;
 }
 
 // The rule for the forward compares estimated times on a whole GB300, whatever

@@ -115,9 +115,20 @@ struct GridConvCall {
 sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const GridConvCall& c, cudaStream_t s);
 
 // x (bf16 NCTHW) -> grid copy of `nck` channels per group (kept channels
-// colidx[ci*taps]/taps when colidx != NULL, else 0..nck-1), `chunks` chunks.
-sadmm_status launch_grid_x(const Grid& gr, const Geometry& g, const void* x, const int* colidx, int nck, int chunks,
-                           __nv_bfloat16* xs, cudaStream_t s);
+// colidx[ci*taps]/taps when colidx != NULL, else 0..nck-1), `chunks` chunks, by
+// bx x by blocks of 256 threads.
+struct GridX {
+    Grid gr;
+    const __nv_bfloat16* x;
+    const int* colidx;
+    __nv_bfloat16* xs;
+    int C, Cg, nck, chunks, taps, bx, by;
+    long long x_total;
+    int* status;
+};
+// False when by passes the grid limit.
+bool grid_x_args(const Grid& gr, const Geometry& g, const void* x, const int* colidx, int nck, int chunks,
+                 __nv_bfloat16* xs, GridX* a);
 
 // ---- grid forward (conv_grid.cu) ----
 // Whether the plan's forward takes the grid; its tiling then, and the bytes of
@@ -158,6 +169,45 @@ SADMM_DEV void grid_decode(const Grid& gr, int q, int& n, int& t, int& h, int& w
     r -= t * gr.HWb;
     h = (int)fdiv((uint32_t)r, gr.w_div);
     w = r - h * gr.Wb;
+}
+
+// Block (bx, by) of the grid copy of x, 256 threads: thread t takes slot
+// 256*bx + t of two chunks of conv group by / pairs (16 loads in flight, each
+// coalesced along the row); s_off: 16 ints of shared memory.
+SADMM_DEV void grid_x_block(const GridX& a, int bx, int by, int* s_off)
+{
+    const int pairs = (a.chunks + 1) / 2;
+    const int g = by / pairs, c0 = (by - g * pairs) * 2;
+    const int thw = a.gr.T * a.gr.H * a.gr.W;
+    if (threadIdx.x < 16) {  // channel plane offsets (-1: zero)
+        const int ci = c0 * 8 + threadIdx.x;
+        int ch = ci < a.nck ? ci : -1;
+        if (ch >= 0 && a.colidx) {
+            const int col = __ldg(a.colidx + ci * a.taps);
+            ch = col >= 0 ? col / a.taps : -1;
+        }
+        s_off[threadIdx.x] = ch >= 0 ? (g * a.Cg + ch) * thw : -1;
+    }
+    __syncthreads();
+    const int s = bx * 256 + threadIdx.x;
+    if (s >= a.gr.slots) return;
+    int n, t, h, w;
+    grid_decode(a.gr, s, n, t, h, w);
+    const bool valid = n < a.gr.N && t >= a.gr.pt && h >= a.gr.ph && w >= a.gr.pw;
+    const long long base = (long long)n * a.C * thw + (long long)(t - a.gr.pt) * (a.gr.H * a.gr.W) +
+                           (long long)(h - a.gr.ph) * a.gr.W + (w - a.gr.pw);
+    const unsigned short* xi = reinterpret_cast<const unsigned short*>(a.x);
+    uint32_t v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const int off = s_off[e];
+        v[e] = (valid && off >= 0 && dbg_in(base + off, a.x_total, a.status)) ? (uint32_t)__ldg(xi + base + off) : 0u;
+    }
+    uint4* dst = reinterpret_cast<uint4*>(a.xs) + ((size_t)g * a.chunks + c0) * a.gr.slots + s;
+    dst[0] = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+    if (c0 + 1 < a.chunks)
+        dst[a.gr.slots] =
+            make_uint4(v[8] | (v[9] << 16), v[10] | (v[11] << 16), v[12] | (v[13] << 16), v[14] | (v[15] << 16));
 }
 
 }  // namespace sadmm
