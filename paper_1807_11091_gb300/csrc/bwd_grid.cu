@@ -13,10 +13,10 @@
 //                  are the copies themselves, read MN-major (core matrices of 8
 //                  channels x 8 pixels); dZ is zero off the output, so the
 //                  padded pixels add nothing.
-//   k_grid_wreduce the slices of the pixel ranges, in order, into dW's kept
-//                  entries, and db's partial sums
 //   k_grid_conv    dx: the slab GEMM over dZ (conv_grid.cu), every element
 //                  written once
+//   k_grid_wreduce the slices of the pixel ranges, in order, into dW's kept
+//                  entries, and db's partial sums
 //
 // A layer of at most 64 channels fills half of the M side or less: its slab is
 // then staged up to 16 / chunks times, each copy a pixel further on, and one
@@ -24,12 +24,13 @@
 // The tensor core truncates as it accumulates (about 1e-8 of the result per
 // step of 16 pixels), so a slice takes at most kGwMaxTiles tiles of 128.
 //
-// AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5;
-// one cold launch each, against the six im2col / GEMM / col2im chunks before,
-// 841 us in all): dZ 28 us (99 MB moved), x copy 9, weight gradient 72 (57
-// cycles per 128 x 64 x 16 MMA: bound by the operands' shared-memory reads, 96
-// of the 128 rows in use), its reduction 14, input gradient 59 (57 cycles per
-// 128 x 48 x 16).  conv3: 8.5 / 7 / 18 / 10 / 19 us.
+// AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5):
+// 841 us as six im2col / GEMM / col2im chunks, 175 us here.  One cold launch each:
+// front 39 us (138 MB moved; each dZ octet is 16 loads of 2 and 4 bytes), weight
+// gradient 72 (57 cycles per 128 x 64 x 16 MMA: bound by the operands'
+// shared-memory reads, 96 of the 128 rows in use), input gradient 60 (57 cycles
+// per 128 x 48 x 16), reduction 14.  conv3, 164 -> 55 us: 13.5 / 20 / 18 / 14;
+// a ResNet-50 3x3 layer of 64 channels at batch 64, 277 -> 58.
 #include <string.h>
 
 #include <algorithm>
@@ -217,10 +218,10 @@ __global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_const
         tmem_relinquish();
     }
     pdl_wait();
-    pdl_trigger();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();  // after every thread's wait: k_grid_front has completed when a dependent starts
     const uint32_t tmem_base = *tmem_holder;
     // two accumulator sets when every item's columns fit half of TMEM
     int most = 0;
@@ -436,7 +437,7 @@ constexpr int kWrCols = 4;
 
 __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbArgs d)
 {
-    pdl_wait();  // after the kernel before it in the stream
+    pdl_wait();  // after the kernel before it in the stream, and the one before that (see launch_grid_bwd)
     pdl_trigger();
     __shared__ float s_v[8][kWrCols][32];
     if ((int)blockIdx.z == d.groups) {  // the last layer of blocks: the bias gradient
@@ -847,6 +848,7 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
     if (db && !dW &&
         launch_pdl(k_grid_db, dim3((unsigned)((g.groups * plan->n_pad + 7) / 8)), dim3(256), 0, s, dd) != cudaSuccess)
         return SADMM_ECUDA;
+    WrArgs r;
     if (dW) {
         GwArgs a;
         memset(&a, 0, sizeof(a));
@@ -877,7 +879,6 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         const int grid = std::min(a.units, device_sm_count());
         if (launch_pdl(k_grid_wgrad, dim3((unsigned)grid), dim3(kGwThreads), b.ws.smem, s, a) != cudaSuccess)
             return SADMM_ECUDA;
-        WrArgs r;
         memset(&r, 0, sizeof(r));
         r.gr = b.gr;
         r.w = b.ws;
@@ -895,12 +896,15 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         r.taps = (int)g.taps;
         r.chan_kind = chan_kind;
         r.K = g.k;
-        if (launch_pdl(k_grid_wreduce,
-                       dim3((unsigned)((plan->n_cols + kWrCols - 1) / kWrCols), (unsigned)((plan->n_pad + 31) / 32),
-                            (unsigned)g.groups + (db ? 1u : 0u)),
-                       dim3(256), 0, s, r, dd) != cudaSuccess)
-            return SADMM_ECUDA;
     }
+    // The input gradient reads what k_grid_front wrote and nothing of k_grid_wgrad's.
+    // Every CTA of k_grid_wgrad lets it start only after its own wait for
+    // k_grid_front, so it does not wait first: its CTAs take the SMs as the weight
+    // gradient's leave them (its two rounds of items end unevenly: AlexNet conv2 at
+    // batch 128 189 -> 176 us, conv3 59.2 -> 55.1, a ResNet-50 3x3 layer at batch 64
+    // 61.1 -> 58.4).  It waits for k_grid_wgrad at its end, for the reduction behind
+    // it.  (The reduction between the two, beside the input gradient's start: 185, 55
+    // and 58 us.)
     if (dx) {
         GridConvCall c;
         memset(&c, 0, sizeof(c));
@@ -920,9 +924,17 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         c.VH = (int)g.h;
         c.VW = (int)g.w;
         c.out_total = g.n * g.c * g.t * g.h * g.w;
+        c.late_wait = dW != nullptr;  // (k_grid_wgrad stands between)
         const sadmm_status st = launch_grid_conv(b.gr, b.cs, c, s);
         if (st != SADMM_OK) return st;
     }
+    if (dW) {
+        if (launch_pdl(k_grid_wreduce,
+                       dim3((unsigned)((plan->n_cols + kWrCols - 1) / kWrCols), (unsigned)((plan->n_pad + 31) / 32),
+                            (unsigned)g.groups + (db ? 1u : 0u)),
+                       dim3(256), 0, s, r, dd) != cudaSuccess)
+            return SADMM_ECUDA;
+        }
     return cudaGetLastError() == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
 }
 

@@ -64,6 +64,8 @@ SADMM_DEV int atom_add_acq_rel_gpu(int* p, int v)
 // completed and its memory is visible, so it comes before the first read of
 // anything an earlier kernel wrote.  pdl_trigger() lets the next kernel of the
 // stream be scheduled once every CTA of this one has issued it (or exited).
+// A kernel's completion means that of every kernel before it: each one waits,
+// at its start or (k_grid_conv's late_wait) at its end.
 SADMM_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 SADMM_DEV void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -57,6 +57,7 @@ struct GcArgs {
     int* status;
     long long out_total;
     long long gstride;  // source elements per group
+    int late_wait;
     int zstride, groups, planes, plane, VT, VH, VW, VHW;
     int units, mtiles, ntiles;
     FastDiv mt_div, nt_div;
@@ -264,11 +265,11 @@ __global__ void __launch_bounds__(kGcThreads, 1)
         tmem_relinquish();
     }
     // Nothing above reads global memory: it overlaps the previous kernel's tail.
-    pdl_wait();
-    pdl_trigger();
+    if (!a.late_wait) pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();  // (every CTA has its TMEM: a dependent's allocation cannot come first)
     const uint32_t tmem_base = *tmem_holder;
     // The weights of a group stay in shared memory when there is one column
     // tile and every group's (as many steps as its channels need) fit.
@@ -518,6 +519,8 @@ __global__ void __launch_bounds__(kGcThreads, 1)
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)a.tmem_cols);
     }
+    // TMEM is free: what this waits for may still need it.
+    if (a.late_wait) pdl_wait();
 }
 
 __global__ void __launch_bounds__(256) k_grid_x(const GridX a)
@@ -625,6 +628,7 @@ sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const Gri
     a.kcounts = c.kcounts;
     a.status = device_status_ptr();
     a.out_total = c.out_total;
+    a.late_wait = c.late_wait ? 1 : 0;
     a.gstride = (long long)c.chunks * gr.slots * 8;
     a.groups = c.groups;
     a.planes = c.planes;

@@ -111,6 +111,10 @@ struct GridConvCall {
     int VT, VH, VW;        // its extents
     long long out_total;
     int ctas;
+    // 1: the kernel before this one in the stream writes nothing it reads, and lets
+    // it start only when the one that wrote its inputs has completed.  It then
+    // waits for that kernel at its end, so that its completion still means both.
+    int late_wait;
 };
 sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const GridConvCall& c, cudaStream_t s);
 

@@ -264,8 +264,6 @@ SADMM_DEV float load_f32<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloa
 template <>
 SADMM_DEV float load_f32<float>(const float* p) { return *p; }
 
-// Row r of a layer: rows past `rows` pack the input-slab plan's weights, row
-// r - rows of conv group 0 through the slab column map scol, into wps [bn][kpad_s].
 // Row r (kept filter i of conv group g) of a pixel-grid plan's weights
 // [g][tile][step][K half][row][8]: a thread writes the 8 channels of one half of
 // a step, -0.0 at pruned columns (a kept weight that is -0.0 as +0.0: no product
@@ -296,6 +294,9 @@ SADMM_DEV void pack_wg_row(const WpLayer& L, int r)
     }
 }
 
+// Row r of a layer: rows past `rows` pack the input-slab plan's weights, row
+// r - rows of conv group 0 through the slab column map scol, into wps
+// [bn][kpad_s]; rows past those the pixel-grid plan's.
 template <typename T>
 SADMM_DEV void pack_wp_row(const WpLayer& L, long long r)
 {
