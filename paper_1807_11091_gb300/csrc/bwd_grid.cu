@@ -25,12 +25,13 @@
 // step of 16 pixels), so a slice takes at most kGwMaxTiles tiles of 128.
 //
 // AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5):
-// 841 us as six im2col / GEMM / col2im chunks, 175 us here.  One cold launch each:
+// 841 us as six im2col / GEMM / col2im chunks, 173 us here.  One cold launch each:
 // front 39 us (138 MB moved; each dZ octet is 16 loads of 2 and 4 bytes), weight
 // gradient 72 (57 cycles per 128 x 64 x 16 MMA: bound by the operands'
 // shared-memory reads, 96 of the 128 rows in use), input gradient 60 (57 cycles
-// per 128 x 48 x 16), reduction 14.  conv3, 164 -> 55 us: 13.5 / 20 / 18 / 14;
-// a ResNet-50 3x3 layer of 64 channels at batch 64, 277 -> 58.
+// per 128 x 48 x 16), reduction 15.  conv3, 164 -> 52 us: 14 / 18 / 20 / 11; a
+// ResNet-50 3x3 layer (64 of 128 channels and filters kept) at batch 64, 277 -> 48:
+// 13 / 17 / 18 / 10.
 #include <string.h>
 
 #include <algorithm>
@@ -62,7 +63,8 @@ struct WgradShape {
     long long slice;  // floats of a pixel range's slice
 };
 
-bool wgrad_shape(const Grid& gr, int nck, int n_pad, int groups, WgradShape* out)
+// `nck` channels and at most `n_pad`, likely `likely`, filters per group.
+bool wgrad_shape(const Grid& gr, int nck, int n_pad, int likely, int groups, WgradShape* out)
 {
     WgradShape w;
     if (nck < 1) return false;
@@ -79,11 +81,25 @@ bool wgrad_shape(const Grid& gr, int nck, int n_pad, int groups, WgradShape* out
     w.rows = w.rep * w.blk * 8;
     w.nft = (n_pad + 255) / 256;
     w.nst = (int)round_up((n_pad + w.nft - 1) / w.nft, 16);
+    w.tiles = (gr.L + 127) / 128;
     const int macro = gr.KH * w.kwg;
-    w.tpg = std::min(std::min(kGwCols / w.nst, macro), 32);
-    for (;; --w.tpg) {  // fewer taps per item until two stages of their slab fit
-        if (w.tpg < 1) return false;
+    const int nl = std::min(w.nst, (int)round_up(likely, 16));
+    // The taps of an item: what fits TMEM and leaves two stages of slabs; below
+    // that, the split of the taps of least estimated time.  Fewer taps an item
+    // mean longer pixel ranges, so fewer slices to write and to add up, for more
+    // slab loads: a 3x3 layer of 64 kept channels and filters at batch 64 runs its
+    // 6 MMA taps as two items of 6 tiles, not one of 3: its slices are 14 MB, not
+    // 28, and its backward takes 48 us, not 53.  Only for a fifth less by the
+    // estimate: AlexNet conv3 as three items of 8 tiles, not two of 6, is 18 % less
+    // by it and measured 53.9 against 53.4 us (SMs without an item start the input
+    // gradient early).
+    const int tmax = std::min(std::min(kGwCols / w.nst, macro), 32);
+    if (tmax < 1) return false;
+    long long best = -1;
+    for (int tgs = (macro + tmax - 1) / tmax; tgs <= macro; ++tgs) {
+        w.tpg = (macro + tgs - 1) / tgs;
         w.tgs = (macro + w.tpg - 1) / w.tpg;
+        if (w.tgs != tgs) continue;
         int span = 0;
         for (int t0 = 0; t0 < macro; t0 += w.tpg) {
             int lo = 1 << 30, hi = 0;
@@ -101,19 +117,31 @@ bool wgrad_shape(const Grid& gr, int nck, int n_pad, int groups, WgradShape* out
         const long long fixed = 1024 + 512 + (long long)(16 - w.rep * w.blk) * w.spa * 16;
         w.stages = (int)std::min<long long>(kGwMaxStages, (kGwSmemLimit - fixed) / w.stage_stride);
         w.smem = (size_t)(fixed + (long long)w.stages * w.stage_stride);
-        if (w.spa < (1 << 14) && w.stages >= 2 && (w.stages >= 3 || w.tpg == 1)) break;
+        if (w.spa >= (1 << 14) || w.stages < 2 || (w.stages < 3 && w.tpg > 1)) continue;
+        const long long types = (long long)groups * w.nft * w.mblks * gr.KT * w.tgs;
+        const long long work = types * w.tiles;
+        const long long waves = std::max<long long>(1, (work + kGwCtas * kGwMaxTiles - 1) / (kGwCtas * kGwMaxTiles));
+        w.tps = (int)std::max<long long>(1, std::min<long long>(kGwMaxTiles, (work + kGwCtas * waves - 1) / (kGwCtas * waves)));
+        w.Z = (w.tiles + w.tps - 1) / w.tps;
+        if (types * w.Z >= (1ll << 30)) continue;
+        w.types = (int)types;
+        w.slice = types * w.rows * w.tpg * w.nst;
+        // Cycles: rounds of items, each its tiles' MMAs (as in conv_grid.cu) or
+        // loads (40 bytes a cycle), then its slice's stores (32 bytes a cycle;
+        // beside the next item's MMAs when two accumulator sets fit), and the
+        // reduction's reads (16 bytes a cycle and SM).
+        const long long cols = (long long)macro * nl / w.tgs;
+        const long long tile = std::max((long long)macro * 8 * (std::max(32 + nl / 4, nl / 2) + 9) / w.tgs,
+                                        (w.a_bytes + nl * 256ll) / 40) + 150;
+        const long long st = w.rows * cols / 8, item = w.tps * tile, rounds = (types * w.Z + kGwCtas - 1) / kGwCtas;
+        const long long cost = (w.tpg * nl <= kGwCols / 2 ? rounds * std::max(item, st) + st : rounds * (item + st)) +
+                               types * w.Z * w.rows * cols * 4 / (kGwCtas * 16);
+        if (best < 0 || cost * 5 < best * 4) {
+            best = cost;
+            *out = w;
+        }
     }
-    const long long types = (long long)groups * w.nft * w.mblks * gr.KT * w.tgs;
-    w.tiles = (gr.L + 127) / 128;
-    const long long work = types * w.tiles;
-    const long long waves = std::max<long long>(1, (work + kGwCtas * kGwMaxTiles - 1) / (kGwCtas * kGwMaxTiles));
-    w.tps = (int)std::max<long long>(1, std::min<long long>(kGwMaxTiles, (work + kGwCtas * waves - 1) / (kGwCtas * waves)));
-    w.Z = (w.tiles + w.tps - 1) / w.tps;
-    if (types * w.Z >= (1ll << 30)) return false;
-    w.types = (int)types;
-    w.slice = types * w.rows * w.tpg * w.nst;
-    *out = w;
-    return true;
+    return best >= 0;
 }
 
 struct GwArgs {
@@ -429,68 +457,104 @@ struct WrArgs {
     long long K;
 };
 
-// dW[f_i][col_j] = sum over the pixel ranges of their slices: eight threads per
-// entry take every eighth range, then their sums are added in order
+// dW[f_i][col_j] = sum over the pixel ranges of their slices: 32 threads per four
+// filters take every 32nd range, then their sums are added in order
 // (deterministic).  Block (bx, by, g): packed columns bx*kWrCols .., packed rows
-// by*32 .. +31; the slices are read along the filters.
+// by*32 .. +31; the slices are read along the filters, 16 bytes a load.
+// Bound by latency: the slices are in L2, so what counts is loads in flight (16 of
+// 16 bytes a thread, the layer's ranges in one pass up to 128 of them) and what is
+// done before the wait.  With eight range lanes of 4-byte loads, four ranges a pass
+// and the tables read after the wait it stood 10 to 14 us behind the layer (AlexNet
+// conv3 55.2 us in all, now 51.7).
 constexpr int kWrCols = 4;
 
 __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbArgs d)
 {
-    pdl_wait();  // after the kernel before it in the stream, and the one before that (see launch_grid_bwd)
-    pdl_trigger();
-    __shared__ float s_v[8][kWrCols][32];
+    __shared__ float s_v[8][kWrCols][40];
     if ((int)blockIdx.z == d.groups) {  // the last layer of blocks: the bias gradient
+        pdl_wait();
+        pdl_trigger();
         db_blocks(d, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
         return;
     }
+    // The plan's tables: k_grid_front read them too and has completed.
     const int g = blockIdx.z, cnt = __ldg(a.counts + 2 * g);
     const int i0 = blockIdx.y * 32, j0 = blockIdx.x * kWrCols;
     if (i0 >= cnt) return;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int i = i0 + tx;
-    const int ft = i / a.w.nst;
+    const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+    const int iq = i0 + tx * 4, ftq = iq / a.w.nst;  // (a tile's filters are a multiple of 16)
     const float* src[kWrCols];
-    int shift[kWrCols], chan[kWrCols];
-    float v[kWrCols];
 #pragma unroll
     for (int e = 0; e < kWrCols; ++e) {
         const int j = j0 + e;
         const int col = j < a.n_cols ? __ldg(a.colidx + j) : -1;
-        v[e] = 0.0f;
-        src[e] = nullptr;
-        if (col < 0 || i >= cnt) continue;
+        src[e] = a.slices;  // (nothing reads what this adds up)
+        if (col < 0 || iq >= cnt) continue;
         const int c = a.chan_kind ? j / a.taps : col / a.taps, tap = col % a.taps;
         const int kw = tap % a.gr.KW, kh = (tap / a.gr.KW) % a.gr.KH, kt = tap / (a.gr.KW * a.gr.KH);
         const int mb = (c >> 3) / a.w.blk, mt = kh * a.w.kwg + kw / a.w.rep;
         const int m = (((kw % a.w.rep) * a.w.blk + ((c >> 3) - mb * a.w.blk)) << 3) + (c & 7);
-        const int type = (((g * a.w.nft + ft) * a.w.mblks + mb) * a.gr.KT + kt) * a.w.tgs + mt / a.w.tpg;
-        chan[e] = c;
-        shift[e] = kt * a.gr.HWb + kh * a.gr.Wb + kw;
+        const int type = (((g * a.w.nft + ftq) * a.w.mblks + mb) * a.gr.KT + kt) * a.w.tgs + mt / a.w.tpg;
         src[e] = a.slices + ((size_t)type * a.w.rows + m) * (size_t)(a.w.tpg * a.w.nst) + (mt % a.w.tpg) * a.w.nst +
-                 (i - ft * a.w.nst);
+                 (iq - ftq * a.w.nst);
     }
-#pragma unroll 4
-    for (int z = ty; z < a.w.Z; z += 8)
+    // the entry this thread writes: four threads to a filter's four columns
+    const int oe = threadIdx.x & 3, oi = i0 + (threadIdx.x >> 2);
+    const int ocol = threadIdx.x < 128 && j0 + oe < a.n_cols ? __ldg(a.colidx + j0 + oe) : -1;
+    const int of = ocol >= 0 && oi < cnt ? __ldg(a.rowmap + g * a.n_pad + oi) : -1;
+    pdl_wait();  // after the kernel before it in the stream, and the one before that (see launch_grid_bwd)
+    pdl_trigger();
+    float v[kWrCols][4];
 #pragma unroll
-        for (int e = 0; e < kWrCols; ++e)
-            if (src[e]) v[e] += __ldcs(src[e] + (size_t)z * a.w.slice);
+    for (int e = 0; e < kWrCols; ++e)
 #pragma unroll
-    for (int e = 0; e < kWrCols; ++e) s_v[ty][e][tx] = v[e];
+        for (int q = 0; q < 4; ++q) v[e][q] = 0.0f;
+#pragma unroll 1
+    for (int z = ty; z < a.w.Z; z += 128) {
+        float4 t[4][kWrCols];  // every load first
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const bool in = z + 32 * r < a.w.Z;
+            const size_t at = (size_t)(z + 32 * r) * a.w.slice;
+#pragma unroll
+            for (int e = 0; e < kWrCols; ++e) {
+                t[r][e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (in) t[r][e] = __ldcs(reinterpret_cast<const float4*>(src[e] + at));
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int e = 0; e < kWrCols; ++e) {
+                v[e][0] += t[r][e].x;
+                v[e][1] += t[r][e].y;
+                v[e][2] += t[r][e].z;
+                v[e][3] += t[r][e].w;
+            }
+    }
+    // the four range lanes of a warp, then the warps in order
+#pragma unroll
+    for (int e = 0; e < kWrCols; ++e)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            v[e][q] += __shfl_xor_sync(0xffffffffu, v[e][q], 8);
+            v[e][q] += __shfl_xor_sync(0xffffffffu, v[e][q], 16);
+            if ((threadIdx.x & 31) < 8) s_v[threadIdx.x >> 5][e][tx * 4 + q] = v[e][q];
+        }
     __syncthreads();
-    if (ty >= kWrCols || i >= cnt) return;
+    if (of < 0) return;
     float acc = 0.0f;
-    for (int z = 0; z < 8; ++z) acc += s_v[z][ty][tx];
 #pragma unroll
-    for (int e = 0; e < kWrCols; ++e) {
-        if (e != ty || !src[e]) continue;
-        if (acc != acc)
-            acc = wgrad_exact(a.xs + (size_t)g * a.xs_gstride + (size_t)(chan[e] >> 3) * a.gr.slots * 8 + (chan[e] & 7),
-                              a.dz + (size_t)g * a.dz_gstride + (size_t)(i >> 3) * a.gr.slots * 8 + (i & 7), shift[e],
-                              a.gr.D0, a.gr.N, a.gr.P, a.gr.HWb, a.gr.Wb, a.gr.OT, a.gr.OH, a.gr.OW);
-        const int f = __ldg(a.rowmap + g * a.n_pad + i);
-        if (f >= 0) a.dW[(long long)f * a.K + __ldg(a.colidx + j0 + e)] = acc;
+    for (int z = 0; z < 8; ++z) acc += s_v[z][oe][oi - i0];
+    if (acc != acc) {
+        const int c = a.chan_kind ? (j0 + oe) / a.taps : ocol / a.taps, tap = ocol % a.taps;
+        const int kw = tap % a.gr.KW, kh = (tap / a.gr.KW) % a.gr.KH, kt = tap / (a.gr.KW * a.gr.KH);
+        acc = wgrad_exact(a.xs + (size_t)g * a.xs_gstride + (size_t)(c >> 3) * a.gr.slots * 8 + (c & 7),
+                          a.dz + (size_t)g * a.dz_gstride + (size_t)(oi >> 3) * a.gr.slots * 8 + (oi & 7),
+                          kt * a.gr.HWb + kh * a.gr.Wb + kw, a.gr.D0, a.gr.N, a.gr.P, a.gr.HWb, a.gr.Wb, a.gr.OT, a.gr.OH,
+                          a.gr.OW);
     }
+    a.dW[(long long)of * a.K + ocol] = acc;
 }
 
 struct DzArgs {
@@ -723,8 +787,9 @@ bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, GridBwd* out)
     if (plan->n_cols < 1 || plan->n_filt < 1 || g.taps > 256) return false;
     if (!grid_of(g, &b.gr)) return false;
     b.nck = plan->colkind == SADMM_COL_CHANNEL ? plan->n_colgroups : (int)g.cg;
+    const int per = (int)((plan->n_filt + g.groups - 1) / g.groups);
     if (!grid_conv_shape(b.gr, plan->n_pad, b.nck, b.nck, (int)g.groups, (int)kGwCtas, &b.cs)) return false;
-    if (!wgrad_shape(b.gr, b.nck, plan->n_pad, (int)g.groups, &b.ws)) return false;
+    if (!wgrad_shape(b.gr, b.nck, plan->n_pad, per, (int)g.groups, &b.ws)) return false;
     b.dchunks = std::max(b.cs.k16 * 2, b.ws.nft * b.ws.nst / 8);
     b.nparts = (b.gr.slots + kDzSlots - 1) / kDzSlots;
     if ((long long)b.nparts * g.groups * b.dchunks + (b.gr.slots / 256 + 1) * g.groups * ((b.ws.nch + 1) / 2) +
