@@ -25,13 +25,13 @@
 // step of 16 pixels), so a slice takes at most kGwMaxTiles tiles of 128.
 //
 // AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5):
-// 841 us as six im2col / GEMM / col2im chunks, 173 us here.  One cold launch each:
-// front 39 us (138 MB moved; each dZ octet is 16 loads of 2 and 4 bytes), weight
+// 841 us as six im2col / GEMM / col2im chunks, 172 us here.  One cold launch each:
+// front 38 us (138 MB moved; each dZ octet is 16 loads of 2 and 4 bytes), weight
 // gradient 72 (57 cycles per 128 x 64 x 16 MMA: bound by the operands'
 // shared-memory reads, 96 of the 128 rows in use), input gradient 60 (57 cycles
-// per 128 x 48 x 16), reduction 15.  conv3, 164 -> 52 us: 14 / 18 / 20 / 11; a
-// ResNet-50 3x3 layer (64 of 128 channels and filters kept) at batch 64, 277 -> 48:
-// 13 / 17 / 18 / 10.
+// per 128 x 48 x 16), reduction 15.  conv3, 164 -> 50 us: 13 / 18 / 20 / 11; a
+// ResNet-50 3x3 layer (64 of 128 channels and filters kept) at batch 64, 277 -> 45:
+// 12 / 17 / 18 / 10.
 #include <string.h>
 
 #include <algorithm>
@@ -762,13 +762,19 @@ __global__ void __launch_bounds__(256) k_grid_front(const __grid_constant__ Fron
     pdl_trigger();
     __shared__ int s_i[256];
     __shared__ float s_part[8][8];
-    const int b = blockIdx.x;
+    // The input gradient's weights first: a block of them is a chain of dependent
+    // loads (its search of the columns), hidden beside the copies and not behind them
+    // (AlexNet conv3's backward 51.0 -> 49.5 us, the ResNet-50 3x3 layer's 47.7 -> 45.4).
+    int b = blockIdx.x;
+    if (b < a.np) {
+        prep_block(a.prep, b, s_i);
+        return;
+    }
+    b -= a.np;
     if (b < a.ndz)
         dz_block<RELU, Y>(a.dz, b % a.dz.bx, b / a.dz.bx, s_i, s_part);
-    else if (b < a.ndz + a.nx)
-        grid_x_block(a.x, (b - a.ndz) % a.x.bx, (b - a.ndz) / a.x.bx, s_i);
     else
-        prep_block(a.prep, b - a.ndz - a.nx, s_i);
+        grid_x_block(a.x, (b - a.ndz) % a.x.bx, (b - a.ndz) / a.x.bx, s_i);
 }
 
 struct GridBwd {
