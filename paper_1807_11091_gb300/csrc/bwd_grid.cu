@@ -25,12 +25,12 @@
 // step of 16 pixels), so a slice takes at most kGwMaxTiles tiles of 128.
 //
 // AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5):
-// 841 us as six im2col / GEMM / col2im chunks, 172 us here.  One cold launch each:
+// 841 us as six im2col / GEMM / col2im chunks, 165 us here.  One cold launch each:
 // front 38 us (138 MB moved; each dZ octet is 16 loads of 2 and 4 bytes), weight
 // gradient 72 (57 cycles per 128 x 64 x 16 MMA: bound by the operands'
 // shared-memory reads, 96 of the 128 rows in use), input gradient 60 (57 cycles
-// per 128 x 48 x 16), reduction 15.  conv3, 164 -> 50 us: 13 / 18 / 20 / 11; a
-// ResNet-50 3x3 layer (64 of 128 channels and filters kept) at batch 64, 277 -> 45:
+// per 128 x 48 x 16), reduction 15.  conv3, 164 -> 49 us: 13 / 18 / 20 / 11; a
+// ResNet-50 3x3 layer (64 of 128 channels and filters kept) at batch 64, 277 -> 43:
 // 12 / 17 / 18 / 10.
 #include <string.h>
 
@@ -461,16 +461,17 @@ struct WrArgs {
 // filters take every 32nd range, then their sums are added in order
 // (deterministic).  Block (bx, by, g): packed columns bx*kWrCols .., packed rows
 // by*32 .. +31; the slices are read along the filters, 16 bytes a load.
-// Bound by latency: the slices are in L2, so what counts is loads in flight (16 of
-// 16 bytes a thread, the layer's ranges in one pass up to 128 of them) and what is
+// Bound by latency: the slices are in L2, so what counts is loads in flight (8 of
+// 16 bytes a thread, and up to 128 of the layer's ranges in one pass) and what is
 // done before the wait.  With eight range lanes of 4-byte loads, four ranges a pass
 // and the tables read after the wait it stood 10 to 14 us behind the layer (AlexNet
-// conv3 55.2 us in all, now 51.7).
-constexpr int kWrCols = 4;
+// conv3 55.2 us in all, 51.7 after; two columns a block instead of four, twice the
+// blocks, 49.9 -> 48.8 and a ResNet-50 3x3 layer's 45.6 -> 43.6, one column the same).
+constexpr int kWrCols = 2;
 
 __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbArgs d)
 {
-    __shared__ float s_v[8][kWrCols][40];
+    __shared__ float s_v[8][kWrCols][48];
     if ((int)blockIdx.z == d.groups) {  // the last layer of blocks: the bias gradient
         pdl_wait();
         pdl_trigger();
@@ -498,9 +499,9 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbAr
         src[e] = a.slices + ((size_t)type * a.w.rows + m) * (size_t)(a.w.tpg * a.w.nst) + (mt % a.w.tpg) * a.w.nst +
                  (iq - ftq * a.w.nst);
     }
-    // the entry this thread writes: four threads to a filter's four columns
-    const int oe = threadIdx.x & 3, oi = i0 + (threadIdx.x >> 2);
-    const int ocol = threadIdx.x < 128 && j0 + oe < a.n_cols ? __ldg(a.colidx + j0 + oe) : -1;
+    // the entry this thread writes: two threads to a filter's two columns
+    const int oe = threadIdx.x & 1, oi = i0 + (threadIdx.x >> 1);
+    const int ocol = threadIdx.x < 64 && j0 + oe < a.n_cols ? __ldg(a.colidx + j0 + oe) : -1;
     const int of = ocol >= 0 && oi < cnt ? __ldg(a.rowmap + g * a.n_pad + oi) : -1;
     pdl_wait();  // after the kernel before it in the stream, and the one before that (see launch_grid_bwd)
     pdl_trigger();
@@ -567,11 +568,15 @@ struct DzArgs {
     __nv_bfloat16* dz;  // NULL: the bias gradient alone
     float* part;        // [groups*n_pad][bx], or NULL
     int bx, by;         // blocks
+    int slots;          // slots of a block
 };
 
 // Grid copy of dZ and the bias gradient's partial sums.  Block (bx, by), 256 threads: slots
-// bx*kDzSlots .. of chunk by % chunks (8 kept filters) of conv group by / chunks.
-constexpr int kDzSlots = 512;
+// bx*slots .. of chunk by % chunks (8 kept filters) of conv group by / chunks.
+// Four slots a thread where that leaves kDzBlocks blocks, else two: the block's
+// bias sums cost as much as a slot (AlexNet conv2's backward 164.5 -> 160.2 us; one
+// slot a thread instead of two 170.7 -> 177.4).
+constexpr int kDzBlocks = 1024;
 
 // One pixel's dZ of a chunk's filters (nf of them, 8 when FULL): every load
 // first, then the products, the running bias sums and the packed octet.
@@ -617,8 +622,8 @@ SADMM_DEV void dz_block(const DzArgs& a, int bx, int by, int* s_off, float (*s_p
         sum[e] = 0.0f;
     }
 #pragma unroll 1
-    for (int k = 0; k < kDzSlots / 256; ++k) {
-        const int s = bx * kDzSlots + k * 256 + threadIdx.x;
+    for (int k = 0; k < a.slots; k += 256) {
+        const int s = bx * a.slots + k + threadIdx.x;
         if (s >= a.gr.slots) break;
         int n = 0, t = 0, h = 0, w = 0;
         const int q = s - a.gr.D0;
@@ -783,7 +788,8 @@ struct GridBwd {
     WgradShape ws;
     int nck;      // channels of x per group that hold a kept column
     int dchunks;  // 8-filter chunks of dZ per group
-    int nparts;   // blocks of k_grid_dz along the slots
+    int dzslots;  // slots of a block of the dZ copy
+    int nparts;   // its blocks along the slots
     size_t off_xs, off_dz, off_wd, off_maps, off_slices, off_part, total;
 };
 
@@ -797,7 +803,8 @@ bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, GridBwd* out)
     if (!grid_conv_shape(b.gr, plan->n_pad, b.nck, b.nck, (int)g.groups, (int)kGwCtas, &b.cs)) return false;
     if (!wgrad_shape(b.gr, b.nck, plan->n_pad, per, (int)g.groups, &b.ws)) return false;
     b.dchunks = std::max(b.cs.k16 * 2, b.ws.nft * b.ws.nst / 8);
-    b.nparts = (b.gr.slots + kDzSlots - 1) / kDzSlots;
+    b.dzslots = b.gr.slots / 1024 * g.groups * b.dchunks >= kDzBlocks ? 1024 : 512;
+    b.nparts = (b.gr.slots + b.dzslots - 1) / b.dzslots;
     if ((long long)b.nparts * g.groups * b.dchunks + (b.gr.slots / 256 + 1) * g.groups * ((b.ws.nch + 1) / 2) +
             2 * g.groups * b.cs.npad + 256 >= (1ll << 31) ||
         g.groups * ((b.ws.nch + 1) / 2) > 65535)
@@ -893,6 +900,7 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
     d.dz = (dW || dx) ? dz : nullptr;
     d.part = db ? part : nullptr;
     d.bx = b.nparts;
+    d.slots = b.dzslots;
     d.by = (int)(g.groups * b.dchunks);
     fa.ndz = d.bx * d.by;
     if (dW) {

@@ -1,9 +1,10 @@
 """The weight gradient's slices on the pixel grid: more ranges than one pass of the
-reduction holds (128), kept filters that are no multiple of its 16-byte loads, and a
-layer whose taps are split between items (longer ranges) at a size where one item
-could hold them; against the fp64 oracle, at the suite's 2e-3 of the largest value
-and, the sums being fp32 sums of exact products in ranges of at most 12 x 128 pixels,
-at 2e-6 in the 2-norm (4.5e-7 measured at most)."""
+reduction holds (128), kept filters that are no multiple of its 16-byte loads, dZ
+copied in blocks of 1024 slots (the last one ragged), and a layer whose taps are
+split between items (longer ranges) at a size where one item could hold them;
+against the fp64 oracle, at the suite's 2e-3 of the largest value and, the sums
+being fp32 sums of exact products in ranges of at most 12 x 128 pixels, at 2e-6 in
+the 2-norm (4.5e-7 measured at most)."""
 import numpy as np
 import pytest
 import torch
@@ -18,6 +19,7 @@ pytestmark = pytest.mark.gpu
 
 CASES = [
     ("ranges_141_filters_18", ConvShape(n=23, c=48, h=28, w=28, f=32, kh=1, kw=1), 18, wl.COL_CHANNEL, 24),
+    ("dz_blocks_of_1024", ConvShape(n=32, c=8, h=33, w=33, f=256, kh=1, kw=1), 250, wl.COL_NONE, 0),
     ("split_taps", ConvShape(n=90, c=64, h=14, w=14, f=50, kh=3, kw=3, ph=1, pw=1), 50, wl.COL_NONE, 0),
     ("split_taps_odd_columns", ConvShape(n=90, c=64, h=14, w=14, f=64, kh=3, kw=3, ph=1, pw=1), 61, wl.COL_SHAPE, 301),
 ]
