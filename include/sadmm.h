@@ -26,7 +26,9 @@
  *    enqueued on it, in order, asynchronously.  The kernels are launched with
  *    programmatic stream serialization: one may be scheduled while the kernel
  *    before it on the stream finishes, and it waits for that kernel to complete
- *    before it reads or writes global memory, so stream order is kept.
+ *    before it reads or writes global memory, so stream order is kept.  (One
+ *    kernel of sadmm_conv_bwd runs beside the kernel of the same call before it
+ *    and waits for it at its end; every kernel of earlier calls is complete then.)
  *  - Arguments are validated on the host before any launch; a bad argument
  *    returns SADMM_EINVAL and enqueues nothing.  A failed launch returns
  *    SADMM_ECUDA.  Shapes the kernels do not support (see each call) return
@@ -464,7 +466,7 @@ sadmm_status sadmm_pack_batch(sadmm_pack_item* items, int n, int wdt, void* stre
  * Requires sm_100-family tensor cores (SADMM_EUNSUPPORTED otherwise) and
  * N*C*T*H*W < 2^31.  Launches that use one plan must not overlap on the GPU
  * (stream-ordered is fine): split-K partial sums, stream-K arrival
- * counters and the slab path's space-to-depth input live in the plan's
+ * counters and the input-slab and pixel-grid copies of x live in the plan's
  * buffer.
  */
 sadmm_status sadmm_conv_fwd(const sadmm_plan* plan, const void* x, const float* bias,
