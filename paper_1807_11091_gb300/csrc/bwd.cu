@@ -403,7 +403,7 @@ long long bwd_chunk_for(const sadmm_plan* plan, const Geometry& g, size_t ws_byt
 // The grid path wherever the layer has a grid and the workspace holds it: over
 // 20 drawn stride-1 layers (1x1 to 5x5, 3-D, batch 1 to 128, densities 0.1 to 1)
 // it took 0.26 to 0.84 of the gathered path's time, AlexNet conv2 at batch 128
-// 841 -> 165 us, conv3 164 -> 49 us, and none took longer.
+// 841 -> 175 us, conv3 164 -> 50 us, and none took longer.
 sadmm_status launch_conv_bwd(const sadmm_plan* plan, const Geometry& g, const void* x, const void* dy, const void* y,
                              int ydt, int relu, float* dW, float* db, float* dx, void* ws, size_t ws_bytes,
                              cudaStream_t s)

@@ -21,16 +21,21 @@
 // A layer of at most 64 channels fills half of the M side or less: its slab is
 // then staged up to 16 / chunks times, each copy a pixel further on, and one
 // MMA covers that many kernel columns.
-// The tensor core truncates as it accumulates (about 1e-8 of the result per
-// step of 16 pixels), so a slice takes at most kGwMaxTiles tiles of 128.
+// The tensor core truncates as it accumulates (about 1e-8 of the result per step
+// of 16), so fp32 registers or slices take over early: dW after kGwMaxTiles tiles
+// of 128 pixels, dx after kDxSeg steps.  Errors against 64 bits (2-norm) of dW /
+// dx: conv2 2.2e-7 / 1.2e-7, conv3 2.1e-7 / 1.0e-7, the ResNet-50 3x3 layer
+// 2.5e-7 / 1.6e-7, beside 2.2, 1.8 and 2.3e-7 of the chunked path's dW.  With 12
+// tiles conv2's dW stood at 4.5e-7 (and its backward at 161 us, not 175), with 54
+// steps the ResNet layer's dx at 3.3e-7 (43.9 us, not 45.2).
 //
 // AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5):
-// 841 us as six im2col / GEMM / col2im chunks, 165 us here.  One cold launch each:
+// 841 us as six im2col / GEMM / col2im chunks, 175 to 180 us here.  One cold launch each:
 // front 38 us (138 MB moved; each dZ octet is 16 loads of 2 and 4 bytes), weight
 // gradient 72 (57 cycles per 128 x 64 x 16 MMA: bound by the operands'
 // shared-memory reads, 96 of the 128 rows in use), input gradient 60 (57 cycles
-// per 128 x 48 x 16), reduction 15.  conv3, 164 -> 49 us: 13 / 18 / 20 / 11; a
-// ResNet-50 3x3 layer (64 of 128 channels and filters kept) at batch 64, 277 -> 43:
+// per 128 x 48 x 16), reduction 15.  conv3, 164 -> 50 us: 13 / 18 / 20 / 11; a
+// ResNet-50 3x3 layer (64 of 128 channels and filters kept) at batch 64, 277 -> 45:
 // 12 / 17 / 18 / 10.
 #include <string.h>
 
@@ -43,7 +48,8 @@ namespace {
 
 constexpr int kGwThreads = 10 * 32;
 constexpr int kGwMaxStages = 4;
-constexpr int kGwMaxTiles = 12;      // 128-pixel tiles summed in TMEM: 96 MMA steps
+constexpr int kGwMaxTiles = 6;       // 128-pixel tiles summed in TMEM: 48 MMA steps
+constexpr int kDxSeg = 27;           // MMA steps of the input gradient summed in TMEM
 constexpr long long kGwCtas = 152;   // work items come in multiples of about this many (fixed: it sizes the workspace)
 constexpr int kGwSmemLimit = 232448;
 constexpr int kGwCols = 512;         // accumulator columns
@@ -89,8 +95,8 @@ bool wgrad_shape(const Grid& gr, int nck, int n_pad, int likely, int groups, Wgr
     // mean longer pixel ranges, so fewer slices to write and to add up, for more
     // slab loads: a 3x3 layer of 64 kept channels and filters at batch 64 runs its
     // 6 MMA taps as two items of 6 tiles, not one of 3: its slices are 14 MB, not
-    // 28, and its backward takes 48 us, not 53.  Only for a fifth less by the
-    // estimate: AlexNet conv3 as three items of 8 tiles, not two of 6, is 18 % less
+    // 28, and its backward took 48 us, not 53.  Only for a fifth less by the
+    // estimate: AlexNet conv3 as three items of 8 tiles, not two of 6, was 18 % less
     // by it and measured 53.9 against 53.4 us (SMs without an item start the input
     // gradient early).
     const int tmax = std::min(std::min(kGwCols / w.nst, macro), 32);
@@ -800,7 +806,7 @@ bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, GridBwd* out)
     if (!grid_of(g, &b.gr)) return false;
     b.nck = plan->colkind == SADMM_COL_CHANNEL ? plan->n_colgroups : (int)g.cg;
     const int per = (int)((plan->n_filt + g.groups - 1) / g.groups);
-    if (!grid_conv_shape(b.gr, plan->n_pad, b.nck, b.nck, (int)g.groups, (int)kGwCtas, &b.cs)) return false;
+    if (!grid_conv_shape(b.gr, plan->n_pad, b.nck, b.nck, (int)g.groups, (int)kGwCtas, kDxSeg, &b.cs)) return false;
     if (!wgrad_shape(b.gr, b.nck, plan->n_pad, per, (int)g.groups, &b.ws)) return false;
     b.dchunks = std::max(b.cs.k16 * 2, b.ws.nft * b.ws.nst / 8);
     b.dzslots = b.gr.slots / 1024 * g.groups * b.dchunks >= kDzBlocks ? 1024 : 512;

@@ -15,7 +15,7 @@
 //   warp 0       slabs: CB/8 bulk copies per stage
 //   warp 1       TMEM allocator, MMA issuer
 //   warp 2       weights: resident, or a ring of a few MMA steps per slot
-//   warps 3-10   epilogue: every `sps` stages (at most about 54 MMA steps) the
+//   warps 3-10   epilogue: every `sps` stages (at most about `seg` MMA steps) the
 //                accumulator is read from TMEM and added to fp32 registers
 //                (the tensor core truncates when it accumulates, about 1e-8 of
 //                the result per step; short chains keep that below 5e-7), the
@@ -38,7 +38,6 @@ constexpr int kGcWarps = 11;
 constexpr int kGcThreads = kGcWarps * 32;
 constexpr int kGcEpiWarps = 8;
 constexpr int kGcMaxA = 4, kGcMaxB = 8;
-constexpr int kGcSegSteps = 54;    // MMA steps accumulated in TMEM before the fp32 registers take over
 constexpr int kGcTables = 2 * 256 * 4;
 constexpr int kGcZcap = 1024;
 constexpr int kGcBars = 512;
@@ -547,10 +546,12 @@ cudaError_t launch_gc(const GcArgs& a, int grid, size_t smem, cudaStream_t s)
 
 }  // namespace
 
-bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups, int sms, GridConvShape* out)
+bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups, int sms, int seg,
+                     GridConvShape* out)
 {
     if (chans < 1 || cols < 1) return false;
     GridConvShape r;
+    r.seg = seg;
     const int taps = gr.KH * gr.KW;
     r.k16 = (chans + 15) / 16;
     const long long ksteps = (long long)r.k16 * gr.KT * taps;
@@ -563,7 +564,7 @@ bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups
     // A block: as many 16s of channels as divide them, keep a stage to one
     // accumulation segment and its slab to 24 KB.
     int m = 4;
-    while (m > 1 && (r.k16 % m != 0 || taps * m > kGcSegSteps || (128 + span) * 32 * m > 24576)) --m;
+    while (m > 1 && (r.k16 % m != 0 || taps * m > seg || (128 + span) * 32 * m > 24576)) --m;
     r.cb = 16 * m;
     const int rsteps = gr.KW * m;
     // The tiling of least estimated time: rounds of items over the SMs, each
@@ -652,7 +653,7 @@ sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const Gri
     a.h16 = sh.cb / 16;
     a.rsteps = gr.KW * a.h16;
     a.spt = gr.KH * a.rsteps;
-    a.sps = std::max(1, kGcSegSteps / a.spt);
+    a.sps = std::max(1, sh.seg / a.spt);
     a.cap_b = sh.cap_b;
     a.stages_a = sh.stages_a;
     a.a_bytes = a.sp * 16 * (sh.cb / 8);
@@ -711,6 +712,10 @@ static sadmm_status launch_grid_x(const Grid& gr, const Geometry& g, const void*
 // half too (125 against 185).
 constexpr long long kRuleSms = 152;
 
+// MMA steps summed in TMEM: AlexNet conv2's error against 64 bits is 2.1e-7 (the
+// gathered kernel's 3.3e-7); with 27 it would be 1.3e-7 and 55.8 us become 61.2.
+constexpr int kFwdSeg = 54;
+
 // Channels of x per conv group that hold a kept column.
 static int fwd_channels(const sadmm_plan* plan, const Geometry& g)
 {
@@ -732,7 +737,7 @@ bool grid_fwd_plan(const Geometry& g, sadmm_plan* plan, size_t* gx, size_t* gw, 
     if (units < kRuleSms) return false;
     const int nck = fwd_channels(plan, g);
     const int per = (int)((plan->n_filt + g.groups - 1) / g.groups);
-    if (!grid_conv_shape(gr, nck, plan->n_pad, per, (int)g.groups, plan->ctas, &sh)) return false;
+    if (!grid_conv_shape(gr, nck, plan->n_pad, per, (int)g.groups, plan->ctas, kFwdSeg, &sh)) return false;
     const int chunks = sh.k16 * 2;
     if (g.groups * sh.k16 > 65535) return false;
     plan->gx_cb = sh.cb;
@@ -748,7 +753,7 @@ bool grid_fwd_plan(const Geometry& g, sadmm_plan* plan, size_t* gx, size_t* gw, 
     // stages (the gather's rate up to 128 filters, the MMAs' above), and the
     // stores, which overlap less when one accumulator set fills TMEM.
     GridConvShape rule;
-    if (!grid_conv_shape(gr, nck, plan->n_pad, per, (int)g.groups, kRuleSms, &rule)) return false;
+    if (!grid_conv_shape(gr, nck, plan->n_pad, per, (int)g.groups, kRuleSms, kFwdSeg, &rule)) return false;
     const long long xb = 2 * g.n * g.groups * (long long)nck * g.t * g.h * g.w + 2 * g.groups * 16ll * sh.k16 * gr.L;
     const long long yb = 4 * g.m * g.f;
     const long long grid_ns = 8000 + xb / 4000 + rule.cycles * 100 / 195 + yb / 60000;
@@ -775,6 +780,7 @@ sadmm_status launch_grid_fwd(const sadmm_plan* plan, const Geometry& g, const vo
     GridConvShape sh;
     memset(&sh, 0, sizeof(sh));
     sh.cb = plan->gx_cb;
+    sh.seg = kFwdSeg;
     sh.k16 = (nck + 15) / 16;
     sh.ksteps = grid_fwd_ksteps(plan, g);
     sh.mt = plan->gx_mt;

@@ -67,6 +67,7 @@ inline bool grid_of(const Geometry& g, Grid* out)
 // of 16 K columns at a time: [group][column tile][step][K half][row][8].
 struct GridConvShape {
     int cb;      // channels per block (multiple of 16)
+    int seg;     // MMA steps summed in TMEM before the fp32 registers take over
     int k16;     // 16-channel groups of the source (padded channels / 16)
     int ksteps;  // MMA steps of 16 K columns
     int mt;      // 128-pixel tiles per work item (1 or 2)
@@ -77,10 +78,12 @@ struct GridConvShape {
     long long cycles;  // its estimated time
 };
 // The tiling for `chans` source channels and at most `cols`, likely `likely`,
-// output columns per group over `groups` groups; false when it does not fit.
+// output columns per group over `groups` groups, summing about `seg` MMA steps in
+// TMEM; false when it does not fit.
 // The blocks of channels (the order of the sums) follow the layer alone, not its
 // batch or the device.
-bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups, int sms, GridConvShape* out);
+bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups, int sms, int seg,
+                     GridConvShape* out);
 
 // Rows of a column tile in the weights' layout: the most columns any group has,
 // to 16, when there is one tile (the groups' counts are known on the device

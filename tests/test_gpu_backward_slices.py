@@ -3,8 +3,8 @@ reduction holds (128), kept filters that are no multiple of its 16-byte loads, d
 copied in blocks of 1024 slots (the last one ragged), and a layer whose taps are
 split between items (longer ranges) at a size where one item could hold them;
 against the fp64 oracle, at the suite's 2e-3 of the largest value and, the sums
-being fp32 sums of exact products in ranges of at most 12 x 128 pixels, at 2e-6 in
-the 2-norm (4.5e-7 measured at most)."""
+being fp32 sums of exact products in ranges of at most 6 x 128 pixels, at 2e-6 in
+the 2-norm (4.5e-7 measured at most, with 12 x 128)."""
 import numpy as np
 import pytest
 import torch
