@@ -487,7 +487,10 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbAr
     // The plan's tables: k_grid_front read them too and has completed.
     const int g = blockIdx.z, cnt = __ldg(a.counts + 2 * g);
     const int i0 = blockIdx.y * 32, j0 = blockIdx.x * kWrCols;
-    if (i0 >= cnt) return;
+    if (i0 >= cnt) {  // still waits: with no kept filter at all these are the launch's only blocks
+        pdl_wait();
+        return;
+    }
     const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
     const int iq = i0 + tx * 4, ftq = iq / a.w.nst;  // (a tile's filters are a multiple of 16)
     const float* src[kWrCols];
