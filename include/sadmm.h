@@ -47,7 +47,7 @@
 extern "C" {
 #endif
 
-#define SADMM_ABI_VERSION 6
+#define SADMM_ABI_VERSION 7
 
 /* Most layers one batched call (sadmm_project_groups_batch,
  * sadmm_admm_update_batch) takes. */

@@ -33,9 +33,16 @@ def test_library_exports_every_declared_entry_point():
 
 
 def test_struct_layout_and_version():
-    assert sadmm.sadmm_abi_version() == 6
+    assert sadmm.sadmm_abi_version() == 7
     assert sadmm.sadmm_plan_struct_size() == ctypes.sizeof(sadmm.Plan)
     assert sadmm.sadmm_status_string(-1) == "invalid argument"
+
+
+def test_version_changes_with_the_plan_struct():
+    """The struct a caller allocates and the version it checks change together: version 6
+    was a struct of 640 bytes, 7 added the pixel-grid forward's fields."""
+    sizes = {6: 640, 7: 696}
+    assert sadmm.sadmm_plan_struct_size() == sizes[sadmm.sadmm_abi_version()]
 
 
 def test_plan_sizes():
