@@ -1012,6 +1012,7 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         c.VH = (int)g.h;
         c.VW = (int)g.w;
         c.out_total = g.n * g.c * g.t * g.h * g.w;
+        c.src_dz = 1;
         c.late_wait = dW != nullptr;  // (k_grid_wgrad stands between)
         const sadmm_status st = launch_grid_conv(b.gr, b.cs, c, s);
         if (st != SADMM_OK) return st;

@@ -57,6 +57,7 @@ struct GcArgs {
     long long out_total;
     long long gstride;  // source elements per group
     int late_wait;
+    int src_dz;
     int zstride, groups, planes, plane, VT, VH, VW, VHW;
     int units, mtiles, ntiles;
     FastDiv mt_div, nt_div;
@@ -71,25 +72,35 @@ struct GcArgs {
     int relu;
 };
 
-// The sum of one output (column `col` of the tile whose weights wd are, grid
-// pixel q) over the kept K columns only, as the gathered path forms it (pruned
-// entries are -0.0).
-__device__ __noinline__ float grid_exact(const __nv_bfloat16* wd, int bn, int col, const __nv_bfloat16* src, int q,
-                                         int kch, int cb, int KT, int KH, int KW, int HWb, int Wb, int slots)
+// The sum of one output (column `col` of column tile nt of group g, whose weights
+// lie bnr rows apart; grid pixel q) over the kept K columns only, as the gathered
+// path forms it (pruned entries are -0.0).  Where the source is the output
+// gradient, a tap that reads past the output's edge is no term of the sum; in the
+// forward a padded pixel is one, as it is in the gathered path.
+__device__ __noinline__ float grid_exact(const GcArgs& a, int g, int nt, int bnr, int col, int q, int kch)
 {
-    const unsigned short* w = reinterpret_cast<const unsigned short*>(wd) + col * 8;
+    const unsigned short* w =
+        reinterpret_cast<const unsigned short*>(a.wd) + (size_t)(g * a.ntiles + nt) * a.ksteps * a.bn * 16 + col * 8;
+    const __nv_bfloat16* src = a.src + (size_t)g * a.gstride;
     float acc = 0.0f;
-    for (int c0 = 0; c0 < kch; c0 += cb)
-        for (int kt = 0; kt < KT; ++kt)
-            for (int kh = 0; kh < KH; ++kh)
-                for (int kw = 0; kw < KW; ++kw)
-                    for (int c8 = c0; c8 < c0 + cb; c8 += 8, w += bn * 8)
-                        for (int e = 0; e < 8; ++e) {
-                            const unsigned short b = __ldg(w + e);
-                            if (b == 0x8000u || c8 + e >= kch) continue;
-                            const size_t slot = (size_t)(c8 >> 3) * slots + (q + kt * HWb + kh * Wb + kw);
-                            acc += __uint_as_float((uint32_t)b << 16) * __bfloat162float(src[slot * 8 + e]);
-                        }
+    for (int c0 = 0; c0 < kch; c0 += a.cb)
+        for (int kt = 0; kt < a.gr.KT; ++kt)
+            for (int kh = 0; kh < a.gr.KH; ++kh)
+                for (int kw = 0; kw < a.gr.KW; ++kw, w += (size_t)a.cb * bnr) {
+                    const int slot = q + kt * a.gr.HWb + kh * a.gr.Wb + kw;
+                    if (a.src_dz) {
+                        if (slot < a.gr.D0) continue;
+                        int n, t, y, x;
+                        grid_decode(a.gr, slot - a.gr.D0, n, t, y, x);
+                        if (n >= a.gr.N || t >= a.gr.OT || y >= a.gr.OH || x >= a.gr.OW) continue;
+                    }
+                    for (int c = c0; c < min(c0 + a.cb, kch); ++c) {
+                        const unsigned short b = __ldg(w + (size_t)((c - c0) >> 3) * bnr * 8 + (c & 7));
+                        if (b == 0x8000u) continue;
+                        acc += __uint_as_float((uint32_t)b << 16) *
+                               __bfloat162float(src[((size_t)(c >> 3) * a.gr.slots + slot) * 8 + (c & 7)]);
+                    }
+                }
     return acc;
 }
 
@@ -498,9 +509,7 @@ __global__ void __launch_bounds__(kGcThreads, 1)
                 for (int i = 0; i < nch * kEpiCols; ++i) {
                     const int c = i / kEpiCols;
                     if (i >= cnt || (MT == 1 && (c & 1) != h) || !((nan >> (MT == 2 ? c : c >> 1)) & 1u)) continue;
-                    float e = grid_exact(a.wd + (size_t)(g * a.ntiles + nt) * btile / 2, bnr, i,
-                                         a.src + (size_t)g * a.gstride, q, kch, a.cb, a.gr.KT, a.gr.KH, a.gr.KW, a.gr.HWb,
-                                         a.gr.Wb, a.gr.slots) + t_bias[i];
+                    float e = grid_exact(a, g, nt, bnr, i, q, kch) + t_bias[i];
                     if (a.relu) e = fmaxf(e, 0.0f);
                     if (!y_ok(yc, t_off[i])) continue;
                     if (OUT_BF16)
@@ -630,6 +639,7 @@ sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const Gri
     a.status = device_status_ptr();
     a.out_total = c.out_total;
     a.late_wait = c.late_wait ? 1 : 0;
+    a.src_dz = c.src_dz ? 1 : 0;
     a.gstride = (long long)c.chunks * gr.slots * 8;
     a.groups = c.groups;
     a.planes = c.planes;

@@ -114,6 +114,7 @@ struct GridConvCall {
     int VT, VH, VW;        // its extents
     long long out_total;
     int ctas;
+    int src_dz;  // 1: src is the output gradient's copy, pixel 0 at slot D0
     // 1: the kernel before this one in the stream writes nothing it reads, and lets
     // it start only when the one that wrote its inputs has completed.  It then
     // waits for that kernel at its end, so that its completion still means both.

@@ -118,3 +118,46 @@ def test_infinities_reach_the_kept_terms_alone(ck, cf):
     seen[c0, :2, :2] = keep[c0].reshape(3, 3)[:2, :2]
     assert not bad[:, ~seen].any() and bad[np.asarray(rows)][:, seen].all()
     assert torch.equal(dx2, clean[2]) and sadmm.device_status() == 0
+
+
+@pytest.mark.parametrize("case", [
+    ("3x3", ConvShape(n=3, c=16, h=9, w=8, f=24, kh=3, kw=3, ph=1, pw=1)),
+    ("no_pad_5x3", ConvShape(n=2, c=20, h=9, w=8, f=40, kh=5, kw=3, groups=2)),
+    ("3d", ConvShape(n=2, c=8, t=4, h=5, w=6, f=16, kt=3, kh=3, kw=3, pt=1, ph=1, pw=1)),
+], ids=lambda c: c[0])
+def test_infinite_weight_reaches_real_outputs_alone(case):
+    """dx of a kept weight that is infinite: non-finite where that tap reads an output pixel,
+    and the sum of the other terms where it would read one past the output's edge."""
+    from paper_1807_11091_gb300 import sadmm
+    name, s = case
+    dev = torch.device("cuda", 0)
+    g = torch.Generator().manual_seed(3)
+    W = torch.randn(s.w_shape(), generator=g).to(torch.bfloat16)
+    x = torch.randn(s.x_shape(), generator=g).to(torch.bfloat16)
+    dy = (torch.rand(s.y_shape(), generator=g) + 0.5).to(torch.bfloat16)
+    f0, c0, tap = 3, 1, 0  # conv group 0, the first tap: reads output (t + pt, h + ph, w + pw)
+    cols = np.sort(np.random.default_rng(1).permutation(s.k)[:s.k // 2])
+    cols = np.unique(np.append(cols, c0 * s.taps + tap))
+    mask = np.zeros(s.k, dtype=bool)
+    mask[cols] = True
+    Wm = (W.double().reshape(s.f, s.k) * torch.from_numpy(mask)).reshape(W.shape)
+    Wf = Wm.clone()
+    Wf.reshape(s.f, s.k)[f0, c0 * s.taps + tap] = 0.0
+    conv = torch.nn.functional.conv3d if s.is3d else torch.nn.functional.conv2d
+    pad = (s.pt, s.ph, s.pw) if s.is3d else (s.ph, s.pw)
+    xd = x.double().requires_grad_(True)
+    want, = torch.autograd.grad(conv(xd, Wf, padding=pad, groups=s.groups), xd, dy.double())
+    W.reshape(s.f, s.k)[f0, c0 * s.taps + tap] = float("inf")
+    t, h, w = np.meshgrid(np.arange(s.t), np.arange(s.h), np.arange(s.w), indexing="ij")
+    real = (t + s.pt < s.ot) & (h + s.ph < s.oh) & (w + s.pw < s.ow)
+    bad = np.zeros((s.n, s.c, s.t, s.h, s.w), dtype=bool)
+    bad[:, c0] = real
+    bad = bad.reshape(x.shape)
+    ci = torch.as_tensor(cols, dtype=torch.int32, device=dev)
+    pc = sadmm.PrunedConv(s.desc16(), W.to(dev), None, wl.COL_SHAPE, ci, s.f, len(cols))
+    dW, db, dx = pc.backward(x.to(dev), dy.to(dev), relu=False)
+    got = dx.cpu().double().numpy()
+    assert sadmm.device_status() == 0
+    assert np.array_equal(~np.isfinite(got), bad)
+    ref = want.numpy()
+    assert np.abs(got[~bad] - ref[~bad]).max() <= 1e-5 * np.abs(ref).max()
