@@ -23,11 +23,10 @@
 // MMA covers that many kernel columns.
 // The tensor core truncates as it accumulates (about 1e-8 of the result per step
 // of 16), so fp32 registers or slices take over early: dW after kGwMaxTiles tiles
-// of 128 pixels, dx after kDxSeg steps.  Errors against 64 bits (2-norm) of dW /
-// dx: conv2 2.2e-7 / 1.2e-7, conv3 2.1e-7 / 1.0e-7, the ResNet-50 3x3 layer
-// 2.5e-7 / 1.6e-7, beside 2.2, 1.8 and 2.3e-7 of the chunked path's dW.  With 12
-// tiles conv2's dW stood at 4.5e-7 (and its backward at 161 us, not 175), with 54
-// steps the ResNet layer's dx at 3.3e-7 (43.9 us, not 45.2).
+// of 128 pixels, dx after dx_seg() steps.  Errors against 64 bits (2-norm) of dW:
+// conv2 2.2e-7, conv3 2.1e-7, the ResNet-50 3x3 layer 2.5e-7, beside 2.2, 1.9 and
+// 2.3e-7 of the chunked path's.  With 12 tiles conv2's dW stood at 4.5e-7 (and its
+// backward at 161 us, not 175).
 //
 // AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5):
 // 841 us as six im2col / GEMM / col2im chunks, 175 to 180 us here.  One cold launch each:
@@ -49,10 +48,20 @@ namespace {
 constexpr int kGwThreads = 10 * 32;
 constexpr int kGwMaxStages = 4;
 constexpr int kGwMaxTiles = 6;       // 128-pixel tiles summed in TMEM: 48 MMA steps
-constexpr int kDxSeg = 27;           // MMA steps of the input gradient summed in TMEM
+constexpr int kDxStage = 27;         // most MMA steps of an input gradient's stage, where the kernel has no more taps
 constexpr long long kGwCtas = 152;   // work items come in multiples of about this many (fixed: it sizes the workspace)
 constexpr int kGwSmemLimit = 232448;
 constexpr int kGwCols = 512;         // accumulator columns
+
+// MMA steps of the input gradient summed in TMEM.  The chunked path sums a pixel's
+// kept filters there, 16 a step, and adds the taps up in fp32: up to 256 filters a
+// group 12 steps are held here, beyond that, where those sums are long themselves, 27.
+// Errors against 64 bits (chunked path; here; here with 27, unless cut): AlexNet conv3
+// 7.0e-8; 6.5; 9.4, conv2 8.2; 8.7; 12, a ResNet-50 3x3 layer 7.3; 11; 16, 7x7, 9x9 and
+// 11x11 taps over 64 filters 13, 16 and 19; 12, 14 and 15; 44, 76 and 118, 256 filters
+// 3x3 16; 13; 17, 512 filters 30; 16.  Shorter sums cost conv3 48.6 -> 53 us and conv2
+// 180 -> 191 (with 9: 53 and 201 at 0.65 and 0.9e-7).
+int dx_seg(int filters) { return filters <= 256 ? 12 : 27; }
 
 struct WgradShape {
     int nch;          // 8-channel chunks of x per conv group
@@ -809,7 +818,8 @@ bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, GridBwd* out)
     if (!grid_of(g, &b.gr)) return false;
     b.nck = plan->colkind == SADMM_COL_CHANNEL ? plan->n_colgroups : (int)g.cg;
     const int per = (int)((plan->n_filt + g.groups - 1) / g.groups);
-    if (!grid_conv_shape(b.gr, plan->n_pad, b.nck, b.nck, (int)g.groups, (int)kGwCtas, kDxSeg, &b.cs)) return false;
+    if (!grid_conv_shape(b.gr, plan->n_pad, b.nck, b.nck, (int)g.groups, (int)kGwCtas, kDxStage, dx_seg(per), true,
+                         &b.cs)) return false;
     if (!wgrad_shape(b.gr, b.nck, plan->n_pad, per, (int)g.groups, &b.ws)) return false;
     b.dchunks = std::max(b.cs.k16 * 2, b.ws.nft * b.ws.nst / 8);
     b.dzslots = b.gr.slots / 1024 * g.groups * b.dchunks >= kDzBlocks ? 1024 : 512;

@@ -15,11 +15,12 @@
 //   warp 0       slabs: CB/8 bulk copies per stage
 //   warp 1       TMEM allocator, MMA issuer
 //   warp 2       weights: resident, or a ring of a few MMA steps per slot
-//   warps 3-10   epilogue: every `sps` stages (at most about `seg` MMA steps) the
-//                accumulator is read from TMEM and added to fp32 registers
+//   warps 3-10   epilogue: every segment (about `seg` MMA steps: whole stages, or
+//                kernel rows of one) the accumulator is read from TMEM and added to
+//                fp32 registers
 //                (the tensor core truncates when it accumulates, about 1e-8 of
 //                the result per step; short chains keep that below 5e-7), the
-//                other TMEM buffer meanwhile taking the next stages; after the
+//                other TMEM buffers meanwhile taking the next stages; after the
 //                last, bias, ReLU and coalesced stores (lane = pixel).
 // A 0 * inf of a pruned weight would put a NaN where the kept sum has none:
 // pruned entries are stored as -0.0 and an output that comes out NaN is summed
@@ -37,7 +38,7 @@ namespace {
 constexpr int kGcWarps = 11;
 constexpr int kGcThreads = kGcWarps * 32;
 constexpr int kGcEpiWarps = 8;
-constexpr int kGcMaxA = 4, kGcMaxB = 8;
+constexpr int kGcMaxA = 4, kGcMaxB = 8, kGcMaxBuf = 4;
 constexpr int kGcTables = 2 * 256 * 4;
 constexpr int kGcZcap = 1024;
 constexpr int kGcBars = 512;
@@ -65,7 +66,11 @@ struct GcArgs {
     int cb, ncb, spt;   // channels per block, blocks (static), MMA steps per stage
     int h16, rsteps;    // 16-channel steps per tap, MMA steps per kernel row (a slot of the weight ring)
     int sp;             // slots of a slab
-    int sps;            // stages per accumulation segment
+    // Accumulation segments: pps stages each or, where a stage is longer than a
+    // segment (cut), pps pieces of psteps MMA steps of its kernel rows; ppst pieces
+    // a stage (1 without cut).
+    int cut, psteps, pps, ppst;
+    int nbuf;  // accumulator buffers
     int cap_b, stages_a, a_bytes, a_stride;
     int cstride;
     int tmem_stride, tmem_cols;
@@ -141,6 +146,13 @@ struct GcPipe {
     int stages_b, bnr;
 };
 
+// The kernel rows gc_issue is instantiated for: KW taps of h16 16-channel steps, at
+// most 14 MMAs.
+inline bool unrolled_row(int kw, int h16)
+{
+    return ((kw == 1 || kw == 3) && h16 <= 4) || ((kw == 5 || kw == 7) && h16 <= 2) || ((kw == 4 || kw == 6) && h16 == 1);
+}
+
 // The issuing warp's run over its work items.  The whole warp runs the loop,
 // every branch on a parameter or a vote, and one elected lane issues.  KW taps
 // of H steps of 16 channels make a kernel row, unrolled: an MMA then issues in
@@ -148,7 +160,7 @@ struct GcPipe {
 // table in the parameters, 103 with the row chosen by a switch inside the loop,
 // 120 and more with bounds the compiler cannot prove uniform).  KW = 0: any
 // other row, one MMA at a time.
-template <int KW, int H, int MT>
+template <int KW, int H, int MT, bool CUT>
 SADMM_DEV void gc_issue(const GcArgs& a, const GcPipe& p, const int mode)
 {
     const bool resident = mode == kResident;
@@ -176,10 +188,11 @@ SADMM_DEV void gc_issue(const GcArgs& a, const GcPipe& p, const int mode)
             cur = g;
         }
         uint32_t d = 0, blo = blo0;
-        int in_seg = 0;
+        int in_seg = 0;  // stages (CUT: pieces) of the segment so far
         for (int st = 0; st < a.ncb * a.gr.KT; ++st) {
             if (uniform(st >= nst)) break;
-            if (in_seg == 0) {
+            const bool last = uniform(st + 1 == nst);
+            if (!CUT && in_seg == 0) {
                 if (!mbar_wait_warp(&p.acc_empty[ab], acc_ph ^ 1u, p.abort_flag, a.status)) { ok = false; break; }
                 d = p.tmem_base + (uint32_t)(ab * MT * a.tmem_stride);
             }
@@ -192,26 +205,41 @@ SADMM_DEV void gc_issue(const GcArgs& a, const GcPipe& p, const int mode)
                     tc_fence_after();
                     blo = blo0 + (uint32_t)(sb * (mode == kRowSlots ? a.rsteps : a.spt)) * bs16;
                 }
-                const uint32_t acc = (in_seg > 0 || kh > 0) ? 1u : 0u;
-                if (KW > 0) {
+                // CUT: a segment ends at a piece of the kernel row (the row itself when it is unrolled)
+                for (int i0 = 0; i0 < (CUT && KW == 0 ? a.rsteps : 1); i0 += (CUT && KW == 0 ? a.psteps : 1)) {
+                    if (CUT && in_seg == 0) {
+                        if (!mbar_wait_warp(&p.acc_empty[ab], acc_ph ^ 1u, p.abort_flag, a.status)) { ok = false; break; }
+                        tc_fence_after();
+                        d = p.tmem_base + (uint32_t)(ab * MT * a.tmem_stride);
+                    }
+                    const uint32_t acc = (in_seg > 0 || (!CUT && kh > 0)) ? 1u : 0u;
+                    if (KW > 0) {
 #pragma unroll
-                    for (int kw = 0; kw < KW; ++kw)
+                        for (int kw = 0; kw < KW; ++kw)
 #pragma unroll
-                        for (int j = 0; j < H; ++j) {
-                            const uint32_t al = ar + kw + j * half, bl = blo + (kw * H + j) * bs16;
-                            const uint32_t ac = (kw || j) ? 1u : acc;
+                            for (int j = 0; j < H; ++j) {
+                                const uint32_t al = ar + kw + j * half, bl = blo + (kw * H + j) * bs16;
+                                const uint32_t ac = (kw || j) ? 1u : acc;
+                                mma_bf16_ss_elect(d, ahi | al, bhi | bl, idesc, ac);
+                                if (MT == 2) mma_bf16_ss_elect(d + (uint32_t)a.tmem_stride, ahi | (al + 128u), bhi | bl, idesc, ac);
+                            }
+                    } else {
+                        const int end = CUT ? min(i0 + a.psteps, a.rsteps) : a.rsteps;
+                        for (int i = i0; i < end; ++i) {
+                            const int kw = i / a.h16;
+                            const uint32_t al = ar + kw + (i - kw * a.h16) * half, bl = blo + i * bs16;
+                            const uint32_t ac = i > i0 ? 1u : acc;
                             mma_bf16_ss_elect(d, ahi | al, bhi | bl, idesc, ac);
                             if (MT == 2) mma_bf16_ss_elect(d + (uint32_t)a.tmem_stride, ahi | (al + 128u), bhi | bl, idesc, ac);
                         }
-                } else {
-                    for (int i = 0; i < a.rsteps; ++i) {
-                        const int kw = i / a.h16;
-                        const uint32_t al = ar + kw + (i - kw * a.h16) * half, bl = blo + i * bs16;
-                        const uint32_t ac = i > 0 ? 1u : acc;
-                        mma_bf16_ss_elect(d, ahi | al, bhi | bl, idesc, ac);
-                        if (MT == 2) mma_bf16_ss_elect(d + (uint32_t)a.tmem_stride, ahi | (al + 128u), bhi | bl, idesc, ac);
+                    }
+                    if (CUT && (++in_seg == a.pps || (last && kh + 1 == a.gr.KH && (KW > 0 || i0 + a.psteps >= a.rsteps)))) {
+                        mma_commit_elect(&p.acc_full[ab]);
+                        if (++ab == a.nbuf) { ab = 0; acc_ph ^= 1u; }
+                        in_seg = 0;
                     }
                 }
+                if (CUT && !ok) break;
                 ar += (uint32_t)a.gr.Wb;
                 blo += (uint32_t)a.rsteps * bs16;
                 if (mode == kRowSlots) {
@@ -226,9 +254,9 @@ SADMM_DEV void gc_issue(const GcArgs& a, const GcPipe& p, const int mode)
             }
             mma_commit_elect(&p.empty_a[s]);
             if (++s == a.stages_a) { s = 0; ph ^= 1u; }
-            if (++in_seg == a.sps || uniform(st + 1 == nst)) {
+            if (!CUT && (++in_seg == a.pps || last)) {
                 mma_commit_elect(&p.acc_full[ab]);
-                if (++ab == 2) { ab = 0; acc_ph ^= 1u; }
+                if (++ab == a.nbuf) { ab = 0; acc_ph ^= 1u; }
                 in_seg = 0;
             }
         }
@@ -252,8 +280,8 @@ __global__ void __launch_bounds__(kGcThreads, 1)
     uint64_t* full_b = empty_a + kGcMaxA;
     uint64_t* empty_b = full_b + kGcMaxB;
     uint64_t* acc_full = empty_b + kGcMaxB;
-    uint64_t* acc_empty = acc_full + 2;
-    uint64_t* b_full = acc_empty + 2;
+    uint64_t* acc_empty = acc_full + kGcMaxBuf;
+    uint64_t* b_full = acc_empty + kGcMaxBuf;
     uint64_t* b_empty = b_full + 1;
     uint64_t* drain = b_empty + 1;
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(drain + 1);
@@ -263,7 +291,7 @@ __global__ void __launch_bounds__(kGcThreads, 1)
     if (threadIdx.x == 0) {
         for (int s = 0; s < kGcMaxA; ++s) { mbar_init(&full_a[s], 1); mbar_init(&empty_a[s], 1); }
         for (int s = 0; s < kGcMaxB; ++s) { mbar_init(&full_b[s], 1); mbar_init(&empty_b[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], kGcEpiWarps); }
+        for (int b = 0; b < kGcMaxBuf; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], kGcEpiWarps); }
         mbar_init(b_full, 1);
         mbar_init(b_empty, 1);
         mbar_init(drain, 1);
@@ -388,17 +416,20 @@ __global__ void __launch_bounds__(kGcThreads, 1)
         const int row = a.gr.KW * 8 + a.h16;
         const int mode = resident ? kResident : stage_slots ? kStageSlots : kRowSlots;
         // (a loop for each, so that the choice is not in them)
-#define SADMM_ISSUE(KW, H)                                                 \
-    if (mode == kResident) gc_issue<KW, H, MT>(a, p, kResident);           \
-    else if (mode == kStageSlots) gc_issue<KW, H, MT>(a, p, kStageSlots);  \
-    else gc_issue<KW, H, MT>(a, p, kRowSlots);
+#define SADMM_MODES(KW, H, CUT)                                               \
+    if (mode == kResident) gc_issue<KW, H, MT, CUT>(a, p, kResident);         \
+    else if (mode == kStageSlots) gc_issue<KW, H, MT, CUT>(a, p, kStageSlots); \
+    else gc_issue<KW, H, MT, CUT>(a, p, kRowSlots);
+#define SADMM_ISSUE(KW, H) if (!OUT_BF16 && a.cut) { SADMM_MODES(KW, H, true) } else { SADMM_MODES(KW, H, false) }
 #define SADMM_ROW(KW, H) if (row == KW * 8 + H) { SADMM_ISSUE(KW, H) } else
         SADMM_ROW(1, 1) SADMM_ROW(1, 2) SADMM_ROW(1, 3) SADMM_ROW(1, 4)
         SADMM_ROW(3, 1) SADMM_ROW(3, 2) SADMM_ROW(3, 3) SADMM_ROW(3, 4)
-        SADMM_ROW(5, 1) SADMM_ROW(5, 2)
+        SADMM_ROW(5, 1) SADMM_ROW(5, 2) SADMM_ROW(7, 1) SADMM_ROW(7, 2)
+        SADMM_ROW(4, 1) SADMM_ROW(6, 1)
         { SADMM_ISSUE(0, 0) }
 #undef SADMM_ROW
 #undef SADMM_ISSUE
+#undef SADMM_MODES
         // Every MMA issued has completed before TMEM is freed.
         mma_commit_elect(drain);
         if (lane == 0) {
@@ -467,7 +498,8 @@ __global__ void __launch_bounds__(kGcThreads, 1)
             for (int k = 0; k < 8; ++k)
 #pragma unroll
                 for (int j = 0; j < kEpiCols; ++j) v[k][j] = 0.0f;
-            for (int st = 0; alive && st < nst; st += a.sps) {
+            const int pieces = nst * a.ppst;
+            for (int pc = 0; alive && pc < pieces; pc += a.pps) {
                 // warp-uniform outcome: the TMEM loads below are .sync.aligned
                 if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[ab], acc_ph, abort_flag, a.status))) {
                     alive = false;
@@ -490,7 +522,7 @@ __global__ void __launch_bounds__(kGcThreads, 1)
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acc_empty[ab]);
-                if (++ab == 2) { ab = 0; acc_ph ^= 1u; }
+                if (++ab == a.nbuf) { ab = 0; acc_ph ^= 1u; }
             }
             uint32_t nan = 0;  // chunks with a NaN
 #pragma unroll
@@ -555,12 +587,13 @@ cudaError_t launch_gc(const GcArgs& a, int grid, size_t smem, cudaStream_t s)
 
 }  // namespace
 
-bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups, int sms, int seg,
+bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups, int sms, int stage, int seg, bool cut,
                      GridConvShape* out)
 {
     if (chans < 1 || cols < 1) return false;
     GridConvShape r;
     r.seg = seg;
+    r.cut = cut;
     const int taps = gr.KH * gr.KW;
     r.k16 = (chans + 15) / 16;
     const long long ksteps = (long long)r.k16 * gr.KT * taps;
@@ -570,10 +603,10 @@ bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups
     const int n16 = (int)round_up(cols, 16);
     if ((long long)(256 + (gr.KH - 1) * gr.Wb + gr.KW) >= (1 << 14)) return false;  // operand stride field
     const long long span = (gr.KH - 1) * gr.Wb + gr.KW - 1;
-    // A block: as many 16s of channels as divide them, keep a stage to one
-    // accumulation segment and its slab to 24 KB.
+    // A block: as many 16s of channels as divide them, keep a stage to `stage`
+    // MMA steps and its slab to 24 KB.
     int m = 4;
-    while (m > 1 && (r.k16 % m != 0 || taps * m > seg || (128 + span) * 32 * m > 24576)) --m;
+    while (m > 1 && (r.k16 % m != 0 || taps * m > stage || (128 + span) * 32 * m > 24576)) --m;
     r.cb = 16 * m;
     const int rsteps = gr.KW * m;
     // The tiling of least estimated time: rounds of items over the SMs, each
@@ -663,14 +696,18 @@ sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const Gri
     a.h16 = sh.cb / 16;
     a.rsteps = gr.KW * a.h16;
     a.spt = gr.KH * a.rsteps;
-    a.sps = std::max(1, sh.seg / a.spt);
+    a.cut = sh.cut && !c.out_bf16 && a.spt > sh.seg ? 1 : 0;  // (the input gradient's: its output is fp32)
+    a.psteps = unrolled_row(gr.KW, a.h16) ? a.rsteps : std::min(a.rsteps, sh.seg);
+    a.pps = std::max(1, sh.seg / (a.cut ? a.psteps : a.spt));
+    a.ppst = a.cut ? gr.KH * ((a.rsteps + a.psteps - 1) / a.psteps) : 1;
     a.cap_b = sh.cap_b;
     a.stages_a = sh.stages_a;
     a.a_bytes = a.sp * 16 * (sh.cb / 8);
     a.a_stride = (int)round_up(a.a_bytes, 128);
     a.tmem_stride = (int)round_up(sh.bn, 32);
+    a.nbuf = std::min(kGcMaxBuf, 512 / (sh.mt * a.tmem_stride));
     int cols = 32;
-    while (cols < 2 * sh.mt * a.tmem_stride) cols <<= 1;
+    while (cols < a.nbuf * sh.mt * a.tmem_stride) cols <<= 1;
     a.tmem_cols = cols;
     a.relu = c.relu ? 1 : 0;
     long long grid = c.ctas > 0 ? c.ctas : device_sm_count();
@@ -722,8 +759,11 @@ static sadmm_status launch_grid_x(const Grid& gr, const Geometry& g, const void*
 // half too (125 against 185).
 constexpr long long kRuleSms = 152;
 
-// MMA steps summed in TMEM: AlexNet conv2's error against 64 bits is 2.1e-7 (the
-// gathered kernel's 3.3e-7); with 27 it would be 1.3e-7 and 55.8 us become 61.2.
+// MMA steps summed in TMEM, whole stages of one kernel frame: AlexNet conv2's error
+// against 64 bits is 2.1e-7 (the gathered kernel's 3.3e-7); with 27 it would be
+// 1.3e-7 and 55.8 us become 61.2.  A longer frame is one segment: 9x9 taps over 32
+// channels, 81 steps, stand at 7.2e-7 where the gathered kernel's sums of all 162
+// stood at 1.6e-6; cut after 54 they take 51 us instead of 44.
 constexpr int kFwdSeg = 54;
 
 // Channels of x per conv group that hold a kept column.
@@ -747,7 +787,7 @@ bool grid_fwd_plan(const Geometry& g, sadmm_plan* plan, size_t* gx, size_t* gw, 
     if (units < kRuleSms) return false;
     const int nck = fwd_channels(plan, g);
     const int per = (int)((plan->n_filt + g.groups - 1) / g.groups);
-    if (!grid_conv_shape(gr, nck, plan->n_pad, per, (int)g.groups, plan->ctas, kFwdSeg, &sh)) return false;
+    if (!grid_conv_shape(gr, nck, plan->n_pad, per, (int)g.groups, plan->ctas, kFwdSeg, kFwdSeg, false, &sh)) return false;
     const int chunks = sh.k16 * 2;
     if (g.groups * sh.k16 > 65535) return false;
     plan->gx_cb = sh.cb;
@@ -763,7 +803,7 @@ bool grid_fwd_plan(const Geometry& g, sadmm_plan* plan, size_t* gx, size_t* gw, 
     // stages (the gather's rate up to 128 filters, the MMAs' above), and the
     // stores, which overlap less when one accumulator set fills TMEM.
     GridConvShape rule;
-    if (!grid_conv_shape(gr, nck, plan->n_pad, per, (int)g.groups, kRuleSms, kFwdSeg, &rule)) return false;
+    if (!grid_conv_shape(gr, nck, plan->n_pad, per, (int)g.groups, kRuleSms, kFwdSeg, kFwdSeg, false, &rule)) return false;
     const long long xb = 2 * g.n * g.groups * (long long)nck * g.t * g.h * g.w + 2 * g.groups * 16ll * sh.k16 * gr.L;
     const long long yb = 4 * g.m * g.f;
     const long long grid_ns = 8000 + xb / 4000 + rule.cycles * 100 / 195 + yb / 60000;

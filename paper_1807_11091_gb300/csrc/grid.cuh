@@ -67,7 +67,8 @@ inline bool grid_of(const Geometry& g, Grid* out)
 // of 16 K columns at a time: [group][column tile][step][K half][row][8].
 struct GridConvShape {
     int cb;      // channels per block (multiple of 16)
-    int seg;     // MMA steps summed in TMEM before the fp32 registers take over
+    int seg;     // MMA steps summed in TMEM before the fp32 registers take over,
+    bool cut;    // also where that ends inside a stage (else a stage is never cut)
     int k16;     // 16-channel groups of the source (padded channels / 16)
     int ksteps;  // MMA steps of 16 K columns
     int mt;      // 128-pixel tiles per work item (1 or 2)
@@ -78,11 +79,11 @@ struct GridConvShape {
     long long cycles;  // its estimated time
 };
 // The tiling for `chans` source channels and at most `cols`, likely `likely`,
-// output columns per group over `groups` groups, summing about `seg` MMA steps in
-// TMEM; false when it does not fit.
+// output columns per group over `groups` groups, stages of at most `stage` MMA steps
+// where the kernel allows and sums of `seg` in TMEM; false when it does not fit.
 // The blocks of channels (the order of the sums) follow the layer alone, not its
 // batch or the device.
-bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups, int sms, int seg,
+bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups, int sms, int stage, int seg, bool cut,
                      GridConvShape* out);
 
 // Rows of a column tile in the weights' layout: the most columns any group has,

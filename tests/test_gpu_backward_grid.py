@@ -161,3 +161,36 @@ def test_infinite_weight_reaches_real_outputs_alone(case):
     assert np.array_equal(~np.isfinite(got), bad)
     ref = want.numpy()
     assert np.abs(got[~bad] - ref[~bad]).max() <= 1e-5 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("case", [
+    # stages longer than a segment: cut at kernel rows, and inside one
+    ("7x7", ConvShape(n=4, c=32, h=28, w=28, f=64, kh=7, kw=7, ph=3, pw=3)),
+    ("11x11", ConvShape(n=4, c=32, h=20, w=20, f=64, kh=11, kw=11, ph=5, pw=5)),
+    ("1x31", ConvShape(n=8, c=16, h=4, w=96, f=32, kh=1, kw=31, ph=0, pw=15)),
+    # unrolled rows, one and two 16-filter groups a stage
+    ("5x5", ConvShape(n=4, c=48, h=27, w=27, f=72, kh=5, kw=5, ph=2, pw=2)),
+    ("3x3", ConvShape(n=4, c=64, h=28, w=28, f=64, kh=3, kw=3, ph=1, pw=1)),
+    ("3d", ConvShape(n=2, c=16, t=6, h=14, w=14, f=64, kt=3, kh=3, kw=3, pt=1, ph=1, pw=1)),
+    # long sums over the filters
+    ("512_filters", ConvShape(n=8, c=32, h=9, w=9, f=512, kh=3, kw=3, ph=1, pw=1)),
+], ids=lambda c: c[0])
+def test_input_gradient_error_against_64_bits(case):
+    """dx in the 2-norm against 64 bits: the tensor core truncates about 1e-8 of a sum per
+    step of 16, and its sums are cut after 12 steps (27 past 256 filters); the fp32 additions
+    of the at most 130 segments add about 1e-7.  Uncut, the 7x7 and 11x11 layers stand at 4
+    to 12e-7."""
+    from paper_1807_11091_gb300 import sadmm
+    name, s = case
+    dev = torch.device("cuda", 0)
+    g = torch.Generator().manual_seed(8)
+    W = (torch.randn(s.w_shape(), generator=g) * 0.1).to(torch.bfloat16).to(dev)
+    x = torch.relu(torch.randn(s.x_shape(), generator=g)).to(torch.bfloat16).to(dev)
+    dy = torch.randn(s.y_shape(), generator=g).to(torch.bfloat16).to(dev)
+    pc = sadmm.PrunedConv(s.desc16(), W, None, wl.COL_NONE, None, s.f, s.k)
+    dx = pc.backward(x, dy, relu=False)[2]
+    assert sadmm.device_status() == 0
+    conv = torch.nn.functional.conv3d if s.is3d else torch.nn.functional.conv2d
+    xd = x.double().requires_grad_(True)
+    ref, = torch.autograd.grad(conv(xd, W.double(), padding=(s.pt, s.ph, s.pw) if s.is3d else (s.ph, s.pw)), xd, dy.double())
+    assert ((dx.double() - ref).norm() / ref.norm()).item() <= (3.5e-7 if s.f > 256 else 2.5e-7)
