@@ -21,21 +21,16 @@
 // A layer of at most 64 channels fills half of the M side or less: its slab is
 // then staged up to 16 / chunks times, each copy a pixel further on, and one
 // MMA covers that many kernel columns.
-// The tensor core truncates as it accumulates (about 1e-8 of the result per step
-// of 16), so fp32 registers or slices take over early: dW after kGwMaxTiles tiles
-// of 128 pixels, dx after dx_seg() steps.  Errors against 64 bits (2-norm) of dW:
-// conv2 2.2e-7, conv3 2.1e-7, the ResNet-50 3x3 layer 2.5e-7, beside 2.2, 1.9 and
-// 2.3e-7 of the chunked path's.  With 12 tiles conv2's dW stood at 4.5e-7 (and its
-// backward at 161 us, not 175).
+// The tensor core truncates as it accumulates, so fp32 registers take over early: dW
+// after kGwSegTiles tiles of 128 pixels (16 MMA steps), dx after dx_seg() steps; an
+// item's sums leave the registers once, for its slice.  Errors against 64 bits (2-norm)
+// of dW, beside the chunked path's: AlexNet conv2 1.4e-7 (2.2), conv3 1.1e-7 (1.9), a
+// ResNet-50 3x3 layer 1.2e-7 (2.3), 64 channels at 224x224 and batch 8 1.5e-7 (2.3);
+// with sums of 32 steps conv3's stand at 1.5e-7, of 48 at 2.1e-7.
 //
-// AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5):
-// 841 us as six im2col / GEMM / col2im chunks, 175 to 180 us here.  One cold launch each:
-// front 38 us (138 MB moved; each dZ octet is 16 loads of 2 and 4 bytes), weight
-// gradient 72 (57 cycles per 128 x 64 x 16 MMA: bound by the operands'
-// shared-memory reads, 96 of the 128 rows in use), input gradient 60 (57 cycles
-// per 128 x 48 x 16), reduction 15.  conv3, 164 -> 50 us: 13 / 18 / 20 / 11; a
-// ResNet-50 3x3 layer (64 of 128 channels and filters kept) at batch 64, 277 -> 45:
-// 12 / 17 / 18 / 10.
+// AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5): 841
+// us as six im2col / GEMM / col2im chunks, 165 us here; conv3 164 -> 57, a ResNet-50
+// 3x3 layer (64 of 128 channels and filters kept) at batch 64 277 -> 42.
 #include <string.h>
 
 #include <algorithm>
@@ -46,12 +41,15 @@ namespace sadmm {
 namespace {
 
 constexpr int kGwThreads = 10 * 32;
-constexpr int kGwMaxStages = 4;
-constexpr int kGwMaxTiles = 6;       // 128-pixel tiles summed in TMEM: 48 MMA steps
+constexpr int kGwMaxStages = 6;
+constexpr int kGwSegTiles = 2;       // 128-pixel tiles summed in TMEM: 8 MMA steps each
+static_assert(kGwSegTiles % 2 == 0, "a segment ends with a stage of one or two tiles");
+constexpr int kGwMaxTiles = 64;      // tiles of an item, summed in registers
 constexpr int kDxStage = 27;         // most MMA steps of an input gradient's stage, where the kernel has no more taps
 constexpr long long kGwCtas = 152;   // work items come in multiples of about this many (fixed: it sizes the workspace)
 constexpr int kGwSmemLimit = 232448;
-constexpr int kGwCols = 512;         // accumulator columns
+constexpr int kGwCols = 256;         // columns of an accumulator; TMEM holds two
+constexpr int kGwChunks = kGwCols / kEpiCols / 2;  // 16-column chunks of an accumulator that a warp holds
 
 // MMA steps of the input gradient summed in TMEM.  The chunked path sums a pixel's
 // kept filters there, 16 a step, and adds the taps up in fp32: up to 256 filters a
@@ -72,11 +70,47 @@ struct WgradShape {
     int tpg, tgs;     // macro taps per item, items per kernel frame
     int types;        // items per pixel range
     int tiles, tps, Z;  // 128-pixel tiles, tiles per range, ranges
-    int spa;          // slots of a staged chunk
-    int stages, a_bytes, stage_stride;
-    size_t smem;
+    int span;         // slots that an item's taps reach beyond its pixels, at most
     long long slice;  // floats of a pixel range's slice
 };
+
+// How the stages lie in shared memory for items of `nr` filters: slabs of one
+// 128-pixel tile, or of two where that leaves two stages.  A bulk copy takes about
+// 66 cycles whatever its size up to 4 KB at least, and a slab is a copy per chunk.
+struct GwStage {
+    int tiles, spa, a_bytes, stride, count;  // tiles and slots a chunk, bytes of the slab and of a stage, stages
+};
+__host__ __device__ inline GwStage gw_stage(const WgradShape& w, int nr)
+{
+    GwStage st;
+    for (st.tiles = 2;; st.tiles = 1) {
+        st.spa = st.tiles * 128 + w.span;
+        st.a_bytes = (w.rep * w.blk * st.spa * 16 + 127) / 128 * 128;
+        st.stride = st.a_bytes + nr * 256 * st.tiles;
+        // (the MMA reads 16 chunks whatever the rows in use: room past the last stage)
+        st.count = (kGwSmemLimit - 1024 - 512 - (16 - w.rep * w.blk) * st.spa * 16) / st.stride;
+        if (st.count > kGwMaxStages) st.count = kGwMaxStages;
+        if (st.count >= 2 || st.tiles == 1) return st;
+    }
+}
+
+// The most slots that the taps of an item span beyond its 128 pixels.
+int wgrad_span(const Grid& gr, const WgradShape& w)
+{
+    const int macro = gr.KH * w.kwg;
+    int span = 0;
+    for (int t0 = 0; t0 < macro; t0 += w.tpg) {
+        const int t1 = std::min(macro, t0 + w.tpg) - 1, r0 = t0 / w.kwg, r1 = t1 / w.kwg;
+        const int first = r0 * gr.Wb + t0 % w.kwg * w.rep, last = r1 * gr.Wb + t1 % w.kwg * w.rep;
+        int lo = std::min(first, last), hi = std::max(first, last);
+        if (r1 > r0) {
+            lo = std::min(lo, (r0 + 1) * gr.Wb);
+            hi = std::max(hi, (r1 - 1) * gr.Wb + (w.kwg - 1) * w.rep);
+        }
+        span = std::max(span, hi - lo);
+    }
+    return span;
+}
 
 // `nck` channels and at most `n_pad`, likely `likely`, filters per group.
 bool wgrad_shape(const Grid& gr, int nck, int n_pad, int likely, int groups, WgradShape* out)
@@ -94,66 +128,53 @@ bool wgrad_shape(const Grid& gr, int nck, int n_pad, int likely, int groups, Wgr
     w.blk = (w.nch + w.mblks - 1) / w.mblks;
     w.kwg = (gr.KW + w.rep - 1) / w.rep;
     w.rows = w.rep * w.blk * 8;
-    w.nft = (n_pad + 255) / 256;
-    w.nst = (int)round_up((n_pad + w.nft - 1) / w.nft, 16);
     w.tiles = (gr.L + 127) / 128;
     const int macro = gr.KH * w.kwg;
-    const int nl = std::min(w.nst, (int)round_up(likely, 16));
-    // The taps of an item: what fits TMEM and leaves two stages of slabs; below
-    // that, the split of the taps of least estimated time.  Fewer taps an item
-    // mean longer pixel ranges, so fewer slices to write and to add up, for more
-    // slab loads: a 3x3 layer of 64 kept channels and filters at batch 64 runs its
-    // 6 MMA taps as two items of 6 tiles, not one of 3: its slices are 14 MB, not
-    // 28, and its backward took 48 us, not 53.  Only for a fifth less by the
-    // estimate: AlexNet conv3 as three items of 8 tiles, not two of 6, was 18 % less
-    // by it and measured 53.9 against 53.4 us (SMs without an item start the input
-    // gradient early).
-    const int tmax = std::min(std::min(kGwCols / w.nst, macro), 32);
-    if (tmax < 1) return false;
+    // The filter tiles (whole, about 128, 96, 64 and 48), the taps of an item (as many
+    // as fill an accumulator with the likely filters, or fewer) and the pixel ranges of
+    // least estimated time.  More columns an item mean fewer slab loads, more ranges
+    // more slices to write and to add up.
+    const int nft0 = (n_pad + kGwCols - 1) / kGwCols;
     long long best = -1;
-    for (int tgs = (macro + tmax - 1) / tmax; tgs <= macro; ++tgs) {
-        w.tpg = (macro + tgs - 1) / tgs;
-        w.tgs = (macro + w.tpg - 1) / w.tpg;
-        if (w.tgs != tgs) continue;
-        int span = 0;
-        for (int t0 = 0; t0 < macro; t0 += w.tpg) {
-            int lo = 1 << 30, hi = 0;
-            for (int t = t0; t < std::min(macro, t0 + w.tpg); ++t) {
-                const int s = (t / w.kwg) * gr.Wb + (t % w.kwg) * w.rep;
-                lo = std::min(lo, s);
-                hi = std::max(hi, s);
+    int seen = 0;
+    for (const int aim : {kGwCols, 128, 96, 64, 48}) {
+        w.nft = std::max(nft0, (n_pad + aim - 1) / aim);
+        if (w.nft == seen) continue;
+        seen = w.nft;
+        w.nst = (int)round_up((n_pad + w.nft - 1) / w.nft, 16);
+        const int nl = w.nft == 1 ? std::min(w.nst, (int)round_up(likely, 16)) : w.nst;
+        const int tmax = std::min(std::min(kGwCols / nl, macro), 32), tg0 = (macro + tmax - 1) / tmax;
+        for (int tgs = tg0; tgs <= std::min(macro, tg0 + 3); ++tgs) {
+            w.tpg = (macro + tgs - 1) / tgs;
+            w.tgs = (macro + w.tpg - 1) / w.tpg;
+            if (w.tgs != tgs) continue;
+            w.span = wgrad_span(gr, w);
+            if (w.span + 256 >= (1 << 14) || gw_stage(w, w.nst).count < 2) continue;
+            const GwStage sg = gw_stage(w, nl);
+            const long long types = (long long)groups * w.nft * w.mblks * gr.KT * w.tgs;
+            // Cycles of a tile: its MMAs (as in conv_grid.cu) or its share of the slab
+            // copies, and 280 a stage for its waits and commits; of an item its tiles,
+            // then its slice's stores (16 bytes a cycle, beside the next item's MMAs);
+            // and the reduction's reads (16 bytes a cycle and SM).
+            const long long cols = (long long)w.tpg * nl;
+            const long long tile = std::max(w.tpg * 8ll * (std::max(32 + nl / 4, nl / 2) + 9),
+                                            66ll * (w.rep * w.blk + nl / 8) / sg.tiles) + 280 / sg.tiles;
+            const long long st = w.rows * cols / 4;
+            for (int waves = 1; waves <= 4; ++waves) {
+                const long long z = std::max<long long>(std::max<long long>(1, kGwCtas * waves / types),
+                                                        (w.tiles + kGwMaxTiles - 1) / kGwMaxTiles);
+                w.tps = (int)((w.tiles + z - 1) / std::min<long long>(z, w.tiles));
+                w.Z = (w.tiles + w.tps - 1) / w.tps;
+                if (types * w.Z >= (1ll << 30)) continue;
+                w.types = (int)types;
+                w.slice = types * w.rows * w.tpg * w.nst;
+                const long long item = w.tps * tile, rounds = (types * w.Z + kGwCtas - 1) / kGwCtas;
+                const long long cost = rounds * std::max(item, st) + st + types * w.Z * w.rows * cols * 4 / (kGwCtas * 16);
+                if (best < 0 || cost < best) {
+                    best = cost;
+                    *out = w;
+                }
             }
-            span = std::max(span, hi - lo);
-        }
-        w.spa = 128 + span;
-        w.a_bytes = (int)round_up((long long)w.rep * w.blk * w.spa * 16, 128);
-        w.stage_stride = w.a_bytes + w.nst / 8 * 2048;
-        // the MMA reads 16 chunks whatever the rows in use: room past the last stage
-        const long long fixed = 1024 + 512 + (long long)(16 - w.rep * w.blk) * w.spa * 16;
-        w.stages = (int)std::min<long long>(kGwMaxStages, (kGwSmemLimit - fixed) / w.stage_stride);
-        w.smem = (size_t)(fixed + (long long)w.stages * w.stage_stride);
-        if (w.spa >= (1 << 14) || w.stages < 2 || (w.stages < 3 && w.tpg > 1)) continue;
-        const long long types = (long long)groups * w.nft * w.mblks * gr.KT * w.tgs;
-        const long long work = types * w.tiles;
-        const long long waves = std::max<long long>(1, (work + kGwCtas * kGwMaxTiles - 1) / (kGwCtas * kGwMaxTiles));
-        w.tps = (int)std::max<long long>(1, std::min<long long>(kGwMaxTiles, (work + kGwCtas * waves - 1) / (kGwCtas * waves)));
-        w.Z = (w.tiles + w.tps - 1) / w.tps;
-        if (types * w.Z >= (1ll << 30)) continue;
-        w.types = (int)types;
-        w.slice = types * w.rows * w.tpg * w.nst;
-        // Cycles: rounds of items, each its tiles' MMAs (as in conv_grid.cu) or
-        // loads (40 bytes a cycle), then its slice's stores (32 bytes a cycle;
-        // beside the next item's MMAs when two accumulator sets fit), and the
-        // reduction's reads (16 bytes a cycle and SM).
-        const long long cols = (long long)macro * nl / w.tgs;
-        const long long tile = std::max((long long)macro * 8 * (std::max(32 + nl / 4, nl / 2) + 9) / w.tgs,
-                                        (w.a_bytes + nl * 256ll) / 40) + 150;
-        const long long st = w.rows * cols / 8, item = w.tps * tile, rounds = (types * w.Z + kGwCtas - 1) / kGwCtas;
-        const long long cost = (w.tpg * nl <= kGwCols / 2 ? rounds * std::max(item, st) + st : rounds * (item + st)) +
-                               types * w.Z * w.rows * cols * 4 / (kGwCtas * 16);
-        if (best < 0 || cost * 5 < best * 4) {
-            best = cost;
-            *out = w;
         }
     }
     return best >= 0;
@@ -178,6 +199,7 @@ struct GwArgs {
 // frame, tap group).
 struct GwItem {
     int z, type, g, ft, mb, kt, t0, nt, nr, base, span;
+    int tp;  // taps that fill an accumulator: more take another pass over the pixels
 };
 SADMM_DEV GwItem gw_item(const GwArgs& a, int u)
 {
@@ -205,6 +227,7 @@ SADMM_DEV GwItem gw_item(const GwArgs& a, int u)
     }
     it.base = lo;
     it.span = hi - lo;
+    it.tp = min(it.nt, it.nr > 0 ? kGwCols / it.nr : 1);
     return it;
 }
 
@@ -257,7 +280,7 @@ __global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_const
         fence_mbar_init();
     }
     if (warp == 1) {
-        tmem_alloc(tmem_holder, (uint32_t)kGwCols);
+        tmem_alloc(tmem_holder, 2u * kGwCols);
         tmem_relinquish();
     }
     pdl_wait();
@@ -266,11 +289,12 @@ __global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_const
     tc_fence_after();
     pdl_trigger();  // after every thread's wait: k_grid_front has completed when a dependent starts
     const uint32_t tmem_base = *tmem_holder;
-    // two accumulator sets when every item's columns fit half of TMEM
+    // The stages hold what the groups' counts need, known on the device alone.
     int most = 0;
     for (int g = 0; g < a.groups; ++g) most = max(most, __ldg(a.counts + 2 * g));
-    const int nbuf = uniform(a.w.tpg * min(a.w.nst, (most + 15) & ~15) <= kGwCols / 2) ? 2 : 1;
-
+    // (a reduction over the warp: the compiler then knows what follows from it as uniform)
+    most = __reduce_max_sync(0xffffffffu, min(a.w.nst, (most + 15) & ~15));
+    const GwStage sg = gw_stage(a.w, most);
     if (warp == 0) {
         int s = 0;
         uint32_t ph = 0, last = 0, issued = 0;
@@ -280,36 +304,39 @@ __global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_const
             if (it.nr == 0) continue;
             const int nb = min(a.w.blk, a.w.nch - it.mb * a.w.blk);  // chunks of this block
             const int na = nb * a.w.rep, nd = it.nr / 8;
-            const uint32_t abytes = (uint32_t)(128 + it.span) * 16u;
             const __nv_bfloat16* xg = a.xs + (size_t)it.g * a.xs_gstride;
             const __nv_bfloat16* dg = a.dz + (size_t)it.g * a.dz_gstride;
-            const int e = min(a.w.tiles, (it.z + 1) * a.w.tps);
-            for (int t = it.z * a.w.tps; t < e; ++t) {
-                if (!mbar_wait_warp(&empty[s], ph ^ 1u, abort_flag, a.status)) { ok = false; break; }
-                if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)na * abytes + (uint32_t)nd * 2048u);
-                __syncwarp();
-                const uint32_t sa = smem_u32(stage0 + (size_t)s * a.w.stage_stride);
-                for (int i = lane; i < na + nd; i += 32) {
-                    if (i < na) {
-                        const int rp = i / nb, c = i - rp * nb;
-                        bulk_load(sa + (uint32_t)((rp * a.w.blk + c) * a.w.spa * 16),
-                                  xg + ((size_t)(it.mb * a.w.blk + c) * a.gr.slots +
-                                        (size_t)(t * 128 + it.kt * a.gr.HWb + it.base + rp)) * 8,
-                                  abytes, &full[s]);
-                    } else {
-                        const int c = i - na;
-                        bulk_load(sa + (uint32_t)(a.w.a_bytes + c * 2048),
-                                  dg + ((size_t)(it.ft * (a.w.nst / 8) + c) * a.gr.slots +
-                                        (size_t)(a.gr.D0 + t * 128)) * 8,
-                                  2048u, &full[s]);
+            const int b = it.z * a.w.tps, e = min(a.w.tiles, b + a.w.tps);
+            for (int t0 = 0; ok && t0 < it.nt; t0 += it.tp) {  // a pass over the pixels for the taps t0 ..
+                for (int t = b; t < e; t += sg.tiles) {
+                    if (!mbar_wait_warp(&empty[s], ph ^ 1u, abort_flag, a.status)) { ok = false; break; }
+                    const int n = min(sg.tiles, e - t);
+                    const uint32_t abytes = (uint32_t)(n * 128 + it.span) * 16u, dbytes = (uint32_t)n * 2048u;
+                    if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)na * abytes + (uint32_t)nd * dbytes);
+                    __syncwarp();
+                    const uint32_t sa = smem_u32(stage0 + (size_t)s * sg.stride);
+                    for (int k = lane; k < na + nd; k += 32) {
+                        if (k < na) {
+                            const int rp = k / nb, c = k - rp * nb;
+                            bulk_load(sa + (uint32_t)((rp * a.w.blk + c) * sg.spa * 16),
+                                      xg + ((size_t)(it.mb * a.w.blk + c) * a.gr.slots +
+                                            (size_t)(t * 128 + it.kt * a.gr.HWb + it.base + rp)) * 8,
+                                      abytes, &full[s]);
+                        } else {
+                            const int c = k - na;
+                            bulk_load(sa + (uint32_t)(sg.a_bytes + c * sg.tiles * 2048),
+                                      dg + ((size_t)(it.ft * (a.w.nst / 8) + c) * a.gr.slots +
+                                            (size_t)(a.gr.D0 + t * 128)) * 8,
+                                      dbytes, &full[s]);
+                        }
                     }
+                    last = (last & ~(1u << s)) | (ph << s);
+                    issued |= 1u << s;
+                    if (++s == sg.count) { s = 0; ph ^= 1u; }
                 }
-                last = (last & ~(1u << s)) | (ph << s);
-                issued |= 1u << s;
-                if (++s == a.w.stages) { s = 0; ph ^= 1u; }
             }
         }
-        for (int q = 0; q < a.w.stages; ++q) {
+        for (int q = 0; q < sg.count; ++q) {
             if (!(issued & (1u << q))) continue;
             const unsigned long long t0 = globaltimer();
             while (!mbar_try_wait(&full[q], (last >> q) & 1u) && globaltimer() - t0 < kWaitLimitNs) {}
@@ -320,37 +347,61 @@ __global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_const
         int s = 0, ab = 0;
         uint32_t ph = 0, acc_ph = 0;
         bool ok = true;
-        const uint64_t ad0 = sdesc_kmajor_none(smem_u32(stage0), 128u, (uint32_t)a.w.spa * 16u);
-        const uint64_t bd0 = sdesc_kmajor_none(smem_u32(stage0) + (uint32_t)a.w.a_bytes, 128u, 2048u);
+        const uint64_t ad0 = sdesc_kmajor_none(smem_u32(stage0), 128u, (uint32_t)sg.spa * 16u);
+        const uint64_t bd0 = sdesc_kmajor_none(smem_u32(stage0) + (uint32_t)sg.a_bytes, 128u, (uint32_t)sg.tiles * 2048u);
         const uint64_t ahi = ad0 & 0xffffffff00000000ull, bhi = bd0 & 0xffffffff00000000ull;
         for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x) {
-            const GwItem it = gw_item(a, u);
-            if (uniform(it.nr == 0)) continue;
+            GwItem it = gw_item(a, u);
+            // (uniform, as above)
+            it.nr = __reduce_max_sync(0xffffffffu, it.nr);
+            it.tp = __reduce_max_sync(0xffffffffu, it.tp);
+            if (it.nr == 0) continue;
             const uint32_t idesc = idesc_bf16_f32(128, it.nr) | (1u << 15) | (1u << 16);  // A and B MN-major
-            if (!mbar_wait_warp(&acc_empty[ab], acc_ph ^ 1u, abort_flag, a.status)) break;
-            const uint32_t d0 = tmem_base + (uint32_t)(ab * (kGwCols / 2));
             const int b = it.z * a.w.tps, e = min(a.w.tiles, b + a.w.tps);
-            for (int t = b; t < e; ++t) {
-                if (!mbar_wait_warp(&full[s], ph, abort_flag, a.status)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t so = (uint32_t)(s * a.w.stage_stride) >> 4;
-                const uint32_t blo = (uint32_t)bd0 + so;
-                for (int j = 0; j < it.nt; ++j) {
-                    const int tap = it.t0 + j;
-                    const uint32_t alo = (uint32_t)ad0 + so +
-                                         (uint32_t)((tap / a.w.kwg) * a.gr.Wb + (tap % a.w.kwg) * a.w.rep - it.base);
-                    const uint32_t d = d0 + (uint32_t)(j * it.nr);
+            for (int t0 = it.t0; ok && t0 < it.t0 + it.nt; t0 += it.tp) {
+                const int np = min(it.tp, it.t0 + it.nt - t0);
+                const uint32_t kq0 = (uint32_t)(t0 % a.w.kwg);
+                const uint32_t to0 = (uint32_t)(t0 / a.w.kwg * a.gr.Wb) + kq0 * (uint32_t)a.w.rep - (uint32_t)it.base;
+                int in_seg = 0;
+                uint32_t d0 = 0;
+                for (int t = b; t < e; t += sg.tiles) {
+                    if (in_seg == 0) {
+                        if (!mbar_wait_warp(&acc_empty[ab], acc_ph ^ 1u, abort_flag, a.status)) { ok = false; break; }
+                        d0 = tmem_base + (uint32_t)(ab * kGwCols);
+                    }
+                    if (!mbar_wait_warp(&full[s], ph, abort_flag, a.status)) { ok = false; break; }
+                    tc_fence_after();
+                    const int n = min(sg.tiles, e - t);
+                    const uint32_t so = (uint32_t)(s * sg.stride) >> 4;
+                    uint32_t to = to0, kq = kq0;  // the tap's shift in the slab, its place in the kernel row
+                    for (int j = 0; j < np; ++j) {
+                        uint32_t alo = (uint32_t)ad0 + so + to, blo = (uint32_t)bd0 + so;
+                        const uint32_t d = d0 + (uint32_t)(j * it.nr);
+                        uint32_t acc = in_seg > 0 ? 1u : 0u;
+                        for (int q = 0; q < n; ++q) {
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)  // 16 grid pixels each
-                        mma_bf16_ss_elect(d, ahi | (alo + kk * 16u), bhi | (blo + kk * 16u), idesc,
-                                          (t > b || kk > 0) ? 1u : 0u);
+                            for (int kk = 0; kk < 8; ++kk)  // 16 grid pixels each
+                                mma_bf16_ss_elect(d, ahi | (alo + kk * 16u), bhi | (blo + kk * 16u), idesc, kk > 0 ? 1u : acc);
+                            acc = 1u;
+                            alo += 128u;
+                            blo += 128u;
+                        }
+                        to += (uint32_t)a.w.rep;
+                        if (++kq == (uint32_t)a.w.kwg) {
+                            kq = 0;
+                            to += (uint32_t)(a.gr.Wb - a.w.kwg * a.w.rep);
+                        }
+                    }
+                    mma_commit_elect(&empty[s]);
+                    if (++s == sg.count) { s = 0; ph ^= 1u; }
+                    in_seg += n;
+                    if (in_seg >= kGwSegTiles || t + n >= e) {
+                        mma_commit_elect(&acc_full[ab]);
+                        if (++ab == 2) { ab = 0; acc_ph ^= 1u; }
+                        in_seg = 0;
+                    }
                 }
-                mma_commit_elect(&empty[s]);
-                if (++s == a.w.stages) { s = 0; ph ^= 1u; }
             }
-            if (!ok) break;
-            mma_commit_elect(&acc_full[ab]);
-            if (++ab == nbuf) { ab = 0; acc_ph ^= 1u; }
         }
         mma_commit_elect(drain);
         if (lane == 0) {
@@ -359,50 +410,77 @@ __global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_const
         }
         __syncwarp();
     } else {
-        // epilogue: the item's accumulator into its slice, lane = channel row
+        // epilogue: the item's segments added up in registers, then written to its
+        // slice; lane = channel row, the two warps of a TMEM lane quadrant take its
+        // 16-column chunks in turn
         const int q4 = warp & 3, h = (warp - 2) >> 2;
         const int row = q4 * 32 + lane;
         int ab = 0;
         uint32_t acc_ph = 0;
-        for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+        bool alive = true;
+        for (int u = blockIdx.x; alive && u < a.units; u += gridDim.x) {
             const GwItem it = gw_item(a, u);
             if (it.nr == 0) continue;
             // the item's taps whose column of this lane's channel is kept: only
             // those are written (found while the MMAs run)
             const uint32_t keep = gw_keep(a, it, row);
-            if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[ab], acc_ph, abort_flag, a.status))) break;
-            tc_fence_after();
-            const uint32_t taddr = tmem_base + (uint32_t)(ab * (kGwCols / 2)) + ((uint32_t)(q4 * 32) << 16);
+            const int per = it.nr / kEpiCols;
+            const int b = it.z * a.w.tps, e = min(a.w.tiles, b + a.w.tps);
             float* dst = a.slices + (size_t)it.z * a.w.slice +
                          ((size_t)it.type * a.w.rows + row) * (size_t)(a.w.tpg * a.w.nst);
-            const int per = it.nr / kEpiCols, n = it.nt * per;
-            if (q4 * 32 < a.w.rows) {
-                for (int k = h; k < n; k += 2) {
-                    uint32_t r[kEpiCols];
-                    tmem_ld_32x32b_x16(taddr + (uint32_t)(k * kEpiCols), r);
-                    tmem_ld_wait();
-                    const int j = k / per;
-                    if ((keep >> j) & 1u) {
-                        float4* d4 = reinterpret_cast<float4*>(dst + j * a.w.nst + (k - j * per) * kEpiCols);
+            for (int p0 = 0; alive && p0 < it.nt; p0 += it.tp) {
+                const int n = min(it.tp, it.nt - p0) * per;
+                float v[kGwChunks][kEpiCols];
 #pragma unroll
-                        for (int e = 0; e < kEpiCols / 4; ++e)
-                            d4[e] = make_float4(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]),
-                                                __uint_as_float(r[4 * e + 2]), __uint_as_float(r[4 * e + 3]));
+                for (int c = 0; c < kGwChunks; ++c)
+#pragma unroll
+                    for (int i = 0; i < kEpiCols; ++i) v[c][i] = 0.0f;
+                for (int t = b; t < e; t += kGwSegTiles) {
+                    // warp-uniform outcome: the TMEM loads below are .sync.aligned
+                    if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[ab], acc_ph, abort_flag, a.status))) {
+                        alive = false;
+                        break;
                     }
+                    tc_fence_after();
+                    if (q4 * 32 < a.w.rows) {
+                        const uint32_t taddr = tmem_base + (uint32_t)(ab * kGwCols) + ((uint32_t)(q4 * 32) << 16);
+#pragma unroll
+                        for (int c = 0; c < kGwChunks; ++c) {
+                            const int k = 2 * c + h;
+                            if (k < n) {
+                                uint32_t r[kEpiCols];
+                                tmem_ld_32x32b_x16(taddr + (uint32_t)(k * kEpiCols), r);
+                                tmem_ld_wait();
+#pragma unroll
+                                for (int i = 0; i < kEpiCols; ++i) v[c][i] += __uint_as_float(r[i]);
+                            }
+                        }
+                    }
+                    tc_fence_before();
                     __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[ab]);
+                    if (++ab == 2) { ab = 0; acc_ph ^= 1u; }
                 }
+                if (!alive) break;
+#pragma unroll
+                for (int c = 0; c < kGwChunks; ++c) {
+                    const int k = 2 * c + h, j = k / per;
+                    if (k < n && ((keep >> (p0 + j)) & 1u)) {
+                        float4* d4 = reinterpret_cast<float4*>(dst + (p0 + j) * a.w.nst + (k - j * per) * kEpiCols);
+#pragma unroll
+                        for (int i = 0; i < kEpiCols / 4; ++i)
+                            d4[i] = make_float4(v[c][4 * i], v[c][4 * i + 1], v[c][4 * i + 2], v[c][4 * i + 3]);
+                    }
+                }
+                __syncwarp();
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[ab]);
-            if (++ab == nbuf) { ab = 0; acc_ph ^= 1u; }
         }
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, (uint32_t)kGwCols);
+        tmem_dealloc(tmem_base, 2u * kGwCols);
     }
 }
 
@@ -975,7 +1053,7 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
             configured_dev = dev;
         }
         const int grid = std::min(a.units, device_sm_count());
-        if (launch_pdl(k_grid_wgrad, dim3((unsigned)grid), dim3(kGwThreads), b.ws.smem, s, a) != cudaSuccess)
+        if (launch_pdl(k_grid_wgrad, dim3((unsigned)grid), dim3(kGwThreads), (size_t)kGwSmemLimit, s, a) != cudaSuccess)
             return SADMM_ECUDA;
         memset(&r, 0, sizeof(r));
         r.gr = b.gr;

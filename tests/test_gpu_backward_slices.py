@@ -1,10 +1,9 @@
-"""The weight gradient's slices on the pixel grid: more ranges than one pass of the
-reduction holds (128), kept filters that are no multiple of its 16-byte loads, dZ
-copied in blocks of 1024 slots (the last one ragged), and a layer whose taps are
-split between items (longer ranges) at a size where one item could hold them;
-against the fp64 oracle, at the suite's 2e-3 of the largest value and, the sums
-being fp32 sums of exact products in ranges of at most 6 x 128 pixels, at 2e-6 in
-the 2-norm (4.5e-7 measured at most, with 12 x 128)."""
+"""The weight gradient on the pixel grid: its slices (kept filters that are no multiple of
+the reduction's 16-byte loads, several pixel ranges), dZ copied in blocks of 1024 slots
+(the last one ragged), a layer whose taps are split between items, and groups that keep
+more filters than an item's taps were set for; against the fp64 oracle, at the suite's
+2e-3 of the largest value and, the sums being fp32 sums of exact products, at 2e-6 in the
+2-norm, or at the bound that a test derives."""
 import numpy as np
 import pytest
 import torch
@@ -45,3 +44,60 @@ def test_weight_gradient(case):
         assert_close(g, want, what=f"{name} {what}")
         assert np.linalg.norm(g - want) <= 2e-6 * np.linalg.norm(want), what
     assert np.all(dW.cpu().numpy()[rdW.reshape(s.f, -1) == 0.0] == 0.0)
+
+
+@pytest.mark.parametrize("case", [
+    ("3x3", ConvShape(n=24, c=64, h=56, w=56, f=64, kh=3, kw=3, ph=1, pw=1)),  # ranges of the most tiles
+    ("1x1", ConvShape(n=16, c=256, h=28, w=28, f=160, kh=1, kw=1)),
+    ("13x13", ConvShape(n=128, c=256, h=13, w=13, f=96, kh=3, kw=3, ph=1, pw=1)),  # two channel blocks
+    ("wide", ConvShape(n=8, c=144, h=14, w=14, f=520, kh=3, kw=3, ph=1, pw=1)),  # filter tiles below 256
+], ids=lambda c: c[0])
+def test_weight_gradient_error_against_64_bits(case):
+    """dW in the 2-norm against 64 bits: the tensor core truncates about 5e-9 of a sum per step
+    of 16 pixels and its sums are 16 steps long, which the at most 32 fp32 additions of a range
+    and those of the ranges raise to 1.6e-7.  Sums of 48 steps stand at 2.0 to 2.7e-7."""
+    from paper_1807_11091_gb300 import sadmm
+    name, s = case
+    dev = torch.device("cuda", 0)
+    g = torch.Generator().manual_seed(12)
+    W = torch.randn(s.w_shape(), generator=g).to(torch.bfloat16).to(dev)
+    x = torch.relu(torch.randn(s.x_shape(), generator=g)).to(torch.bfloat16).to(dev)
+    dy = torch.randn(s.y_shape(), generator=g).to(torch.bfloat16).to(dev)
+    pc = sadmm.PrunedConv(s.desc16(), W, None, wl.COL_NONE, None, s.f, s.k)
+    dW = pc.backward(x, dy, relu=False, want_dx=False)[0]
+    assert sadmm.device_status() == 0
+    ref = _dw64(s, x, dy)
+    assert ((dW.double().reshape(s.f, -1) - ref).norm() / ref.norm()).item() <= 1.8e-7
+
+
+def _dw64(s, x, dy):
+    Wd = torch.zeros(s.w_shape(), dtype=torch.float64, device=x.device, requires_grad=True)
+    y = torch.nn.functional.conv2d(x.double(), Wd, padding=(s.ph, s.pw), groups=s.groups)
+    return torch.autograd.grad(y, Wd, dy.double())[0].reshape(s.f, -1)
+
+
+@pytest.mark.parametrize("kept", [(128, 2), (3, 128), (128, 0), (64, 66)], ids=str)
+def test_weight_gradient_of_uneven_groups(kept):
+    """The taps of an item are set for the filters a group is likely to keep; a group that keeps
+    more takes several passes over the pixels, one that keeps none has no items."""
+    from paper_1807_11091_gb300 import sadmm
+    s = ConvShape(n=6, c=48, h=15, w=14, f=256, kh=5, kw=5, ph=2, pw=2, groups=2)
+    dev = torch.device("cuda", 0)
+    g = torch.Generator().manual_seed(13)
+    W = torch.randn(s.w_shape(), generator=g).to(torch.bfloat16).to(dev)
+    x = torch.relu(torch.randn(s.x_shape(), generator=g)).to(torch.bfloat16).to(dev)
+    dy = torch.randn(s.y_shape(), generator=g).to(torch.bfloat16).to(dev)
+    rows = np.concatenate([np.arange(kept[0]), 128 + np.arange(kept[1])]).astype(np.int32)
+    pc = sadmm.PrunedConv(s.desc16(), W, torch.as_tensor(rows, device=dev), wl.COL_NONE, None, len(rows), s.k)
+    dW, _, dx = pc.backward(x, dy, relu=False)
+    assert sadmm.device_status() == 0
+    ref = _dw64(s, x, dy)
+    keep = torch.zeros(s.f, 1, dtype=torch.float64, device=dev)
+    keep[torch.as_tensor(rows, device=dev).long()] = 1.0
+    ref = ref * keep
+    assert ((dW.double().reshape(s.f, -1) - ref).norm() / ref.norm()).item() <= 1.8e-7
+    assert not dW.reshape(s.f, -1)[keep[:, 0] == 0].any()
+    xd = x.double().requires_grad_(True)
+    Wd = (W.double().reshape(s.f, -1) * keep).reshape(W.shape)
+    rdx, = torch.autograd.grad(torch.nn.functional.conv2d(xd, Wd, padding=(2, 2), groups=2), xd, dy.double())
+    assert ((dx.double() - rdx).norm() / rdx.norm()).item() <= 2.5e-7
