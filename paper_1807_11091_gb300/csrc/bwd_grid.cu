@@ -550,21 +550,21 @@ struct WrArgs {
     long long K;
 };
 
-// dW[f_i][col_j] = sum over the pixel ranges of their slices: 32 threads per four
-// filters take every 32nd range, then their sums are added in order
-// (deterministic).  Block (bx, by, g): packed columns bx*kWrCols .., packed rows
+// dW[f_i][col_j] = sum over the pixel ranges of their slices: LANES threads per two
+// columns of four filters take every LANES-th range, then their sums are added in order
+// (deterministic).  Block (bx, by, g): 64 / LANES packed columns, packed rows
 // by*32 .. +31; the slices are read along the filters, 16 bytes a load.
-// Bound by latency: the slices are in L2, so what counts is loads in flight (8 of
-// 16 bytes a thread, and up to 128 of the layer's ranges in one pass) and what is
-// done before the wait.  With eight range lanes of 4-byte loads, four ranges a pass
-// and the tables read after the wait it stood 10 to 14 us behind the layer (AlexNet
-// conv3 55.2 us in all, 51.7 after; two columns a block instead of four, twice the
-// blocks, 49.9 -> 48.8 and a ResNet-50 3x3 layer's 45.6 -> 43.6, one column the same).
+// Bound by latency: what counts is loads in flight (8 of 16 bytes a thread, four ranges)
+// and what is done before the wait.  A thread has work for all of them when the lanes
+// follow the ranges: with 32 lanes whatever their number, 512 filters x 512 channels 3x3
+// over 8 images of 7x7, one range, stood at 217 us of the backward's 256.
 constexpr int kWrCols = 2;
 
+template <int LANES>
 __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbArgs d)
 {
-    __shared__ float s_v[8][kWrCols][48];
+    __shared__ float s_v[64][33];  // [part of the ranges][column][filter]
+    __shared__ int s_f[32];        // the rows' filters
     if ((int)blockIdx.z == d.groups) {  // the last layer of blocks: the bias gradient
         pdl_wait();
         pdl_trigger();
@@ -572,18 +572,20 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbAr
         return;
     }
     // The plan's tables: k_grid_front read them too and has completed.
+    constexpr int ncol = 32 * kWrCols / LANES;
     const int g = blockIdx.z, cnt = __ldg(a.counts + 2 * g);
-    const int i0 = blockIdx.y * 32, j0 = blockIdx.x * kWrCols;
+    const int i0 = blockIdx.y * 32, j0 = blockIdx.x * ncol;
     if (i0 >= cnt) {  // still waits: with no kept filter at all these are the launch's only blocks
         pdl_wait();
         return;
     }
     const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+    const int rl = ty & (LANES - 1), jt = ty / LANES * kWrCols;  // range lane, first column in the block
     const int iq = i0 + tx * 4, ftq = iq / a.w.nst;  // (a tile's filters are a multiple of 16)
     const float* src[kWrCols];
 #pragma unroll
     for (int e = 0; e < kWrCols; ++e) {
-        const int j = j0 + e;
+        const int j = j0 + jt + e;
         const int col = j < a.n_cols ? __ldg(a.colidx + j) : -1;
         src[e] = a.slices;  // (nothing reads what this adds up)
         if (col < 0 || iq >= cnt) continue;
@@ -595,10 +597,10 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbAr
         src[e] = a.slices + ((size_t)type * a.w.rows + m) * (size_t)(a.w.tpg * a.w.nst) + (mt % a.w.tpg) * a.w.nst +
                  (iq - ftq * a.w.nst);
     }
-    // the entry this thread writes: two threads to a filter's two columns
-    const int oe = threadIdx.x & 1, oi = i0 + (threadIdx.x >> 1);
-    const int ocol = threadIdx.x < 64 && j0 + oe < a.n_cols ? __ldg(a.colidx + j0 + oe) : -1;
-    const int of = ocol >= 0 && oi < cnt ? __ldg(a.rowmap + g * a.n_pad + oi) : -1;
+    // the column of the entries this thread writes (ncol divides the block), their filters
+    const int oe = threadIdx.x & (ncol - 1);
+    const int ocol = j0 + oe < a.n_cols ? __ldg(a.colidx + j0 + oe) : -1;
+    if (threadIdx.x < 32) s_f[threadIdx.x] = i0 + (int)threadIdx.x < cnt ? __ldg(a.rowmap + g * a.n_pad + i0 + threadIdx.x) : -1;
     pdl_wait();  // after the kernel before it in the stream, and the one before that (see launch_grid_bwd)
     pdl_trigger();
     float v[kWrCols][4];
@@ -607,12 +609,12 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbAr
 #pragma unroll
         for (int q = 0; q < 4; ++q) v[e][q] = 0.0f;
 #pragma unroll 1
-    for (int z = ty; z < a.w.Z; z += 128) {
+    for (int z = rl; z < a.w.Z; z += 4 * LANES) {
         float4 t[4][kWrCols];  // every load first
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const bool in = z + 32 * r < a.w.Z;
-            const size_t at = (size_t)(z + 32 * r) * a.w.slice;
+            const bool in = z + r * LANES < a.w.Z;
+            const size_t at = (size_t)(z + r * LANES) * a.w.slice;
 #pragma unroll
             for (int e = 0; e < kWrCols; ++e) {
                 t[r][e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -629,29 +631,35 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbAr
                 v[e][3] += t[r][e].w;
             }
     }
-    // the four range lanes of a warp, then the warps in order
+    // the range lanes of a warp (four values of ty), then the warps in order
+    constexpr int parts = LANES > 4 ? LANES / 4 : 1;
 #pragma unroll
     for (int e = 0; e < kWrCols; ++e)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            v[e][q] += __shfl_xor_sync(0xffffffffu, v[e][q], 8);
-            v[e][q] += __shfl_xor_sync(0xffffffffu, v[e][q], 16);
-            if ((threadIdx.x & 31) < 8) s_v[threadIdx.x >> 5][e][tx * 4 + q] = v[e][q];
+            const float p = __shfl_xor_sync(0xffffffffu, v[e][q], 8);
+            if (LANES > 1) v[e][q] += p;
+            const float p2 = __shfl_xor_sync(0xffffffffu, v[e][q], 16);
+            if (LANES > 2) v[e][q] += p2;
+            if ((rl & 3) == 0) s_v[(rl >> 2) * ncol + jt + e][tx * 4 + q] = v[e][q];
         }
     __syncthreads();
-    if (of < 0) return;
-    float acc = 0.0f;
-#pragma unroll
-    for (int z = 0; z < 8; ++z) acc += s_v[z][oe][oi - i0];
-    if (acc != acc) {
-        const int c = a.chan_kind ? (j0 + oe) / a.taps : ocol / a.taps, tap = ocol % a.taps;
-        const int kw = tap % a.gr.KW, kh = (tap / a.gr.KW) % a.gr.KH, kt = tap / (a.gr.KW * a.gr.KH);
-        acc = wgrad_exact(a.xs + (size_t)g * a.xs_gstride + (size_t)(c >> 3) * a.gr.slots * 8 + (c & 7),
-                          a.dz + (size_t)g * a.dz_gstride + (size_t)(oi >> 3) * a.gr.slots * 8 + (oi & 7),
-                          kt * a.gr.HWb + kh * a.gr.Wb + kw, a.gr.D0, a.gr.N, a.gr.P, a.gr.HWb, a.gr.Wb, a.gr.OT, a.gr.OH,
-                          a.gr.OW);
+    if (ocol < 0) return;
+    for (int i = threadIdx.x / ncol; i < 32; i += 256 / ncol) {
+        const int of = s_f[i], oi = i0 + i;
+        if (of < 0) continue;
+        float acc = 0.0f;
+        for (int z = 0; z < parts; ++z) acc += s_v[z * ncol + oe][i];
+        if (acc != acc) {
+            const int c = a.chan_kind ? (j0 + oe) / a.taps : ocol / a.taps, tap = ocol % a.taps;
+            const int kw = tap % a.gr.KW, kh = (tap / a.gr.KW) % a.gr.KH, kt = tap / (a.gr.KW * a.gr.KH);
+            acc = wgrad_exact(a.xs + (size_t)g * a.xs_gstride + (size_t)(c >> 3) * a.gr.slots * 8 + (c & 7),
+                              a.dz + (size_t)g * a.dz_gstride + (size_t)(oi >> 3) * a.gr.slots * 8 + (oi & 7),
+                              kt * a.gr.HWb + kh * a.gr.Wb + kw, a.gr.D0, a.gr.N, a.gr.P, a.gr.HWb, a.gr.Wb, a.gr.OT, a.gr.OH,
+                              a.gr.OW);
+        }
+        a.dW[(long long)of * a.K + ocol] = acc;
     }
-    a.dW[(long long)of * a.K + ocol] = acc;
 }
 
 struct DzArgs {
@@ -1106,12 +1114,22 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         if (st != SADMM_OK) return st;
     }
     if (dW) {
-        if (launch_pdl(k_grid_wreduce,
-                       dim3((unsigned)((plan->n_cols + kWrCols - 1) / kWrCols), (unsigned)((plan->n_pad + 31) / 32),
-                            (unsigned)g.groups + (db ? 1u : 0u)),
-                       dim3(256), 0, s, r, dd) != cudaSuccess)
-            return SADMM_ECUDA;
-        }
+        // As many range lanes as give each four ranges, or more while there are fewer
+        // than two blocks an SM (idle lanes cost nothing then: with one range and lanes
+        // for it alone, 2 images of 8x8 with 16 channels took 14.1 us, not 11.7).
+        const long long rows = (plan->n_pad + 31) / 32 * g.groups;
+        auto xblocks = [&](int lanes) { return (plan->n_cols * lanes + 32 * kWrCols - 1) / (32 * kWrCols); };
+        int lanes = 1;
+        while (lanes < 32 && (lanes * 4 < b.ws.Z || xblocks(lanes) * rows < 2 * kGwCtas)) lanes *= 2;
+        const dim3 wgrid((unsigned)xblocks(lanes), (unsigned)((plan->n_pad + 31) / 32), (unsigned)g.groups + (db ? 1u : 0u));
+        const auto kern = lanes == 1   ? k_grid_wreduce<1>
+                          : lanes == 2 ? k_grid_wreduce<2>
+                          : lanes == 4 ? k_grid_wreduce<4>
+                          : lanes == 8 ? k_grid_wreduce<8>
+                          : lanes == 16 ? k_grid_wreduce<16>
+                                        : k_grid_wreduce<32>;
+        if (launch_pdl(kern, wgrid, dim3(256), 0, s, r, dd) != cudaSuccess) return SADMM_ECUDA;
+    }
     return cudaGetLastError() == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
 }
 

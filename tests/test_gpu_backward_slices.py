@@ -101,3 +101,32 @@ def test_weight_gradient_of_uneven_groups(kept):
     Wd = (W.double().reshape(s.f, -1) * keep).reshape(W.shape)
     rdx, = torch.autograd.grad(torch.nn.functional.conv2d(xd, Wd, padding=(2, 2), groups=2), xd, dy.double())
     assert ((dx.double() - rdx).norm() / rdx.norm()).item() <= 2.5e-7
+
+
+@pytest.mark.parametrize("n,c,f,hw,kc", [
+    (1, 256, 300, 7, 2301), (1, 128, 300, 7, 1151), (1, 64, 300, 7, 570), (8, 40, 100, 14, 353), (4, 16, 20, 9, 143),
+    (64, 64, 64, 28, 301), (128, 256, 96, 13, 577),
+], ids=lambda v: str(v))
+def test_slice_reduction_by_ranges_and_blocks(n, c, f, hw, kc):
+    """The reduction's range lanes follow the ranges (one range of a wide layer to 47 of a
+    narrow one) and its blocks; columns and filters that are no multiple of a block's."""
+    from paper_1807_11091_gb300 import sadmm
+    s = ConvShape(n=n, c=c, h=hw, w=hw, f=f, kh=3, kw=3, ph=1, pw=1)
+    dev = torch.device("cuda", 0)
+    g = torch.Generator().manual_seed(14)
+    W = torch.randn(s.w_shape(), generator=g).to(torch.bfloat16).to(dev)
+    x = torch.relu(torch.randn(s.x_shape(), generator=g)).to(torch.bfloat16).to(dev)
+    dy = torch.randn(s.y_shape(), generator=g).to(torch.bfloat16).to(dev)
+    rows, cols = np.sort(np.random.default_rng(1).permutation(f)[:f - 3]), np.sort(np.random.default_rng(2).permutation(s.k)[:kc])
+    fi, ci = (torch.as_tensor(a.astype(np.int32), device=dev) for a in (rows, cols))
+    pc = sadmm.PrunedConv(s.desc16(), W, fi, wl.COL_SHAPE, ci, f - 3, kc)
+    dW, db, _ = pc.backward(x, dy, relu=False)
+    assert sadmm.device_status() == 0
+    keep = torch.zeros(f, s.k, dtype=torch.float64, device=dev)
+    keep[fi.long()[:, None], ci.long()[None, :]] = 1.0
+    ref = _dw64(s, x, dy) * keep
+    dW = dW.double().reshape(f, -1)
+    assert ((dW - ref).norm() / ref.norm()).item() <= 1.8e-7
+    assert not dW[keep == 0].any()
+    rdb = dy.double().sum((0, 2, 3)) * (keep.sum(1) > 0)
+    assert (db.double() - rdb).abs().max().item() <= 1e-5 * rdb.abs().max().item()
