@@ -527,10 +527,12 @@ sadmm_status sadmm_project_groups_noalloc(const sadmm_conv_desc* d, const void* 
                                           void* stream);
 
 /* Device bytes of scratch for sadmm_conv_bwd's default path.  A stride-1 layer
- * whose pads are below its kernel extents runs whole on a zero-padded pixel grid
+ * whose pads are below its kernel extents runs on a zero-padded pixel grid
  * (copies of x and dZ, a partial dW per pixel range); any other layer takes its
  * output pixels in chunks of at most 32768 (sized so a chunk's gathered bf16
- * operands and fp32 products stay in L2).  0 on a bad plan. */
+ * operands and fp32 products stay in L2).  The grid takes the whole batch, or
+ * equal shares of its images in turn, so that this is never more than 256 MiB
+ * and what chunks of 32768 pixels take, whichever is more.  0 on a bad plan. */
 size_t sadmm_conv_bwd_workspace_size(const sadmm_plan* plan);
 
 /* Device bytes of scratch for chunks of `chunk_pixels` output pixels (rounded
@@ -568,7 +570,7 @@ size_t sadmm_conv_bwd_workspace_size_chunk(const sadmm_plan* plan, long long chu
  *          dx fp32 [N][C][T][H][W] or NULL.  Every element of each is written.
  *   workspace  ws_bytes of device scratch, 1024-byte aligned: at least
  *          sadmm_conv_bwd_workspace_size_chunk(plan, 256) (else SADMM_EINVAL);
- *          sadmm_conv_bwd_workspace_size(plan) gives the largest chunks.
+ *          sadmm_conv_bwd_workspace_size(plan) gives the default path.
  */
 sadmm_status sadmm_conv_bwd(const sadmm_plan* plan, const void* x, const void* dy, const void* y, int ydt,
                             int relu, float* dW, float* db, float* dx, void* workspace, size_t ws_bytes,

@@ -379,10 +379,23 @@ int pick_bn(long long n)
 
 }  // namespace
 
+// The most workspace the grid path takes: what the chunked path takes by default, or
+// kGridBwdCap.  Its copies of x and dZ grow with the batch; a layer that needs more
+// takes its images in several passes, which cost a ramp of four launches each: 64
+// channels at 224x224 and batch 64 1178 us whole in 908 MB, 1257 in four passes of 256
+// MiB, 1345 of 128, 1402 of 64; 128 channels at 112x112 and batch 128 1421, 1488, 1624
+// and 1624.
+constexpr size_t kGridBwdCap = size_t(256) << 20;
+
+static size_t grid_cap(const sadmm_plan* plan, const Geometry& g)
+{
+    return std::max(kGridBwdCap, layout(geometry(plan, g, kBwdMaxChunk)).total);
+}
+
 size_t bwd_workspace_bytes(const sadmm_plan* plan, const Geometry& g, long long chunk)
 {
     if (chunk <= 0) {
-        const size_t grid = grid_bwd_bytes(plan, g);
+        const size_t grid = grid_bwd_bytes(plan, g, grid_cap(plan, g));
         if (grid > 0) return std::max(grid, layout(geometry(plan, g, 256)).total);
     }
     return layout(geometry(plan, g, chunk > 0 ? chunk : kBwdMaxChunk)).total;
@@ -409,8 +422,8 @@ sadmm_status launch_conv_bwd(const sadmm_plan* plan, const Geometry& g, const vo
                              cudaStream_t s)
 {
     if (g.m >= (1ll << 31)) return SADMM_EUNSUPPORTED;  // pixel indices decode in 32 bits
-    const size_t grid = grid_bwd_bytes(plan, g);
-    if (grid > 0 && grid <= ws_bytes) return launch_grid_bwd(plan, g, x, dy, y, ydt, relu, dW, db, dx, ws, s);
+    const size_t cap = grid_cap(plan, g), grid = grid_bwd_bytes(plan, g, cap);
+    if (grid > 0 && grid <= ws_bytes) return launch_grid_bwd(plan, g, cap, x, dy, y, ydt, relu, dW, db, dx, ws, s);
     const long long chunk = bwd_chunk_for(plan, g, ws_bytes);
     if (chunk <= 0) return SADMM_EINVAL;
     BwdGeo b = geometry(plan, g, chunk);

@@ -506,6 +506,7 @@ struct DbArgs {
     const int* zeromap;
     const int* counts;
     int nparts, groups, n_pad, Fg;
+    int more;  // 1: added to db, which an earlier pass over other images wrote
     float* db;
 };
 
@@ -520,9 +521,9 @@ SADMM_DEV void db_blocks(const DbArgs& a, int b, int nb)
         float s = 0.0f;
         for (int k = lane; k < a.nparts; k += 32) s += __ldg(a.part + (size_t)r * a.nparts + k);
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) a.db[f] = s;
+        if (lane == 0) a.db[f] = a.more ? a.db[f] + s : s;
     }
-    for (int z = b * 256 + threadIdx.x; z < a.groups * a.Fg; z += nb * 256) {
+    for (int z = b * 256 + threadIdx.x; !a.more && z < a.groups * a.Fg; z += nb * 256) {
         const int g = z / a.Fg;
         if (z - g * a.Fg < __ldg(a.counts + 2 * g + 1)) a.db[__ldg(a.zeromap + z)] = 0.0f;
     }
@@ -547,6 +548,7 @@ struct WrArgs {
     long long xs_gstride, dz_gstride;
     float* dW;
     int n_pad, n_cols, taps, chan_kind;
+    int more;  // 1: added to dW, which an earlier pass over other images wrote
     long long K;
 };
 
@@ -658,7 +660,8 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbAr
                               kt * a.gr.HWb + kh * a.gr.Wb + kw, a.gr.D0, a.gr.N, a.gr.P, a.gr.HWb, a.gr.Wb, a.gr.OT, a.gr.OH,
                               a.gr.OW);
         }
-        a.dW[(long long)of * a.K + ocol] = acc;
+        float* dst = a.dW + (long long)of * a.K + ocol;
+        *dst = a.more ? *dst + acc : acc;
     }
 }
 
@@ -887,6 +890,7 @@ __global__ void __launch_bounds__(256) k_grid_front(const __grid_constant__ Fron
 }
 
 struct GridBwd {
+    int images;   // of a pass
     Grid gr;
     GridConvShape cs;
     WgradShape ws;
@@ -897,9 +901,11 @@ struct GridBwd {
     size_t off_xs, off_dz, off_wd, off_maps, off_slices, off_part, total;
 };
 
-bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, GridBwd* out)
+// One pass over the images of g.
+bool grid_bwd_pass(const sadmm_plan* plan, const Geometry& g, GridBwd* out)
 {
     GridBwd b;
+    b.images = (int)g.n;
     if (plan->n_cols < 1 || plan->n_filt < 1 || g.taps > 256) return false;
     if (!grid_of(g, &b.gr)) return false;
     b.nck = plan->colkind == SADMM_COL_CHANNEL ? plan->n_colgroups : (int)g.cg;
@@ -931,19 +937,37 @@ bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, GridBwd* out)
     return true;
 }
 
-}  // namespace
-
-size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g)
+// The layer in as few passes over equal shares of its images as keep the workspace
+// within `cap` bytes; false when one image does not.
+bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, size_t cap, GridBwd* out)
 {
-    GridBwd b;
-    return grid_bwd_shape(plan, g, &b) ? b.total : 0;
+    Geometry p = g;
+    for (long long passes = 1;;) {
+        p.n = (g.n + passes - 1) / passes;
+        p.m = p.n * p.plane;
+        const bool fits = grid_bwd_pass(plan, p, out);
+        if (fits && out->total <= cap) return true;
+        if (p.n == 1) return false;
+        // the workspace is about proportional to the images; at least one image fewer
+        const long long next = fits ? (long long)((double)passes * out->total / cap) : 2 * passes;
+        passes = std::min(g.n, std::max(next, (g.n + p.n - 2) / (p.n - 1)));
+    }
 }
 
-sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const void* x, const void* dy, const void* y,
-                             int ydt, int relu, float* dW, float* db, float* dx, void* ws, cudaStream_t s)
+}  // namespace
+
+size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g, size_t cap)
 {
     GridBwd b;
-    if (!grid_bwd_shape(plan, g, &b)) return SADMM_EINVAL;
+    return grid_bwd_shape(plan, g, cap, &b) ? b.total : 0;
+}
+
+// The images of g, a pass's or the last fewer, in b's workspace; `more`: dW and db add
+// to what the passes before left.
+static sadmm_status launch_pass(const sadmm_plan* plan, const Geometry& g, const GridBwd& b, const void* x, const void* dy,
+                                const void* y, int ydt, int relu, float* dW, float* db, float* dx, void* ws, bool more,
+                                cudaStream_t s)
+{
     const char* base = static_cast<const char*>(plan->dev);
     char* w = static_cast<char*>(ws);
     const int* rowmap = reinterpret_cast<const int*>(base + plan->off_rowmap);
@@ -978,7 +1002,7 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         p.nck = b.nck;
         p.chan_kind = chan_kind;
         p.ncpad = b.cs.npad;
-        p.rows = dx ? (int)g.groups * b.cs.npad : 0;
+        p.rows = dx && !more ? (int)g.groups * b.cs.npad : 0;  // (they stay for the passes after the first)
         p.bn = b.cs.bn;
         p.cb = b.cs.cb;
         p.ksteps = b.cs.ksteps;
@@ -987,8 +1011,8 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         p.zmap = zmap;
         p.counts2 = counts2;
         p.zero = dW;
-        p.zero_n = dW ? g.f * g.k : 0;
-        p.zblocks = dW ? (int)std::min<long long>(256, (p.zero_n + 2047) / 2048) : 0;
+        p.zero_n = dW && !more ? g.f * g.k : 0;
+        p.zblocks = p.zero_n > 0 ? (int)std::min<long long>(256, (p.zero_n + 2047) / 2048) : 0;
         fa.np = p.rows * kPrepSplit + p.zblocks;
     }
     DzArgs& d = fa.dz;
@@ -1029,6 +1053,7 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
     dd.n_pad = plan->n_pad;
     dd.Fg = (int)g.fg;
     dd.db = db;
+    dd.more = more ? 1 : 0;
     if (db && !dW &&
         launch_pdl(k_grid_db, dim3((unsigned)((g.groups * plan->n_pad + 7) / 8)), dim3(256), 0, s, dd) != cudaSuccess)
         return SADMM_ECUDA;
@@ -1079,6 +1104,7 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         r.n_cols = plan->n_cols;
         r.taps = (int)g.taps;
         r.chan_kind = chan_kind;
+        r.more = more ? 1 : 0;
         r.K = g.k;
     }
     // The input gradient reads what k_grid_front wrote and nothing of k_grid_wgrad's.
@@ -1131,6 +1157,33 @@ sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const vo
         if (launch_pdl(kern, wgrid, dim3(256), 0, s, r, dd) != cudaSuccess) return SADMM_ECUDA;
     }
     return cudaGetLastError() == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
+}
+
+sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, size_t cap, const void* x, const void* dy,
+                             const void* y, int ydt, int relu, float* dW, float* db, float* dx, void* ws, cudaStream_t s)
+{
+    GridBwd b;
+    if (!grid_bwd_shape(plan, g, cap, &b)) return SADMM_EINVAL;
+    Geometry p = g;
+    const long long xn = g.c * g.t * g.h * g.w, yn = g.f * g.plane;  // elements of an image
+    for (long long n0 = 0; n0 < g.n; n0 += b.images) {
+        p.n = std::min<long long>(b.images, g.n - n0);
+        p.m = p.n * p.plane;
+        if (p.n < b.images) {  // the last pass: fewer pixels, and ranges, in the same layout
+            if (!grid_of(p, &b.gr)) return SADMM_EINVAL;
+            b.ws.tiles = (b.gr.L + 127) / 128;
+            b.ws.Z = (b.ws.tiles + b.ws.tps - 1) / b.ws.tps;
+            b.nparts = (b.gr.slots + b.dzslots - 1) / b.dzslots;
+        }
+        const char* yp = static_cast<const char*>(y);
+        const sadmm_status st =
+            launch_pass(plan, p, b, static_cast<const __nv_bfloat16*>(x) + n0 * xn,
+                        static_cast<const __nv_bfloat16*>(dy) + n0 * yn,
+                        yp ? yp + n0 * yn * (ydt == SADMM_BF16 ? 2 : 4) : nullptr, ydt, relu, dW, db,
+                        dx ? dx + n0 * xn : nullptr, ws, n0 > 0, s);
+        if (st != SADMM_OK) return st;
+    }
+    return SADMM_OK;
 }
 
 }  // namespace sadmm

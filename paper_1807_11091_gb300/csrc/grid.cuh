@@ -148,9 +148,11 @@ sadmm_status launch_grid_fwd(const sadmm_plan* plan, const Geometry& g, const vo
                              void* y, int ydt, cudaStream_t s);
 
 // ---- grid backward (bwd_grid.cu) ----
-size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g);  // 0: the layer takes the gathered backward
-sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, const void* x, const void* dy, const void* y,
-                             int ydt, int relu, float* dW, float* db, float* dx, void* ws, cudaStream_t s);
+// The workspace, at most cap bytes: a layer that needs more takes its images in several
+// passes.  0: the layer has no grid, or one image of it needs more.
+size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g, size_t cap);
+sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, size_t cap, const void* x, const void* dy,
+                             const void* y, int ydt, int relu, float* dW, float* db, float* dx, void* ws, cudaStream_t s);
 
 // ------------------------------------------------------------- device side --
 

@@ -613,8 +613,9 @@ class PrunedConv:
     def backward(self, x, dy, y=None, relu=True, want_dw=True, want_db=True, want_dx=True, stream=None,
                  chunk_pixels=0):
         """Runs sadmm_conv_bwd; returns (dW, db, dx) fp32 device tensors (None where not requested).
-        chunk_pixels > 0 sizes the workspace for chunks of that many output pixels
-        (default: chunks of up to 32768 pixels)."""
+        The scratch is sadmm_conv_bwd_workspace_size's; chunk_pixels > 0 sizes it for
+        chunks of that many output pixels instead (the pixel grid still runs where
+        that holds it)."""
         torch = _torch()
         n, c, t, h, w, f, g, kt, kh, kw = self.desc16[:10]
         dev = dy.device

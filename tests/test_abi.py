@@ -270,3 +270,17 @@ def test_pack_batch_rejects_bad_items_on_host():
     assert sadmm.sadmm_pack_batch([item(pl) for pl in plans], 0, None) == sadmm.SADMM_EINVAL
     # nothing was bound: every rejected call enqueues nothing
     assert not p.dev and not q.dev
+
+
+@pytest.mark.parametrize("n,c,hw,f,k,cf", [(128, 128, 112, 128, 3, 1.0), (128, 128, 112, 128, 3, 0.1), (128, 512, 56, 512, 3, 0.1),
+                                           (64, 64, 224, 64, 3, 0.5), (128, 96, 27, 256, 5, 0.5), (256, 64, 56, 256, 1, 1.0),
+                                           (1, 512, 224, 512, 3, 1.0), (1024, 16, 8, 16, 3, 1.0)])
+def test_backward_scratch_is_bounded(n, c, hw, f, k, cf):
+    """The default scratch of a backward does not grow with the batch past 256 MiB, or past
+    what 32768-pixel chunks take."""
+    s = wl.ConvShape(n=n, c=c, h=hw, w=hw, f=f, kh=k, kw=k, ph=k // 2, pw=k // 2)
+    kc = wl.retained(cf, s.k)
+    st, p = sadmm.sadmm_plan_init(sadmm.make_desc(s.desc16()), f, wl.COL_SHAPE, kc)
+    assert st == 0
+    chunks = sadmm.sadmm_conv_bwd_workspace_size_chunk(p, 32768)
+    assert 0 < sadmm.sadmm_conv_bwd_workspace_size(p) <= max(chunks, 256 << 20)
