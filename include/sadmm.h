@@ -528,7 +528,8 @@ sadmm_status sadmm_project_groups_noalloc(const sadmm_conv_desc* d, const void* 
 
 /* Device bytes of scratch for sadmm_conv_bwd's default path.  A stride-1 layer
  * whose pads are below its kernel extents runs on a zero-padded pixel grid
- * (copies of x and dZ, a partial dW per pixel range); any other layer takes its
+ * (copies of x and dZ, a partial dW per pixel range) unless few of many
+ * channels' columns are kept; any other layer takes its
  * output pixels in chunks of at most 32768 (sized so a chunk's gathered bf16
  * operands and fp32 products stay in L2).  The grid takes the whole batch, or
  * equal shares of its images in turn, so that this is never more than 256 MiB

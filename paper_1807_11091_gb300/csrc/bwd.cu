@@ -387,15 +387,42 @@ int pick_bn(long long n)
 // and 1624.
 constexpr size_t kGridBwdCap = size_t(256) << 20;
 
-static size_t grid_cap(const sadmm_plan* plan, const Geometry& g)
+// The chunked path's estimated time: launches a layer and a chunk of a conv group, and
+// what its passes move per gathered pixel (dZ twice, im2col and col2im a packed column),
+// its two GEMMs' share that the passes do not hide, dx zeroed and dW's partial sums.
+// Fitted to 96 layers (those that take less than three times the grid's time): 0.8 to
+// 1.2 of what they measured.
+static long long chunked_ns(const BwdGeo& b)
 {
-    return std::max(kGridBwdCap, layout(geometry(plan, g, kBwdMaxChunk)).total);
+    const long long chunks = (b.M + b.mc - 1) / b.mc * b.groups, pix = chunks * b.mc;
+    const long long dwn = (long long)b.F * b.Cg * b.taps + (long long)b.groups * b.fr * b.k_pad;
+    return 26000 + 22000 * chunks + (pix * (25ll * (b.fr + b.fk) + 32ll * b.k_pad) + 27 * ((long long)b.N * b.x_chw + dwn)) / 10000 +
+           pix / 64 * (16ll * b.kr * b.fk + 40ll * b.fr * b.k_pad) / 10000000 * 64;
+}
+
+// The grid path where the layer has a grid that is estimated to be no slower, its
+// workspace then (0: the chunked path).  The grid contracts over every tap and channel,
+// the chunked path over the kept columns alone.  Of 207 layers measured both ways (1x1 to
+// 11x11, 3-D, 1 to 32 groups, batch 1 to 128, 2 to 100 % of the columns) the grid is the
+// faster on 187, up to 14 times (AlexNet conv2 at batch 128 841 -> 163 us, conv3 164 ->
+// 55), and the slower where few of many channels' columns are kept: 1024 -> 1024 3x3 at
+// 14x14 and batch 32 with 2 % of them 296 us against 158, 512 -> 512 at 28x28 and batch
+// 64 473 against 335.  The rule takes the slower path on four, at most 18 % the
+// slower, and on one of 120 drawn layers, by 9 %.
+static size_t grid_bytes(const sadmm_plan* plan, const Geometry& g, size_t* cap)
+{
+    const BwdGeo b = geometry(plan, g, kBwdMaxChunk);
+    *cap = std::max(kGridBwdCap, layout(b).total);
+    long long ns = 0;
+    const size_t bytes = grid_bwd_bytes(plan, g, *cap, &ns);
+    return bytes > 0 && chunked_ns(b) + 8000 < ns ? 0 : bytes;
 }
 
 size_t bwd_workspace_bytes(const sadmm_plan* plan, const Geometry& g, long long chunk)
 {
     if (chunk <= 0) {
-        const size_t grid = grid_bwd_bytes(plan, g, grid_cap(plan, g));
+        size_t cap;
+        const size_t grid = grid_bytes(plan, g, &cap);
         if (grid > 0) return std::max(grid, layout(geometry(plan, g, 256)).total);
     }
     return layout(geometry(plan, g, chunk > 0 ? chunk : kBwdMaxChunk)).total;
@@ -413,16 +440,14 @@ long long bwd_chunk_for(const sadmm_plan* plan, const Geometry& g, size_t ws_byt
     return 0;
 }
 
-// The grid path wherever the layer has a grid and the workspace holds it: over
-// 20 drawn stride-1 layers (1x1 to 5x5, 3-D, batch 1 to 128, densities 0.1 to 1)
-// it took 0.26 to 0.84 of the gathered path's time, AlexNet conv2 at batch 128
-// 841 -> 175 us, conv3 164 -> 50 us, and none took longer.
+// (The grid path where grid_bytes chooses it and the workspace holds it.)
 sadmm_status launch_conv_bwd(const sadmm_plan* plan, const Geometry& g, const void* x, const void* dy, const void* y,
                              int ydt, int relu, float* dW, float* db, float* dx, void* ws, size_t ws_bytes,
                              cudaStream_t s)
 {
     if (g.m >= (1ll << 31)) return SADMM_EUNSUPPORTED;  // pixel indices decode in 32 bits
-    const size_t cap = grid_cap(plan, g), grid = grid_bwd_bytes(plan, g, cap);
+    size_t cap;
+    const size_t grid = grid_bytes(plan, g, &cap);
     if (grid > 0 && grid <= ws_bytes) return launch_grid_bwd(plan, g, cap, x, dy, y, ydt, relu, dW, db, dx, ws, s);
     const long long chunk = bwd_chunk_for(plan, g, ws_bytes);
     if (chunk <= 0) return SADMM_EINVAL;

@@ -72,6 +72,7 @@ struct WgradShape {
     int tiles, tps, Z;  // 128-pixel tiles, tiles per range, ranges
     int span;         // slots that an item's taps reach beyond its pixels, at most
     long long slice;  // floats of a pixel range's slice
+    long long cycles;  // estimated time
 };
 
 // How the stages lie in shared memory for items of `nr` filters: slabs of one
@@ -173,7 +174,7 @@ bool wgrad_shape(const Grid& gr, int nck, int n_pad, int likely, int groups, Wgr
                 const long long item = w.tps * tile, rounds = (types * w.Z + kGwCtas - 1) / kGwCtas;
                 const long long cost = rounds * std::max(item, st) + st + types * w.Z * w.rows * cols * 4 / (kGwCtas * 16);
                 if (best < 0 || cost < best) {
-                    best = cost;
+                    best = w.cycles = cost;
                     *out = w;
                 }
             }
@@ -958,10 +959,16 @@ bool grid_bwd_shape(const sadmm_plan* plan, const Geometry& g, size_t cap, GridB
 
 }  // namespace
 
-size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g, size_t cap)
+// The estimate, fitted with the chunked path's (bwd.cu): launches, the two contractions'
+// cycles at 1.95 GHz, and the copies; 0.8 to 1.15 of what 96 layers measured that take
+// more than a third of the chunked path's time, less of the others.
+size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g, size_t cap, long long* ns)
 {
     GridBwd b;
-    return grid_bwd_shape(plan, g, cap, &b) ? b.total : 0;
+    if (!grid_bwd_shape(plan, g, cap, &b)) return 0;
+    const long long copies = 16ll * g.groups * b.gr.slots * (b.ws.nch + b.dchunks);
+    *ns = (g.n + b.images - 1) / b.images * (16000 + (b.ws.cycles + b.cs.cycles * 5 / 4) * 100 / 195 + copies / 2000);
+    return b.total;
 }
 
 // The images of g, a pass's or the last fewer, in b's workspace; `more`: dW and db add

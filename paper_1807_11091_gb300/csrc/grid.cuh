@@ -149,8 +149,9 @@ sadmm_status launch_grid_fwd(const sadmm_plan* plan, const Geometry& g, const vo
 
 // ---- grid backward (bwd_grid.cu) ----
 // The workspace, at most cap bytes: a layer that needs more takes its images in several
-// passes.  0: the layer has no grid, or one image of it needs more.
-size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g, size_t cap);
+// passes.  0: the layer has no grid, or one image of it needs more.  *ns: its estimated
+// time.
+size_t grid_bwd_bytes(const sadmm_plan* plan, const Geometry& g, size_t cap, long long* ns);
 sadmm_status launch_grid_bwd(const sadmm_plan* plan, const Geometry& g, size_t cap, const void* x, const void* dy,
                              const void* y, int ydt, int relu, float* dW, float* db, float* dx, void* ws, cudaStream_t s);
 

@@ -284,3 +284,17 @@ def test_backward_scratch_is_bounded(n, c, hw, f, k, cf):
     assert st == 0
     chunks = sadmm.sadmm_conv_bwd_workspace_size_chunk(p, 32768)
     assert 0 < sadmm.sadmm_conv_bwd_workspace_size(p) <= max(chunks, 256 << 20)
+
+
+@pytest.mark.parametrize("n,c,hw,f,k,cf,grid", [
+    (32, 1024, 14, 1024, 3, 0.02, False), (64, 512, 28, 512, 3, 0.02, False), (8, 512, 14, 512, 5, 0.05, False),
+    (32, 1024, 14, 1024, 3, 1.0, True), (64, 512, 28, 512, 3, 0.5, True), (128, 96, 27, 256, 5, 0.1, True),
+    (2, 92, 7, 178, 1, 0.3, True),  # a call of four launches, not of a dozen
+])
+def test_backward_takes_the_grid_where_it_is_faster(n, c, hw, f, k, cf, grid):
+    """The grid contracts over every tap and channel: where few of many channels' columns are
+    kept the chunked path is the default, and with it its workspace."""
+    s = wl.ConvShape(n=n, c=c, h=hw, w=hw, f=f, kh=k, kw=k, ph=k // 2, pw=k // 2)
+    st, p = sadmm.sadmm_plan_init(sadmm.make_desc(s.desc16()), f, wl.COL_SHAPE, wl.retained(cf, s.k))
+    assert st == 0
+    assert (sadmm.sadmm_conv_bwd_workspace_size(p) != sadmm.sadmm_conv_bwd_workspace_size_chunk(p, 32768)) == grid
