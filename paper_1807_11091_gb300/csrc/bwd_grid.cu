@@ -487,22 +487,6 @@ __global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_const
     }
 }
 
-// The weight gradient of one kept entry over the layer's output pixels alone:
-// what its grid sum is, unless a padded pixel's zero met an infinity or a NaN.
-__device__ __noinline__ float wgrad_exact(const __nv_bfloat16* xc, const __nv_bfloat16* dc, int shift, int D0, int N, int P,
-                                          int HWb, int Wb, int OT, int OH, int OW)
-{
-    float acc = 0.0f;
-    for (int n = 0; n < N; ++n)
-        for (int t = 0; t < OT; ++t)
-            for (int h = 0; h < OH; ++h)
-                for (int w = 0; w < OW; ++w) {
-                    const size_t q = (size_t)n * P + (size_t)t * HWb + h * Wb + w;
-                    acc += __bfloat162float(dc[(q + D0) * 8]) * __bfloat162float(xc[(q + shift) * 8]);
-                }
-    return acc;
-}
-
 struct DbArgs {
     const float* part;  // NULL: no bias gradient
     const int* rowmap;
@@ -555,6 +539,58 @@ struct WrArgs {
     long long K;
 };
 
+// Where the slices of packed row i, K column col (packed column j) of group g lie, in
+// the first range.
+SADMM_DEV size_t wr_slice(const WrArgs& a, int g, int i, int j, int col)
+{
+    const int c = a.chan_kind ? j / a.taps : col / a.taps, tap = col % a.taps;
+    const int kw = tap % a.gr.KW, kh = (tap / a.gr.KW) % a.gr.KH, kt = tap / (a.gr.KW * a.gr.KH);
+    const int mb = (c >> 3) / a.w.blk, mt = kh * a.w.kwg + kw / a.w.rep, ft = i / a.w.nst;
+    const int m = (((kw % a.w.rep) * a.w.blk + ((c >> 3) - mb * a.w.blk)) << 3) + (c & 7);
+    const int type = (((g * a.w.nft + ft) * a.w.mblks + mb) * a.gr.KT + kt) * a.w.tgs + mt / a.w.tpg;
+    return ((size_t)type * a.w.rows + m) * (size_t)(a.w.tpg * a.w.nst) + (mt % a.w.tpg) * a.w.nst + (i - ft * a.w.nst);
+}
+
+// One entry of the weight gradient whose sum came out NaN, by a warp: a range's slice is
+// NaN where a padded pixel's zero met an infinity or a NaN of x, which is no term of the
+// sum, so such a range is added up again over its output pixels alone, until one of its
+// terms is NaN itself.  Every lane returns the sum.
+__device__ __noinline__ float wgrad_exact(const WrArgs& a, int g, int i, int j, int col)
+{
+    const int lane = threadIdx.x & 31;
+    const int c = a.chan_kind ? j / a.taps : col / a.taps, tap = col % a.taps;
+    const int kw = tap % a.gr.KW, kh = (tap / a.gr.KW) % a.gr.KH, kt = tap / (a.gr.KW * a.gr.KH);
+    const int shift = kt * a.gr.HWb + kh * a.gr.Wb + kw;
+    const __nv_bfloat16* xc = a.xs + (size_t)g * a.xs_gstride + (size_t)(c >> 3) * a.gr.slots * 8 + (c & 7);
+    const __nv_bfloat16* dc = a.dz + (size_t)g * a.dz_gstride + (size_t)(i >> 3) * a.gr.slots * 8 + (i & 7);
+    const float* src = a.slices + wr_slice(a, g, i, j, col);
+    float acc = 0.0f;  // of the lane's ranges and pixels
+    for (int z0 = 0; z0 < a.w.Z; z0 += 32) {
+        const float v = z0 + lane < a.w.Z ? __ldcg(src + (size_t)(z0 + lane) * a.w.slice) : 0.0f;
+        uint32_t bad = __ballot_sync(0xffffffffu, v != v);
+        if (v == v) acc += v;
+        for (; bad; bad &= bad - 1) {
+            const int z = z0 + __ffs(bad) - 1;
+            const int end = min(a.w.tiles, (z + 1) * a.w.tps) * 128;
+            float sum = 0.0f;
+            for (int q0 = z * a.w.tps * 128; q0 < end; q0 += 128) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int q = q0 + 32 * k + lane;
+                    int n, t, h, w;
+                    grid_decode(a.gr, q, n, t, h, w);
+                    if (n < a.gr.N && t < a.gr.OT && h < a.gr.OH && w < a.gr.OW)
+                        sum += __bfloat162float(dc[(size_t)(q + a.gr.D0) * 8]) * __bfloat162float(xc[(size_t)(q + shift) * 8]);
+                }
+                if (__any_sync(0xffffffffu, sum != sum)) return __uint_as_float(0x7fffffffu);
+            }
+            acc += sum;
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return acc;
+}
+
 // dW[f_i][col_j] = sum over the pixel ranges of their slices: LANES threads per two
 // columns of four filters take every LANES-th range, then their sums are added in order
 // (deterministic).  Block (bx, by, g): 64 / LANES packed columns, packed rows
@@ -566,7 +602,7 @@ struct WrArgs {
 constexpr int kWrCols = 2;
 
 template <int LANES>
-__global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbArgs d)
+__global__ void __launch_bounds__(256) k_grid_wreduce(const __grid_constant__ WrArgs a, const DbArgs d)
 {
     __shared__ float s_v[64][33];  // [part of the ranges][column][filter]
     __shared__ int s_f[32];        // the rows' filters
@@ -586,7 +622,7 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbAr
     }
     const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
     const int rl = ty & (LANES - 1), jt = ty / LANES * kWrCols;  // range lane, first column in the block
-    const int iq = i0 + tx * 4, ftq = iq / a.w.nst;  // (a tile's filters are a multiple of 16)
+    const int iq = i0 + tx * 4;  // (a filter tile is a multiple of 16)
     const float* src[kWrCols];
 #pragma unroll
     for (int e = 0; e < kWrCols; ++e) {
@@ -594,13 +630,7 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbAr
         const int col = j < a.n_cols ? __ldg(a.colidx + j) : -1;
         src[e] = a.slices;  // (nothing reads what this adds up)
         if (col < 0 || iq >= cnt) continue;
-        const int c = a.chan_kind ? j / a.taps : col / a.taps, tap = col % a.taps;
-        const int kw = tap % a.gr.KW, kh = (tap / a.gr.KW) % a.gr.KH, kt = tap / (a.gr.KW * a.gr.KH);
-        const int mb = (c >> 3) / a.w.blk, mt = kh * a.w.kwg + kw / a.w.rep;
-        const int m = (((kw % a.w.rep) * a.w.blk + ((c >> 3) - mb * a.w.blk)) << 3) + (c & 7);
-        const int type = (((g * a.w.nft + ftq) * a.w.mblks + mb) * a.gr.KT + kt) * a.w.tgs + mt / a.w.tpg;
-        src[e] = a.slices + ((size_t)type * a.w.rows + m) * (size_t)(a.w.tpg * a.w.nst) + (mt % a.w.tpg) * a.w.nst +
-                 (iq - ftq * a.w.nst);
+        src[e] = a.slices + wr_slice(a, g, iq, j, col);
     }
     // the column of the entries this thread writes (ncol divides the block), their filters
     const int oe = threadIdx.x & (ncol - 1);
@@ -649,20 +679,18 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const WrArgs a, const DbAr
             if ((rl & 3) == 0) s_v[(rl >> 2) * ncol + jt + e][tx * 4 + q] = v[e][q];
         }
     __syncthreads();
-    if (ocol < 0) return;
-    for (int i = threadIdx.x / ncol; i < 32; i += 256 / ncol) {
-        const int of = s_f[i], oi = i0 + i;
-        if (of < 0) continue;
+    for (int i = threadIdx.x / ncol; i < 32; i += 256 / ncol) {  // (a warp's lanes alike)
+        const int of = ocol >= 0 ? s_f[i] : -1;
         float acc = 0.0f;
-        for (int z = 0; z < parts; ++z) acc += s_v[z * ncol + oe][i];
-        if (acc != acc) {
-            const int c = a.chan_kind ? (j0 + oe) / a.taps : ocol / a.taps, tap = ocol % a.taps;
-            const int kw = tap % a.gr.KW, kh = (tap / a.gr.KW) % a.gr.KH, kt = tap / (a.gr.KW * a.gr.KH);
-            acc = wgrad_exact(a.xs + (size_t)g * a.xs_gstride + (size_t)(c >> 3) * a.gr.slots * 8 + (c & 7),
-                              a.dz + (size_t)g * a.dz_gstride + (size_t)(oi >> 3) * a.gr.slots * 8 + (oi & 7),
-                              kt * a.gr.HWb + kh * a.gr.Wb + kw, a.gr.D0, a.gr.N, a.gr.P, a.gr.HWb, a.gr.Wb, a.gr.OT, a.gr.OH,
-                              a.gr.OW);
+        if (of >= 0)
+            for (int z = 0; z < parts; ++z) acc += s_v[z * ncol + oe][i];
+        for (uint32_t bad = __ballot_sync(0xffffffffu, acc != acc); bad; bad &= bad - 1) {
+            const int l = __ffs(bad) - 1;
+            const float e = wgrad_exact(a, g, __shfl_sync(0xffffffffu, i0 + i, l), __shfl_sync(0xffffffffu, j0 + oe, l),
+                                        __shfl_sync(0xffffffffu, ocol, l));
+            if ((int)(threadIdx.x & 31) == l) acc = e;
         }
+        if (of < 0) continue;
         float* dst = a.dW + (long long)of * a.K + ocol;
         *dst = a.more ? *dst + acc : acc;
     }

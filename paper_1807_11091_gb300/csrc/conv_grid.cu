@@ -77,35 +77,105 @@ struct GcArgs {
     int relu;
 };
 
-// The sum of one output (column `col` of column tile nt of group g, whose weights
-// lie bnr rows apart; grid pixel q) over the kept K columns only, as the gathered
-// path forms it (pruned entries are -0.0).  Where the source is the output
-// gradient, a tap that reads past the output's edge is no term of the sum; in the
-// forward a padded pixel is one, as it is in the gathered path.
-__device__ __noinline__ float grid_exact(const GcArgs& a, int g, int nt, int bnr, int col, int q, int kch)
+// ---- outputs that come out NaN, summed again ----
+// Their K columns lie in octets u: 8 channels of a tap, in the weights' order.
+SADMM_DEV int gc_octets(const GcArgs& a, int kch)
 {
-    const unsigned short* w =
-        reinterpret_cast<const unsigned short*>(a.wd) + (size_t)(g * a.ntiles + nt) * a.ksteps * a.bn * 16 + col * 8;
-    const __nv_bfloat16* src = a.src + (size_t)g * a.gstride;
-    float acc = 0.0f;
+    return (kch + a.cb - 1) / a.cb * a.gr.KT * a.gr.KH * a.gr.KW * (a.cb / 8);
+}
+
+// The kept terms (pruned entries are -0.0) of octet u of one output of grid pixel q:
+// column `col` of the tile whose weights lie at wt, bnr rows apart.  Where the source is
+// the output gradient, a tap that reads past the output's edge is no term; in the forward
+// a padded pixel is one, as it is in the gathered path.
+SADMM_DEV float gc_terms(const GcArgs& a, const uint4* wt, const uint4* src, int bnr, int col, int u, int q, int kch)
+{
+    const int per = a.cb / 8, t = u / per, taps = a.gr.KT * a.gr.KH * a.gr.KW;
+    const int blk = t / taps, tap = t - blk * taps, kw = tap % a.gr.KW, r = tap / a.gr.KW;
+    const int c = blk * a.cb + (u - t * per) * 8;
+    const int slot = q + r / a.gr.KH * a.gr.HWb + r % a.gr.KH * a.gr.Wb + kw;
+    if (c >= kch) return 0.0f;
+    const uint4 w4 = __ldg(wt + (size_t)u * bnr + col), x4 = src[(size_t)(c >> 3) * a.gr.slots + slot];
+    const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w}, x[4] = {x4.x, x4.y, x4.z, x4.w};
+    float sum = 0.0f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const uint32_t wb = (e & 1) ? w[e >> 1] & 0xffff0000u : w[e >> 1] << 16;
+        const uint32_t xb = (e & 1) ? x[e >> 1] & 0xffff0000u : x[e >> 1] << 16;
+        if (wb != 0x80000000u && c + e < kch) sum += __uint_as_float(wb) * __uint_as_float(xb);
+    }
+    if (sum != sum && a.src_dz) {
+        int n = a.gr.N, t0 = 0, y0 = 0, x0 = 0;
+        if (slot >= a.gr.D0) grid_decode(a.gr, slot - a.gr.D0, n, t0, y0, x0);
+        if (n >= a.gr.N || t0 >= a.gr.OT || y0 >= a.gr.OH || x0 >= a.gr.OW) return 0.0f;
+    }
+    return sum;
+}
+
+// The first octets of grid pixel q, of four taps at most, whose source holds an infinity
+// or a NaN (-1: no more): where a NaN of any of its outputs that is a kept term's shows
+// first.  (One a tap: what is pruned is pruned for every filter.)
+__device__ __noinline__ int4 grid_scan(const GcArgs& a, const uint4* src, int q, int kch)
+{
+    int4 f = make_int4(-1, -1, -1, -1);
+    int u = 0;
     for (int c0 = 0; c0 < kch; c0 += a.cb)
         for (int kt = 0; kt < a.gr.KT; ++kt)
             for (int kh = 0; kh < a.gr.KH; ++kh)
-                for (int kw = 0; kw < a.gr.KW; ++kw, w += (size_t)a.cb * bnr) {
-                    const int slot = q + kt * a.gr.HWb + kh * a.gr.Wb + kw;
-                    if (a.src_dz) {
-                        if (slot < a.gr.D0) continue;
-                        int n, t, y, x;
-                        grid_decode(a.gr, slot - a.gr.D0, n, t, y, x);
-                        if (n >= a.gr.N || t >= a.gr.OT || y >= a.gr.OH || x >= a.gr.OW) continue;
-                    }
-                    for (int c = c0; c < min(c0 + a.cb, kch); ++c) {
-                        const unsigned short b = __ldg(w + (size_t)((c - c0) >> 3) * bnr * 8 + (c & 7));
-                        if (b == 0x8000u) continue;
-                        acc += __uint_as_float((uint32_t)b << 16) *
-                               __bfloat162float(src[((size_t)(c >> 3) * a.gr.slots + slot) * 8 + (c & 7)]);
+                for (int kw = 0; kw < a.gr.KW; ++kw) {
+                    const uint4* p = src + (size_t)(c0 >> 3) * a.gr.slots + (q + kt * a.gr.HWb + kh * a.gr.Wb + kw);
+                    bool found = false;
+                    for (int c8 = 0; c8 < a.cb / 8; ++c8, ++u, p += a.gr.slots) {
+                        if (found) continue;
+                        const uint4 x = *p;
+                        bool bad = false;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const uint32_t v = e == 0 ? x.x : e == 1 ? x.y : e == 2 ? x.z : x.w;
+                            bad |= (v & 0x7f80u) == 0x7f80u || (v & 0x7f800000u) == 0x7f800000u;
+                        }
+                        if (!bad) continue;
+                        found = true;
+                        if (f.x < 0) f.x = u;
+                        else if (f.y < 0) f.y = u;
+                        else if (f.z < 0) f.z = u;
+                        else {
+                            f.w = u;
+                            return f;
+                        }
                     }
                 }
+    return f;
+}
+
+// Whether a kept term of the octets f is NaN: the output is then.
+__device__ __noinline__ bool grid_nan_at(const GcArgs& a, const uint4* wt, const uint4* src, int bnr, int col, int q, int kch,
+                                         int4 f)
+{
+    bool nan = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int u = k == 0 ? f.x : k == 1 ? f.y : k == 2 ? f.z : f.w;
+        if (nan || u < 0) continue;
+        const float t = gc_terms(a, wt, src, bnr, col, u, q, kch);
+        nan = t != t;
+    }
+    return nan;
+}
+
+// The sum of one output over the kept K columns only, as the gathered path forms it, by a
+// warp; every lane returns it.  NaN as soon as a term is.
+__device__ __noinline__ float grid_exact(const GcArgs& a, const uint4* wt, const uint4* src, int bnr, int col, int q, int kch)
+{
+    const int units = gc_octets(a, kch), lane = threadIdx.x & 31;
+    float acc = 0.0f;
+    for (int u0 = 0; u0 < units; u0 += 64) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (u0 + 32 * k + lane < units) acc += gc_terms(a, wt, src, bnr, col, u0 + 32 * k + lane, q, kch);
+        if (__any_sync(0xffffffffu, acc != acc)) return __uint_as_float(0x7fffffffu);
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     return acc;
 }
 
@@ -524,7 +594,7 @@ __global__ void __launch_bounds__(kGcThreads, 1)
                 if (lane == 0) mbar_arrive(&acc_empty[ab]);
                 if (++ab == a.nbuf) { ab = 0; acc_ph ^= 1u; }
             }
-            uint32_t nan = 0;  // chunks with a NaN
+            uint32_t nan[4] = {0u, 0u, 0u, 0u};  // NaN columns, 16 bits a chunk
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
                 const int c = MT == 2 ? k : 2 * k + h;
@@ -532,22 +602,48 @@ __global__ void __launch_bounds__(kGcThreads, 1)
                     bool bad = false;
 #pragma unroll
                     for (int j = 0; j < kEpiCols; ++j) bad |= v[k][j] != v[k][j];
-                    if (bad) nan |= 1u << k;
+                    if (bad) {
+#pragma unroll
+                        for (int j = 0; j < kEpiCols; ++j)
+                            nan[k >> 1] |= (v[k][j] != v[k][j] ? 1u : 0u) << ((k & 1) * 16 + j);
+                    }
                     store_cols<OUT_BF16>(v[k], c * kEpiCols, cnt, t_off, t_bias, a.relu, yf, yh, yc);
                 }
             }
-            if (nan) {
+            // NaN columns: what a lane finds to be a kept term's stands, the others are
+            // summed again by the warp
+            if (__any_sync(0xffffffffu, (nan[0] | nan[1] | nan[2] | nan[3]) != 0)) {
                 const int kch = a.kcounts ? __ldg(a.kcounts + 2 * g) : a.ncb * a.cb;
-                for (int i = 0; i < nch * kEpiCols; ++i) {
-                    const int c = i / kEpiCols;
-                    if (i >= cnt || (MT == 1 && (c & 1) != h) || !((nan >> (MT == 2 ? c : c >> 1)) & 1u)) continue;
-                    float e = grid_exact(a, g, nt, bnr, i, q, kch) + t_bias[i];
-                    if (a.relu) e = fmaxf(e, 0.0f);
-                    if (!y_ok(yc, t_off[i])) continue;
-                    if (OUT_BF16)
-                        yh[t_off[i]] = __float2bfloat16_rn(e);
-                    else
-                        yf[t_off[i]] = e;
+                const uint4* wt = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(a.wd) +
+                                                                 (size_t)(g * a.ntiles + nt) * btile);
+                const uint4* src = reinterpret_cast<const uint4*>(a.src + (size_t)g * a.gstride);
+                int4 first = make_int4(-1, -1, -1, -1);
+                if (nan[0] | nan[1] | nan[2] | nan[3]) first = grid_scan(a, src, q, kch);
+#pragma unroll
+                for (int k2 = 0; k2 < 4; ++k2) {
+                    uint32_t left = 0;
+                    for (uint32_t bits = nan[k2]; bits; bits &= bits - 1) {
+                        const int bit = __ffs(bits) - 1, k = 2 * k2 + (bit >> 4);
+                        const int i = (MT == 2 ? k : 2 * k + h) * kEpiCols + (bit & 15);
+                        if (i < cnt && !grid_nan_at(a, wt, src, bnr, i, q, kch, first)) left |= 1u << bit;
+                    }
+                    __syncwarp();
+                    for (uint32_t lanes = __ballot_sync(0xffffffffu, left != 0); lanes; lanes &= lanes - 1) {
+                        const int l = __ffs(lanes) - 1;
+                        const int ql = __shfl_sync(0xffffffffu, q, l);
+                        for (uint32_t bits = __shfl_sync(0xffffffffu, left, l); bits; bits &= bits - 1) {
+                            const int bit = __ffs(bits) - 1, k = 2 * k2 + (bit >> 4);
+                            const int i = (MT == 2 ? k : 2 * k + h) * kEpiCols + (bit & 15);
+                            float e = grid_exact(a, wt, src, bnr, i, ql, kch) + t_bias[i];
+                            if (lane != l || !y_ok(yc, t_off[i])) continue;
+                            if (a.relu) e = fmaxf(e, 0.0f);
+                            if (OUT_BF16)
+                                yh[t_off[i]] = __float2bfloat16_rn(e);
+                            else
+                                yf[t_off[i]] = e;
+                        }
+                        __syncwarp();
+                    }
                 }
             }
             __syncwarp();
