@@ -468,7 +468,9 @@ __global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_const
 #pragma unroll
                 for (int c = 0; c < kGwChunks; ++c) {
                     const int k = 2 * c + h, j = k / per;
-                    if (k < n && ((keep >> (p0 + j)) & 1u)) {
+                    if (k < n && ((keep >> (p0 + j)) & 1u) &&
+                        dbg_in(dst + (p0 + j) * a.w.nst + (k - j * per) * kEpiCols + kEpiCols - 1 - a.slices,
+                               a.w.Z * a.w.slice, a.status)) {
                         float4* d4 = reinterpret_cast<float4*>(dst + (p0 + j) * a.w.nst + (k - j * per) * kEpiCols);
 #pragma unroll
                         for (int i = 0; i < kEpiCols / 4; ++i)
@@ -495,6 +497,8 @@ struct DbArgs {
     int nparts, groups, n_pad, Fg;
     int more;  // 1: added to db, which an earlier pass over other images wrote
     float* db;
+    int F;
+    int* status;
 };
 
 // db, by blocks b, b + nb, ... of 256 threads: a warp per packed row adds its
@@ -508,11 +512,13 @@ SADMM_DEV void db_blocks(const DbArgs& a, int b, int nb)
         float s = 0.0f;
         for (int k = lane; k < a.nparts; k += 32) s += __ldg(a.part + (size_t)r * a.nparts + k);
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) a.db[f] = a.more ? a.db[f] + s : s;
+        if (lane == 0 && dbg_in(f, a.F, a.status)) a.db[f] = a.more ? a.db[f] + s : s;
     }
     for (int z = b * 256 + threadIdx.x; !a.more && z < a.groups * a.Fg; z += nb * 256) {
         const int g = z / a.Fg;
-        if (z - g * a.Fg < __ldg(a.counts + 2 * g + 1)) a.db[__ldg(a.zeromap + z)] = 0.0f;
+        if (z - g * a.Fg >= __ldg(a.counts + 2 * g + 1)) continue;
+        const int f = __ldg(a.zeromap + z);
+        if (dbg_in(f, a.F, a.status)) a.db[f] = 0.0f;
     }
 }
 
@@ -536,7 +542,8 @@ struct WrArgs {
     float* dW;
     int n_pad, n_cols, taps, chan_kind;
     int more;  // 1: added to dW, which an earlier pass over other images wrote
-    long long K;
+    long long K, dw_total;
+    int* status;
 };
 
 // Where the slices of packed row i, K column col (packed column j) of group g lie, in
@@ -653,7 +660,8 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const __grid_constant__ Wr
 #pragma unroll
             for (int e = 0; e < kWrCols; ++e) {
                 t[r][e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (in) t[r][e] = __ldcs(reinterpret_cast<const float4*>(src[e] + at));
+                if (in && dbg_in(src[e] + at + 3 - a.slices, a.w.Z * a.w.slice, a.status))
+                    t[r][e] = __ldcs(reinterpret_cast<const float4*>(src[e] + at));
             }
         }
 #pragma unroll
@@ -691,6 +699,7 @@ __global__ void __launch_bounds__(256) k_grid_wreduce(const __grid_constant__ Wr
             if ((int)(threadIdx.x & 31) == l) acc = e;
         }
         if (of < 0) continue;
+        if (!dbg_in((long long)of * a.K + ocol, a.dw_total, a.status)) continue;
         float* dst = a.dW + (long long)of * a.K + ocol;
         *dst = a.more ? *dst + acc : acc;
     }
@@ -707,6 +716,8 @@ struct DzArgs {
     float* part;        // [groups*n_pad][bx], or NULL
     int bx, by;         // blocks
     int slots;          // slots of a block
+    long long y_total, dz_total;  // elements of dY, octets of the copy
+    int* status;
 };
 
 // Grid copy of dZ and the bias gradient's partial sums.  Block (bx, by), 256 threads: slots
@@ -719,14 +730,15 @@ constexpr int kDzBlocks = 1024;
 // One pixel's dZ of a chunk's filters (nf of them, 8 when FULL): every load
 // first, then the products, the running bias sums and the packed octet.
 template <bool RELU, typename Y, bool FULL>
-SADMM_DEV void dz_octet(const unsigned short* dp, const Y* yp, const int (&off)[8], int nf, float (&sum)[8], uint32_t (&o)[4])
+SADMM_DEV void dz_octet(const unsigned short* dp, const Y* yp, const YCheck& in, const int (&off)[8], int nf, float (&sum)[8],
+                        uint32_t (&o)[4])
 {
     uint32_t dyv[8];
     Y yv[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-        dyv[e] = (FULL || e < nf) ? (uint32_t)__ldg(dp + off[e]) : 0u;
-        if (RELU) yv[e] = (FULL || e < nf) ? __ldg(yp + off[e]) : Y(0);
+        dyv[e] = (FULL || e < nf) && y_ok(in, off[e]) ? (uint32_t)__ldg(dp + off[e]) : 0u;
+        if (RELU) yv[e] = (FULL || e < nf) && y_ok(in, off[e]) ? __ldg(yp + off[e]) : Y(0);
     }
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -772,12 +784,13 @@ SADMM_DEV void dz_block(const DzArgs& a, int bx, int by, int* s_off, float (*s_p
             const long long base = (long long)n * a.F * a.plane + (t * a.gr.OH + h) * a.gr.OW + w;
             const unsigned short* dp = reinterpret_cast<const unsigned short*>(a.dy) + base;
             const Y* yp = static_cast<const Y*>(a.y) + base;
-            if (nf == 8) dz_octet<RELU, Y, true>(dp, yp, off, 8, sum, o);
-            else dz_octet<RELU, Y, false>(dp, yp, off, nf, sum, o);
+            const YCheck in{base, a.y_total, a.status};
+            if (nf == 8) dz_octet<RELU, Y, true>(dp, yp, in, off, 8, sum, o);
+            else dz_octet<RELU, Y, false>(dp, yp, in, off, nf, sum, o);
         }
-        if (a.dz)
-            reinterpret_cast<uint4*>(a.dz)[((size_t)g * a.chunks + ck) * a.gr.slots + s] =
-                make_uint4(o[0], o[1], o[2], o[3]);
+        const size_t at = ((size_t)g * a.chunks + ck) * a.gr.slots + s;
+        if (a.dz && dbg_in((long long)at, a.dz_total, a.status))
+            reinterpret_cast<uint4*>(a.dz)[at] = make_uint4(o[0], o[1], o[2], o[3]);
     }
     if (!a.part) return;
 #pragma unroll
@@ -1067,6 +1080,9 @@ static sadmm_status launch_pass(const sadmm_plan* plan, const Geometry& g, const
     d.part = db ? part : nullptr;
     d.bx = b.nparts;
     d.slots = b.dzslots;
+    d.y_total = g.n * g.f * g.plane;
+    d.dz_total = g.groups * b.dchunks * (long long)b.gr.slots;
+    d.status = device_status_ptr();
     d.by = (int)(g.groups * b.dchunks);
     fa.ndz = d.bx * d.by;
     if (dW) {
@@ -1090,6 +1106,8 @@ static sadmm_status launch_pass(const sadmm_plan* plan, const Geometry& g, const
     dd.n_pad = plan->n_pad;
     dd.Fg = (int)g.fg;
     dd.db = db;
+    dd.F = (int)g.f;
+    dd.status = device_status_ptr();
     dd.more = more ? 1 : 0;
     if (db && !dW &&
         launch_pdl(k_grid_db, dim3((unsigned)((g.groups * plan->n_pad + 7) / 8)), dim3(256), 0, s, dd) != cudaSuccess)
@@ -1143,6 +1161,8 @@ static sadmm_status launch_pass(const sadmm_plan* plan, const Geometry& g, const
         r.chan_kind = chan_kind;
         r.more = more ? 1 : 0;
         r.K = g.k;
+        r.dw_total = g.f * g.k;
+        r.status = device_status_ptr();
     }
     // The input gradient reads what k_grid_front wrote and nothing of k_grid_wgrad's.
     // Every CTA of k_grid_wgrad lets it start only after its own wait for

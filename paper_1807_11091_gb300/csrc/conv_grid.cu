@@ -829,6 +829,7 @@ bool grid_x_args(const Grid& gr, const Geometry& g, const void* x, const int* co
     a->chunks = chunks;
     a->taps = (int)g.taps;
     a->x_total = g.n * g.c * g.t * g.h * g.w;
+    a->xs_total = g.groups * chunks * (long long)gr.slots;
     a->status = device_status_ptr();
     a->bx = (gr.slots + 255) / 256;
     a->by = (int)(g.groups * ((chunks + 1) / 2));

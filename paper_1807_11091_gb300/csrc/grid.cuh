@@ -132,7 +132,7 @@ struct GridX {
     const int* colidx;
     __nv_bfloat16* xs;
     int C, Cg, nck, chunks, taps, bx, by;
-    long long x_total;
+    long long x_total, xs_total;  // elements of x, octets of the copy
     int* status;
 };
 // False when by passes the grid limit.
@@ -215,9 +215,11 @@ SADMM_DEV void grid_x_block(const GridX& a, int bx, int by, int* s_off)
         const int off = s_off[e];
         v[e] = (valid && off >= 0 && dbg_in(base + off, a.x_total, a.status)) ? (uint32_t)__ldg(xi + base + off) : 0u;
     }
-    uint4* dst = reinterpret_cast<uint4*>(a.xs) + ((size_t)g * a.chunks + c0) * a.gr.slots + s;
+    const size_t at = ((size_t)g * a.chunks + c0) * a.gr.slots + s;
+    uint4* dst = reinterpret_cast<uint4*>(a.xs) + at;
+    if (!dbg_in((long long)at, a.xs_total, a.status)) return;
     dst[0] = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
-    if (c0 + 1 < a.chunks)
+    if (c0 + 1 < a.chunks && dbg_in((long long)at + a.gr.slots, a.xs_total, a.status))
         dst[a.gr.slots] =
             make_uint4(v[8] | (v[9] << 16), v[10] | (v[11] << 16), v[12] | (v[13] << 16), v[14] | (v[15] << 16));
 }
