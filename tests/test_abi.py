@@ -298,3 +298,18 @@ def test_backward_takes_the_grid_where_it_is_faster(n, c, hw, f, k, cf, grid):
     st, p = sadmm.sadmm_plan_init(sadmm.make_desc(s.desc16()), f, wl.COL_SHAPE, wl.retained(cf, s.k))
     assert st == 0
     assert (sadmm.sadmm_conv_bwd_workspace_size(p) != sadmm.sadmm_conv_bwd_workspace_size_chunk(p, 32768)) == grid
+
+
+def test_stream_without_the_private_torch_calls(monkeypatch):
+    """A torch without the calls that read the raw stream is asked for its stream object."""
+    import torch
+
+    class Stream:
+        cuda_stream = 1234
+
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.delattr(torch._C, name, raising=False)
+    assert sadmm._stream() == 1234
+    assert sadmm._stream(Stream) == 1234
