@@ -389,9 +389,10 @@ def _stream(stream=None) -> int:
     it, which are not public: 0.3 us instead of 3)."""
     torch = _torch()
     if stream is None and torch.cuda.is_initialized():
-        raw, device = (getattr(torch._C, f, None) for f in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
-        if raw is not None and device is not None:
-            return raw(device())
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:
+            pass
     s = stream if stream is not None else torch.cuda.current_stream()
     return int(s.cuda_stream)
 
