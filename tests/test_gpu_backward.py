@@ -110,14 +110,57 @@ def test_backward_without_relu():
     assert_close(dx, rdx, what="no relu dx")
 
 
+def _assert_chunked(s, kf, ck, kc):
+    """The layer's backward runs in pixel chunks by default, on no input slab."""
+    from paper_1807_11091_gb300 import sadmm
+    st, p = sadmm.sadmm_plan_init(sadmm.make_desc(s.desc16()), kf, ck, kc if ck != wl.COL_NONE else s.k)
+    assert st == 0 and p.xs_mode == 0
+    assert sadmm.sadmm_conv_bwd_workspace_size(p) == sadmm.sadmm_conv_bwd_workspace_size_chunk(p, 32768)
+
+
+# the chunked path's forms: each takes a stride, which the pixel grid does not
+CHUNKED = [
+    ("ragged", ConvShape(n=3, c=5, h=21, w=25, f=37, kh=3, kw=3, sh=2, sw=2, ph=1, pw=1), 0.7, wl.COL_SHAPE, 0.4),
+    ("groups2_5x5", ConvShape(n=2, c=8, h=17, w=17, f=12, kh=5, kw=5, sh=2, sw=2, ph=2, pw=2, groups=2), 0.5, wl.COL_SHAPE,
+     0.5),
+    ("c3d", ConvShape(n=2, c=4, t=5, h=11, w=13, f=20, kt=3, kh=3, kw=3, sh=2, sw=2, pt=1, ph=1, pw=1), 1.0, wl.COL_SHAPE, 0.3),
+    ("c3d_45_taps", ConvShape(n=2, c=4, t=6, h=13, w=16, f=16, kt=3, kh=3, kw=5, sh=2, sw=2, pt=1, ph=1, pw=2), 0.75,
+     wl.COL_SHAPE, 0.4),
+    ("channel_3x3", ConvShape(n=2, c=48, h=17, w=17, f=80, kh=3, kw=3, sh=2, sw=2, ph=1, pw=1, groups=2), 0.5, wl.COL_CHANNEL,
+     0.5),
+    ("two_filter_tiles", ConvShape(n=2, c=16, h=19, w=19, f=300, kh=3, kw=3, sh=2, sw=2, ph=1, pw=1), 1.0, wl.COL_SHAPE, 0.9),
+    # a full 32768-pixel chunk, split as the wide layers' are, then a ragged one, two conv groups
+    ("full_chunks", ConvShape(n=44, c=96, h=55, w=55, f=256, kh=5, kw=5, sh=2, sw=2, ph=2, pw=2, groups=2), 0.5, wl.COL_SHAPE,
+     0.5),
+]
+
+
+@pytest.mark.parametrize("case", CHUNKED, ids=lambda c: c[0])
+def test_backward_in_chunks_matches_oracle(case):
+    name, s, ff, ck, cf = case
+    kf, kc = wl.retained(ff, s.f), wl.retained(cf, s.cg if ck == wl.COL_CHANNEL else s.k)
+    _assert_chunked(s, kf, ck, kc)
+    if name == "full_chunks":
+        assert s.n * s.oh * s.ow > 32768
+    t = wl.gen_tensors(s, seed=13)
+    (dW, db, dx), (rdW, rdb, rdx), rows, cols = _backward(s, t, kf, ck, kc)
+    assert_close(dW, rdW, what=f"{name} dW")
+    assert_close(db, rdb, what=f"{name} db")
+    assert_close(dx, rdx, what=f"{name} dx")
+    keep = oracle.masked_weights(np.ones(t["W"].shape), rows, ck, cols, s.taps).reshape(s.f, -1) != 0
+    assert np.all(dW[~keep] == 0.0)
+    assert np.all(db[np.setdiff1d(np.arange(s.f), rows)] == 0.0)
+
+
 @pytest.mark.parametrize("chunk", [32768, 9984, 256])
 def test_backward_several_pixel_chunks(chunk):
-    """41772 output pixels in chunks as large as a smaller workspace holds:
-    32768 + a ragged 9004, five chunks, or 164 chunks of 256, so the weight
-    gradient accumulates per pixel split across chunks."""
-    s = ConvShape(n=3, c=6, h=120, w=120, f=24, kh=3, kw=3)
+    """42483 output pixels (a stride of 2: no pixel grid) in chunks as large as a
+    smaller workspace holds: 32768 + a ragged 9715, five chunks, or 166 chunks of
+    256, so the weight gradient accumulates per pixel split across chunks."""
+    s = ConvShape(n=3, c=6, h=239, w=239, f=24, kh=3, kw=3, sh=2, sw=2)
     kf, kc = wl.retained(0.75, s.f), wl.retained(0.6, s.k)
     assert s.n * s.oh * s.ow > 32768
+    _assert_chunked(s, kf, wl.COL_SHAPE, kc)
     t = wl.gen_tensors(s, seed=21)
     (dW, db, dx), (rdW, rdb, rdx), rows, cols = _backward(s, t, kf, wl.COL_SHAPE, kc, chunk_pixels=chunk)
     assert_close(dW, rdW, what=f"chunks of {chunk}: dW")
@@ -160,13 +203,14 @@ def _raw_backward(pc, x, dy, y, want_dw, want_dx):
     return dW, db, dx
 
 
-def test_backward_weight_gradient_deterministic_and_partial_calls():
+@pytest.mark.parametrize("case", [CASES[1], CHUNKED[1]], ids=["grid", "chunked"])
+def test_backward_weight_gradient_deterministic_and_partial_calls(case):
     """dW and db come out bit-identical on every call (fixed-order sums); a call
     that asks for the weight gradient only, the input gradient only, or the bias
     gradient only gives what the full call gives (dx up to its atomic
     summation order)."""
     from paper_1807_11091_gb300 import sadmm
-    name, s, ff, ck, cf = CASES[1]
+    name, s, ff, ck, cf = case
     kf, kc = wl.retained(ff, s.f), wl.retained(cf, s.k)
     t = wl.gen_tensors(s, seed=31)
     dev = torch.device("cuda", 0)
@@ -224,18 +268,15 @@ def test_backward_weight_gradient_on_the_slab(case):
     assert np.array_equal(dW, dW2)
 
 
-@pytest.mark.parametrize("li,batch", [(0, 16), (1, 72)], ids=["conv1_b16_slab_many_runs", "conv2_b72_full_chunks"])
+@pytest.mark.parametrize("li,batch", [(0, 16), (1, 72)], ids=["conv1_b16_slab_many_runs", "conv2_b72"])
 def test_backward_alexnet_at_benchmarked_paths(li, batch):
     """The paths the benchmark's batch-128 backward takes, at batches the fp64
     oracle finishes in seconds: CONV1's weight gradient on the slab over 378
     output tiles (2.5 runs per CTA, one fp32 slice each, summed in CTA order);
-    CONV2 (two conv groups) in a full 32768-pixel chunk, with the benchmark's
-    weight-gradient split for that chunk, then a ragged second chunk."""
+    CONV2 (two conv groups) on the pixel grid, in ranges of dozens of tiles."""
     L = wl.subset_layer(wl.alexnet()[li], batch)
     s = L.shape
     t = wl.gen_tensors(s, seed=L.seed)
-    if li == 1:
-        assert s.n * s.oh * s.ow > 32768
     (dW, db, dx), (rdW, rdb, rdx), rows, cols = _backward(s, t, L.k_filters, L.colkind, L.k_cols, seed=li)
     assert_close(dW, rdW, what=f"{L.name} batch {batch} dW")
     assert_close(db, rdb, what=f"{L.name} batch {batch} db")
