@@ -594,7 +594,8 @@ __global__ void __launch_bounds__(kGcThreads, 1)
                 if (lane == 0) mbar_arrive(&acc_empty[ab]);
                 if (++ab == a.nbuf) { ab = 0; acc_ph ^= 1u; }
             }
-            uint32_t nan[4] = {0u, 0u, 0u, 0u};  // NaN columns, 16 bits a chunk
+            uint32_t nan = 0;         // chunks with NaN columns
+            uint32_t nan_cols[8];     // theirs, 16 bits a chunk (in local memory: read by a runtime index)
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
                 const int c = MT == 2 ? k : 2 * k + h;
@@ -603,37 +604,38 @@ __global__ void __launch_bounds__(kGcThreads, 1)
 #pragma unroll
                     for (int j = 0; j < kEpiCols; ++j) bad |= v[k][j] != v[k][j];
                     if (bad) {
+                        uint32_t m = 0;
 #pragma unroll
-                        for (int j = 0; j < kEpiCols; ++j)
-                            nan[k >> 1] |= (v[k][j] != v[k][j] ? 1u : 0u) << ((k & 1) * 16 + j);
+                        for (int j = 0; j < kEpiCols; ++j) m |= (v[k][j] != v[k][j] ? 1u : 0u) << j;
+                        nan |= 1u << k;
+                        nan_cols[k] = m;
                     }
                     store_cols<OUT_BF16>(v[k], c * kEpiCols, cnt, t_off, t_bias, a.relu, yf, yh, yc);
                 }
             }
             // NaN columns: what a lane finds to be a kept term's stands, the others are
             // summed again by the warp
-            if (__any_sync(0xffffffffu, (nan[0] | nan[1] | nan[2] | nan[3]) != 0)) {
+            if (__any_sync(0xffffffffu, nan != 0)) {
                 const int kch = a.kcounts ? __ldg(a.kcounts + 2 * g) : a.ncb * a.cb;
                 const uint4* wt = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(a.wd) +
                                                                  (size_t)(g * a.ntiles + nt) * btile);
                 const uint4* src = reinterpret_cast<const uint4*>(a.src + (size_t)g * a.gstride);
                 int4 first = make_int4(-1, -1, -1, -1);
-                if (nan[0] | nan[1] | nan[2] | nan[3]) first = grid_scan(a, src, q, kch);
-#pragma unroll
-                for (int k2 = 0; k2 < 4; ++k2) {
+                if (nan) first = grid_scan(a, src, q, kch);
+#pragma unroll 1
+                for (int k = 0; k < 8; ++k) {
+                    const int c0 = (MT == 2 ? k : 2 * k + h) * kEpiCols;
                     uint32_t left = 0;
-                    for (uint32_t bits = nan[k2]; bits; bits &= bits - 1) {
-                        const int bit = __ffs(bits) - 1, k = 2 * k2 + (bit >> 4);
-                        const int i = (MT == 2 ? k : 2 * k + h) * kEpiCols + (bit & 15);
-                        if (i < cnt && !grid_nan_at(a, wt, src, bnr, i, q, kch, first)) left |= 1u << bit;
+                    for (uint32_t bits = (nan >> k) & 1u ? nan_cols[k] : 0u; bits; bits &= bits - 1) {
+                        const int i = c0 + __ffs(bits) - 1;
+                        if (i < cnt && !grid_nan_at(a, wt, src, bnr, i, q, kch, first)) left |= bits & (0u - bits);
                     }
                     __syncwarp();
                     for (uint32_t lanes = __ballot_sync(0xffffffffu, left != 0); lanes; lanes &= lanes - 1) {
                         const int l = __ffs(lanes) - 1;
                         const int ql = __shfl_sync(0xffffffffu, q, l);
                         for (uint32_t bits = __shfl_sync(0xffffffffu, left, l); bits; bits &= bits - 1) {
-                            const int bit = __ffs(bits) - 1, k = 2 * k2 + (bit >> 4);
-                            const int i = (MT == 2 ? k : 2 * k + h) * kEpiCols + (bit & 15);
+                            const int i = c0 + __ffs(bits) - 1;
                             float e = grid_exact(a, wt, src, bnr, i, ql, kch) + t_bias[i];
                             if (lane != l || !y_ok(yc, t_off[i])) continue;
                             if (a.relu) e = fmaxf(e, 0.0f);

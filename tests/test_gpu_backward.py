@@ -118,7 +118,8 @@ def _assert_chunked(s, kf, ck, kc):
     assert sadmm.sadmm_conv_bwd_workspace_size(p) == sadmm.sadmm_conv_bwd_workspace_size_chunk(p, 32768)
 
 
-# the chunked path's forms: each takes a stride, which the pixel grid does not
+# the chunked path's forms: each takes a stride, which the pixel grid does not, or keeps
+# few of many channels' columns
 CHUNKED = [
     ("ragged", ConvShape(n=3, c=5, h=21, w=25, f=37, kh=3, kw=3, sh=2, sw=2, ph=1, pw=1), 0.7, wl.COL_SHAPE, 0.4),
     ("groups2_5x5", ConvShape(n=2, c=8, h=17, w=17, f=12, kh=5, kw=5, sh=2, sw=2, ph=2, pw=2, groups=2), 0.5, wl.COL_SHAPE,
@@ -129,6 +130,7 @@ CHUNKED = [
     ("channel_3x3", ConvShape(n=2, c=48, h=17, w=17, f=80, kh=3, kw=3, sh=2, sw=2, ph=1, pw=1, groups=2), 0.5, wl.COL_CHANNEL,
      0.5),
     ("two_filter_tiles", ConvShape(n=2, c=16, h=19, w=19, f=300, kh=3, kw=3, sh=2, sw=2, ph=1, pw=1), 1.0, wl.COL_SHAPE, 0.9),
+    ("sparse_wide_stride1", ConvShape(n=1, c=1024, h=14, w=14, f=1024, kh=3, kw=3, ph=1, pw=1), 1.0, wl.COL_SHAPE, 0.02),
     # a full 32768-pixel chunk, split as the wide layers' are, then a ragged one, two conv groups
     ("full_chunks", ConvShape(n=44, c=96, h=55, w=55, f=256, kh=5, kw=5, sh=2, sw=2, ph=2, pw=2, groups=2), 0.5, wl.COL_SHAPE,
      0.5),
