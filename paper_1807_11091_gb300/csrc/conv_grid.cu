@@ -220,7 +220,9 @@ struct GcPipe {
 // most 14 MMAs.
 inline bool unrolled_row(int kw, int h16)
 {
-    return ((kw == 1 || kw == 3) && h16 <= 4) || ((kw == 5 || kw == 7) && h16 <= 2) || ((kw == 4 || kw == 6) && h16 == 1);
+    if (kw == 1 || kw == 3) return h16 <= 4;
+    if (kw == 5 || kw == 7) return h16 <= 2;
+    return h16 == 1 && (kw == 4 || kw == 6 || kw == 9 || kw == 11);
 }
 
 // The issuing warp's run over its work items.  The whole warp runs the loop,
@@ -495,7 +497,7 @@ __global__ void __launch_bounds__(kGcThreads, 1)
         SADMM_ROW(1, 1) SADMM_ROW(1, 2) SADMM_ROW(1, 3) SADMM_ROW(1, 4)
         SADMM_ROW(3, 1) SADMM_ROW(3, 2) SADMM_ROW(3, 3) SADMM_ROW(3, 4)
         SADMM_ROW(5, 1) SADMM_ROW(5, 2) SADMM_ROW(7, 1) SADMM_ROW(7, 2)
-        SADMM_ROW(4, 1) SADMM_ROW(6, 1)
+        SADMM_ROW(4, 1) SADMM_ROW(6, 1) SADMM_ROW(9, 1) SADMM_ROW(11, 1)
         { SADMM_ISSUE(0, 0) }
 #undef SADMM_ROW
 #undef SADMM_ISSUE
