@@ -705,8 +705,9 @@ bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups
     const long long span = (gr.KH - 1) * gr.Wb + gr.KW - 1;
     // A block: as many 16s of channels as divide them, keep a stage to `stage`
     // MMA steps and its slab to 24 KB.
+    // (and, where sums are cut, a kernel row unrolled: its issue is the slower otherwise)
     int m = 4;
-    while (m > 1 && (r.k16 % m != 0 || taps * m > stage || (128 + span) * 32 * m > 24576)) --m;
+    while (m > 1 && (r.k16 % m != 0 || taps * m > stage || (cut && unrolled_row(gr.KW, 1) && !unrolled_row(gr.KW, m)) || (128 + span) * 32 * m > 24576)) --m;
     r.cb = 16 * m;
     const int rsteps = gr.KW * m;
     // The tiling of least estimated time: rounds of items over the SMs, each
