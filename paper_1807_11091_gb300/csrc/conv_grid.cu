@@ -705,9 +705,21 @@ bool grid_conv_shape(const Grid& gr, int chans, int cols, int likely, int groups
     const long long span = (gr.KH - 1) * gr.Wb + gr.KW - 1;
     // A block: as many 16s of channels as divide them, keep a stage to `stage`
     // MMA steps and its slab to 24 KB.
-    // (and, where sums are cut, a kernel row unrolled: its issue is the slower otherwise)
-    int m = 4;
-    while (m > 1 && (r.k16 % m != 0 || taps * m > stage || (cut && unrolled_row(gr.KW, 1) && !unrolled_row(gr.KW, m)) || (128 + span) * 32 * m > 24576)) --m;
+    // Where sums are cut, a kernel row that is unrolled (its issue is the slower
+    // otherwise) and of which whole rows fill a segment best: the rest of one is a
+    // segment more to read (AlexNet conv3: 12 steps of 2 rows, not 9 of 1).
+    int m = 1;
+    for (int k = 2, filled = 0; k <= 4; ++k) {
+        if (r.k16 % k != 0 || taps * k > stage || (128 + span) * 32 * k > 24576) continue;
+        if (cut) {
+            if (unrolled_row(gr.KW, 1) && !unrolled_row(gr.KW, k)) continue;
+            if (filled == 0) filled = std::max(gr.KW, seg / gr.KW * gr.KW);
+            const int f = std::max(1, seg / (gr.KW * k)) * gr.KW * k;
+            if (taps * k > seg && f < filled) continue;
+            filled = std::max(filled, f);
+        }
+        m = k;
+    }
     r.cb = 16 * m;
     const int rsteps = gr.KW * m;
     // The tiling of least estimated time: rounds of items over the SMs, each
