@@ -64,7 +64,8 @@ int dx_seg(int filters) { return filters <= 256 ? 12 : 27; }
 struct WgradShape {
     int nch;          // 8-channel chunks of x per conv group
     int blk, mblks;   // chunks per M block, blocks
-    int rep, kwg;     // kernel columns per MMA, groups of them per kernel row
+    int rep, kwg;     // kernel columns per MMA, groups of them (macro taps) per kernel row
+    int kws;          // a row's macro taps as items take them: kwg, or to a multiple of tpg where no item spans rows
     int rows;         // M rows in use: rep * blk * 8
     int nst, nft;     // filters per N tile, tiles
     int tpg, tgs;     // macro taps per item, items per kernel frame
@@ -95,18 +96,19 @@ __host__ __device__ inline GwStage gw_stage(const WgradShape& w, int nr)
     }
 }
 
-// The most slots that the taps of an item span beyond its 128 pixels.
+// The most slots that the taps of an item span beyond its pixels.
 int wgrad_span(const Grid& gr, const WgradShape& w)
 {
-    const int macro = gr.KH * w.kwg;
+    if (w.kws % w.tpg == 0) return (std::min(w.tpg, w.kwg) - 1) * w.rep;  // (no item spans rows)
+    const int macro = gr.KH * w.kws;
     int span = 0;
     for (int t0 = 0; t0 < macro; t0 += w.tpg) {
-        const int t1 = std::min(macro, t0 + w.tpg) - 1, r0 = t0 / w.kwg, r1 = t1 / w.kwg;
-        const int first = r0 * gr.Wb + t0 % w.kwg * w.rep, last = r1 * gr.Wb + t1 % w.kwg * w.rep;
+        const int t1 = std::min(macro, t0 + w.tpg) - 1, r0 = t0 / w.kws, r1 = t1 / w.kws;
+        const int first = r0 * gr.Wb + t0 % w.kws * w.rep, last = r1 * gr.Wb + t1 % w.kws * w.rep;
         int lo = std::min(first, last), hi = std::max(first, last);
         if (r1 > r0) {
             lo = std::min(lo, (r0 + 1) * gr.Wb);
-            hi = std::max(hi, (r1 - 1) * gr.Wb + (w.kwg - 1) * w.rep);
+            hi = std::max(hi, (r1 - 1) * gr.Wb + (w.kws - 1) * w.rep);
         }
         span = std::max(span, hi - lo);
     }
@@ -145,10 +147,14 @@ bool wgrad_shape(const Grid& gr, int nck, int n_pad, int likely, int groups, Wgr
         w.nst = (int)round_up((n_pad + w.nft - 1) / w.nft, 16);
         const int nl = w.nft == 1 ? std::min(w.nst, (int)round_up(likely, 16)) : w.nst;
         const int tmax = std::min(std::min(kGwCols / nl, macro), 32), tg0 = (macro + tmax - 1) / tmax;
-        for (int tgs = tg0; tgs <= std::min(macro, tg0 + 3); ++tgs) {
+        for (int tgs = tg0, by_row = 0; tgs <= std::min(macro, tg0 + 3); tgs += by_row, by_row ^= 1) {
             w.tpg = (macro + tgs - 1) / tgs;
-            w.tgs = (macro + w.tpg - 1) / w.tpg;
-            if (w.tgs != tgs) continue;
+            if ((macro + w.tpg - 1) / w.tpg != tgs) continue;
+            // also with items that span no rows, whose slabs are shorter (AlexNet conv3 in
+            // pairs of taps fits stages of two tiles so)
+            w.kws = by_row ? (int)round_up(w.kwg, w.tpg) : w.kwg;
+            if (by_row && (w.kws == w.kwg || w.tpg > w.kwg)) continue;
+            w.tgs = (gr.KH * w.kws + w.tpg - 1) / w.tpg;
             w.span = wgrad_span(gr, w);
             if (w.span + 256 >= (1 << 14) || gw_stage(w, w.nst).count < 2) continue;
             const GwStage sg = gw_stage(w, nl);
@@ -219,12 +225,13 @@ SADMM_DEV GwItem gw_item(const GwArgs& a, int u)
     it.ft = r % a.w.nft;
     it.g = r / a.w.nft;
     it.t0 = tg * a.w.tpg;
-    it.nt = min(a.w.tpg, a.gr.KH * a.w.kwg - it.t0);
+    it.nt = min(a.w.tpg, a.gr.KH * a.w.kws - it.t0);
+    if (a.w.kws % a.w.tpg == 0) it.nt = min(it.nt, a.w.kwg - it.t0 % a.w.kws);
     const int cnt = min(a.w.nst, __ldg(a.counts + 2 * it.g) - it.ft * a.w.nst);
     it.nr = cnt > 0 ? (cnt + 15) & ~15 : 0;
     int lo = 1 << 30, hi = 0;
     for (int t = it.t0; t < it.t0 + it.nt; ++t) {
-        const int s = (t / a.w.kwg) * a.gr.Wb + (t % a.w.kwg) * a.w.rep;
+        const int s = (t / a.w.kws) * a.gr.Wb + (t % a.w.kws) * a.w.rep;
         lo = min(lo, s);
         hi = max(hi, s);
     }
@@ -242,7 +249,7 @@ SADMM_DEV uint32_t gw_keep(const GwArgs& a, const GwItem& it, int row)
     if (row >= a.w.rows || c >= a.nck) return 0;
     uint32_t keep = 0;
     for (int j = 0; j < it.nt; ++j) {
-        const int t = it.t0 + j, kh = t / a.w.kwg, kw = (t - kh * a.w.kwg) * a.w.rep + rp;
+        const int t = it.t0 + j, kh = t / a.w.kws, kw = (t - kh * a.w.kws) * a.w.rep + rp;
         if (kw >= a.gr.KW) continue;
         bool ok = true;
         if (a.colidx) {
@@ -363,8 +370,8 @@ __global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_const
             const int b = it.z * a.w.tps, e = min(a.w.tiles, b + a.w.tps);
             for (int t0 = it.t0; ok && t0 < it.t0 + it.nt; t0 += it.tp) {
                 const int np = min(it.tp, it.t0 + it.nt - t0);
-                const uint32_t kq0 = (uint32_t)(t0 % a.w.kwg);
-                const uint32_t to0 = (uint32_t)(t0 / a.w.kwg * a.gr.Wb) + kq0 * (uint32_t)a.w.rep - (uint32_t)it.base;
+                const uint32_t kq0 = (uint32_t)(t0 % a.w.kws);
+                const uint32_t to0 = (uint32_t)(t0 / a.w.kws * a.gr.Wb) + kq0 * (uint32_t)a.w.rep - (uint32_t)it.base;
                 int in_seg = 0;
                 uint32_t d0 = 0;
                 for (int t = b; t < e; t += sg.tiles) {
@@ -390,9 +397,9 @@ __global__ void __launch_bounds__(kGwThreads, 1) k_grid_wgrad(const __grid_const
                             blo += 128u;
                         }
                         to += (uint32_t)a.w.rep;
-                        if (++kq == (uint32_t)a.w.kwg) {
+                        if (++kq == (uint32_t)a.w.kws) {
                             kq = 0;
-                            to += (uint32_t)(a.gr.Wb - a.w.kwg * a.w.rep);
+                            to += (uint32_t)(a.gr.Wb - a.w.kws * a.w.rep);
                         }
                     }
                     mma_commit_elect(&empty[s]);
@@ -552,7 +559,7 @@ SADMM_DEV size_t wr_slice(const WrArgs& a, int g, int i, int j, int col)
 {
     const int c = a.chan_kind ? j / a.taps : col / a.taps, tap = col % a.taps;
     const int kw = tap % a.gr.KW, kh = (tap / a.gr.KW) % a.gr.KH, kt = tap / (a.gr.KW * a.gr.KH);
-    const int mb = (c >> 3) / a.w.blk, mt = kh * a.w.kwg + kw / a.w.rep, ft = i / a.w.nst;
+    const int mb = (c >> 3) / a.w.blk, mt = kh * a.w.kws + kw / a.w.rep, ft = i / a.w.nst;
     const int m = (((kw % a.w.rep) * a.w.blk + ((c >> 3) - mb * a.w.blk)) << 3) + (c & 7);
     const int type = (((g * a.w.nft + ft) * a.w.mblks + mb) * a.gr.KT + kt) * a.w.tgs + mt / a.w.tpg;
     return ((size_t)type * a.w.rows + m) * (size_t)(a.w.tpg * a.w.nst) + (mt % a.w.tpg) * a.w.nst + (i - ft * a.w.nst);
