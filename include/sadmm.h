@@ -390,7 +390,9 @@ sadmm_status sadmm_sparse_conv_fwd(const sadmm_conv_desc* d, const void* plan, c
  * the pruned columns.  A product of a pruned column never reaches the output,
  * infinities and NaN included: the sums are the gathered path's, in another
  * order.  The plan still holds the gathered packing (the chunked backward and
- * larger strides use it).  Both passes belong to SADMM_FWD_REST.
+ * larger strides use it).  Both passes belong to SADMM_FWD_REST.  The copy takes 2
+ * bytes per channel and grid pixel of the batch out of dev_bytes (96 channels of
+ * 27x27 at batch 128: 22 MB, 64 of 224x224 at batch 64: 415 MB).
  */
 sadmm_status sadmm_plan_init(sadmm_plan* plan, const sadmm_conv_desc* d,
                              int n_filt, int colkind, int n_colgroups);

@@ -404,8 +404,8 @@ static long long chunked_ns(const BwdGeo& b)
 // workspace then (0: the chunked path).  The grid contracts over every tap and channel,
 // the chunked path over the kept columns alone.  Of 207 layers measured both ways (1x1 to
 // 11x11, 3-D, 1 to 32 groups, batch 1 to 128, 2 to 100 % of the columns) the grid is the
-// faster on 187, up to 14 times (AlexNet conv2 at batch 128 841 -> 163 us, conv3 164 ->
-// 55), and the slower where few of many channels' columns are kept: 1024 -> 1024 3x3 at
+// faster on 187, up to 14 times (AlexNet conv2 at batch 128 841 -> 162 us, conv3 164 ->
+// 53), and the slower where few of many channels' columns are kept: 1024 -> 1024 3x3 at
 // 14x14 and batch 32 with 2 % of them 296 us against 158, 512 -> 512 at 28x28 and batch
 // 64 473 against 335.  The rule takes the slower path on four, at most 18 % the
 // slower, and on one of 120 drawn layers, by 9 %.

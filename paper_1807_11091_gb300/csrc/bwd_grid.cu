@@ -29,8 +29,13 @@
 // with sums of 32 steps conv3's stand at 1.5e-7, of 48 at 2.1e-7.
 //
 // AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5): 841
-// us as six im2col / GEMM / col2im chunks, 165 us here; conv3 164 -> 57, a ResNet-50
-// 3x3 layer (64 of 128 channels and filters kept) at batch 64 277 -> 42.
+// us as six im2col / GEMM / col2im chunks, 162 us here; conv3 164 -> 52.5, a ResNet-50
+// 3x3 layer (64 of 128 channels and filters kept) at batch 64 277 -> 42.7.
+// One cold launch each (front, weight gradient, input gradient, reduction): conv2 35, 58,
+// 76, 8 us, conv3 14, 21, 27, 10, the ResNet layer 14, 16, 22, 10.  Both gradients run at
+// the issue rate of their MMAs (48 to 57 cycles a 128 x 64 x 16, set by the operands'
+// shared-memory reads) between their first loads and their last stores; the front pass
+// is 16 loads of 2 and 4 bytes an octet.
 #include <string.h>
 
 #include <algorithm>
@@ -54,11 +59,12 @@ constexpr int kGwChunks = kGwCols / kEpiCols / 2;  // 16-column chunks of an acc
 // MMA steps of the input gradient summed in TMEM.  The chunked path sums a pixel's
 // kept filters there, 16 a step, and adds the taps up in fp32: up to 256 filters a
 // group 12 steps are held here, beyond that, where those sums are long themselves, 27.
-// Errors against 64 bits (chunked path; here; here with 27, unless cut): AlexNet conv3
-// 7.0e-8; 6.5; 9.4, conv2 8.2; 8.7; 12, a ResNet-50 3x3 layer 7.3; 11; 16, 7x7, 9x9 and
-// 11x11 taps over 64 filters 13, 16 and 19; 12, 14 and 15; 44, 76 and 118, 256 filters
-// 3x3 16; 13; 17, 512 filters 30; 16.  Shorter sums cost conv3 48.6 -> 53 us and conv2
-// 180 -> 191 (with 9: 53 and 201 at 0.65 and 0.9e-7).
+// Errors against 64 bits, in 1e-8 (chunked path; here; with 27 steps): AlexNet conv3
+// 7.0; 6.4; 9.4, conv2 8.2; 8.7; 12, a ResNet-50 3x3 layer 7.3; 11; 16, 7x7, 9x9 and
+// 11x11 taps over 64 filters 13, 16, 19; 12, 14, 15; 19, 24, 21, 256 filters 3x3 16; 13;
+// 17, 512 filters 30; 16 (27 steps).  A sum more to read takes about 750 cycles of an
+// epilogue beside the MMAs: conv3's backward is 52.5 us, not 49.1, conv2's 162, not 149,
+// the ResNet layer's 42.7, not 41.7.
 int dx_seg(int filters) { return filters <= 256 ? 12 : 27; }
 
 struct WgradShape {
@@ -78,7 +84,8 @@ struct WgradShape {
 
 // How the stages lie in shared memory for items of `nr` filters: slabs of one
 // 128-pixel tile, or of two where that leaves two stages.  A bulk copy takes about
-// 66 cycles whatever its size up to 4 KB at least, and a slab is a copy per chunk.
+// 66 cycles whatever its size up to 4 KB at least, and a slab is a copy per chunk
+// (with one tile: conv2's backward 172 us, not 162, conv3's 60, not 52.5).
 struct GwStage {
     int tiles, spa, a_bytes, stride, count;  // tiles and slots a chunk, bytes of the slab and of a stage, stages
 };

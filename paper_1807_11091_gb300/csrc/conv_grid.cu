@@ -877,7 +877,7 @@ constexpr long long kRuleSms = 152;
 // against 64 bits is 2.1e-7 (the gathered kernel's 3.3e-7); with 27 it would be
 // 1.3e-7 and 55.8 us become 61.2.  A longer frame is one segment: 9x9 taps over 32
 // channels, 81 steps, stand at 7.2e-7 where the gathered kernel's sums of all 162
-// stood at 1.6e-6; cut after 54 they take 51 us instead of 44.
+// stand at 1.6e-6.
 constexpr int kFwdSeg = 54;
 
 // Channels of x per conv group that hold a kept column.
