@@ -29,10 +29,10 @@
 // with sums of 32 steps conv3's stand at 1.5e-7, of 48 at 2.1e-7.
 //
 // AlexNet conv2 at batch 128 (two groups of 64 kept filters x 48 channels, 5x5): 841
-// us as six im2col / GEMM / col2im chunks, 162 us here; conv3 164 -> 52.5, a ResNet-50
-// 3x3 layer (64 of 128 channels and filters kept) at batch 64 277 -> 42.7.
+// us as six im2col / GEMM / col2im chunks, 161 us here; conv3 164 -> 52, a ResNet-50
+// 3x3 layer (64 of 128 channels and filters kept) at batch 64 277 -> 42.2.
 // One cold launch each (front, weight gradient, input gradient, reduction): conv2 35, 58,
-// 76, 8 us, conv3 14, 21, 27, 10, the ResNet layer 14, 16, 22, 10.  Both gradients run at
+// 74, 8 us, conv3 14, 21, 27, 10, the ResNet layer 14, 17, 21, 11.  Both gradients run at
 // the issue rate of their MMAs (48 to 57 cycles a 128 x 64 x 16, set by the operands'
 // shared-memory reads) between their first loads and their last stores; the front pass
 // is 16 loads of 2 and 4 bytes an octet.
@@ -63,8 +63,8 @@ constexpr int kGwChunks = kGwCols / kEpiCols / 2;  // 16-column chunks of an acc
 // 7.0; 6.4; 9.4, conv2 8.2; 8.7; 12, a ResNet-50 3x3 layer 7.3; 11; 16, 7x7, 9x9 and
 // 11x11 taps over 64 filters 13, 16, 19; 12, 14, 15; 19, 24, 21, 256 filters 3x3 16; 13;
 // 17, 512 filters 30; 16 (27 steps).  A sum more to read takes about 750 cycles of an
-// epilogue beside the MMAs: conv3's backward is 52.5 us, not 49.1, conv2's 162, not 149,
-// the ResNet layer's 42.7, not 41.7.
+// epilogue beside the MMAs: conv3's backward was 52.5 us, not 49.1, conv2's 162, not 149,
+// the ResNet layer's 42.7, not 41.7 (with loads one by one: 52.0, 161 and 42.2 now).
 int dx_seg(int filters) { return filters <= 256 ? 12 : 27; }
 
 struct WgradShape {

@@ -335,7 +335,193 @@ SADMM_DEV void gc_issue(const GcArgs& a, const GcPipe& p, const int mode)
     }
 }
 
-template <bool OUT_BF16, int MT>
+// What the epilogue warps share.
+struct GcEpi {
+    uint64_t* acc_full;  // then acc_empty
+    volatile int* abort_flag;
+    int* t_off;          // [256], then t_bias [256], z_off [kGcZcap]
+    uint32_t tmem_base;
+    int bnr;
+};
+
+// The epilogue warps' run over the work items; a warp holds NCH chunks of 16 columns.
+// With four, a segment's loads leave TMEM together: one by one each takes about 125
+// cycles (AlexNet conv2's backward 162.5 -> 160.7 us, conv3's 53.0 -> 52.0, a 1x1 layer's
+// of 256 channels and 64 filters at 56x56 164 -> 154).  Eight leave no registers for that (two in flight spilled 80 bytes and AlexNet
+// conv2's forward took 60 us instead of 52), and both forms in the forward's kernel cost
+// it 1 %, so the input gradient, whose segments are the short ones, has its own.
+template <bool OUT_BF16, int MT, int NCH>
+SADMM_DEV void gc_epilogue(const GcArgs& a, const GcEpi& ep)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int* t_off = ep.t_off;
+    float* t_bias = reinterpret_cast<float*>(t_off + 256);
+    int* z_off = t_off + 512;
+    // Two warps per TMEM lane quadrant: with one pixel tile they take its
+    // 16-column chunks in turn, with two a tile each.
+    const int q4 = warp & 3;
+    const int h = (warp - 3) >> 2;
+    const int et = threadIdx.x - 3 * 32;
+    int ab = 0, key = -1;
+    uint32_t acc_ph = 0;
+    bool alive = true;
+    for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+        int g, nt, mt;
+        gc_unit(a, u, g, nt, mt);
+        const int cnt = min(a.bn, __ldg(a.counts + 2 * g) - nt * a.bn);
+        const int zc = nt == 0 ? __ldg(a.counts + 2 * g + 1) : 0;
+        if (g * a.ntiles + nt != key) {
+            key = g * a.ntiles + nt;
+            asm volatile("bar.sync 1, %0;" ::"n"(kGcEpiWarps * 32) : "memory");  // the old tables are read
+            for (int i = et; i < cnt; i += kGcEpiWarps * 32) {
+                const int p = __ldg(a.colmap + g * a.cstride + nt * a.bn + i);
+                t_off[i] = p >= 0 ? p * a.plane : 0;
+                t_bias[i] = (p >= 0 && a.bias) ? __ldg(a.bias + p) : 0.0f;
+            }
+            for (int z = et; z < min(zc, kGcZcap); z += kGcEpiWarps * 32)
+                z_off[z] = __ldg(a.zmap + g * a.zstride + z) * a.plane;
+            asm volatile("bar.sync 1, %0;" ::"n"(kGcEpiWarps * 32) : "memory");
+        }
+        const int q = mt * (MT * 128) + (MT == 2 ? h * 128 : 0) + q4 * 32 + lane;
+        int n, t, hh, w;
+        grid_decode(a.gr, q, n, t, hh, w);
+        const bool valid = q < a.gr.L && t < a.VT && hh < a.VH && w < a.VW;
+        const long long pix =
+            valid ? (long long)n * a.planes * a.plane + (long long)t * a.VHW + (long long)hh * a.VW + w : 0;
+        float* yf = reinterpret_cast<float*>(a.out) + pix;
+        __nv_bfloat16* yh = reinterpret_cast<__nv_bfloat16*>(a.out) + pix;
+        const YCheck yc{pix, a.out_total, a.status};
+        // zero planes, while the item's MMAs run: 16 at a time, the table read
+        // four offsets to a load
+        if (alive && valid) {
+            const int zt = min(zc, kGcZcap) & ~15;
+            for (int z = MT == 2 ? 0 : 16 * h; z < zt; z += MT == 2 ? 16 : 32) {
+#pragma unroll
+                for (int j = 0; j < 16; j += 4) {
+                    const int4 o = *reinterpret_cast<const int4*>(z_off + z + j);
+                    zero_at<OUT_BF16>(yf, yh, yc, o.x);
+                    zero_at<OUT_BF16>(yf, yh, yc, o.y);
+                    zero_at<OUT_BF16>(yf, yh, yc, o.z);
+                    zero_at<OUT_BF16>(yf, yh, yc, o.w);
+                }
+            }
+            for (int z = zt + (MT == 2 ? 0 : h); z < zc; z += MT == 2 ? 1 : 2)
+                zero_at<OUT_BF16>(yf, yh, yc, z < kGcZcap ? z_off[z] : __ldg(a.zmap + g * a.zstride + z) * a.plane);
+        }
+        if (cnt <= 0) continue;
+        const int nch = (cnt + kEpiCols - 1) / kEpiCols;
+        const int nst = gc_blocks(a, g) * a.gr.KT;
+        float v[NCH][kEpiCols];
+#pragma unroll
+        for (int k = 0; k < NCH; ++k)
+#pragma unroll
+            for (int j = 0; j < kEpiCols; ++j) v[k][j] = 0.0f;
+        const int pieces = nst * a.ppst;
+        for (int pc = 0; alive && pc < pieces; pc += a.pps) {
+            // warp-uniform outcome: the TMEM loads below are .sync.aligned
+            if (!__all_sync(0xffffffffu, mbar_wait(&ep.acc_full[ab], acc_ph, ep.abort_flag, a.status))) {
+                alive = false;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t taddr = ep.tmem_base + (uint32_t)((ab * MT + (MT == 2 ? h : 0)) * a.tmem_stride) +
+                                   ((uint32_t)(q4 * 32) << 16);
+            if (NCH <= 4) {
+                uint32_t r[NCH][kEpiCols];
+#pragma unroll
+                for (int k = 0; k < NCH; ++k) {
+                    const int c = MT == 2 ? k : 2 * k + h;
+                    if (c < nch) tmem_ld_32x32b_x16(taddr + (uint32_t)(c * kEpiCols), r[k]);
+                }
+                tmem_ld_wait();
+                tc_fence_before();  // the buffer is free before the additions
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ep.acc_full[kGcMaxBuf + ab]);
+#pragma unroll
+                for (int k = 0; k < NCH; ++k) {
+                    if ((MT == 2 ? k : 2 * k + h) < nch) {
+#pragma unroll
+                        for (int j = 0; j < kEpiCols; ++j) v[k][j] += __uint_as_float(r[k][j]);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < NCH; ++k) {
+                    const int c = MT == 2 ? k : 2 * k + h;
+                    if (c < nch) {
+                        uint32_t r[kEpiCols];
+                        tmem_ld_32x32b_x16(taddr + (uint32_t)(c * kEpiCols), r);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int j = 0; j < kEpiCols; ++j) v[k][j] += __uint_as_float(r[j]);
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ep.acc_full[kGcMaxBuf + ab]);
+            }
+            if (++ab == a.nbuf) { ab = 0; acc_ph ^= 1u; }
+        }
+        uint32_t nan = 0;         // chunks with NaN columns
+        uint32_t nan_cols[NCH];     // theirs, 16 bits a chunk (in local memory: read by a runtime index)
+#pragma unroll
+        for (int k = 0; k < NCH; ++k) {
+            const int c = MT == 2 ? k : 2 * k + h;
+            if (alive && valid && c < nch) {
+                bool bad = false;
+#pragma unroll
+                for (int j = 0; j < kEpiCols; ++j) bad |= v[k][j] != v[k][j];
+                if (bad) {
+                    uint32_t m = 0;
+#pragma unroll
+                    for (int j = 0; j < kEpiCols; ++j) m |= (v[k][j] != v[k][j] ? 1u : 0u) << j;
+                    nan |= 1u << k;
+                    nan_cols[k] = m;
+                }
+                store_cols<OUT_BF16>(v[k], c * kEpiCols, cnt, t_off, t_bias, a.relu, yf, yh, yc);
+            }
+        }
+        // NaN columns: what a lane finds to be a kept term's stands, the others are
+        // summed again by the warp
+        if (__any_sync(0xffffffffu, nan != 0)) {
+            const int kch = a.kcounts ? __ldg(a.kcounts + 2 * g) : a.ncb * a.cb;
+            const uint4* wt = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(a.wd) +
+                                                             (size_t)(g * a.ntiles + nt) * a.ksteps * a.bn * 32);
+            const uint4* src = reinterpret_cast<const uint4*>(a.src + (size_t)g * a.gstride);
+            int4 first = make_int4(-1, -1, -1, -1);
+            if (nan) first = grid_scan(a, src, q, kch);
+#pragma unroll 1
+            for (int k = 0; k < NCH; ++k) {
+                const int c0 = (MT == 2 ? k : 2 * k + h) * kEpiCols;
+                uint32_t left = 0;
+                for (uint32_t bits = (nan >> k) & 1u ? nan_cols[k] : 0u; bits; bits &= bits - 1) {
+                    const int i = c0 + __ffs(bits) - 1;
+                    if (i < cnt && !grid_nan_at(a, wt, src, ep.bnr, i, q, kch, first)) left |= bits & (0u - bits);
+                }
+                __syncwarp();
+                for (uint32_t lanes = __ballot_sync(0xffffffffu, left != 0); lanes; lanes &= lanes - 1) {
+                    const int l = __ffs(lanes) - 1;
+                    const int ql = __shfl_sync(0xffffffffu, q, l);
+                    for (uint32_t bits = __shfl_sync(0xffffffffu, left, l); bits; bits &= bits - 1) {
+                        const int i = c0 + __ffs(bits) - 1;
+                        float e = grid_exact(a, wt, src, ep.bnr, i, ql, kch) + t_bias[i];
+                        if (lane != l || !y_ok(yc, t_off[i])) continue;
+                        if (a.relu) e = fmaxf(e, 0.0f);
+                        if (OUT_BF16)
+                            yh[t_off[i]] = __float2bfloat16_rn(e);
+                        else
+                            yf[t_off[i]] = e;
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// DX: the input gradient, whose sums may be cut.
+template <bool OUT_BF16, int MT, bool DX>
 __global__ void __launch_bounds__(kGcThreads, 1)
     k_grid_conv(const __grid_constant__ GcArgs a)
 {
@@ -492,7 +678,7 @@ __global__ void __launch_bounds__(kGcThreads, 1)
     if (mode == kResident) gc_issue<KW, H, MT, CUT>(a, p, kResident);         \
     else if (mode == kStageSlots) gc_issue<KW, H, MT, CUT>(a, p, kStageSlots); \
     else gc_issue<KW, H, MT, CUT>(a, p, kRowSlots);
-#define SADMM_ISSUE(KW, H) if (!OUT_BF16 && a.cut) { SADMM_MODES(KW, H, true) } else { SADMM_MODES(KW, H, false) }
+#define SADMM_ISSUE(KW, H) if (DX && a.cut) { SADMM_MODES(KW, H, true) } else { SADMM_MODES(KW, H, false) }
 #define SADMM_ROW(KW, H) if (row == KW * 8 + H) { SADMM_ISSUE(KW, H) } else
         SADMM_ROW(1, 1) SADMM_ROW(1, 2) SADMM_ROW(1, 3) SADMM_ROW(1, 4)
         SADMM_ROW(3, 1) SADMM_ROW(3, 2) SADMM_ROW(3, 3) SADMM_ROW(3, 4)
@@ -511,147 +697,11 @@ __global__ void __launch_bounds__(kGcThreads, 1)
         __syncwarp();
     } else {
         // --------------------------------------------------------- epilogue
-        // Two warps per TMEM lane quadrant: with one pixel tile they take its
-        // 16-column chunks in turn, with two a tile each.
-        const int q4 = warp & 3;
-        const int h = (warp - 3) >> 2;
-        const int et = threadIdx.x - 3 * 32;
-        int ab = 0, key = -1;
-        uint32_t acc_ph = 0;
-        bool alive = true;
-        for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
-            int g, nt, mt;
-            gc_unit(a, u, g, nt, mt);
-            const int cnt = min(a.bn, __ldg(a.counts + 2 * g) - nt * a.bn);
-            const int zc = nt == 0 ? __ldg(a.counts + 2 * g + 1) : 0;
-            if (g * a.ntiles + nt != key) {
-                key = g * a.ntiles + nt;
-                asm volatile("bar.sync 1, %0;" ::"n"(kGcEpiWarps * 32) : "memory");  // the old tables are read
-                for (int i = et; i < cnt; i += kGcEpiWarps * 32) {
-                    const int p = __ldg(a.colmap + g * a.cstride + nt * a.bn + i);
-                    t_off[i] = p >= 0 ? p * a.plane : 0;
-                    t_bias[i] = (p >= 0 && a.bias) ? __ldg(a.bias + p) : 0.0f;
-                }
-                for (int z = et; z < min(zc, kGcZcap); z += kGcEpiWarps * 32)
-                    z_off[z] = __ldg(a.zmap + g * a.zstride + z) * a.plane;
-                asm volatile("bar.sync 1, %0;" ::"n"(kGcEpiWarps * 32) : "memory");
-            }
-            const int q = mt * (MT * 128) + (MT == 2 ? h * 128 : 0) + q4 * 32 + lane;
-            int n, t, hh, w;
-            grid_decode(a.gr, q, n, t, hh, w);
-            const bool valid = q < a.gr.L && t < a.VT && hh < a.VH && w < a.VW;
-            const long long pix =
-                valid ? (long long)n * a.planes * a.plane + (long long)t * a.VHW + (long long)hh * a.VW + w : 0;
-            float* yf = reinterpret_cast<float*>(a.out) + pix;
-            __nv_bfloat16* yh = reinterpret_cast<__nv_bfloat16*>(a.out) + pix;
-            const YCheck yc{pix, a.out_total, a.status};
-            // zero planes, while the item's MMAs run: 16 at a time, the table read
-            // four offsets to a load
-            if (alive && valid) {
-                const int zt = min(zc, kGcZcap) & ~15;
-                for (int z = MT == 2 ? 0 : 16 * h; z < zt; z += MT == 2 ? 16 : 32) {
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4) {
-                        const int4 o = *reinterpret_cast<const int4*>(z_off + z + j);
-                        zero_at<OUT_BF16>(yf, yh, yc, o.x);
-                        zero_at<OUT_BF16>(yf, yh, yc, o.y);
-                        zero_at<OUT_BF16>(yf, yh, yc, o.z);
-                        zero_at<OUT_BF16>(yf, yh, yc, o.w);
-                    }
-                }
-                for (int z = zt + (MT == 2 ? 0 : h); z < zc; z += MT == 2 ? 1 : 2)
-                    zero_at<OUT_BF16>(yf, yh, yc, z < kGcZcap ? z_off[z] : __ldg(a.zmap + g * a.zstride + z) * a.plane);
-            }
-            if (cnt <= 0) continue;
-            const int nch = (cnt + kEpiCols - 1) / kEpiCols;
-            const int nst = gc_blocks(a, g) * a.gr.KT;
-            float v[8][kEpiCols];
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-#pragma unroll
-                for (int j = 0; j < kEpiCols; ++j) v[k][j] = 0.0f;
-            const int pieces = nst * a.ppst;
-            for (int pc = 0; alive && pc < pieces; pc += a.pps) {
-                // warp-uniform outcome: the TMEM loads below are .sync.aligned
-                if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[ab], acc_ph, abort_flag, a.status))) {
-                    alive = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t taddr = tmem_base + (uint32_t)((ab * MT + (MT == 2 ? h : 0)) * a.tmem_stride) +
-                                       ((uint32_t)(q4 * 32) << 16);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int c = MT == 2 ? k : 2 * k + h;
-                    if (c < nch) {
-                        uint32_t r[kEpiCols];
-                        tmem_ld_32x32b_x16(taddr + (uint32_t)(c * kEpiCols), r);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int j = 0; j < kEpiCols; ++j) v[k][j] += __uint_as_float(r[j]);
-                    }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&acc_empty[ab]);
-                if (++ab == a.nbuf) { ab = 0; acc_ph ^= 1u; }
-            }
-            uint32_t nan = 0;         // chunks with NaN columns
-            uint32_t nan_cols[8];     // theirs, 16 bits a chunk (in local memory: read by a runtime index)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int c = MT == 2 ? k : 2 * k + h;
-                if (alive && valid && c < nch) {
-                    bool bad = false;
-#pragma unroll
-                    for (int j = 0; j < kEpiCols; ++j) bad |= v[k][j] != v[k][j];
-                    if (bad) {
-                        uint32_t m = 0;
-#pragma unroll
-                        for (int j = 0; j < kEpiCols; ++j) m |= (v[k][j] != v[k][j] ? 1u : 0u) << j;
-                        nan |= 1u << k;
-                        nan_cols[k] = m;
-                    }
-                    store_cols<OUT_BF16>(v[k], c * kEpiCols, cnt, t_off, t_bias, a.relu, yf, yh, yc);
-                }
-            }
-            // NaN columns: what a lane finds to be a kept term's stands, the others are
-            // summed again by the warp
-            if (__any_sync(0xffffffffu, nan != 0)) {
-                const int kch = a.kcounts ? __ldg(a.kcounts + 2 * g) : a.ncb * a.cb;
-                const uint4* wt = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(a.wd) +
-                                                                 (size_t)(g * a.ntiles + nt) * btile);
-                const uint4* src = reinterpret_cast<const uint4*>(a.src + (size_t)g * a.gstride);
-                int4 first = make_int4(-1, -1, -1, -1);
-                if (nan) first = grid_scan(a, src, q, kch);
-#pragma unroll 1
-                for (int k = 0; k < 8; ++k) {
-                    const int c0 = (MT == 2 ? k : 2 * k + h) * kEpiCols;
-                    uint32_t left = 0;
-                    for (uint32_t bits = (nan >> k) & 1u ? nan_cols[k] : 0u; bits; bits &= bits - 1) {
-                        const int i = c0 + __ffs(bits) - 1;
-                        if (i < cnt && !grid_nan_at(a, wt, src, bnr, i, q, kch, first)) left |= bits & (0u - bits);
-                    }
-                    __syncwarp();
-                    for (uint32_t lanes = __ballot_sync(0xffffffffu, left != 0); lanes; lanes &= lanes - 1) {
-                        const int l = __ffs(lanes) - 1;
-                        const int ql = __shfl_sync(0xffffffffu, q, l);
-                        for (uint32_t bits = __shfl_sync(0xffffffffu, left, l); bits; bits &= bits - 1) {
-                            const int i = c0 + __ffs(bits) - 1;
-                            float e = grid_exact(a, wt, src, bnr, i, ql, kch) + t_bias[i];
-                            if (lane != l || !y_ok(yc, t_off[i])) continue;
-                            if (a.relu) e = fmaxf(e, 0.0f);
-                            if (OUT_BF16)
-                                yh[t_off[i]] = __float2bfloat16_rn(e);
-                            else
-                                yf[t_off[i]] = e;
-                        }
-                        __syncwarp();
-                    }
-                }
-            }
-            __syncwarp();
-        }
+        const GcEpi ep{acc_full, abort_flag, t_off, tmem_base, bnr};
+        if (DX && (a.bn / kEpiCols * MT + 1) / 2 <= 4)  // a warp's chunks
+            gc_epilogue<OUT_BF16, MT, 4>(a, ep);
+        else
+            gc_epilogue<OUT_BF16, MT, 8>(a, ep);
     }
     tc_fence_before();
     __syncthreads();
@@ -670,10 +720,10 @@ __global__ void __launch_bounds__(256) k_grid_x(const GridX a)
     grid_x_block(a, blockIdx.x, blockIdx.y, s_off);
 }
 
-template <bool OUT_BF16, int MT>
+template <bool OUT_BF16, int MT, bool DX>
 cudaError_t launch_gc(const GcArgs& a, int grid, size_t smem, cudaStream_t s)
 {
-    auto kern = k_grid_conv<OUT_BF16, MT>;
+    auto kern = k_grid_conv<OUT_BF16, MT, DX>;
     static int configured_dev = -1;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -809,7 +859,7 @@ sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const Gri
     a.h16 = sh.cb / 16;
     a.rsteps = gr.KW * a.h16;
     a.spt = gr.KH * a.rsteps;
-    a.cut = sh.cut && !c.out_bf16 && a.spt > sh.seg ? 1 : 0;  // (the input gradient's: its output is fp32)
+    a.cut = sh.cut && c.src_dz && a.spt > sh.seg ? 1 : 0;
     a.psteps = unrolled_row(gr.KW, a.h16) ? a.rsteps : std::min(a.rsteps, sh.seg);
     a.pps = std::max(1, sh.seg / (a.cut ? a.psteps : a.spt));
     a.ppst = a.cut ? gr.KH * ((a.rsteps + a.psteps - 1) / a.psteps) : 1;
@@ -826,10 +876,12 @@ sadmm_status launch_grid_conv(const Grid& gr, const GridConvShape& sh, const Gri
     long long grid = c.ctas > 0 ? c.ctas : device_sm_count();
     if (grid > units) grid = units;
     cudaError_t e;
-    if (sh.mt == 2)
-        e = c.out_bf16 ? launch_gc<true, 2>(a, (int)grid, sh.smem, s) : launch_gc<false, 2>(a, (int)grid, sh.smem, s);
+    if (c.src_dz)  // (its output is fp32)
+        e = sh.mt == 2 ? launch_gc<false, 2, true>(a, (int)grid, sh.smem, s) : launch_gc<false, 1, true>(a, (int)grid, sh.smem, s);
+    else if (sh.mt == 2)
+        e = c.out_bf16 ? launch_gc<true, 2, false>(a, (int)grid, sh.smem, s) : launch_gc<false, 2, false>(a, (int)grid, sh.smem, s);
     else
-        e = c.out_bf16 ? launch_gc<true, 1>(a, (int)grid, sh.smem, s) : launch_gc<false, 1>(a, (int)grid, sh.smem, s);
+        e = c.out_bf16 ? launch_gc<true, 1, false>(a, (int)grid, sh.smem, s) : launch_gc<false, 1, false>(a, (int)grid, sh.smem, s);
     return e == cudaSuccess ? SADMM_OK : SADMM_ECUDA;
 }
 
